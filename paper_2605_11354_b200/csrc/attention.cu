@@ -3,31 +3,40 @@
 //
 // One CTA owns 128 query rows of one (b, h): at block 64 a PAIR of query blocks (two M=64 problems interleaved in the
 // two 16-lane halves of every TMEM sub-partition, each with its own list of critical key blocks), at block 128 one
-// query block (M=128).  Work advances in steps of 64 keys.  Per step t (w = t & 1):
-//   TMA      K tile(s) (e4m3, 64-byte rows, 64B swizzle) and V tile(s) (dequantised fp16, 128B swizzle) -> rings of four
-//   tcgen05  S[w] = Q K^T          kind::f8f6f4, fp32 accumulators in TMEM (64 columns, two buffers)
-//   softmax  warpgroup w, one thread per query row (TMEM lane = thread): the 64 scores are read once into registers,
-//            row maximum, lazy rescale, exp2, row sum; the probabilities go back to TMEM as packed fp16 (P[w], 32 columns)
-//   tcgen05  O += P[w] V           kind::f16 with the A operand read from TMEM, V as MN-major B operand from shared
-//                                  memory, ONE fp32 accumulator in TMEM (64 columns) for all steps
-// The two softmax warpgroups take the even and the odd steps.  Each owns a score buffer and a probability buffer, so
-// Q K^T of step t+2 is issued as soon as warpgroup w has read S[w], and P V of step t runs under the exponentials of
-// the following steps: the softmax threads do not wait for a product in the steady state, and with two CTAs per SM every
-// SM sub-partition holds four softmax warps in different phases, which is what keeps the exponential unit fed.
-// Both warpgroups accumulate into the same O, so they share one reference maximum per row: the thread that handles
-// step t reads the reference left by step t-1 from a shared-memory slot (written early in that step, right after its
-// row maximum is known), applies the lazy-rescale rule and publishes the reference of step t.  Row sums are kept
-// per warpgroup, brought to the final reference and added in the epilogue.
+// query block (M=128).  Work advances in steps of 64 keys.  Per step t:
+//   TMA      K tile(s) (e4m3, 64-byte rows, 64B swizzle) and V tile(s) (dequantised fp16, 128B swizzle) -> rings of two
+//   tcgen05  S = Q K^T             kind::f8f6f4, fp32 accumulators in TMEM (64 columns)
+//   softmax  one thread per query row (TMEM lane = thread): the 64 scores are read into registers and S is released at
+//            once (Q K^T of step t+1 runs under the exponentials of step t); exp2, row sum; the probabilities go back
+//            to TMEM as packed fp16 (P, 32 columns)
+//   tcgen05  O += P V              kind::f16 with the A operand read from TMEM, V as MN-major B operand from shared
+//                                  memory, one fp32 accumulator in TMEM (64 columns), under the exponentials of step t+1
+// so the softmax warps never wait for a product in the steady state.  The exponential unit is the bound (16 per clock
+// and SM: 512 clocks per step); the products of a step take 384 clocks of tensor pipe at block 64 (M = 64 runs at half
+// rate) and 192 at block 128.  A warp alone needs some 1100 clocks for its 32 x 64 scores (loads, stores and barriers
+// included), so two warps per scheduler are the least that can keep the unit busy and three do it comfortably: S, P and O
+// take 160 TMEM columns (an allocation of 128 and one of 32), 74 KB of shared memory and 80 registers per thread, and
+// THREE CTAs fit on an SM.  Measured at 10 % of 2147 key blocks: 650 clocks per step and SM (two CTAs with two softmax
+// warpgroups each on alternate steps of one tile, as before: 757).
+// A CTA takes tile after tile: it asks the hardware's work scheduler for a CTA that has not been launched yet and computes
+// that one's tile itself (taken only where the grid is larger than the chip holds).  The next tile's Q, K and V tiles and
+// its first scores are then under way while the softmax warps write this tile's output, and what lies between two tiles
+// of a CTA (5.5 k clocks of 13 k: launch, barriers, TMEM allocation, first loads) is paid once.  Barriers are never
+// re-initialised: rings and parities run on a count through all tiles.
+// The code (48 KB) is kept below the instruction cache's limit (at 62 KB the same kernel is 8 % slower): waits with their
+// rare part out of line, loops not unrolled, warp-uniform values made known to the compiler.
 // P is carried in fp16 (not e4m3): one e4m3 term has a 2.6 % rounding error per probability, which alone is ten
 // times the output tolerance.  V travels as the dequantised value in fp16 (2^-12 relative rounding).
 // Tail: phi(Q) (bf16) times the aggregated, projected summaries G_i (bf16) as one more MMA, divided by
-// phi(Q) . zeta_i, added to the normalised softmax output and stored (each warpgroup handles 32 of the 64 columns).
+// phi(Q) . zeta_i, added to the normalised softmax output and stored.
 //
-// Warp roles (384 threads): warp 0 = TMA producer, warp 1 = Q K^T issuer, warp 2 = P V issuer (one thread each; all
-// their waits block on mbarriers, nothing polls), warp 3 idle, warps 4-7 / 8-11 = softmax warpgroups 0 / 1.  The
-// control warps give registers back (setmaxnreg) so that a softmax thread can hold a whole row of scores.
+// Warp roles (256 threads): warp 0 = TMA producer, warp 1 = Q K^T issuer, warp 2 = P V issuer (and the linear product)
+// (all lanes run the loops, one elected lane issues; all waits block on mbarriers in the order in which the events
+// occur), warp 3 idle, warps 4-7 = softmax.  The control warps give registers back (setmaxnreg) so that a softmax
+// thread can hold a whole row of scores next to its probabilities.
 // Every wait is bounded (1 s); on expiry the CTA sets *device_status and all roles leave their loops.
 #include <atomic>
+#include <type_traits>
 #include <utility>
 
 #include "common.cuh"
@@ -39,50 +48,47 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kStages = 4;   // K ring; also the number of P V completion barriers (step t uses number t % 4)
-constexpr int kVStages = 3;  // V ring
-constexpr int kSetThreads = 128;                 // one softmax warpgroup
-constexpr int kSoftmaxThreads = 2 * kSetThreads;
 constexpr int kCtrlWarps = 4;
-constexpr int kThreads = kCtrlWarps * 32 + kSoftmaxThreads;
-constexpr int kCtrlRegs = 32, kSoftmaxRegs = 104;  // 128 * 32 + 256 * 104 = 384 * 80, the launch allocation
-constexpr uint32_t kBackoffNs = 64;  // sleep between polls of the single-thread roles
+constexpr int kSoftmaxWarps = 4;
+constexpr int kThreads = (kCtrlWarps + kSoftmaxWarps) * 32;
+constexpr int kCtasPerSm = 3;
+constexpr int kCtrlRegs = 48, kSoftmaxRegs = 112;  // 128 * 48 + 128 * 112 = 256 * 80, the launch allocation
 constexpr int kStepKeys = 64;
-constexpr uint32_t kTmemCols = 256;
-// TMEM columns: S buffers at 0 and 64, O at 128, P buffers (packed fp16, 32 columns each) at 192 and 224; the linear
-// branch's product reuses S buffer 0.
-constexpr uint32_t kColS = 0, kColO = 128, kColP = 192, kColL = 0;
+constexpr int kStages = 2;  // K ring and V ring
+// TMEM: 64 columns of scores (later the product of the linear branch) and 64 of O in one allocation, 32 columns of
+// probabilities (packed fp16) in another.
+constexpr uint32_t kColsSO = 128, kColsP = 32, kColO = 64;
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kRescaleThreshold = 8.0f;  // lazy rescale: keep the old reference max until it is beaten by 2^8
-constexpr float kNoMax = -1.0e30f;         // reference maximum of a row that has seen no valid key yet
+constexpr float kRescaleThreshold = 8.0f;  // lazy rescale: keep the old reference until it is beaten by 2^8
+constexpr float kNoMax = -1.0e30f;    // reference maximum of a row that has seen no valid key yet
+constexpr int kScalSlots = 4;
 
-// shared-memory map (bytes from a 1024-aligned base)
-constexpr uint32_t kQBytes = 8192, kKStage = 8192, kVStage = 16384;
-constexpr uint32_t kOffQ = 0;
-constexpr uint32_t kOffK = kOffQ + kQBytes;
-constexpr uint32_t kOffV = kOffK + kStages * kKStage;
-constexpr uint32_t kOffPhi = kOffV + kVStages * kVStage;  // phi(Q) as bf16 A operand of the linear product (16 KB)
-constexpr uint32_t kOffZeta = kOffPhi + 16384;            // zeta_i of the linear branch (256 B per query block)
-constexpr uint32_t kOffRef = kOffZeta + 512;              // per row: {reference maximum, number of steps published}
-constexpr uint32_t kOffX = kOffRef + 1024;                // epilogue exchange between the warpgroups (2 x 128 x 8 B)
-constexpr uint32_t kOffScal = kOffX + 2048;               // per step and query block: {exponent factor, valid keys}, ring of 8
-constexpr uint32_t kOffBar = kOffScal + 128;
-constexpr uint32_t kSmemBytes = kOffBar + 512;  // two CTAs per SM: 2 * (110592 + 1024 reserved) <= 232448
-// after the main loop the rings are reused: aggregated summaries G_i in K stages 0-1 (16 KB), the output rows in the
-// V ring (32 KB)
-constexpr uint32_t kOffG = kOffK;
-constexpr uint32_t kOffOut = kOffV;
+// shared-memory map (bytes from a 1024-aligned base); a step's tiles take half a stage at block 128 (one key block's)
+constexpr uint32_t kStageK = 8192, kStageV = 16384;
+constexpr uint32_t kOffQ = 0;                           // 8 KB
+constexpr uint32_t kOffK = kOffQ + 8192;
+constexpr uint32_t kOffV = kOffK + kStages * kStageK;
+constexpr uint32_t kOffPhi = kOffV + kStages * kStageV;  // phi(Q) as bf16 A operand of the linear product (16 KB); after
+                                                         // that product the output rows, each warp in its own rows' place
+constexpr uint32_t kOffZeta = kOffPhi + 16384;           // zeta_i of the linear branch (256 B per query block), two tiles
+constexpr uint32_t kOffScal = kOffZeta + 1024;           // per step and query block: {exponent factor, valid keys}
+constexpr uint32_t kOffNext = kOffScal + kScalSlots * 16;  // answer of the work scheduler (16 B), tile numbers (4 x 4 B)
+constexpr uint32_t kOffBar = kOffNext + 32;
+constexpr uint32_t kSmemBytes = kOffBar + 256;           // three CTAs per SM: 3 * (75104 + 1024 reserved) <= 233472
+constexpr int kTileSlots = 4;
 
 struct Bars {
-  uint64_t q_full, z_full, g_full, phi_full, l_full, x_full;
-  uint64_t k_full[kStages], v_full[kVStages];  // TMA -> issuer
-  uint64_t k_free[kStages];                   // Q K^T of the step in this stage complete -> producer
-  uint64_t pv_done[kStages];                  // P V of step t (number t % 4) complete -> producer, softmax
-  uint64_t qk_done[2];                        // S buffer written -> softmax
-  uint64_t s_empty[2], p_full[2];             // softmax -> issuer
-  uint32_t tmem_base;
+  uint64_t q_full, phi_full, next_full;
+  uint64_t tile_full[kTileSlots];             // tile number of the CTA's next tile known
+  uint64_t k_full[kStages], v_full[kStages];  // TMA -> issuer
+  uint64_t s_full[kStages];                   // Q K^T number n complete (n % 2) -> softmax, producer (K stage free)
+  uint64_t v_done[kStages];                   // product number n of the V ring complete (n % 2) -> softmax (P free, O or
+                                              // the linear product valid), producer (V stage free)
+  uint64_t s_free, p_full;                    // softmax -> issuers: score columns read / probabilities stored
+  uint32_t tmem_so, tmem_p;
   int abort;
 };
+static_assert(sizeof(Bars) <= 256, "barrier block");
 
 struct AttnParams {
   const float* q_scales;
@@ -91,9 +97,10 @@ struct AttnParams {
   const float* zeta;    // [B*H*Nb][64]
   void* out;
   long long out_stride_b, out_stride_h, out_stride_n;
-  int heads, tokens, nb, k_crit, k_marg, phi, out_dtype;
+  int heads, tokens, nb, tiles_per_head, k_crit, k_marg, phi, out_dtype;
   // output through TMA stores (map_o): position of the token / head / batch dimension among the map's dimensions
   // 1..3 (they are ordered by stride); tma_out = 0: plain stores
+  int steal;  // more tiles than CTAs fit on the chip: CTAs take over the tiles of CTAs not yet launched
   int tma_out, dim_token, dim_head, dim_batch;
   int* status;
 };
@@ -121,9 +128,6 @@ __device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uin
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-
-// One aligned 8-byte word of shared memory, read / written by a single instruction that the compiler may neither
-// drop nor reorder against other volatile accesses.
 __device__ __forceinline__ uint2 lds_volatile_v2(uint32_t addr) {
   uint2 v;
   asm volatile("ld.volatile.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
@@ -132,25 +136,22 @@ __device__ __forceinline__ uint2 lds_volatile_v2(uint32_t addr) {
 __device__ __forceinline__ void sts_volatile_v2(uint32_t addr, uint32_t x, uint32_t y) {
   asm volatile("st.volatile.shared.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(x), "r"(y) : "memory");
 }
-
-// Polls a row's reference slot until `count` steps have been published (bounded like every other wait).
-static __device__ __noinline__ bool reference_wait_slow(uint32_t slot, int count, uint2& v, volatile int* abort_flag, int* status) {
-  const uint64_t t0 = global_timer_ns();
-  uint32_t polls = 0;
-  while (true) {
-    v = lds_volatile_v2(slot);
-    if (static_cast<int>(v.y) == count) return true;
-    if ((++polls & 0x3Fu) == 0) {
-      if (*abort_flag != 0) return false;
-      if (global_timer_ns() - t0 > kWaitLimitNs) {
-        *abort_flag = 309;
-        if (status != nullptr) atomicCAS(status, 0, 309);
-        return false;
-      }
-    }
-  }
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
 }
-// Scales the 64 accumulator columns of this thread's TMEM lane by alpha (lazy rescale of O; rare).
+__device__ __forceinline__ void sts128(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+// Hides where a value comes from: what is derived from it is then computed where it is used instead of being kept in
+// registers (dozens of them) around the loop over the tiles.
+__device__ __forceinline__ void opaque(uint32_t& v) { asm volatile("" : "+r"(v)); }
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+
+// Scales the 64 accumulator columns of this thread's TMEM lane by alpha (rare).
 static __device__ __noinline__ void rescale_accumulator(uint32_t o_addr, float alpha) {
 #pragma unroll 1
   for (int part = 0; part < 4; ++part) {
@@ -161,28 +162,76 @@ static __device__ __noinline__ void rescale_accumulator(uint32_t o_addr, float a
     for (int k = 0; k < 16; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * alpha);
     tmem_st16(o_addr + part * 16, o);
   }
+  tmem_wait_st();
 }
 
-// exp2 of 32 scaled scores, packed to fp16 pairs; returns the sum.  Arguments and sums run on pairs of columns
-// (packed fp32x2 fma / add).
-__device__ __forceinline__ float exp_half_row(const uint32_t (&x)[32], float c, float neg_ref, uint32_t* packed) {
-  const uint64_t c2 = pack_f32x2(c, c), shift2 = pack_f32x2(neg_ref, neg_ref);
-  uint64_t sum2[2] = {0ull, 0ull};  // bit pattern of (0.f, 0.f)
+// 2^a for a pair of arguments on the fused-multiply-add units: a = n + f with n = round(a) (adding 1.5 * 2^23 leaves n in
+// the low mantissa bits) and |f| <= 1/2, 2^f by a degree-5 polynomial (minimax in the relative error by a Remez
+// exchange; 2.1e-7 in fp32 arithmetic over all of [-1/2, 1/2], the size of the hardware approximation's own error),
+// n added to the exponent field.  Arguments are at most the rescale threshold; from below they are clamped to stay inside
+// the exponent range (a value that small is zero as a probability).
+__device__ __forceinline__ void exp2_pair_fma(uint64_t a2, float& p0, float& p1) {
+  float a0, a1;
+  unpack_f32x2(a2, a0, a1);
+  a2 = pack_f32x2(fmaxf(a0, -125.f), fmaxf(a1, -125.f));
+  auto both = [](float v) { return pack_f32x2(v, v); };
+  const uint64_t t2 = add_f32x2(a2, both(12582912.f));
+  const uint64_t f2 = fma_f32x2(add_f32x2(t2, both(-12582912.f)), both(-1.f), a2);
+  uint64_t q = fma_f32x2(both(0.0013276472454890609f), f2, both(0.009675540961325169f));
+  q = fma_f32x2(q, f2, both(0.05550713092088699f));
+  q = fma_f32x2(q, f2, both(0.24022120237350464f));
+  q = fma_f32x2(q, f2, both(0.6931469440460205f));
+  q = fma_f32x2(q, f2, both(1.0000001192092896f));
+  float t0, t1, q0, q1;
+  unpack_f32x2(t2, t0, t1);
+  unpack_f32x2(q, q0, q1);
+  p0 = __uint_as_float(__float_as_uint(q0) + (__float_as_uint(t0) << 23));
+  p1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(t1) << 23));
+}
+
+// exp2 of 32 scaled scores, packed to fp16 pairs; adds them to two running pairs of sums.  Arguments and sums run on
+// pairs of columns (packed fp32x2 fma / add).  Every eighth pair goes to the multiply-add units (2 % faster at 16 heads of
+// 10992 tokens and 1 % at 137400 than none; every fourth costs more instructions than it saves and is slower than none).
+__device__ __forceinline__ void exp_half_row(const uint32_t (&x)[32], uint64_t c2, uint64_t shift2, uint32_t* packed,
+                                             uint64_t (&sum2)[2]) {
 #pragma unroll
   for (int k = 0; k < 32; k += 2) {
-    float a0, a1;
-    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(x[k]), __uint_as_float(x[k + 1])), c2, shift2), a0, a1);
-    const float p0 = ex2(a0), p1 = ex2(a1);
+    const uint64_t a2 = fma_f32x2(pack_f32x2(__uint_as_float(x[k]), __uint_as_float(x[k + 1])), c2, shift2);
+    float p0, p1;
+    if (((k >> 1) & 7) == 7) {
+      exp2_pair_fma(a2, p0, p1);
+    } else {
+      float a0, a1;
+      unpack_f32x2(a2, a0, a1);
+      p0 = ex2(a0);
+      p1 = ex2(a1);
+    }
     sum2[(k >> 1) & 1] = add_f32x2(sum2[(k >> 1) & 1], pack_f32x2(p0, p1));
     packed[k >> 1] = pack_half2(p0, p1);
   }
-  float s0, s1;
-  unpack_f32x2(add_f32x2(sum2[0], sum2[1]), s0, s1);
-  return s0 + s1;
+}
+
+// Work stealing: asks for the cancellation of a CTA of this grid that has not been launched yet (the answer arrives in
+// shared memory and is counted on `bar`); taken_cta returns the number of the cancelled CTA, whose tile the asking CTA then
+// computes itself, or -1 when none was left.
+__device__ __forceinline__ void request_next_cta(uint32_t answer, uint64_t* bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+               ::"r"(answer), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ int taken_cta(uint32_t answer) {
+  uint32_t x, ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+      "ld.shared.b128 r, [%2];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+      "selp.u32 %1, 1, 0, p;\n\tmov.u32 %0, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, r;\n\t}"
+      : "=r"(x), "=r"(ok) : "r"(answer) : "memory");
+  return ok != 0 ? static_cast<int>(x) : -1;
 }
 
 template <int BS>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_g,
                  const __grid_constant__ CUtensorMap map_o, const AttnParams p) {
@@ -190,7 +239,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr int kHalves = kPair ? 2 : 1;             // independent M=64 problems per CTA
   constexpr int kStepsPerBlock = BS / kStepKeys;     // 1 or 2
   constexpr int kM = kPair ? 64 : 128;
-  constexpr uint32_t kKTx = kHalves * 4096, kVTx = kHalves * 8192;
+  constexpr uint32_t kTxK = kHalves * 4096, kTxV = kHalves * 8192;  // bytes of a step's tiles
 
   extern __shared__ __align__(1024) uint8_t smem[];
   Bars* bars = reinterpret_cast<Bars*>(smem + kOffBar);
@@ -201,264 +250,280 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     return;
   }
 
-  // A wait that expired in an earlier CTA of this launch stops the rest of the grid before it touches anything.
-  if (p.status != nullptr && *reinterpret_cast<volatile int*>(p.status) != 0) return;
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tiles_per_head = kPair ? (p.nb + 1) / 2 : p.nb;
-  const int bh = blockIdx.x / tiles_per_head;
-  const int tile = blockIdx.x % tiles_per_head;
-  const int i_q[2] = {kPair ? 2 * tile : tile, kPair ? min(2 * tile + 1, p.nb - 1) : tile};
-  const size_t bh_rows = static_cast<size_t>(bh) * p.nb;
+  // (a shuffle from lane 0 tells the compiler that a value is the same in all lanes)
+  const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int steps = p.k_crit * kStepsPerBlock;
+  const int v_steps = steps + (p.k_marg > 0 ? 1 : 0);  // V-ring entries of a tile: the steps' V tiles, then G
+  // a tile's (b, h) and its query blocks (the second of an odd pair is a copy that is not stored)
+  struct Tile {
+    int bh, i_q[2];
+  };
+  auto tile_at = [&](int id) {
+    Tile t;
+    t.bh = id / p.tiles_per_head;
+    const int i = id - t.bh * p.tiles_per_head;
+    t.i_q[0] = kPair ? 2 * i : i;
+    t.i_q[1] = kPair ? min(2 * i + 1, p.nb - 1) : i;
+    return t;
+  };
 
   if (threadIdx.x == 0) {
     mbar_init(&bars->q_full, 1);
-    mbar_init(&bars->z_full, 1);
-    mbar_init(&bars->x_full, kSoftmaxThreads);
-    mbar_init(&bars->g_full, 1);
-    mbar_init(&bars->phi_full, kSoftmaxThreads);
-    mbar_init(&bars->l_full, 1);
-    for (int s = 0; s < kVStages; ++s) mbar_init(&bars->v_full[s], 1);
+    mbar_init(&bars->phi_full, kSoftmaxWarps);
+    mbar_init(&bars->next_full, 1);
+    mbar_init(&bars->s_free, kSoftmaxWarps);
+    mbar_init(&bars->p_full, kSoftmaxWarps);
+    for (int s = 0; s < kTileSlots; ++s) mbar_init(&bars->tile_full[s], 1);
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&bars->k_full[s], 1);
-      mbar_init(&bars->k_free[s], 1);
-      mbar_init(&bars->pv_done[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&bars->qk_done[b], 1);
-      mbar_init(&bars->s_empty[b], kSetThreads);
-      mbar_init(&bars->p_full[b], kSetThreads);
+      mbar_init(&bars->v_full[s], 1);
+      mbar_init(&bars->s_full[s], 1);
+      mbar_init(&bars->v_done[s], 1);
     }
     bars->abort = 0;
     mbar_fence_init();
   }
   if (warp == 1) {
-    tmem_alloc(&bars->tmem_base, kTmemCols);
+    tmem_alloc(&bars->tmem_so, kColsSO);
+    tmem_alloc(&bars->tmem_p, kColsP);
     tmem_relinquish();
   }
-  if (threadIdx.x >= kCtrlWarps * 32 && threadIdx.x < kCtrlWarps * 32 + 128)
-    reinterpret_cast<uint2*>(smem + kOffRef)[threadIdx.x - kCtrlWarps * 32] = make_uint2(__float_as_uint(kNoMax), 0u);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = bars->tmem_base;
+  const uint32_t tmem_so = __shfl_sync(0xFFFFFFFFu, bars->tmem_so, 0), tmem_p = __shfl_sync(0xFFFFFFFFu, bars->tmem_p, 0);
+  volatile int* const tile_ids = reinterpret_cast<volatile int*>(smem + kOffNext + 16);
+  // number of the CTA's tile after `it` tiles (-1: none is left, -2: a wait has expired), from the producer
+  auto next_tile = [&](int it, int code, auto role) {
+    if (!mbar_wait_far<decltype(role)::value>(&bars->tile_full[it % kTileSlots], (it / kTileSlots) & 1, abort_flag, p.status, code)) return -2;
+    return __shfl_sync(0xFFFFFFFFu, tile_ids[it % kTileSlots], 0);
+  };
   // each branch below starts by giving registers back (control warps) or taking them (softmax warps)
 
   if (warp < kCtrlWarps) {
   setmaxnreg_dec<kCtrlRegs>();
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer
-    // All 32 lanes run the loops and the waits, so that control flow, step counters and addresses are the same in every
+    // All 32 lanes run the loop and the waits, so that control flow, step counters and addresses are the same in every
     // lane (the compiler can then keep them in the warp's uniform registers, which is where TMA and tcgen05
     // instructions take their operands from); one elected lane issues.
-    {
-      const bool leader = elect_one();
-      if (leader) {
-        tma_prefetch_desc(&map_q);
-        tma_prefetch_desc(&map_k);
-        tma_prefetch_desc(&map_v);
-        mbar_arrive_expect_tx(&bars->q_full, kQBytes);
-        if (kPair) {
-          tma_load_2d(smem + kOffQ, &map_q, &bars->q_full, 0, static_cast<int>((bh_rows + i_q[0]) * 64));
-          tma_load_2d(smem + kOffQ + 4096, &map_q, &bars->q_full, 0, static_cast<int>((bh_rows + i_q[1]) * 64));
-        } else {
-          tma_load_2d(smem + kOffQ, &map_q, &bars->q_full, 0, static_cast<int>((bh_rows + i_q[0]) * 128));
-          tma_load_2d(smem + kOffQ + 4096, &map_q, &bars->q_full, 0, static_cast<int>((bh_rows + i_q[0]) * 128 + 64));
-        }
-      }
-      const float sq0 = __ldg(p.q_scales + bh_rows + i_q[0]) * (kLog2e * 0.125f);
-      const float sq1 = __ldg(p.q_scales + bh_rows + i_q[1]) * (kLog2e * 0.125f);
-      // Key blocks and their scales are fetched 32 steps at a time, lane l holding those of step 32 c + l, and handed
-      // to the issuing lane by a shuffle: no global load (let alone two dependent ones) sits in the per-step path.
-      int jl[2] = {0, 0};
-      float sl[2] = {0.f, 0.f};
-      auto refill = [&](int first) {
-        const int tt = first + lane;
-        if (tt < steps) {
-          for (int hf = 0; hf < kHalves; ++hf) {
-            jl[hf] = ldg_pinned(p.crit_idx + (bh_rows + i_q[hf]) * p.k_crit + (kPair ? tt : tt / 2));
-            sl[hf] = ldg_pinned(p.k_scales + bh_rows + jl[hf]);
-          }
-        }
-      };
+    const bool leader = elect_one();
+    const uint32_t answer = smem_u32(smem + kOffNext);
+    // Key blocks and their scales are fetched 32 steps at a time, lane l holding those of step 32 c + l, and handed
+    // to the issuing lane by a shuffle: no global load sits in the per-step path.
+    int jl[2] = {0, 0};
+    float sl[2] = {0.f, 0.f};
+    float sq[2] = {0.f, 0.f};
+    // The K cursor runs one step ahead of the V cursor (Q K^T of step t+1 is issued under the exponentials of step t, before
+    // P V of step t): the events the two wait for alternate in time in exactly this order, so blocking waits lose nothing.
+    bool ok = true;
+    int kc = 0, vc = 0;  // ring entries so far, through all tiles
+    auto wait_all = [&](uint64_t* bar, uint32_t parity, int code) {
+      return __all_sync(0xFFFFFFFFu, mbar_wait_far<1>(bar, parity, abort_flag, p.status, code));
+    };
+    auto wait_v_stage = [&]() {
+      return vc < kStages || wait_all(&bars->v_done[vc % kStages], (vc / kStages - 1) & 1, 102);
+    };
+    int id = blockIdx.x;
+#pragma unroll 1
+    for (int it = 0; id >= 0; ++it) {
+      const Tile tile = tile_at(id);
+      const size_t bh_rows = static_cast<size_t>(tile.bh) * p.nb;
       // tile row (in the code tensors) of a step in key block j
       auto tile_row = [&](int t, int j) {
         if (kPair) return static_cast<int>((bh_rows + j) * 64);
         return static_cast<int>((bh_rows + j) * 128 + (t & 1) * 64);
       };
-      // The K cursor runs one step ahead of the V cursor (a K stage is free after the Q K^T of four steps earlier,
-      // a V stage only after the P V of three steps earlier, and Q K^T of step t is issued before P V of step t-1).
-      // The events the two cursors wait for alternate in time in exactly this order, so blocking waits lose nothing.
-      // Together with the K tile of a step the producer leaves the step's scalars for the softmax threads: the
-      // factor that turns a raw score into a base-2 exponent and the number of valid keys (ring of eight: the slot of
-      // step t is rewritten for step t+8, when the softmax threads of step t+2 have long released the scores, which
-      // they read after the scalars).
-      bool ok = true;
-      int sv = 0;              // V stage of the V cursor's step (tv % 3)
-      int jv[2] = {0, 0};      // key blocks of the V cursor's step (those of the K cursor one iteration earlier)
-      for (int i = 0; ok && i <= steps; ++i) {
-        const int tk = i, tv = i - 1;
+      if (leader && p.steal) {
+        mbar_arrive_expect_tx(&bars->next_full, 16);
+        request_next_cta(answer, &bars->next_full);
+      }
+      if (it > 0) {  // the previous tile's last Q K^T and phi(Q) have read the Q tile
+        if (steps > 0) ok = wait_all(&bars->s_full[(kc - 1) % kStages], ((kc - 1) / kStages) & 1, 104);
+        if (p.k_marg > 0) ok = ok && wait_all(&bars->phi_full, (it - 1) & 1, 105);
+        if (!ok) break;
+      }
+      if (leader) {
+        mbar_arrive_expect_tx(&bars->q_full, 8192);
+        for (int x = 0; x < 2; ++x)
+          tma_load_2d(smem + kOffQ + x * 4096, &map_q, &bars->q_full, 0,
+                      static_cast<int>(kPair ? (bh_rows + tile.i_q[x]) * 64 : (bh_rows + tile.i_q[0]) * 128 + x * 64));
+      }
+      int jv[2] = {0, 0};  // key blocks of the V cursor's step
+#pragma unroll 1
+      for (int t = 0; t <= steps; ++t) {
         int jk[2] = {0, 0};
-        if (tk < steps) {
-          if ((tk & 31) == 0) refill(tk);
-          float sk[2];
+        if (t < steps) {
+          const bool refill = (t & 31) == 0;
+          if (refill) {
+            const int tt = min(t + lane, steps - 1);
+            for (int hf = 0; hf < kHalves; ++hf)
+              jl[hf] = ldg_pinned(p.crit_idx + (bh_rows + tile.i_q[hf]) * p.k_crit + (kPair ? tt : tt / 2));
+          }
+          const int st = kc % kStages;
+          if (kc >= kStages) ok = wait_all(&bars->s_full[st], (kc / kStages - 1) & 1, 101);
+          if (!ok) break;
+          for (int hf = 0; hf < kHalves; ++hf) jk[hf] = __shfl_sync(0xFFFFFFFFu, jl[hf], t & 31);
+          if (leader) {
+            mbar_expect_tx(&bars->k_full[st], kTxK);
+            for (int hf = 0; hf < kHalves; ++hf)
+              tma_load_2d(smem + kOffK + st * kStageK + hf * 4096, &map_k, &bars->k_full[st], 0, tile_row(t, jk[hf]));
+          }
+          // The step's scalars for the softmax threads, on their way while the tiles travel: the factor that turns a raw
+          // score into a base-2 exponent and the number of valid keys.  The slot of entry n is rewritten for entry n + 4,
+          // when Q K^T of entry n + 2 has completed and with it the softmax threads' reads of entry n.
+          if (refill) {
+            for (int hf = 0; hf < kHalves; ++hf) sl[hf] = ldg_pinned(p.k_scales + bh_rows + jl[hf]);
+            if (t == 0)
+              for (int hf = 0; hf < kHalves; ++hf) sq[hf] = ldg_pinned(p.q_scales + bh_rows + tile.i_q[hf]) * (kLog2e * 0.125f);
+          }
           for (int hf = 0; hf < kHalves; ++hf) {
-            jk[hf] = __shfl_sync(0xFFFFFFFFu, jl[hf], tk & 31);
-            sk[hf] = __shfl_sync(0xFFFFFFFFu, sl[hf], tk & 31);
+            const float skf = __shfl_sync(0xFFFFFFFFu, sl[hf], t & 31);
+            int valid = p.tokens - jk[hf] * BS - (kPair ? 0 : (t & 1) * kStepKeys);
+            valid = max(0, min(kStepKeys, valid));
+            if (leader)
+              sts_volatile_v2(smem_u32(smem + kOffScal) + (kc % kScalSlots) * 16 + hf * 8, __float_as_uint(sq[hf] * skf),
+                              static_cast<uint32_t>(valid));
           }
-          const int st = tk % kStages;
-          if (tk >= kStages)
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&bars->k_free[st], ((tk - kStages) / kStages) & 1, abort_flag, p.status, 101, kBackoffNs));
-          if (!ok) break;
-          if (leader) {
-            for (int hf = 0; hf < kHalves; ++hf) {
-              int valid = p.tokens - jk[hf] * BS - (kPair ? 0 : (tk & 1) * kStepKeys);
-              valid = max(0, min(kStepKeys, valid));
-              sts_volatile_v2(smem_u32(smem + kOffScal) + (tk & 7) * 16 + hf * 8,
-                              __float_as_uint((hf ? sq1 : sq0) * sk[hf]), static_cast<uint32_t>(valid));
-            }
-            mbar_arrive_expect_tx(&bars->k_full[st], kKTx);
-            for (int hf = 0; hf < kHalves; ++hf)
-              tma_load_2d(smem + kOffK + st * kKStage + hf * 4096, &map_k, &bars->k_full[st], 0, tile_row(tk, jk[hf]));
-          }
+          if (leader) mbar_arrive(&bars->k_full[st]);
+          ++kc;
         }
-        if (tv >= 0) {
-          // the stage of step tv held step tv - 3 before
-          if (tv >= kVStages)
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(&bars->pv_done[(tv - kVStages) % kStages], ((tv - kVStages) / kStages) & 1,
-                                                   abort_flag, p.status, 102, kBackoffNs));
-          if (!ok) break;
+        if (t > 0) {
+          const int st = vc % kStages;
+          if (!(ok = wait_v_stage())) break;
           if (leader) {
-            mbar_arrive_expect_tx(&bars->v_full[sv], kVTx);
+            mbar_arrive_expect_tx(&bars->v_full[st], kTxV);
             for (int hf = 0; hf < kHalves; ++hf)
-              tma_load_2d(smem + kOffV + sv * kVStage + hf * 8192, &map_v, &bars->v_full[sv], 0, tile_row(tv, jv[hf]));
+              tma_load_2d(smem + kOffV + st * kStageV + hf * 8192, &map_v, &bars->v_full[st], 0, tile_row(t - 1, jv[hf]));
           }
-          if (++sv == kVStages) sv = 0;
+          ++vc;
         }
         for (int hf = 0; hf < kHalves; ++hf) jv[hf] = jk[hf];
       }
       if (ok && p.k_marg > 0) {
-        // The aggregated summaries go to K stages 0 and 1, which are free once the last Q K^T products have
-        // completed: well before the last P V products, so this load is off the tail's critical path.
-        for (int u = max(0, steps - kStages); u < steps && ok; ++u)
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(&bars->k_free[u % kStages], (u / kStages) & 1, abort_flag, p.status, 103, kBackoffNs));
-        // G and zeta come from the kernel enqueued just before this one, which may still be running when this kernel
-        // was launched to overlap with it: everything above reads older results only.
-        wait_for_prior_grid();
+        // The aggregated summaries follow the last V tile through its ring.  G and zeta come from the kernel enqueued
+        // just before this one, which may still be running when this kernel was launched to overlap with it: everything
+        // above reads older results only.
+        const int st = vc % kStages;
+        ok = wait_v_stage();
+        if (it == 0) wait_for_prior_grid();
         if (ok && leader) {
-          mbar_arrive_expect_tx(&bars->z_full, kHalves * 256);
-          for (int hf = 0; hf < kHalves; ++hf)
-            bulk_load(smem + kOffZeta + hf * 256, p.zeta + (bh_rows + i_q[hf]) * kHeadDim, 256, &bars->z_full);
-          mbar_arrive_expect_tx(&bars->g_full, kHalves * 8192);
-          for (int hf = 0; hf < kHalves; ++hf)
-            tma_load_2d(smem + kOffG + hf * 8192, &map_g, &bars->g_full, 0, static_cast<int>((bh_rows + i_q[hf]) * 64));
+          mbar_arrive_expect_tx(&bars->v_full[st], kHalves * (256 + 8192));
+          for (int hf = 0; hf < kHalves; ++hf) {
+            bulk_load(smem + kOffZeta + (it & 1) * 512 + hf * 256, p.zeta + (bh_rows + tile.i_q[hf]) * kHeadDim, 256, &bars->v_full[st]);
+            tma_load_2d(smem + kOffV + st * kStageV + hf * 8192, &map_g, &bars->v_full[st], 0,
+                        static_cast<int>((bh_rows + tile.i_q[hf]) * 64));
+          }
         }
+        ++vc;
+      }
+      if (!ok) break;
+      id = -1;
+      if (p.steal) {
+        if (!(ok = wait_all(&bars->next_full, it & 1, 106))) break;
+        id = __shfl_sync(0xFFFFFFFFu, taken_cta(answer), 0);
+      }
+      fence_proxy_async_smem();  // the answer has been read before the next one may be written
+      __syncwarp();
+      if (leader) {
+        tile_ids[it % kTileSlots] = id;
+        mbar_arrive(&bars->tile_full[it % kTileSlots]);
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------ Q K^T issuer
-    // One thread issues a small tcgen05.mma about every 55 clocks and pays some 100 clocks per barrier it looks
-    // at, so the two products of a step have an issuing warp each (this one and the next); a single issuer for
-    // both was measured to be the bottleneck of the whole kernel.  Operand descriptors are built once and advanced by
-    // adding byte offsets (in 16-byte units) to their address field.  As in the producer, all lanes run the loop
-    // and one elected lane issues.
-    {
-      const bool leader = elect_one();
-      constexpr uint32_t idesc_qk = instr_desc(0, kM, 64, 0, 0);   // e4m3 x e4m3, both K-major
-      constexpr uint32_t idesc_lin = instr_desc(1, kM, 64, 0, 0);  // bf16 x bf16, both K-major
-      const uint32_t q_addr = smem_u32(smem + kOffQ);
-      const uint64_t k_desc0 = smem_desc(smem_u32(smem + kOffK), 16, 512, kSwizzle64);
-      bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(&bars->q_full, 0, abort_flag, p.status, 201, kBackoffNs));
-      uint64_t q_desc[2][kHalves];
-#pragma unroll
-      for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-        for (int hf = 0; hf < kHalves; ++hf)
-          q_desc[kk][hf] = smem_desc(q_addr + (kPair ? hf * 4096 : 0) + kk * 32, 16, 512, kSwizzle64);
-      // S[t&1] = Q K(t)^T needs the K tile of step t and S[t&1] drained by the softmax threads of step t-2; it runs
-      // one step ahead of the softmax threads, so the scores of step t are waiting when step t-1 is finished.
-      for (int t = 0; ok && t < steps; ++t) {
-        const int st = t % kStages;
-        ok = mbar_wait(&bars->k_full[st], (t / kStages) & 1, abort_flag, p.status, 202, kBackoffNs);
-        if (ok && t >= 2)
-          ok = mbar_wait(&bars->s_empty[t & 1], ((t - 2) >> 1) & 1, abort_flag, p.status, 203, kBackoffNs);
+    const bool leader = elect_one();
+    constexpr uint32_t idesc_qk = instr_desc(0, kM, 64, 0, 0);  // e4m3 x e4m3, both K-major
+    const uint64_t q_desc = smem_desc(smem_u32(smem + kOffQ), 16, 512, kSwizzle64);
+    const uint64_t k_desc0 = smem_desc(smem_u32(smem + kOffK), 16, 512, kSwizzle64);
+    bool ok = true;
+    int kc = 0, sc = 0;  // products issued, releases of the score columns waited for, through all tiles
+#pragma unroll 1
+    for (int it = 0, id = 0; id >= 0 && steps > 0; id = next_tile(it, 210, std::integral_constant<int, 1>{}), ++it) {
+      ok = mbar_wait_far<1>(&bars->q_full, it & 1, abort_flag, p.status, 201);
+#pragma unroll 1
+      for (int t = 0; t < steps; ++t, ++kc) {
+        const int st = kc % kStages;
+        ok = ok && mbar_wait_far<1>(&bars->k_full[st], (kc / kStages) & 1, abort_flag, p.status, 202);
+        if (t > 0 || it > 0) {  // the scores of the step before (in a tile's first step: the linear product) have been read
+          ok = ok && mbar_wait_far<1>(&bars->s_free, sc & 1, abort_flag, p.status, 203);
+          ++sc;
+        }
         ok = __all_sync(0xFFFFFFFFu, ok);
         if (!ok) break;
-        const uint32_t s_tmem = tmem + kColS + (t & 1) * 64;
-        const uint64_t k_desc = k_desc0 + static_cast<uint64_t>((st * kKStage) >> 4);
+        const uint64_t k_desc = k_desc0 + static_cast<uint64_t>((st * kStageK) >> 4);
         tc_fence_after();
         if (leader) {
 #pragma unroll
           for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
             for (int hf = 0; hf < kHalves; ++hf)
-              mma_f8(s_tmem + ((hf * 16u) << 16), q_desc[kk][hf], k_desc + ((hf * 4096 + kk * 32) >> 4), idesc_qk, kk);
+              mma_f8(tmem_so + ((hf * 16u) << 16), q_desc + ((hf * 4096 + kk * 32) >> 4), k_desc + ((hf * 4096 + kk * 32) >> 4),
+                     idesc_qk, kk);
           }
-          mma_commit(&bars->qk_done[t & 1]);
-          mma_commit(&bars->k_free[st]);
+          mma_commit(&bars->s_full[st]);
         }
       }
-      if (ok && p.k_marg > 0) {
-        // the linear product lands in score buffer 0: the scores of the last even step must have been read (the loop
-        // above has only waited for those of steps up to steps - 3)
-        ok = mbar_wait(&bars->g_full, 0, abort_flag, p.status, 206, kBackoffNs) &&
-             mbar_wait(&bars->phi_full, 0, abort_flag, p.status, 207, kBackoffNs);
-        if (ok && steps > 0) {
-          const int t_even = (steps - 1) & ~1;
-          ok = mbar_wait(&bars->s_empty[0], (t_even >> 1) & 1, abort_flag, p.status, 208, kBackoffNs);
-        }
-        ok = __all_sync(0xFFFFFFFFu, ok);
-        if (ok) {
-          tc_fence_after();
-          const uint32_t phi_addr = smem_u32(smem + kOffPhi), g_addr = smem_u32(smem + kOffG);
-          if (leader) {
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-#pragma unroll
-              for (int hf = 0; hf < kHalves; ++hf) {
-                const uint64_t a = smem_desc(phi_addr + (kPair ? hf * 8192 : 0) + kk * 32, 16, 1024, kSwizzle128);
-                const uint64_t bd = smem_desc(g_addr + hf * 8192 + kk * 32, 16, 1024, kSwizzle128);
-                mma_f16(tmem + kColL + ((hf * 16u) << 16), a, bd, idesc_lin, kk);
-              }
-            }
-            mma_commit(&bars->l_full);
-          }
-        }
+      if (!ok) break;
+      if (p.k_marg > 0) {  // the release of the last scores, which the linear product takes up, passes by here
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait_far<1>(&bars->s_free, sc & 1, abort_flag, p.status, 208));
+        ++sc;
+        if (!ok) break;
       }
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------------------------------ P V issuer
-    {
-      const bool leader = elect_one();
-      constexpr uint32_t idesc_pv = instr_desc(0, kM, 64, 0, 1);  // f16 x f16, P from TMEM, V MN-major
-      const uint64_t v_desc0 = smem_desc(smem_u32(smem + kOffV), 8192, 1024, kSwizzle128);
-      const uint32_t o_tmem = tmem + kColO;
-      bool ok = true;
-      int sv = 0;
-      uint32_t v_par = 0;  // V stage of step t (t % 3) and the parity of its barrier ((t / 3) & 1)
-      for (int t = 0; ok && t < steps; ++t) {  // O += P[t&1] V(t)
-        ok = mbar_wait(&bars->v_full[sv], v_par, abort_flag, p.status, 205, kBackoffNs) &&
-             mbar_wait(&bars->p_full[t & 1], (t >> 1) & 1, abort_flag, p.status, 204, kBackoffNs);
+    const bool leader = elect_one();
+    constexpr uint32_t idesc_pv = instr_desc(0, kM, 64, 0, 1);   // f16 x f16, P from TMEM, V MN-major
+    constexpr uint32_t idesc_lin = instr_desc(1, kM, 64, 0, 0);  // bf16 x bf16, both K-major
+    const uint64_t v_desc0 = smem_desc(smem_u32(smem + kOffV), 8192, 1024, kSwizzle128);
+    const uint32_t o_tmem = tmem_so + kColO;
+    bool ok = true;
+    int vc = 0, pc = 0;  // V-ring entries, probability tiles, through all tiles
+#pragma unroll 1
+    for (int it = 0, id = 0; id >= 0; id = next_tile(it, 211, std::integral_constant<int, 1>{}), ++it) {
+#pragma unroll 1
+      for (int t = 0; t < steps; ++t, ++vc, ++pc) {  // O += P V(t)
+        const int st = vc % kStages;
+        ok = mbar_wait_far<1>(&bars->v_full[st], (vc / kStages) & 1, abort_flag, p.status, 205) &&
+             mbar_wait_far<1>(&bars->p_full, pc & 1, abort_flag, p.status, 204);
         ok = __all_sync(0xFFFFFFFFu, ok);
         if (!ok) break;
-        const uint32_t p_tmem = tmem + kColP + (t & 1) * 32;
-        const uint64_t v_desc = v_desc0 + static_cast<uint64_t>((sv * kVStage) >> 4);
+        const uint64_t v_desc = v_desc0 + static_cast<uint64_t>((st * kStageV) >> 4);
         tc_fence_after();
         if (leader) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
 #pragma unroll
             for (int hf = 0; hf < kHalves; ++hf)
-              mma_f16_ts(o_tmem + ((hf * 16u) << 16), p_tmem + ((hf * 16u) << 16) + kk * 8,
+              mma_f16_ts(o_tmem + ((hf * 16u) << 16), tmem_p + ((hf * 16u) << 16) + kk * 8,
                          v_desc + ((hf * 8192 + kk * 2048) >> 4), idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
           }
-          mma_commit(&bars->pv_done[t % kStages]);
+          mma_commit(&bars->v_done[st]);
         }
-        if (++sv == kVStages) {
-          sv = 0;
-          v_par ^= 1u;
+      }
+      if (!ok) break;
+      if (p.k_marg > 0) {
+        // phi(Q) G into the score columns (released by the softmax threads: this step's probabilities, waited for above,
+        // were made from the last scores)
+        const int st = vc % kStages;
+        ok = mbar_wait_far<1>(&bars->phi_full, it & 1, abort_flag, p.status, 207) &&
+             mbar_wait_far<1>(&bars->v_full[st], (vc / kStages) & 1, abort_flag, p.status, 206);
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        if (leader) {
+          const uint64_t a0 = smem_desc(smem_u32(smem + kOffPhi), 16, 1024, kSwizzle128);
+          const uint64_t b0 = smem_desc(smem_u32(smem + kOffV) + st * kStageV, 16, 1024, kSwizzle128);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+#pragma unroll
+            for (int hf = 0; hf < kHalves; ++hf)
+              mma_f16(tmem_so + ((hf * 16u) << 16), a0 + ((hf * 8192 + kk * 32) >> 4), b0 + ((hf * 8192 + kk * 32) >> 4), idesc_lin, kk);
+          }
+          mma_commit(&bars->v_done[st]);
         }
+        ++vc;
       }
     }
   }
@@ -466,45 +531,44 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // ------------------------------------------------------------------------------------------ softmax + epilogue
     setmaxnreg_inc<kSoftmaxRegs>();
     const int quarter = warp & 3;                       // TMEM sub-partition this warp may touch
-    const int w = (warp - kCtrlWarps) >> 2;             // warpgroup: steps t with (t & 1) == w
     const int hf = kPair ? (lane >> 4) : 0;             // which query block of the pair this thread serves
     const int row_in_block = kPair ? quarter * 16 + (lane & 15) : quarter * 32 + lane;
     const int p_row = kPair ? hf * 64 + row_in_block : row_in_block;  // row inside the 128-row tile
-    const int iq = i_q[hf];
-    const size_t q_tile = bh_rows + iq;
-    const uint32_t lane_addr = tmem + ((static_cast<uint32_t>(quarter) * 32u) << 16);
-    const uint32_t s_addr = lane_addr + kColS + w * 64, p_addr = lane_addr + kColP + w * 32, o_addr = lane_addr + kColO;
-    const float sq = __ldg(p.q_scales + q_tile);
+    const uint32_t lane_off = (static_cast<uint32_t>(quarter) * 32u) << 16;
+    const uint32_t s_addr = tmem_so + lane_off, o_addr = tmem_so + kColO + lane_off, p_addr = tmem_p + lane_off;
     const uint32_t scal_slot = smem_u32(smem + kOffScal) + hf * 8;
-    const uint32_t ref_slot = smem_u32(smem + kOffRef) + p_row * 8;
-
-    float m_seen = kNoMax, l = 0.f;  // reference this warpgroup's row sum is relative to; the row sum
-    bool ok = true;
-
-    // Waits until `count` steps have published their reference for this row and returns it.  The slot is one aligned
-    // 8-byte word written by a single store, so value and count are always seen together.
-    auto reference_after = [&](int count, float& m) -> bool {
-      uint2 v = lds_volatile_v2(ref_slot);
-      if (static_cast<int>(v.y) != count && !reference_wait_slow(ref_slot, count, v, abort_flag, p.status)) return false;
-      m = __uint_as_float(v.x);
-      return true;
-    };
-
-    // linear branch, first part: this thread's 32 columns (warpgroup w -> columns 32 w ..) of phi(q) as bf16 A operand
-    // of the linear product.  It needs the Q tile only, so it is computed while the first key tiles are on their way
-    // and the softmax threads would be idle; the operand has a shared-memory region of its own and the linear product
-    // can then be issued as soon as the aggregated summaries have arrived and the last scores have been read.  The
-    // denominators phi(q) . zeta_i follow in the epilogue, from the operand's own rounded values.
-    // The query row comes from the Q tile in shared memory (64-byte rows, 64B swizzle: 16-byte chunk c of row r sits at
-    // chunk c ^ ((r >> 1) & 3)).
-    // The loops over 16-column chunks here and in the epilogue are deliberately NOT unrolled: the kernel's code has to
-    // stay within the instruction cache of an SM, which its fully unrolled form exceeded several times over (the
-    // kernel was then bound by instruction fetch from the GPC-level cache, not by any arithmetic unit).
-    float den = 0.f;
     const int swz = p_row & 7;
+    // hands the probabilities of the step just finished to the P V issuer
+    auto publish = [&]() {
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->p_full);
+    };
+    bool ok = true;
+    int kc = 0, vc = 0;  // Q K^T products and V-ring products so far, through all tiles
+#pragma unroll 1
+    for (int it = 0, id = blockIdx.x; id >= 0; id = next_tile(it, 310, std::integral_constant<int, 0>{}), ++it) {
+    // shared-memory addresses of this thread's row: phi(q) / staged output, and the query
+    uint32_t phi_row = smem_u32(smem + kOffPhi) + p_row * 128, q_row = smem_u32(smem + kOffQ) + p_row * 64;
+    opaque(phi_row);
+    opaque(q_row);
+    const Tile tile = tile_at(id);
+    const int iq = tile.i_q[hf];
+    const size_t bh_rows = static_cast<size_t>(tile.bh) * p.nb;
+
+    // linear branch, first part: phi(q) as bf16 A operand of the linear product.  It needs the Q tile only, so it is
+    // computed while the first key tiles are on their way and the softmax threads would be idle; the denominators
+    // phi(q) . zeta_i follow in the epilogue, from the operand's own rounded values.
+    // The query row comes from the Q tile in shared memory (64-byte rows, 64B swizzle: 16-byte chunk c of row r sits at
+    // chunk c ^ ((r >> 1) & 3)).  The loops over chunks are not unrolled: the kernel's code has to stay within the
+    // instruction cache.
     if (p.k_marg > 0) {
-      ok = mbar_wait_far(&bars->q_full, 0, abort_flag, p.status, 307);
-      const uint8_t* qrow = smem + kOffQ + p_row * 64;
+      const float sq = __ldg(p.q_scales + bh_rows + iq);
+      if (!(ok = mbar_wait_far(&bars->q_full, it & 1, abort_flag, p.status, 307))) break;
+      // the previous tile's output rows, staged where this warp's rows of phi(q) go, must have been read
+      if (lane == 0) bulk_wait_group_read0();
+      __syncwarp();
       const int qswz = (p_row >> 1) & 3;
       // phi = softmax over the components: any common shift of the exponents cancels in the ratio numerator /
       // denominator.  448 * scale bounds every component of the block, so it serves as the shift without a pass over
@@ -514,26 +578,23 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const float cq = sq * kLog2e;
       float shift = 448.f * cq;
       if (phi_softmax && 896.f * cq > 100.f) {
-        float mxq[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        float mxq = -INFINITY;
 #pragma unroll 1
-        for (int c4 = 0; c4 < 4; ++c4) {  // row maximum over the 64 components
-          const uint4 raw = *reinterpret_cast<const uint4*>(qrow + ((c4 ^ qswz) << 4));
+        for (int c4 = 0; c4 < 4; ++c4) {
+          const uint4 raw = lds128(q_row + ((c4 ^ qswz) << 4));
           const uint32_t words[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
           for (int xw = 0; xw < 4; ++xw) {
             float fv[4];
             e4m3x4_to_float(words[xw], fv);
-#pragma unroll
-            for (int y = 0; y < 4; ++y) mxq[y] = fmaxf(mxq[y], fv[y]);
+            mxq = fmaxf(max3(mxq, fv[0], fv[1]), fmaxf(fv[2], fv[3]));
           }
         }
-        shift = fmaxf(fmaxf(mxq[0], mxq[1]), fmaxf(mxq[2], mxq[3])) * cq;  // sq > 0 commutes with max
+        shift = mxq * cq;  // sq > 0 commutes with max
       }
-      uint8_t* const phirow = smem + kOffPhi + p_row * 128;
 #pragma unroll 1
-      for (int cc = 0; cc < 2; ++cc) {  // this warpgroup's two chunks of 16 components
-        const int c4 = 2 * w + cc;
-        const uint4 raw = *reinterpret_cast<const uint4*>(qrow + ((c4 ^ qswz) << 4));
+      for (int c4 = 0; c4 < 4; ++c4) {
+        const uint4 raw = lds128(q_row + ((c4 ^ qswz) << 4));
         const uint32_t words[4] = {raw.x, raw.y, raw.z, raw.w};
         uint32_t pk8[8];
 #pragma unroll
@@ -553,260 +614,216 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             pk8[xw * 2 + (y >> 1)] = pack_bf162(e0, e1);
           }
         }
-        *reinterpret_cast<uint4*>(phirow + (((c4 * 2) ^ swz) << 4)) = make_uint4(pk8[0], pk8[1], pk8[2], pk8[3]);
-        *reinterpret_cast<uint4*>(phirow + (((c4 * 2 + 1) ^ swz) << 4)) = make_uint4(pk8[4], pk8[5], pk8[6], pk8[7]);
+        sts128(phi_row + (((c4 * 2) ^ swz) << 4), pk8[0], pk8[1], pk8[2], pk8[3]);
+        sts128(phi_row + (((c4 * 2 + 1) ^ swz) << 4), pk8[4], pk8[5], pk8[6], pk8[7]);
       }
       fence_proxy_async_smem();
-      mbar_arrive(&bars->phi_full);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->phi_full);
     }
 
-
-    // barrier of the P V product two steps back (the one that frees P[w]): its stage alternates between w and w + 2,
-    // its parity flips every second iteration; both are carried along instead of being recomputed from t
-    uint64_t* const pv_bar0 = &bars->pv_done[w];
-    uint32_t pv_off = 0, pv_par = 0, pv_flip = 0, qk_par = 0;
-
-    for (int t = w; t < steps; t += 2) {
-      if (!(ok = mbar_wait_far(&bars->qk_done[w], qk_par, abort_flag, p.status, 301))) break;
-      qk_par ^= 1u;
+    float m_ref = kNoMax, l = 0.f;  // the row's reference, and its sum relative to it
+#pragma unroll 1
+    for (int t = 0; t < steps; ++t, ++kc) {
+      if (!(ok = mbar_wait_far(&bars->s_full[kc % kStages], (kc / kStages) & 1, abort_flag, p.status, 301))) break;
       tc_fence_after();
-      // the step's scalars, left by the producer before it requested the K tile
-      const uint2 scal = lds_volatile_v2(scal_slot + (t & 7) * 16);
+      uint32_t xa[32], xb[32];
+      tmem_ld32(s_addr, xa);
+      tmem_ld32(s_addr + 32, xb);
+      if (t > 0) publish();  // the store of step t-1 has had this step's wait and loads to complete under
+      // the step's scalars, left by the producer before it completed the K stage
+      const uint2 scal = lds_volatile_v2(scal_slot + (kc % kScalSlots) * 16);
       const float c = __uint_as_float(scal.x);
       const int valid = static_cast<int>(scal.y);
-      uint32_t xa[32], xb[32];
-      float mx4[4];
-      {
-        tmem_ld32(s_addr, xa);
-        tmem_ld32(s_addr + 32, xb);
-        tmem_wait_ld();
-        // the whole row of scores is in registers: the issuer may overwrite S[w] with step t+2 right away
-        tc_fence_before();
-        mbar_arrive(&bars->s_empty[w]);
-        if (valid < kStepKeys) {
-#pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            if (k >= valid) xa[k] = 0xFF800000u;  // -inf
-            if (32 + k >= valid) xb[k] = 0xFF800000u;
-          }
-        }
-        // row maximum of the raw scores (c > 0 commutes with max), four independent chains
-#pragma unroll
-        for (int q = 0; q < 4; ++q) mx4[q] = fmaxf(__uint_as_float(xa[q]), __uint_as_float(xb[q]));
-#pragma unroll
-        for (int k = 4; k < 32; k += 4) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) mx4[q] = max3(mx4[q], __uint_as_float(xa[k + q]), __uint_as_float(xb[k + q]));
-        }
-      }
-      // a step without any valid key (second half of a short last block) leaves the reference where it is
-      const float tile_max = fmaxf(max3(fmaxf(mx4[0], mx4[1]), mx4[2], mx4[3]) * c, kNoMax);
-
-      // the row's reference after step t-1 (published early in that step by the other warpgroup), the lazy-rescale
-      // decision of this step, and its publication for step t+1
-      float m_ref = kNoMax;
-      if (t > 0 && !(ok = reference_after(t, m_ref))) break;
-      if (m_ref != m_seen) l *= ex2(m_seen - m_ref);  // bring this warpgroup's row sum to the current reference
-      bool need = false;
-      float alpha = 1.f;
-      if (t == 0) {
-        m_ref = tile_max;
-      } else if (tile_max > m_ref + kRescaleThreshold) {
-        need = true;
-        alpha = ex2(m_ref - tile_max);
-        m_ref = tile_max;
-        l *= alpha;
-      }
-      m_seen = m_ref;
-      sts_volatile_v2(ref_slot, __float_as_uint(m_ref), static_cast<uint32_t>(t + 1));
-
-      // P[w] is free once the P V product of step t-2 has completed (long ago in the steady state)
-      if (t >= 2) {
-        if (!(ok = mbar_wait_far(pv_bar0 + pv_off, pv_par, abort_flag, p.status, 302))) break;
-        pv_off ^= 2u;
-        pv_par ^= pv_flip;
-        pv_flip ^= 1u;
-      }
-      tc_fence_after();
-      {
-        // the second half of the row is read again instead of being held across the first half's exponentials;
-        // S[w] is released once it is in registers
-        uint32_t packed[16];
-        l += exp_half_row(xa, c, -m_ref, packed);
-        tmem_st16(p_addr, packed);
-        l += exp_half_row(xb, c, -m_ref, packed);
-        tmem_st16(p_addr + 16, packed);
-      }
-      if (__any_sync(0xFFFFFFFFu, need)) {
-        // O is being accumulated into by the P V product of step t-1: wait for it, then scale the rows whose
-        // reference moved.  The product of this step waits for this thread's arrival below.
-        if (!(ok = mbar_wait_far(&bars->pv_done[(t - 1) % kStages], ((t - 1) / kStages) & 1, abort_flag, p.status, 303))) break;
-        tc_fence_after();
-        rescale_accumulator(o_addr, alpha);
-      }
-      tmem_wait_st();
+      tmem_wait_ld();
+      // the whole row of scores is in registers: the issuer may overwrite S with step t+1 right away
       tc_fence_before();
-      mbar_arrive(&bars->p_full[w]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->s_free);
+      if (valid < kStepKeys) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          if (k >= valid) xa[k] = 0xFF800000u;  // -inf
+          if (32 + k >= valid) xb[k] = 0xFF800000u;
+        }
+      }
+      // row maximum of the raw scores (c > 0 commutes with max), eight independent chains; a step without any valid key
+      // (second half of a short last block) leaves the reference where it is
+      float mx[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) mx[q] = fmaxf(__uint_as_float(xa[q]), __uint_as_float(xb[q]));
+#pragma unroll
+      for (int k = 8; k < 32; k += 8) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) mx[q] = max3(mx[q], __uint_as_float(xa[k + q]), __uint_as_float(xb[k + q]));
+      }
+      const float top = fmaxf(max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7])) * c, kNoMax);
+      // lazy rescale: the reference of a row moves only when it is beaten by 2^8 (and in the first step)
+      if (__any_sync(0xFFFFFFFFu, top > m_ref + kRescaleThreshold)) {
+        const float m_new = top > m_ref + kRescaleThreshold ? top : m_ref;
+        const float alpha = ex2(m_ref - m_new);
+        l *= alpha;
+        m_ref = m_new;
+        if (t > 0) {
+          // O is being accumulated into by the P V product of step t-1: wait for it first
+          const int u = vc + t - 1;
+          if (!(ok = mbar_wait_far(&bars->v_done[u % kStages], (u / kStages) & 1, abort_flag, p.status, 303))) break;
+          tc_fence_after();
+          rescale_accumulator(o_addr, alpha);
+        }
+      }
+      uint32_t packed[32];
+      {
+        const uint64_t c2 = pack_f32x2(c, c), shift2 = pack_f32x2(-m_ref, -m_ref);
+        uint64_t sum2[2] = {0ull, 0ull};  // bit pattern of (0.f, 0.f)
+        exp_half_row(xa, c2, shift2, packed, sum2);
+        exp_half_row(xb, c2, shift2, packed + 16, sum2);
+        float s0, s1;
+        unpack_f32x2(add_f32x2(sum2[0], sum2[1]), s0, s1);
+        l += s0 + s1;
+      }
+      // P is free once the P V product of step t-1 has completed (long ago in the steady state)
+      if (t > 0) {
+        const int u = vc + t - 1;
+        if (!(ok = mbar_wait_far(&bars->v_done[u % kStages], (u / kStages) & 1, abort_flag, p.status, 302))) break;
+        tc_fence_after();
+      }
+      tmem_st32(p_addr, packed);
     }
+    if (!ok) break;
+    if (steps > 0) publish();
 
-    // linear branch, second part: partial denominator phi(q) . zeta_i over this thread's 32 columns, with the same
-    // rounded values as the numerator's operand (read back from shared memory); zeta_i arrives with the aggregated
-    // summaries at the end of the producer's work
-    if (ok && p.k_marg > 0) {
-      ok = mbar_wait_far(&bars->z_full, 0, abort_flag, p.status, 308);
-      const uint8_t* const phirow = smem + kOffPhi + p_row * 128;
+    // linear branch, second part: the denominator phi(q) . zeta_i, with the same rounded values as the numerator's operand;
+    // zeta_i arrives with the aggregated summaries behind the last V tile
+    const int v_last = vc + v_steps - 1;  // the tile's last product
+    float den = 0.f;
+    if (p.k_marg > 0) {
+      if (!(ok = mbar_wait_far(&bars->v_full[v_last % kStages], (v_last / kStages) & 1, abort_flag, p.status, 308))) break;
+      const uint32_t zeta = smem_u32(smem + kOffZeta) + (it & 1) * 512 + hf * 256;
       float den4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-      for (int ch = 0; ch < 4; ++ch) {  // 16-byte chunks of eight components
-        const int c8 = 4 * w + ch;
-        const uint4 raw = *reinterpret_cast<const uint4*>(phirow + ((c8 ^ swz) << 4));
-        const uint32_t words[4] = {raw.x, raw.y, raw.z, raw.w};
-        const float4* zeta = reinterpret_cast<const float4*>(smem + kOffZeta + hf * 256 + c8 * 32);
+      for (int c8 = 0; c8 < 8; ++c8) {  // 16-byte chunks of eight components
+        const uint4 rw = lds128(phi_row + ((c8 ^ swz) << 4));
+        const uint32_t words[4] = {rw.x, rw.y, rw.z, rw.w};
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
-          const float4 z = zeta[half];
-          den4[0] = fmaf(__uint_as_float(words[2 * half] << 16), z.x, den4[0]);
-          den4[1] = fmaf(__uint_as_float(words[2 * half] & 0xFFFF0000u), z.y, den4[1]);
-          den4[2] = fmaf(__uint_as_float(words[2 * half + 1] << 16), z.z, den4[2]);
-          den4[3] = fmaf(__uint_as_float(words[2 * half + 1] & 0xFFFF0000u), z.w, den4[3]);
+          const uint4 z = lds128(zeta + c8 * 32 + half * 16);
+          den4[0] = fmaf(__uint_as_float(words[2 * half] << 16), __uint_as_float(z.x), den4[0]);
+          den4[1] = fmaf(__uint_as_float(words[2 * half] & 0xFFFF0000u), __uint_as_float(z.y), den4[1]);
+          den4[2] = fmaf(__uint_as_float(words[2 * half + 1] << 16), __uint_as_float(z.z), den4[2]);
+          den4[3] = fmaf(__uint_as_float(words[2 * half + 1] & 0xFFFF0000u), __uint_as_float(z.w), den4[3]);
         }
       }
       den = (den4[0] + den4[1]) + (den4[2] + den4[3]);
+      // (the last P V product is the one before)
+      if (steps > 0 && !(ok = mbar_wait_far(&bars->v_done[(v_last - 1) % kStages], ((v_last - 1) / kStages) & 1, abort_flag, p.status, 304))) break;
     }
-
-    // the two threads of a row (one per warpgroup) bring their row sums to the final reference and swap them together
-    // with the partial denominators
-    float inv_l = 0.f;
-    if (ok) {
-      float m_fin = kNoMax;
-      if (steps > 0) ok = reference_after(steps, m_fin);
-      if (ok) {
-        if (m_fin != m_seen) l *= ex2(m_seen - m_fin);
-        float2* xbuf = reinterpret_cast<float2*>(smem + kOffX);
-        xbuf[w * 128 + p_row] = make_float2(l, den);
-        mbar_arrive(&bars->x_full);
-        ok = mbar_wait_far(&bars->x_full, 0, abort_flag, p.status, 306);
-        if (ok) {
-          const float2 other = xbuf[(w ^ 1) * 128 + p_row];
-          inv_l = steps > 0 ? 1.f / (l + other.x) : 0.f;
-          den += other.y;
-        }
-      }
-    }
-    // the last P V product (commits are cumulative: it covers every earlier one), then the linear product
-    if (ok && steps > 0)
-      ok = mbar_wait_far(&bars->pv_done[(steps - 1) % kStages], ((steps - 1) / kStages) & 1, abort_flag, p.status, 304);
-    if (ok && p.k_marg > 0) ok = mbar_wait_far(&bars->l_full, 0, abort_flag, p.status, 305);
+    if (v_steps > 0 && !(ok = mbar_wait_far(&bars->v_done[v_last % kStages], (v_last / kStages) & 1, abort_flag, p.status, 305))) break;
+    vc += v_steps;
     tc_fence_after();
 
-    ok = __all_sync(0xFFFFFFFFu, ok);  // the store below synchronises the warp
-    if (ok) {
-      const int bb = bh / p.heads, h = bh % p.heads;
-      const float l_scale = p.k_marg > 0 ? 1.f / den : 0.f;
-      // The thread's 32 output values go to the V ring (free: every P V product has completed), 16-byte chunks
-      // swizzled by the row so that neither these writes nor the row-wise reads below conflict; then each store
-      // instruction of the warp writes whole half rows (fp32: four rows x 128 bytes, 16-bit: eight rows x 64 bytes).
-      const bool wide = p.out_dtype == LITE3R_F32;
-      const bool to_bf16 = p.out_dtype == LITE3R_BF16;
-      const uint32_t row_bytes = wide ? 256u : 128u;
-      // With TMA stores every warp stages its 32 half rows in a tile of its own (row = lane, 128 bytes with the 128B
-      // swizzle for fp32, 64 bytes with the 64B swizzle for the 16-bit types), which is the layout the store engine
-      // reads; otherwise whole rows of the 128-row tile, chunks swizzled by the row.
-      const bool tma_out = p.tma_out != 0;
-      const uint32_t half_bytes = wide ? 128u : 64u;
-      uint8_t* const warp_tile = smem + kOffOut + (warp - kCtrlWarps) * 4096;
-      const int tswz = wide ? (lane & 7) : ((lane >> 1) & 3);
-      uint8_t* const orow = tma_out ? warp_tile + lane * half_bytes : smem + kOffOut + p_row * row_bytes;
+    // Output, 128 bytes of a row at a time (32 fp32 columns or 64 of a 16-bit type).  The warp stages its rows where it
+    // kept its rows of phi(q) (the linear product has read them) in the layout the store engine reads: 128-byte rows with the
+    // 128B swizzle.
+    const int bb = tile.bh / p.heads, h = tile.bh - bb * p.heads;
+    const float inv_l = steps > 0 ? 1.f / l : 0.f;
+    const float l_scale = p.k_marg > 0 ? 1.f / den : 0.f;
+    const bool wide = p.out_dtype == LITE3R_F32;
+    const bool to_bf16 = p.out_dtype == LITE3R_BF16;
+    if (p.k_marg == 0) {  // the previous tile's rows must have been read (next to a linear branch phi(q) has waited for that)
+      if (lane == 0) bulk_wait_group_read0();
+      __syncwarp();
+    }
 #pragma unroll 1
-      for (int cc = 0; cc < 2; ++cc) {  // 16 columns at a time
-        float acc[16];
-        uint32_t v[16];
-        if (steps > 0) {
-          tmem_ld16(o_addr + w * 32 + cc * 16, v);
-          tmem_wait_ld();
-#pragma unroll
-          for (int k = 0; k < 16; ++k) acc[k] = __uint_as_float(v[k]) * inv_l;
-        } else {
-#pragma unroll
-          for (int k = 0; k < 16; ++k) acc[k] = 0.f;
-        }
-        if (p.k_marg > 0) {
-          tmem_ld16(lane_addr + kColL + w * 32 + cc * 16, v);
-          tmem_wait_ld();
-#pragma unroll
-          for (int k = 0; k < 16; ++k) acc[k] = fmaf(__uint_as_float(v[k]), l_scale, acc[k]);
-        }
-        if (wide) {
-#pragma unroll
-          for (int ch = 0; ch < 4; ++ch)
-            *reinterpret_cast<float4*>(orow + ((tma_out ? ((cc * 4 + ch) ^ tswz) : ((w * 8 + cc * 4 + ch) ^ swz)) << 4)) =
-                make_float4(acc[4 * ch], acc[4 * ch + 1], acc[4 * ch + 2], acc[4 * ch + 3]);
-        } else {
-#pragma unroll
-          for (int ch = 0; ch < 2; ++ch) {
-            uint32_t pk[4];
-#pragma unroll
-            for (int y = 0; y < 4; ++y)
-              pk[y] = to_bf16 ? pack_bf162(acc[8 * ch + 2 * y], acc[8 * ch + 2 * y + 1])
-                              : pack_half2(acc[8 * ch + 2 * y], acc[8 * ch + 2 * y + 1]);
-            *reinterpret_cast<uint4*>(orow + ((tma_out ? ((cc * 2 + ch) ^ tswz) : ((w * 4 + cc * 2 + ch) ^ swz)) << 4)) =
-                make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          }
-        }
+    for (int half = 0; half < 2; ++half) {  // 32 columns
+      uint32_t v[32], u[32];
+      tmem_ld32(o_addr + half * 32, v);
+      tmem_ld32(s_addr + half * 32, u);
+      if (wide && half == 1) {  // the first half's rows have been read by the store engine (or by the lanes that stored them)
+        if (lane == 0) bulk_wait_group_read0();
+        __syncwarp();
       }
-      if (tma_out) {
-        // two boxes of 16 rows x 32 columns per warp: lanes 0-15 and 16-31 hold 16 consecutive tokens each (of the two
-        // query blocks of a pair, or of the two halves of the warp's 32 rows); rows past the end of the sequence are
-        // clipped by the store engine, the copy of the last block in an odd pair is not stored at all
+      tmem_wait_ld();
+      if (p.k_marg > 0 && half == 1) {  // the linear product has been read: the score columns are free for the next tile
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->s_free);
+      }
+      // (without a critical block O, without a linear branch its product was never written)
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const float o = steps > 0 ? __uint_as_float(v[k]) : 0.f, lin = p.k_marg > 0 ? __uint_as_float(u[k]) : 0.f;
+        v[k] = __float_as_uint(fmaf(lin, l_scale, o * inv_l));
+      }
+      if (wide) {
+#pragma unroll
+        for (int ch = 0; ch < 8; ++ch)
+          sts128(phi_row + ((ch ^ swz) << 4), v[4 * ch], v[4 * ch + 1], v[4 * ch + 2], v[4 * ch + 3]);
+      } else {
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int y = 0; y < 4; ++y)
+            pk[y] = to_bf16 ? pack_bf162(__uint_as_float(v[8 * ch + 2 * y]), __uint_as_float(v[8 * ch + 2 * y + 1]))
+                            : pack_half2(__uint_as_float(v[8 * ch + 2 * y]), __uint_as_float(v[8 * ch + 2 * y + 1]));
+          sts128(phi_row + (((half * 4 + ch) ^ swz) << 4), pk[0], pk[1], pk[2], pk[3]);
+        }
+        if (half == 0) continue;
+      }
+      if (p.tma_out != 0) {
+        // boxes of 16 tokens x 128 bytes: lanes 0-15 and 16-31 hold 16 consecutive tokens each (of the two query blocks
+        // of a pair, or of the two halves of the warp's 32 rows); rows past the end of the sequence are clipped by the
+        // store engine, the copy of the last block in an odd pair is not stored at all
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
 #pragma unroll
           for (int g2 = 0; g2 < 2; ++g2) {
-            const int token0 = kPair ? i_q[g2] * BS + quarter * 16 : i_q[0] * BS + quarter * 32 + 16 * g2;
-            if (token0 >= p.tokens || (kPair && g2 == 1 && i_q[1] == i_q[0])) continue;
-            int c[4] = {w * 32, 0, 0, 0};
+            const int token0 = kPair ? tile.i_q[g2] * BS + quarter * 16 : tile.i_q[0] * BS + quarter * 32 + 16 * g2;
+            if (token0 >= p.tokens || (kPair && g2 == 1 && tile.i_q[1] == tile.i_q[0])) continue;
+            int c[4] = {0, 0, 0, 0};
             c[p.dim_token] = token0;
             c[p.dim_head] = h;
             c[p.dim_batch] = bb;
-            tma_store_4d(&map_o, warp_tile + g2 * 16 * half_bytes, c[0], c[1], c[2], c[3]);
+            const int row0 = kPair ? g2 * 64 + quarter * 16 : quarter * 32 + g2 * 16;
+            tma_store_4d(&map_o, smem + kOffPhi + row0 * 128, wide ? half * 32 : 0, c[1], c[2], c[3]);
           }
           bulk_commit_group();
-          bulk_wait_group_read0();  // the tile must stay in place until the engine has read it
+        }
+      } else {
+        __syncwarp();
+        const int ch = lane & 7;
+        const uint32_t elem = wide ? 4u : 2u;
+        uint8_t* const out_bh = static_cast<uint8_t*>(p.out) +
+                                (static_cast<long long>(bb) * p.out_stride_b + static_cast<long long>(h) * p.out_stride_h) * elem +
+                                (wide ? half * 128 : 0) + ch * 16;
+        const long long row_pitch = p.out_stride_n * static_cast<long long>(elem);
+        const bool second_block_is_copy = kPair && tile.i_q[1] == tile.i_q[0];
+#pragma unroll 1
+        for (int r = lane >> 3; r < 32; r += 4) {  // row of this warp's block: thread r computed it
+          const int r_hf = kPair ? (r >> 4) : 0;
+          const int r_in_block = kPair ? quarter * 16 + (r & 15) : quarter * 32 + r;
+          const int r_p = kPair ? r_hf * 64 + r_in_block : r_in_block;
+          const int r_token = tile.i_q[r_hf] * BS + r_in_block;
+          const uint4 val = *reinterpret_cast<const uint4*>(smem + kOffPhi + r_p * 128 + ((ch ^ (r_p & 7)) << 4));
+          if (r_token < p.tokens && !(second_block_is_copy && r_hf == 1))
+            *reinterpret_cast<uint4*>(out_bh + r_token * row_pitch) = val;
         }
         __syncwarp();
-      } else {
-      __syncwarp();
-      const int chunk_shift = wide ? 3 : 2;       // 8 or 4 chunks of 16 bytes per half row
-      const int ch = lane & ((1 << chunk_shift) - 1);
-      const int half_chunks = 1 << chunk_shift;
-      const int rows_per_pass = 32 >> chunk_shift;  // 4 or 8
-      const uint32_t elem = wide ? 4u : 2u;
-      uint8_t* const out_bh = static_cast<uint8_t*>(p.out) +
-                              (static_cast<long long>(bb) * p.out_stride_b + static_cast<long long>(h) * p.out_stride_h) * elem +
-                              w * 32 * elem + ch * 16;
-      const long long row_pitch = p.out_stride_n * static_cast<long long>(elem);
-      const bool second_block_is_copy = kPair && i_q[1] == i_q[0];
-#pragma unroll 1
-      for (int r = lane >> chunk_shift; r < 32; r += rows_per_pass) {  // row of this warp's block: thread r computed it
-        const int r_hf = kPair ? (r >> 4) : 0;
-        const int r_in_block = kPair ? quarter * 16 + (r & 15) : quarter * 32 + r;
-        const int r_p = kPair ? r_hf * 64 + r_in_block : r_in_block;
-        const int r_token = i_q[r_hf] * BS + r_in_block;
-        const uint4 val = *reinterpret_cast<const uint4*>(smem + kOffOut + r_p * row_bytes +
-                                                          (((w * half_chunks + ch) ^ (r_p & 7)) << 4));
-        if (r_token < p.tokens && !(second_block_is_copy && r_hf == 1))
-          *reinterpret_cast<uint4*>(out_bh + r_token * row_pitch) = val;
-      }
       }
     }
+    tc_fence_before();  // O and the linear product have been read (ordered before the next tile's arrivals)
+    }  // tiles
+    if (lane == 0) bulk_wait_group_read0();  // the staged rows must stay in place until the engine has read them
   }
 
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, kTmemCols);
+    tmem_dealloc(tmem_p, kColsP);
+    tmem_dealloc(tmem_so, kColsSO);
   }
 }
 
@@ -848,7 +865,7 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
     cache.block = BS;
   }
   // The output goes through TMA stores when a tiled map can describe it: the token, head and batch dimensions ordered
-  // by stride (dimensions of extent 1 last), 16 tokens x 32 columns per box.  If the driver refuses the map the kernel
+  // by stride (dimensions of extent 1 last), 16 tokens x 128 bytes per box.  If the driver refuses the map the kernel
   // falls back to plain stores.
   if (cache.out != a.out || cache.out_dtype != a.out_dtype || cache.out_strides[0] != a.out_stride_n ||
       cache.out_strides[1] != a.out_stride_h || cache.out_strides[2] != a.out_stride_b || cache.out_dims[0] != s.tokens ||
@@ -868,7 +885,7 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
       for (int j = i + 1; j < 3; ++j)
         if (before(dm[j], dm[i])) std::swap(dm[i], dm[j]);
     uint64_t dims[4] = {kHeadDim, 0, 0, 0}, strides[3];
-    uint32_t box[4] = {32, 1, 1, 1};
+    uint32_t box[4] = {128u / elem, 1, 1, 1};  // 128 bytes of a row
     uint64_t packed = static_cast<uint64_t>(kHeadDim) * elem;  // stride a dimension would have if packed after the previous ones
     bool ok = (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0;
     for (int i = 0; i < 3; ++i) {
@@ -890,8 +907,7 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
       const CUtensorMapDataType type = a.out_dtype == LITE3R_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                        : a.out_dtype == LITE3R_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                                                     : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-      const CUtensorMapSwizzle swz = a.out_dtype == LITE3R_F32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
-      cache.out_ok = make_tensor_map_4d(&cache.o, type, a.out, dims, strides, box, swz) == LITE3R_OK ? 1 : 0;
+      cache.out_ok = make_tensor_map_4d(&cache.o, type, a.out, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) == LITE3R_OK ? 1 : 0;
     }
     cache.out = a.out;
     cache.out_dtype = a.out_dtype;
@@ -921,6 +937,7 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   p.heads = s.heads;
   p.tokens = s.tokens;
   p.nb = nb;
+  p.tiles_per_head = BS == 64 ? (nb + 1) / 2 : nb;
   p.k_crit = a.k_crit;
   p.k_marg = a.k_marg;
   p.phi = a.phi;
@@ -928,7 +945,10 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   p.status = a.device_status;
   st = ensure_dynamic_smem(attention_kernel<BS>, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
-  const int ctas = s.batch * s.heads * (BS == 64 ? (nb + 1) / 2 : nb);
+  const int ctas = s.batch * s.heads * p.tiles_per_head;
+  int sms = 0;
+  if ((st = sm_count(&sms)) != LITE3R_OK) return st;
+  p.steal = ctas > sms * kCtasPerSm ? 1 : 0;
   if (a.overlap_prior) {
     // programmatic dependent launch: the kernel may start while the preceding one (which announces it early) is
     // still running, and waits for its completion itself before it reads that kernel's results

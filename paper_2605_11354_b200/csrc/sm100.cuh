@@ -42,16 +42,18 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
-// One try: the thread may be suspended by the hardware until the phase completes or `hint_ns` have passed, so a
-// waiting warp does not burn issue slots that the working warps of the SM need.
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity, uint32_t hint_ns = 20000u) {
+// One try: the thread may be suspended by the hardware, for a time limit of its own, until the phase completes, so a
+// waiting warp does not burn issue slots that the working warps of the SM need.  Without a suspend-time hint on
+// purpose: given one, the wait is made of short polls with sleeps in between, which cost issue slots (a third of the
+// attention kernel's instructions) and wake up late.
+__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(hint_ns)
+      : "r"(smem_u32(bar)), "r"(parity)
       : "memory");
   return ok != 0;
 }
@@ -79,42 +81,53 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // backoff_ns > 0 makes the thread sleep between polls: for single-thread roles whose waits are long, so that their
 // polling does not take issue slots from the working warps.
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // 1 s
+// What a waiting thread looks at every few polls: returns the time at which the wait began (since = 0: now), or 0 when
+// the wait is over without success.
+__device__ __forceinline__ uint64_t wait_check(uint64_t since, volatile int* abort_flag, int* status, int code, uint64_t limit_ns) {
+  if (*abort_flag != 0) return 0;
+  if (status != nullptr && *reinterpret_cast<volatile int*>(status) != 0) {  // another CTA already gave up
+    *abort_flag = code;
+    return 0;
+  }
+  const uint64_t now = global_timer_ns();
+  if (since == 0) return now;
+  if (now - since <= limit_ns) return since;
+  *abort_flag = code;
+  if (status != nullptr) atomicCAS(status, 0, code);
+  return 0;
+}
 __device__ __forceinline__ bool mbar_wait_loop(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                int code, uint32_t backoff_ns, uint64_t limit_ns) {
-  const uint64_t t0 = global_timer_ns();
+  uint64_t since = 0;
   uint32_t polls = 0;
   while (true) {
     if (backoff_ns != 0) __nanosleep(backoff_ns);
     if (mbar_try_wait(bar, parity)) return true;
-    if ((++polls & 0xFu) == 0) {
-      if (*abort_flag != 0) return false;
-      if (status != nullptr && *reinterpret_cast<volatile int*>(status) != 0) {  // another CTA already gave up
-        *abort_flag = code;
-        return false;
-      }
-      if (global_timer_ns() - t0 > limit_ns) {
-        *abort_flag = code;
-        if (status != nullptr) atomicCAS(status, 0, code);
-        return false;
-      }
-    }
+    if ((++polls & 0x3Fu) == 0 && (since = wait_check(since, abort_flag, status, code, limit_ns)) == 0) return false;
   }
 }
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                           int code, uint32_t backoff_ns = 0, uint64_t limit_ns = kWaitLimitNs) {
-  if (mbar_test(bar, parity)) return true;
+  if (mbar_try_wait(bar, parity)) return true;  // woken by the hardware; the clock is read only after that
   return mbar_wait_loop(bar, parity, abort_flag, status, code, backoff_ns, limit_ns);
 }
-// The same wait with its polling loop in a function of its own (not inlined): a wait that succeeds at once costs the
-// caller two instructions, which keeps a hot loop with several waits small enough for the instruction caches.
-static __device__ __noinline__ bool mbar_wait_loop_far(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                                       int* status, int code) {
-  return mbar_wait_loop(bar, parity, abort_flag, status, code, 0, kWaitLimitNs);
+// The same wait with everything but its polls in a function of its own (not inlined): a wait costs its caller a handful
+// of instructions, which keeps a kernel with many waits small enough for the instruction caches.  kRole gives warps
+// with different register budgets (setmaxnreg) a copy each.
+template <int kRole>
+static __device__ __noinline__ uint64_t wait_check_far(uint64_t since, volatile int* abort_flag, int* status, int code) {
+  return wait_check(since, abort_flag, status, code, kWaitLimitNs);
 }
+template <int kRole = 0>
 __device__ __forceinline__ bool mbar_wait_far(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                               int code) {
-  if (mbar_test(bar, parity)) return true;
-  return mbar_wait_loop_far(bar, parity, abort_flag, status, code);
+  uint64_t since = 0;
+  uint32_t polls = 0;
+#pragma unroll 1
+  while (!mbar_try_wait(bar, parity)) {
+    if ((++polls & 0x3Fu) == 0 && (since = wait_check_far<kRole>(since, abort_flag, status, code)) == 0) return false;
+  }
+  return true;
 }
 
 // Bounded idling for a single-thread role that polls several barriers without blocking on any of them: call
