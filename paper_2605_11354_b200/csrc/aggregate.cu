@@ -48,7 +48,6 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed cha
   extern __shared__ __align__(1024) uint8_t smem[];
   Bars* bars = reinterpret_cast<Bars*>(smem + kOffBar);
   volatile int* abort_flag = &bars->abort;
-  if (status != nullptr && *reinterpret_cast<volatile int*>(status) != 0) return;
   if ((smem_u32(smem) & 1023u) != 0) {
     if (threadIdx.x == 0 && status != nullptr) atomicCAS(status, 0, 901);
     return;
@@ -92,8 +91,10 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed cha
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
-  // The attention kernel that follows needs this kernel's results only at its very end: it may be scheduled as soon
-  // as every CTA of this grid has its tensor memory (it waits for the grid's completion itself before it reads G and zeta).
+  wait_for_prior_grid();
+  // The attention kernel that follows needs this kernel's results only at the end of a tile: it may be scheduled as soon
+  // as every CTA of this grid has its tensor memory and knows the summaries complete (it waits for this grid's completion
+  // itself before it reads G and zeta).
   sm100::launch_dependents();
 
   if (warp == 0) {
@@ -253,25 +254,13 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed cha
 }  // namespace
 
 lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls, const lite3r_shape& s, int nb,
-                               __nv_bfloat16* g16, float* zeta, int* device_status, cudaStream_t stream) {
+                               __nv_bfloat16* g16, float* zeta, int* device_status, bool after_wait, cudaStream_t stream) {
   const uint64_t rows = static_cast<uint64_t>(s.batch) * s.heads * nb;
-  // the tensor map of the summaries is kept from the calling thread's previous call while buffer and size repeat
-  struct MapCache {
-    alignas(64) CUtensorMap map;
-    const void* base = nullptr;
-    uint64_t rows = 0;
-  };
-  thread_local MapCache cache;
+  const CUtensorMap* const map = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hws, kSummaryRow, rows, 64, 64,
+                                                    CU_TENSOR_MAP_SWIZZLE_128B);
+  if (map == nullptr) return LITE3R_ERR_CUDA;
+  const CUtensorMap map_s = *map;
   lite3r_status st;
-  if (cache.base != hws || cache.rows != rows) {
-    cache.base = nullptr;
-    st = make_tensor_map_2d(&cache.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hws, kSummaryRow, rows, 64, 64,
-                            CU_TENSOR_MAP_SWIZZLE_128B);
-    if (st != LITE3R_OK) return st;
-    cache.base = hws;
-    cache.rows = rows;
-  }
-  const CUtensorMap& map_s = cache.map;
   st = ensure_dynamic_smem(aggregate_mma_kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
   if (rows > 0x7FFFFFFFull - kTileM) return LITE3R_ERR_UNSUPPORTED;
@@ -300,8 +289,12 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   const double time_flat = static_cast<double>((ctas_flat + slots - 1) / slots) * (kFixed + flat_chunks);
   const int flat = time_flat < time_inside ? 1 : 0;
   const dim3 grid(ceil_div(kSummaryRow, kTileN), flat ? ceil_div(total_rows, kTileM) : ceil_div(nb, kTileM), flat ? 1 : bh);
-  aggregate_mma_kernel<<<grid, kThreads, kSmemBytes, stream>>>(map_s, cls, nb, total_rows, flat, g16, zeta, device_status);
-  return after_launch();
+  if (after_wait) {
+    aggregate_mma_kernel<<<grid, kThreads, kSmemBytes, stream>>>(map_s, cls, nb, total_rows, flat, g16, zeta, device_status);
+    return after_launch();
+  }
+  return launch_dependent(aggregate_mma_kernel, grid, kThreads, static_cast<int>(kSmemBytes), stream, map_s, cls, nb, total_rows,
+                          flat, g16, zeta, device_status);
 }
 
 }  // namespace lite3r

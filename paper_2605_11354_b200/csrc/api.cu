@@ -2,6 +2,8 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstring>
+#include <memory>
 #include <mutex>
 #include <unordered_map>
 
@@ -119,48 +121,66 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-lite3r_status make_tensor_map_2d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base,
-                                 uint64_t inner, uint64_t rows, uint32_t box_inner, uint32_t box_rows,
-                                 CUtensorMapSwizzle swizzle) {
-  EncodeTiledFn fn = encode_fn();
-  if (fn == nullptr) return LITE3R_ERR_CUDA;
-  const cuuint64_t dims[2] = {inner, rows};
-  const cuuint64_t strides[1] = {inner * static_cast<cuuint64_t>(elem_bytes)};
-  const cuuint32_t box[2] = {box_inner, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = fn(map, type, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? LITE3R_OK : LITE3R_ERR_CUDA;
-}
+namespace {
+// Everything a descriptor depends on; unused extents stay 0.
+struct MapKey {
+  const void* base;
+  uint64_t dims[4], strides[3];
+  uint32_t box[4];
+  int type, rank, swizzle, l2;
+};
+struct MapSlot {
+  alignas(64) CUtensorMap map;
+  MapKey key;
+};
+constexpr uint32_t kMapSlots = 512, kMapWays = 4;  // per thread; 512 x 256 bytes
 
-lite3r_status make_tensor_map_3d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base,
-                                 uint64_t inner, uint64_t rows, uint64_t planes, uint32_t box_inner, uint32_t box_rows,
-                                 CUtensorMapSwizzle swizzle) {
+const CUtensorMap* cached_map(const MapKey& key) {
+  thread_local std::unique_ptr<MapSlot[]> slots;
+  thread_local uint32_t next_way = 0;
+  if (!slots) slots.reset(new MapSlot[kMapSlots]());
+  const uint64_t* words = reinterpret_cast<const uint64_t*>(&key);
+  static_assert(sizeof(MapKey) % 8 == 0, "hashed by words");
+  uint64_t h = 0;
+  for (size_t i = 0; i < sizeof(MapKey) / 8; ++i) h = (h ^ words[i]) * 0x9E3779B97F4A7C15ull, h ^= h >> 29;
+  MapSlot* const set = slots.get() + (h % (kMapSlots / kMapWays)) * kMapWays;
+  for (uint32_t w = 0; w < kMapWays; ++w)
+    if (std::memcmp(&set[w].key, &key, sizeof(MapKey)) == 0) return &set[w].map;
   EncodeTiledFn fn = encode_fn();
-  if (fn == nullptr) return LITE3R_ERR_CUDA;
-  const cuuint64_t dims[3] = {inner, rows, planes};
-  const cuuint64_t strides[2] = {inner * static_cast<cuuint64_t>(elem_bytes),
-                                 inner * rows * static_cast<cuuint64_t>(elem_bytes)};
-  const cuuint32_t box[3] = {box_inner, box_rows, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = fn(map, type, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? LITE3R_OK : LITE3R_ERR_CUDA;
-}
-
-// Rank-4 map over a tensor whose innermost dimension is contiguous: extents dims[0..3], byte strides of dimensions
-// 1..3 (multiples of 16), box of box[0..3] elements.
-lite3r_status make_tensor_map_4d(CUtensorMap* map, CUtensorMapDataType type, const void* base, const uint64_t dims[4],
-                                 const uint64_t strides_bytes[3], const uint32_t box[4], CUtensorMapSwizzle swizzle) {
-  EncodeTiledFn fn = encode_fn();
-  if (fn == nullptr) return LITE3R_ERR_CUDA;
-  const cuuint64_t d[4] = {dims[0], dims[1], dims[2], dims[3]};
-  const cuuint64_t st[3] = {strides_bytes[0], strides_bytes[1], strides_bytes[2]};
-  const cuuint32_t bx[4] = {box[0], box[1], box[2], box[3]};
+  if (fn == nullptr) return nullptr;
+  MapSlot& slot = set[next_way++ % kMapWays];
+  slot.key = MapKey{};  // stays invalid if the driver refuses
   const cuuint32_t estr[4] = {1, 1, 1, 1};
-  const CUresult r = fn(map, type, 4, const_cast<void*>(base), d, st, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
-                        CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? LITE3R_OK : LITE3R_ERR_CUDA;
+  cuuint64_t dims[4], strides[3];
+  for (int i = 0; i < 4; ++i) dims[i] = key.dims[i];
+  for (int i = 0; i < 3; ++i) strides[i] = key.strides[i];
+  if (fn(&slot.map, static_cast<CUtensorMapDataType>(key.type), static_cast<cuuint32_t>(key.rank), const_cast<void*>(key.base), dims,
+         strides, key.box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, static_cast<CUtensorMapSwizzle>(key.swizzle),
+         static_cast<CUtensorMapL2promotion>(key.l2), CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return nullptr;
+  slot.key = key;
+  return &slot.map;
+}
+}  // namespace
+
+const CUtensorMap* make_tensor_map_2d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
+                                      uint64_t rows, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle) {
+  return cached_map({base, {inner, rows, 0, 0}, {inner * static_cast<uint64_t>(elem_bytes), 0, 0}, {box_inner, box_rows, 0, 0},
+                     type, 2, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B});
+}
+
+const CUtensorMap* make_tensor_map_3d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
+                                      uint64_t rows, uint64_t planes, uint32_t box_inner, uint32_t box_rows,
+                                      CUtensorMapSwizzle swizzle) {
+  const uint64_t pitch = inner * static_cast<uint64_t>(elem_bytes);
+  return cached_map({base, {inner, rows, planes, 0}, {pitch, pitch * rows, 0}, {box_inner, box_rows, 1, 0}, type, 3, swizzle,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B});
+}
+
+const CUtensorMap* make_tensor_map_4d(CUtensorMapDataType type, const void* base, const uint64_t dims[4],
+                                      const uint64_t strides_bytes[3], const uint32_t box[4], CUtensorMapSwizzle swizzle) {
+  return cached_map({base, {dims[0], dims[1], dims[2], dims[3]}, {strides_bytes[0], strides_bytes[1], strides_bytes[2]},
+                     {box[0], box[1], box[2], box[3]}, type, 4, swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE});
 }
 
 Counts class_counts(int nb, double crit, double neg) {
@@ -466,7 +486,6 @@ lite3r_status lite3r_proj_lin_backward(const void* o_lin, const void* d_out, con
   if (workspace_bytes < train_workspace_bytes(*shape)) return LITE3R_ERR_WORKSPACE;
   if ((st = check_device()) != LITE3R_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  if (device_status != nullptr && (st = record_cuda(cudaMemsetAsync(device_status, 0, sizeof(int), cs))) != LITE3R_OK) return st;
   return launch_proj_lin_backward(static_cast<const __nv_bfloat16*>(o_lin), static_cast<const __nv_bfloat16*>(d_out), *shape,
                                   d_proj, static_cast<float*>(workspace), device_status, cs);
 }
@@ -513,7 +532,6 @@ lite3r_status lite3r_linear_fp8(const unsigned char* x_codes, const float* x_sca
   if (y == nullptr || !aligned(y, 16) || y_stride < d_out || (y_stride % 8)) return LITE3R_ERR_INVALID_ARG;
   if ((st = check_device()) != LITE3R_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  if (device_status != nullptr && (st = record_cuda(cudaMemsetAsync(device_status, 0, sizeof(int), cs))) != LITE3R_OK) return st;
   return launch_linear_fp8(x_codes, x_scales, w_codes, w_scales, bias, rows, d_in, d_out, y, static_cast<int>(y_dtype),
                            y_stride, device_status, cs);
 }
@@ -533,7 +551,6 @@ lite3r_status lite3r_qkv_project_fp8(const unsigned char* x_codes, const float* 
     if ((st = check_fp8(&out[i], true, false)) != LITE3R_OK) return st;
   if ((st = check_device()) != LITE3R_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  if (device_status != nullptr && (st = record_cuda(cudaMemsetAsync(device_status, 0, sizeof(int), cs))) != LITE3R_OK) return st;
   return launch_qkv_project(x_codes, x_scales, w_codes, w_scales, bias, *shape, d_model, out, device_status, cs);
 }
 

@@ -15,7 +15,7 @@
 // and SM: 512 clocks per step); the products of a step take 384 clocks of tensor pipe at block 64 (M = 64 runs at half
 // rate) and 192 at block 128.  A warp alone needs some 1100 clocks for its 32 x 64 scores (loads, stores and barriers
 // included), so two warps per scheduler are the least that can keep the unit busy and three do it comfortably: S, P and O
-// take 160 TMEM columns (an allocation of 128 and one of 32), 74 KB of shared memory and 80 registers per thread, and
+// take 160 TMEM columns, 74 KB of shared memory and 80 registers per thread, and
 // THREE CTAs fit on an SM.  Measured at 10 % of 2147 key blocks: 650 clocks per step and SM (two CTAs with two softmax
 // warpgroups each on alternate steps of one tile, as before: 757).
 // A CTA takes tile after tile: it asks the hardware's work scheduler for a CTA that has not been launched yet and computes
@@ -55,9 +55,11 @@ constexpr int kCtasPerSm = 3;
 constexpr int kCtrlRegs = 48, kSoftmaxRegs = 112;  // 128 * 48 + 128 * 112 = 256 * 80, the launch allocation
 constexpr int kStepKeys = 64;
 constexpr int kStages = 2;  // K ring and V ring
-// TMEM: 64 columns of scores (later the product of the linear branch) and 64 of O in one allocation, 32 columns of
-// probabilities (packed fp16) in another.
-constexpr uint32_t kColsSO = 128, kColsP = 32, kColO = 64;
+// TMEM: 64 columns of scores (later the product of the linear branch), 64 of O, 32 of probabilities (packed fp16), each an
+// allocation of its own, the smallest first: three CTAs then fit in whatever order they come and beside whatever an earlier
+// kernel's last CTAs still hold.  (With one allocation of 128 columns and one of 32, a 32 left in the middle by such a
+// start kept the third CTA out of an SM for the whole grid: 6 % at 16 heads of 137400 tokens.)
+constexpr uint32_t kColsS = 64, kColsO = 64, kColsP = 32;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleThreshold = 8.0f;  // lazy rescale: keep the old reference until it is beaten by 2^8
 constexpr float kNoMax = -1.0e30f;    // reference maximum of a row that has seen no valid key yet
@@ -85,7 +87,7 @@ struct Bars {
   uint64_t v_done[kStages];                   // product number n of the V ring complete (n % 2) -> softmax (P free, O or
                                               // the linear product valid), producer (V stage free)
   uint64_t s_free, p_full;                    // softmax -> issuers: score columns read / probabilities stored
-  uint32_t tmem_so, tmem_p;
+  uint32_t tmem_s, tmem_o, tmem_p;
   int abort;
 };
 static_assert(sizeof(Bars) <= 256, "barrier block");
@@ -100,6 +102,7 @@ struct AttnParams {
   int heads, tokens, nb, tiles_per_head, k_crit, k_marg, phi, out_dtype;
   // output through TMA stores (map_o): position of the token / head / batch dimension among the map's dimensions
   // 1..3 (they are ordered by stride); tma_out = 0: plain stores
+  int wait_first;  // the preceding launch must have completed before anything is read
   int steal;  // more tiles than CTAs fit on the chip: CTAs take over the tiles of CTAs not yet launched
   int tma_out, dim_token, dim_head, dim_batch;
   int* status;
@@ -284,14 +287,17 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     mbar_fence_init();
   }
   if (warp == 1) {
-    tmem_alloc(&bars->tmem_so, kColsSO);
     tmem_alloc(&bars->tmem_p, kColsP);
+    tmem_alloc(&bars->tmem_s, kColsS);
+    tmem_alloc(&bars->tmem_o, kColsO);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_so = __shfl_sync(0xFFFFFFFFu, bars->tmem_so, 0), tmem_p = __shfl_sync(0xFFFFFFFFu, bars->tmem_p, 0);
+  const uint32_t tmem_s = __shfl_sync(0xFFFFFFFFu, bars->tmem_s, 0), tmem_o = __shfl_sync(0xFFFFFFFFu, bars->tmem_o, 0);
+  const uint32_t tmem_p = __shfl_sync(0xFFFFFFFFu, bars->tmem_p, 0);
+  if (p.wait_first) wait_for_prior_grid();
   volatile int* const tile_ids = reinterpret_cast<volatile int*>(smem + kOffNext + 16);
   // number of the CTA's tile after `it` tiles (-1: none is left, -2: a wait has expired), from the producer
   auto next_tile = [&](int it, int code, auto role) {
@@ -458,7 +464,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
             for (int hf = 0; hf < kHalves; ++hf)
-              mma_f8(tmem_so + ((hf * 16u) << 16), q_desc + ((hf * 4096 + kk * 32) >> 4), k_desc + ((hf * 4096 + kk * 32) >> 4),
+              mma_f8(tmem_s + ((hf * 16u) << 16), q_desc + ((hf * 4096 + kk * 32) >> 4), k_desc + ((hf * 4096 + kk * 32) >> 4),
                      idesc_qk, kk);
           }
           mma_commit(&bars->s_full[st]);
@@ -477,7 +483,6 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     constexpr uint32_t idesc_pv = instr_desc(0, kM, 64, 0, 1);   // f16 x f16, P from TMEM, V MN-major
     constexpr uint32_t idesc_lin = instr_desc(1, kM, 64, 0, 0);  // bf16 x bf16, both K-major
     const uint64_t v_desc0 = smem_desc(smem_u32(smem + kOffV), 8192, 1024, kSwizzle128);
-    const uint32_t o_tmem = tmem_so + kColO;
     bool ok = true;
     int vc = 0, pc = 0;  // V-ring entries, probability tiles, through all tiles
 #pragma unroll 1
@@ -496,7 +501,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int kk = 0; kk < 4; ++kk) {
 #pragma unroll
             for (int hf = 0; hf < kHalves; ++hf)
-              mma_f16_ts(o_tmem + ((hf * 16u) << 16), tmem_p + ((hf * 16u) << 16) + kk * 8,
+              mma_f16_ts(tmem_o + ((hf * 16u) << 16), tmem_p + ((hf * 16u) << 16) + kk * 8,
                          v_desc + ((hf * 8192 + kk * 2048) >> 4), idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
           }
           mma_commit(&bars->v_done[st]);
@@ -519,7 +524,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int kk = 0; kk < 4; ++kk) {
 #pragma unroll
             for (int hf = 0; hf < kHalves; ++hf)
-              mma_f16(tmem_so + ((hf * 16u) << 16), a0 + ((hf * 8192 + kk * 32) >> 4), b0 + ((hf * 8192 + kk * 32) >> 4), idesc_lin, kk);
+              mma_f16(tmem_s + ((hf * 16u) << 16), a0 + ((hf * 8192 + kk * 32) >> 4), b0 + ((hf * 8192 + kk * 32) >> 4), idesc_lin, kk);
           }
           mma_commit(&bars->v_done[st]);
         }
@@ -535,7 +540,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int row_in_block = kPair ? quarter * 16 + (lane & 15) : quarter * 32 + lane;
     const int p_row = kPair ? hf * 64 + row_in_block : row_in_block;  // row inside the 128-row tile
     const uint32_t lane_off = (static_cast<uint32_t>(quarter) * 32u) << 16;
-    const uint32_t s_addr = tmem_so + lane_off, o_addr = tmem_so + kColO + lane_off, p_addr = tmem_p + lane_off;
+    const uint32_t s_addr = tmem_s + lane_off, o_addr = tmem_o + lane_off, p_addr = tmem_p + lane_off;
     const uint32_t scal_slot = smem_u32(smem + kOffScal) + hf * 8;
     const int swz = p_row & 7;
     // hands the probabilities of the step just finished to the P V issuer
@@ -823,7 +828,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_p, kColsP);
-    tmem_dealloc(tmem_so, kColsSO);
+    tmem_dealloc(tmem_s, kColsS);
+    tmem_dealloc(tmem_o, kColsO);
   }
 }
 
@@ -836,96 +842,59 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   const lite3r_shape& s = a.shape;
   const int nb = ceil_div(s.tokens, BS);
   const uint64_t tiles = static_cast<uint64_t>(s.batch) * s.heads * nb;
-  // The four tensor maps depend on the buffers and the shape only; a caller that runs the same buffers again (the
-  // usual serving loop) reuses the encoded maps of its previous call (one entry per calling thread).
-  struct MapCache {
-    alignas(64) CUtensorMap q, k, v, g, o;
-    const void* key[4] = {nullptr, nullptr, nullptr, nullptr};
-    uint64_t tiles = 0;
-    int block = 0;
-    // the output map
-    const void* out = nullptr;
-    long long out_strides[3] = {0, 0, 0};
-    int out_dims[3] = {0, 0, 0}, out_dtype = -1, out_ok = 0, dim_token = 1, dim_head = 2, dim_batch = 3;
-  };
-  thread_local MapCache cache;
-  lite3r_status st;
-  if (cache.key[0] != a.q_codes || cache.key[1] != a.k_codes || cache.key[2] != a.v16 || cache.key[3] != a.g16 ||
-      cache.tiles != tiles || cache.block != BS) {
-    cache.key[0] = nullptr;  // stays invalid if an encode below fails
-    if ((st = make_tensor_map_2d(&cache.q, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.q_codes, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B)) != LITE3R_OK) return st;
-    if ((st = make_tensor_map_2d(&cache.k, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.k_codes, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B)) != LITE3R_OK) return st;
-    if ((st = make_tensor_map_2d(&cache.v, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, a.v16, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
-    if ((st = make_tensor_map_2d(&cache.g, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.g16, 64, tiles * 64, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
-    cache.key[0] = a.q_codes;
-    cache.key[1] = a.k_codes;
-    cache.key[2] = a.v16;
-    cache.key[3] = a.g16;
-    cache.tiles = tiles;
-    cache.block = BS;
-  }
+  const CUtensorMap* const ptrs[4] = {
+      make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.q_codes, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B),
+      make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.k_codes, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B),
+      make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, a.v16, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B),
+      make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.g16, 64, tiles * 64, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)};
+  for (const CUtensorMap* m : ptrs)
+    if (m == nullptr) return LITE3R_ERR_CUDA;
+  const CUtensorMap map_q = *ptrs[0], map_k = *ptrs[1], map_v = *ptrs[2], map_g = *ptrs[3];
+  lite3r_status st = LITE3R_OK;
+  AttnParams p;
   // The output goes through TMA stores when a tiled map can describe it: the token, head and batch dimensions ordered
   // by stride (dimensions of extent 1 last), 16 tokens x 128 bytes per box.  If the driver refuses the map the kernel
   // falls back to plain stores.
-  if (cache.out != a.out || cache.out_dtype != a.out_dtype || cache.out_strides[0] != a.out_stride_n ||
-      cache.out_strides[1] != a.out_stride_h || cache.out_strides[2] != a.out_stride_b || cache.out_dims[0] != s.tokens ||
-      cache.out_dims[1] != s.heads || cache.out_dims[2] != s.batch) {
-    const int elem = a.out_dtype == LITE3R_F32 ? 4 : 2;
-    struct Dim {
-      long long stride;
-      int extent, which;  // which: 0 token, 1 head, 2 batch
-    } dm[3] = {{a.out_stride_n, s.tokens, 0}, {a.out_stride_h, s.heads, 1}, {a.out_stride_b, s.batch, 2}};
-    // order: extents above 1 by ascending stride, then the extent-1 dimensions (whose stride does not matter)
-    auto before = [](const Dim& x, const Dim& y) {
-      if ((x.extent > 1) != (y.extent > 1)) return x.extent > 1;
-      if (x.extent > 1 && x.stride != y.stride) return x.stride < y.stride;
-      return x.which < y.which;
-    };
-    for (int i = 0; i < 3; ++i)
-      for (int j = i + 1; j < 3; ++j)
-        if (before(dm[j], dm[i])) std::swap(dm[i], dm[j]);
-    uint64_t dims[4] = {kHeadDim, 0, 0, 0}, strides[3];
-    uint32_t box[4] = {128u / elem, 1, 1, 1};  // 128 bytes of a row
-    uint64_t packed = static_cast<uint64_t>(kHeadDim) * elem;  // stride a dimension would have if packed after the previous ones
-    bool ok = (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0;
-    for (int i = 0; i < 3; ++i) {
-      dims[i + 1] = static_cast<uint64_t>(dm[i].extent);
-      strides[i] = dm[i].extent > 1 ? static_cast<uint64_t>(dm[i].stride) * elem : packed;
-      ok = ok && strides[i] > 0 && (strides[i] & 15u) == 0;
-      packed = strides[i] * dims[i + 1];
-      if (dm[i].which == 0) {
-        box[i + 1] = 16;
-        cache.dim_token = i + 1;
-      } else if (dm[i].which == 1) {
-        cache.dim_head = i + 1;
-      } else {
-        cache.dim_batch = i + 1;
-      }
+  const int elem = a.out_dtype == LITE3R_F32 ? 4 : 2;
+  struct Dim {
+    long long stride;
+    int extent, which;  // which: 0 token, 1 head, 2 batch
+  } dm[3] = {{a.out_stride_n, s.tokens, 0}, {a.out_stride_h, s.heads, 1}, {a.out_stride_b, s.batch, 2}};
+  // order: extents above 1 by ascending stride, then the extent-1 dimensions (whose stride does not matter)
+  auto before = [](const Dim& x, const Dim& y) {
+    if ((x.extent > 1) != (y.extent > 1)) return x.extent > 1;
+    if (x.extent > 1 && x.stride != y.stride) return x.stride < y.stride;
+    return x.which < y.which;
+  };
+  for (int i = 0; i < 3; ++i)
+    for (int j = i + 1; j < 3; ++j)
+      if (before(dm[j], dm[i])) std::swap(dm[i], dm[j]);
+  uint64_t dims[4] = {kHeadDim, 0, 0, 0}, strides[3];
+  uint32_t box[4] = {128u / elem, 1, 1, 1};  // 128 bytes of a row
+  uint64_t packed = static_cast<uint64_t>(kHeadDim) * elem;  // stride a dimension would have if packed after the previous ones
+  bool describable = (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0;
+  for (int i = 0; i < 3; ++i) {
+    dims[i + 1] = static_cast<uint64_t>(dm[i].extent);
+    strides[i] = dm[i].extent > 1 ? static_cast<uint64_t>(dm[i].stride) * elem : packed;
+    describable = describable && strides[i] > 0 && (strides[i] & 15u) == 0;
+    packed = strides[i] * dims[i + 1];
+    if (dm[i].which == 0) {
+      box[i + 1] = 16;
+      p.dim_token = i + 1;
+    } else if (dm[i].which == 1) {
+      p.dim_head = i + 1;
+    } else {
+      p.dim_batch = i + 1;
     }
-    cache.out_ok = 0;
-    if (ok) {
-      const CUtensorMapDataType type = a.out_dtype == LITE3R_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                       : a.out_dtype == LITE3R_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
-                                                                    : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-      cache.out_ok = make_tensor_map_4d(&cache.o, type, a.out, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) == LITE3R_OK ? 1 : 0;
-    }
-    cache.out = a.out;
-    cache.out_dtype = a.out_dtype;
-    cache.out_strides[0] = a.out_stride_n;
-    cache.out_strides[1] = a.out_stride_h;
-    cache.out_strides[2] = a.out_stride_b;
-    cache.out_dims[0] = s.tokens;
-    cache.out_dims[1] = s.heads;
-    cache.out_dims[2] = s.batch;
   }
-  const CUtensorMap &map_q = cache.q, &map_k = cache.k, &map_v = cache.v, &map_g = cache.g;
-  const bool tma_out = cache.out_ok != 0 && g_plain_stores.load(std::memory_order_relaxed) == 0;
-  const CUtensorMap& map_o = tma_out ? cache.o : cache.q;  // any valid map when it is not used
-  AttnParams p;
-  p.tma_out = tma_out ? 1 : 0;
-  p.dim_token = cache.dim_token;
-  p.dim_head = cache.dim_head;
-  p.dim_batch = cache.dim_batch;
+  const CUtensorMap* out_map = nullptr;
+  if (describable && g_plain_stores.load(std::memory_order_relaxed) == 0)
+    out_map = make_tensor_map_4d(a.out_dtype == LITE3R_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                 : a.out_dtype == LITE3R_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                              : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
+                                 a.out, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+  p.tma_out = out_map != nullptr ? 1 : 0;
+  const CUtensorMap map_o = out_map != nullptr ? *out_map : map_q;  // any valid map when it is not used
   p.q_scales = a.q_scales;
   p.k_scales = a.k_scales;
   p.crit_idx = a.crit_idx;
@@ -949,25 +918,11 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   int sms = 0;
   if ((st = sm_count(&sms)) != LITE3R_OK) return st;
   p.steal = ctas > sms * kCtasPerSm ? 1 : 0;
-  if (a.overlap_prior) {
-    // programmatic dependent launch: the kernel may start while the preceding one (which announces it early) is
-    // still running, and waits for its completion itself before it reads that kernel's results
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(ctas));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, attention_kernel<BS>, map_q, map_k, map_v, map_g, map_o, p);
-    if (err != cudaSuccess) return record_cuda(err);
-    return after_launch();
-  }
-  attention_kernel<BS><<<ctas, kThreads, kSmemBytes, stream>>>(map_q, map_k, map_v, map_g, map_o, p);
-  return after_launch();
+  // With a linear branch the launch before this one is the aggregation, whose results are needed only at a tile's end: the
+  // kernel then runs beside it and waits for its completion itself.  Otherwise it waits before it reads anything.
+  p.wait_first = a.overlap_prior ? 0 : 1;
+  return launch_dependent(attention_kernel<BS>, dim3(static_cast<unsigned>(ctas)), kThreads, static_cast<int>(kSmemBytes), stream,
+                          map_q, map_k, map_v, map_g, map_o, p);
 }
 
 }  // namespace

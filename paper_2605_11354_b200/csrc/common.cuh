@@ -41,6 +41,26 @@ lite3r_status ensure_dynamic_smem(K* kernel, int bytes) {
   return ensure_smem_limit(reinterpret_cast<const void*>(kernel), bytes);
 }
 
+// Enqueues a kernel as a programmatic dependent of the launch before it in the stream: it may start while that one is
+// still running, and waits (griddepcontrol.wait) before it touches anything that one reads or writes.  Every kernel of
+// the library that is launched this way lets its own successor start early as soon as its set-up is done.
+template <typename... Params, typename... Args>
+lite3r_status launch_dependent(void (*kernel)(Params...), dim3 grid, int block, int smem_bytes, cudaStream_t stream,
+                               const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(static_cast<unsigned>(block));
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem_bytes);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const lite3r_status st = record_cuda(cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...));
+  return st == LITE3R_OK ? after_launch() : st;
+}
+
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 struct Counts {
@@ -126,19 +146,30 @@ lite3r_status launch_attention(const AttentionLaunch& a, cudaStream_t stream);
 void set_attention_plain_stores(int on);  // test hook, see lite3r_attention_plain_stores
 
 // Per-key-block summaries ((H_j W)^T | z_j) in bf16, one kSummaryRow-wide row per (b, h, key block).
+// Clears *device_status; after_wait as in launch_aggregate.
 lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const float* proj, long long proj_head_stride,
                              const lite3r_shape& s, int phi, __nv_bfloat16* hws, __half* v16, int* device_status,
-                             cudaStream_t stream);
+                             bool after_wait, cudaStream_t stream);
 
 // Marginal aggregation G_i = sum over marginal j of the summary rows, as a 0/1-mask GEMM on tensor cores.
+// after_wait: the stream has just waited for an event (the launch is then an ordinary one).
 lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls, const lite3r_shape& s, int nb,
-                               __nv_bfloat16* g16, float* zeta, int* device_status, cudaStream_t stream);
+                               __nv_bfloat16* g16, float* zeta, int* device_status, bool after_wait, cudaStream_t stream);
 
 // TMA descriptor of a row-major 2-D tensor [rows][inner] (row pitch = inner * elem_bytes, a multiple of 16 bytes)
-// with a box of box_inner x box_rows elements.
-lite3r_status make_tensor_map_2d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base,
-                                 uint64_t inner, uint64_t rows, uint32_t box_inner, uint32_t box_rows,
-                                 CUtensorMapSwizzle swizzle);
+// with a box of box_inner x box_rows elements.  The make_tensor_map functions return a descriptor kept by the calling
+// thread (valid until the thread has asked for a few hundred others): descriptors depend on their arguments only, and a
+// caller that runs the same buffers again, or those of many layers in turn, finds them encoded.  NULL: refused.
+const CUtensorMap* make_tensor_map_2d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
+                                      uint64_t rows, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle);
+// The same for a 3-D tensor [planes][rows][inner] with a box of box_inner x box_rows x 1 (rows past the end of a plane
+// are zero-filled, so a tile never runs into the next plane).
+const CUtensorMap* make_tensor_map_3d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
+                                      uint64_t rows, uint64_t planes, uint32_t box_inner, uint32_t box_rows,
+                                      CUtensorMapSwizzle swizzle);
+// Rank 4, extents dims[0..3], byte strides of dimensions 1..3 (multiples of 16), box of box[0..3] elements.
+const CUtensorMap* make_tensor_map_4d(CUtensorMapDataType type, const void* base, const uint64_t dims[4],
+                                      const uint64_t strides_bytes[3], const uint32_t box[4], CUtensorMapSwizzle swizzle);
 
 // The FP8 linear layer in front of the attention (linear.cu).
 lite3r_status launch_rowquant(const void* x, int dtype, long long row_stride, int rows, int cols, uint8_t* codes,
@@ -149,14 +180,6 @@ lite3r_status launch_linear_fp8(const uint8_t* x_codes, const float* x_scales, c
 lite3r_status launch_qkv_project(const uint8_t* x_codes, const float* x_scales, const uint8_t* w_codes,
                                  const float* w_scales, const float* bias, const lite3r_shape& s, int d_model,
                                  const lite3r_fp8* out, int* device_status, cudaStream_t stream);
-
-// The same for a 3-D tensor [planes][rows][inner] with a box of box_inner x box_rows x 1 (rows past the end of a plane
-// are zero-filled, so a tile never runs into the next plane).
-lite3r_status make_tensor_map_4d(CUtensorMap* map, CUtensorMapDataType type, const void* base, const uint64_t dims[4],
-                                 const uint64_t strides_bytes[3], const uint32_t box[4], CUtensorMapSwizzle swizzle);
-lite3r_status make_tensor_map_3d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base,
-                                 uint64_t inner, uint64_t rows, uint64_t planes, uint32_t box_inner, uint32_t box_rows,
-                                 CUtensorMapSwizzle swizzle);
 
 // Training side of the linear-branch projection (train.cu).
 size_t train_workspace_bytes(const lite3r_shape& s);

@@ -19,7 +19,10 @@ namespace {
 // ------------------------------------------------------------------------------------------------ prep
 // Dequantised V (code value x block scale) as fp16, the B operand of the P V tensor-core product.
 __global__ void __launch_bounds__(256) prep_kernel(const uint8_t* __restrict__ v_codes, const float* __restrict__ v_scales,
-                                                   size_t words, int words_per_tile, __half* __restrict__ v16) {
+                                                   size_t words, int words_per_tile, __half* __restrict__ v16, int* status) {
+  sm100::wait_for_prior_grid();
+  sm100::launch_dependents();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && status != nullptr) *status = 0;
   const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
   for (size_t w = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; w < words; w += stride) {
     const uint4 packed = __ldg(reinterpret_cast<const uint4*>(v_codes) + w);
@@ -123,21 +126,22 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
     int sms = 0;
     if ((st = sm_count(&sms)) != LITE3R_OK) return st;
     const int blocks = static_cast<int>(std::min<size_t>((words + 255) / 256, static_cast<size_t>(sms) * 8));
-    prep_kernel<<<blocks, 256, 0, stream>>>(a.v.codes, a.v.scales, words, BS * kHeadDim / 16, w.v16);
-    if ((st = after_launch()) != LITE3R_OK) return st;
+    st = launch_dependent(prep_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, stream, a.v.codes, a.v.scales, words,
+                          BS * kHeadDim / 16, w.v16, a.device_status);
+    if (st != LITE3R_OK) return st;
     profile_mark(1, stream);
   }
   if ((phases & 1) && a.plan.k_marg > 0) {
     profile_mark(2, stream);
     st = launch_summary(a.k, a.v, a.proj, a.proj_head_stride, s, a.phi, w.hws, a.plan.k_crit > 0 ? w.v16 : nullptr,
-                        a.device_status, stream);
+                        a.device_status, phases != 3, stream);
     if (st != LITE3R_OK) return st;
     profile_mark(3, stream);
   }
   if (!(phases & 2)) return st;
   if (a.plan.k_marg > 0) {
     profile_mark(4, stream);
-    if ((st = launch_aggregate(w.hws, plan.cls, s, nb, w.g16, w.zeta, a.device_status, stream)) != LITE3R_OK) return st;
+    if ((st = launch_aggregate(w.hws, plan.cls, s, nb, w.g16, w.zeta, a.device_status, phases != 3, stream)) != LITE3R_OK) return st;
     profile_mark(5, stream);
   }
   AttentionLaunch att;
@@ -188,7 +192,10 @@ void forward_workspace_offsets(const lite3r_shape& s, const Counts& c, bool plan
 }
 
 lite3r_status launch_forward(const ForwardArgs& a, int phases, cudaStream_t stream) {
-  if ((phases & 1) && a.device_status != nullptr) {  // the status word is cleared where the forward begins
+  // The status word is cleared where the forward begins: by its first kernel (the first CTA, before any wait of the forward
+  // can have expired), or here where no kernel precedes the attention kernel.
+  const bool first_kernel_clears = a.plan.k_marg > 0 || (a.plan.k_crit > 0 && !a.linear_only);
+  if ((phases & 1) && a.device_status != nullptr && !first_kernel_clears) {
     lite3r_status st = record_cuda(cudaMemsetAsync(a.device_status, 0, sizeof(int), stream));
     if (st != LITE3R_OK) return st;
   }

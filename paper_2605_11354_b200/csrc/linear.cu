@@ -49,6 +49,8 @@ __device__ __forceinline__ uint32_t quantise_pair(float a, float b, float scale)
 template <typename SrcT>
 __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ x, long long row_stride, int rows, int cols,
                                                        uint8_t* __restrict__ codes, float* __restrict__ scales) {
+  wait_for_prior_grid();
+  launch_dependents();
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int segs = cols >> 3;
@@ -202,7 +204,6 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     if (threadIdx.x == 0 && p.status != nullptr) atomicCAS(p.status, 0, 900);
     return;
   }
-  if (p.status != nullptr && *reinterpret_cast<volatile int*>(p.status) != 0) return;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // row tiles never run through a batch boundary in the fused form (a tile belongs to one sequence)
@@ -247,6 +248,9 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  wait_for_prior_grid();
+  launch_dependents();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && p.status != nullptr) *p.status = 0;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -259,7 +263,7 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         for (int k = 0; ok && k < k_steps; ++k, ++kc) {
           const int st = kc % kStages;
           if (kc >= kStages)
-            ok = mbar_wait(&bars->empty[st], ((kc - kStages) / kStages) & 1, abort_flag, p.status, 601, 32);
+            ok = mbar_wait_clearing(&bars->empty[st], ((kc - kStages) / kStages) & 1, abort_flag, p.status, 601, 32);
           if (!ok) break;
           mbar_arrive_expect_tx(&bars->full[st], kStageBytes);
           tma_load_2d(smem + st * kStageBytes, &map_x, &bars->full[st], k * kTileK, t.row0);
@@ -277,11 +281,11 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       for (int tile_id = blockIdx.x; ok && tile_id < p.tiles; tile_id += gridDim.x, ++it) {
         const int ab = it & 1;
         // the accumulator was last used two tiles ago: wait until the epilogue warps have read it out
-        if (it >= 2) ok = mbar_wait(&bars->acc_empty[ab], ((it - 2) >> 1) & 1, abort_flag, p.status, 604);
+        if (it >= 2) ok = mbar_wait_clearing(&bars->acc_empty[ab], ((it - 2) >> 1) & 1, abort_flag, p.status, 604);
         tc_fence_after();
         for (int k = 0; ok && k < k_steps; ++k, ++kc) {
           const int st = kc % kStages;
-          ok = mbar_wait(&bars->full[st], (kc / kStages) & 1, abort_flag, p.status, 602);
+          ok = mbar_wait_clearing(&bars->full[st], (kc / kStages) & 1, abort_flag, p.status, 602);
           if (!ok) break;
           tc_fence_after();
           const uint64_t off = static_cast<uint64_t>((st * kStageBytes) >> 4);
@@ -319,7 +323,7 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       bia[tid] = (p.bias != nullptr && col + tid < p.d_out) ? __ldg(p.bias + col + tid) : 0.f;
     }
     named_barrier_sync(bar_id, 128);
-    ok = mbar_wait(&bars->acc_full[ab], (it >> 1) & 1, abort_flag, p.status, 603);
+    ok = mbar_wait_clearing(&bars->acc_full[ab], (it >> 1) & 1, abort_flag, p.status, 603);
     tc_fence_after();
     ok = __all_sync(0xFFFFFFFFu, ok);
     if (!ok) break;
@@ -507,12 +511,13 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 }
 
 lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const LinearParams& p, cudaStream_t stream) {
-  alignas(64) CUtensorMap map_x, map_w;
+  const CUtensorMap* const px = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, x_codes, p.d_in, p.rows, kTileK, kTileM,
+                                                   CU_TENSOR_MAP_SWIZZLE_128B);
+  const CUtensorMap* const pw = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, w_codes, p.d_in, p.d_out, kTileK, kTileN,
+                                                   CU_TENSOR_MAP_SWIZZLE_128B);
+  if (px == nullptr || pw == nullptr) return LITE3R_ERR_CUDA;
+  const CUtensorMap map_x = *px, map_w = *pw;
   lite3r_status st;
-  if ((st = make_tensor_map_2d(&map_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, x_codes, p.d_in, p.rows, kTileK, kTileM,
-                               CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
-  if ((st = make_tensor_map_2d(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, w_codes, p.d_in, p.d_out, kTileK, kTileN,
-                               CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
   if ((st = ensure_dynamic_smem(linear_fp8_kernel, static_cast<int>(kSmemBytes))) != LITE3R_OK) return st;
   const int row_tiles = p.fused ? p.batch * ceil_div(p.tokens, kTileM) : ceil_div(p.rows, kTileM);
   LinearParams q = p;
@@ -521,8 +526,8 @@ lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const 
   int sms = 0;
   if ((st = sm_count(&sms)) != LITE3R_OK) return st;
   const int grid = q.tiles < sms ? q.tiles : sms;
-  linear_fp8_kernel<<<grid, kThreads, kSmemBytes, stream>>>(map_x, map_w, q);
-  return after_launch();
+  return launch_dependent(linear_fp8_kernel, dim3(static_cast<unsigned>(grid)), kThreads, static_cast<int>(kSmemBytes), stream, map_x,
+                          map_w, q);
 }
 
 }  // namespace
@@ -533,11 +538,12 @@ lite3r_status launch_rowquant(const void* x, int dtype, long long row_stride, in
   lite3r_status st = sm_count(&sms);
   if (st != LITE3R_OK) return st;
   const int blocks = std::min(ceil_div(rows, 8), sms * 8);
+  const dim3 grid(static_cast<unsigned>(blocks));
   if (dtype == LITE3R_BF16)
-    rowquant_kernel<<<blocks, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(x), row_stride, rows, cols, codes, scales);
-  else
-    rowquant_kernel<<<blocks, 256, 0, stream>>>(static_cast<const float*>(x), row_stride, rows, cols, codes, scales);
-  return after_launch();
+    return launch_dependent(rowquant_kernel<__nv_bfloat16>, grid, 256, 0, stream, static_cast<const __nv_bfloat16*>(x), row_stride,
+                            rows, cols, codes, scales);
+  return launch_dependent(rowquant_kernel<float>, grid, 256, 0, stream, static_cast<const float*>(x), row_stride, rows, cols, codes,
+                          scales);
 }
 
 lite3r_status launch_linear_fp8(const uint8_t* x_codes, const float* x_scales, const uint8_t* w_codes,

@@ -25,6 +25,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "sm100.cuh"
 
 namespace lite3r {
 
@@ -225,6 +226,8 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
   const int lane = threadIdx.x & 31;
   const size_t bh_rows = static_cast<size_t>(bh) * nb;
 
+  sm100::wait_for_prior_grid();
+  sm100::launch_dependents();
   if constexpr (kDirect) {
     // Phase A, R rows x 8 key blocks per warp and step as fp64 tensor-core products (m8n8k4, 16 k-steps over the 64
     // columns, one 8-row tile after the other against the same B values): the integer products and sums stay below
@@ -528,6 +531,8 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
     return ((valid == block && block_pow2) ? num * inv_block : num / static_cast<double>(valid)) + 0.0;
   };
 
+  sm100::wait_for_prior_grid();
+  sm100::launch_dependents();
   {
     // Phase A: fp64 tensor-core products of the exactly widened int32 column sums (see plan_kernel).
     const int tile = warp % kRowTiles, grp = warp / kRowTiles;
@@ -835,10 +840,9 @@ lite3r_status launch_compact(const lite3r_fp8& q, const lite3r_fp8& k, const lit
   lite3r_status st = ensure_dynamic_smem(plan_compact_kernel<R>, static_cast<int>(smem));
   if (st != LITE3R_OK) return st;
   const int row_tiles = ceil_div(nb, R);
-  plan_compact_kernel<R><<<s.batch * s.heads * row_tiles, R * 32, smem, stream>>>(q.colsum, k.colsum, k.scales, s.tokens,
-                                                                                   s.block, nb, c.k_crit, c.k_marg, c.k_neg,
-                                                                                   plan.cls, plan.crit_idx, plan.marg_idx);
-  return after_launch();
+  return launch_dependent(plan_compact_kernel<R>, dim3(static_cast<unsigned>(s.batch * s.heads * row_tiles)), R * 32,
+                          static_cast<int>(smem), stream, q.colsum, k.colsum, k.scales, s.tokens, s.block, nb, c.k_crit, c.k_marg,
+                          c.k_neg, plan.cls, plan.crit_idx, plan.marg_idx);
 }
 
 size_t plan_smem_bytes(int nb, int rows) {
@@ -858,10 +862,9 @@ lite3r_status launch_rows(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r
   lite3r_status st = ensure_dynamic_smem(plan_kernel<R>, static_cast<int>(smem));
   if (st != LITE3R_OK) return st;
   const int row_tiles = ceil_div(nb, R);
-  plan_kernel<R><<<s.batch * s.heads * row_tiles, R * 32, smem, stream>>>(q.colsum, k.colsum, k.scales, s.tokens,
-                                                                           s.block, nb, c.k_crit, c.k_marg, c.k_neg,
-                                                                           plan.cls, plan.crit_idx, plan.marg_idx);
-  return after_launch();
+  return launch_dependent(plan_kernel<R>, dim3(static_cast<unsigned>(s.batch * s.heads * row_tiles)), R * 32,
+                          static_cast<int>(smem), stream, q.colsum, k.colsum, k.scales, s.tokens, s.block, nb, c.k_crit, c.k_marg,
+                          c.k_neg, plan.cls, plan.crit_idx, plan.marg_idx);
 }
 
 }  // namespace

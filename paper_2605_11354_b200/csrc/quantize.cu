@@ -146,6 +146,8 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const __grid_constan
     }
   };
 
+  sm100::wait_for_prior_grid();
+  sm100::launch_dependents();
 #pragma unroll
   for (int d = 0; d < kDepth - 1; ++d) fetch(d);
 
@@ -296,8 +298,8 @@ lite3r_status launch(const QuantBatch& batch, const lite3r_shape& s, cudaStream_
   }
   const long long all = static_cast<long long>(tiles) * batch.count;
   const int grid = static_cast<int>(all < static_cast<long long>(sms) * per_sm ? all : static_cast<long long>(sms) * per_sm);
-  quantize_kernel<BS, SrcT, kThreads><<<grid, kThreads, kSmem, stream>>>(batch, s.heads, s.tokens, nb, tiles);
-  return after_launch();
+  return launch_dependent(quantize_kernel<BS, SrcT, kThreads>, dim3(static_cast<unsigned>(grid)), kThreads, kSmem, stream, batch,
+                          s.heads, s.tokens, nb, tiles);
 }
 
 }  // namespace

@@ -27,7 +27,9 @@ __device__ __forceinline__ bool elect_one() {
 // Programmatic dependent launch.  launch_dependents: the next kernel in the stream, if it was launched with the
 // programmatic-serialization attribute, may start once every CTA of this grid has got here (or exited).
 // wait_for_prior_grid: blocks until the preceding grid has completed and its writes are visible; a no-op in a kernel
-// that was launched the ordinary way.
+// that was launched the ordinary way.  A kernel lets its successor start only after its own wait and after its TMEM
+// allocation: at most two launches are then ever under way, no buffer is read (and kept in a first-level cache) by a
+// kernel two launches back while it is rewritten, and a successor's allocation never comes before this kernel's.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -130,30 +132,14 @@ __device__ __forceinline__ bool mbar_wait_far(uint64_t* bar, uint32_t parity, vo
   return true;
 }
 
-// Bounded idling for a single-thread role that polls several barriers without blocking on any of them: call
-// idle() whenever a round of polls made no progress and progress() whenever one did.  idle() sleeps briefly and
-// returns false once nothing has moved for the wait limit or another role of the CTA (or another CTA) gave up.
-struct IdleGuard {
-  uint64_t since = 0;
-  uint32_t polls = 0;
-  __device__ __forceinline__ void progress() { polls = 0; }
-  __device__ __forceinline__ bool idle(volatile int* abort_flag, int* status, int code, uint32_t backoff_ns) {
-    if (backoff_ns != 0) __nanosleep(backoff_ns);
-    if (polls == 0) since = global_timer_ns();
-    if ((++polls & 0xFu) != 0) return true;
-    if (*abort_flag != 0) return false;
-    if (status != nullptr && *reinterpret_cast<volatile int*>(status) != 0) {
-      *abort_flag = code;
-      return false;
-    }
-    if (global_timer_ns() - since > kWaitLimitNs) {
-      *abort_flag = code;
-      if (status != nullptr) atomicCAS(status, 0, code);
-      return false;
-    }
-    return true;
-  }
-};
+// The wait of a kernel that clears the status word itself (its first CTA does, long before any wait can expire): the word
+// is written when a wait expires but not looked at, since it may still hold what an earlier call left.
+__device__ __forceinline__ bool mbar_wait_clearing(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
+                                                   int code, uint32_t backoff_ns = 0) {
+  if (mbar_wait(bar, parity, abort_flag, nullptr, code, backoff_ns)) return true;
+  if (status != nullptr) atomicCAS(status, 0, code);
+  return false;
+}
 
 // ------------------------------------------------------------------------------------------------ TMA
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {

@@ -95,7 +95,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
     if (threadIdx.x == 0 && p.status != nullptr) atomicCAS(p.status, 0, 902);
     return;
   }
-  if (p.status != nullptr && *reinterpret_cast<volatile int*>(p.status) != 0) return;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // contiguous, balanced share of the rounds
@@ -120,6 +119,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  wait_for_prior_grid();
+  launch_dependents();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && p.status != nullptr) *p.status = 0;
 
   if (warp == 4) {
     // ------------------------------------------------------------------------------------------ MMA issuer
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
       bool ok = true;
       for (int r = r_begin; r < r_end && ok; ++r) {
         const uint32_t ph = static_cast<uint32_t>(r - r_begin) & 1u;
-        if (!(ok = mbar_wait(&bars->ab_full, ph, abort_flag, p.status, 501))) break;
+        if (!(ok = mbar_wait_clearing(&bars->ab_full, ph, abort_flag, p.status, 501))) break;
         tc_fence_after();
 #pragma unroll
         for (int hf = 0; hf < kTilesPerRound; ++hf) {
@@ -159,7 +161,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
             mma_f16(tmem + kColZ + lane_off, a, o, idesc_z, kk);
           }
         }
-        if (!(ok = mbar_wait(&bars->h_full, ph, abort_flag, p.status, 502))) break;
+        if (!(ok = mbar_wait_clearing(&bars->h_full, ph, abort_flag, p.status, 502))) break;
         tc_fence_after();
 #pragma unroll
         for (int hf = 0; hf < kTilesPerRound; ++hf) {
@@ -339,7 +341,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
       mbar_arrive(&bars->ab_full);
 
       // H row: TMEM -> scaled fp16 -> B operand of MMA 2; z row -> global
-      if (!(ok = mbar_wait(&bars->h_done, ph, abort_flag, p.status, 503))) break;
+      if (!(ok = mbar_wait_clearing(&bars->h_done, ph, abort_flag, p.status, 503))) break;
       tc_fence_after();
       {
         uint32_t lo[32], hi[32];
@@ -368,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
       mbar_arrive(&bars->h_full);
 
       // (H W)^T row e': TMEM -> bf16 -> global
-      if (!(ok = mbar_wait(&bars->hw_done, ph, abort_flag, p.status, 504))) break;
+      if (!(ok = mbar_wait_clearing(&bars->hw_done, ph, abort_flag, p.status, 504))) break;
       tc_fence_after();
       {
         uint32_t lo[32], hi[32];
@@ -415,19 +417,22 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
 }
 
 template <int BS>
-lite3r_status launch(const SummaryParams& p, int sm_count, cudaStream_t stream) {
+lite3r_status launch(const SummaryParams& p, int sm_count, bool after_wait, cudaStream_t stream) {
   lite3r_status st = ensure_dynamic_smem(summary_kernel<BS>, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
   const int grid = p.rounds < sm_count * kCtasPerSm ? p.rounds : sm_count * kCtasPerSm;
-  summary_kernel<BS><<<grid, kThreads, kSmemBytes, stream>>>(p);
-  return after_launch();
+  if (after_wait) {
+    summary_kernel<BS><<<grid, kThreads, kSmemBytes, stream>>>(p);
+    return after_launch();
+  }
+  return launch_dependent(summary_kernel<BS>, dim3(static_cast<unsigned>(grid)), kThreads, static_cast<int>(kSmemBytes), stream, p);
 }
 
 }  // namespace
 
 lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const float* proj, long long proj_head_stride,
                              const lite3r_shape& s, int phi, __nv_bfloat16* hws, __half* v16, int* device_status,
-                             cudaStream_t stream) {
+                             bool after_wait, cudaStream_t stream) {
   SummaryParams p;
   p.k_codes = k.codes;
   p.k_scales = k.scales;
@@ -447,7 +452,7 @@ lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const flo
   int sms = 0;
   lite3r_status st = sm_count(&sms);
   if (st != LITE3R_OK) return st;
-  return s.block == 64 ? launch<64>(p, sms, stream) : launch<128>(p, sms, stream);
+  return s.block == 64 ? launch<64>(p, sms, after_wait, stream) : launch<128>(p, sms, after_wait, stream);
 }
 
 }  // namespace lite3r

@@ -19,6 +19,8 @@ using namespace sm100;
 
 // ------------------------------------------------------------------------------------------------ identity (64 x 64)
 __global__ void fill_identity_kernel(float* dst) {
+  wait_for_prior_grid();
+  launch_dependents();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < kHeadDim * kHeadDim) dst[i] = (i / kHeadDim == i % kHeadDim) ? 1.f : 0.f;
 }
@@ -49,6 +51,8 @@ __global__ void __launch_bounds__(kMseThreads) mse_kernel(const T* __restrict__ 
                                                           double* __restrict__ partials) {
   __shared__ double s_sum[kMseThreads / 32];
   double acc = 0.0;
+  wait_for_prior_grid();
+  launch_dependents();
   const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
   for (size_t g = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; g < groups; g += stride) {
     float a[8], b[8];
@@ -80,14 +84,16 @@ __global__ void __launch_bounds__(kMseThreads) mse_kernel(const T* __restrict__ 
 // Adds the block partials in a fixed order: thread t takes partials t, t + 256, ..., then a fixed tree over the threads.
 // One thread doing it alone is a chain of up to 2048 dependent fp64 additions behind as many loads: 47 us for the
 // 1184 partials of a 16 x 10992 x 64 tensor, where the pass over the tensor itself takes 16 us.
-__global__ void __launch_bounds__(kMseThreads) mse_finish_kernel(const double* __restrict__ partials, int n, double inv_count,
+__global__ void __launch_bounds__(kMseThreads) mse_finish_kernel(const double* partials, int n, double inv_count,
                                                                  double* __restrict__ loss) {
   __shared__ double s_sum[kMseThreads / 32];
   double t = 0.0;
+  wait_for_prior_grid();
+  launch_dependents();
 #pragma unroll
   for (int k = 0; k < kMaxMseBlocks / kMseThreads; ++k) {  // independent loads, then additions in order
     const int i = threadIdx.x + k * kMseThreads;
-    t += i < n ? __ldg(partials + i) : 0.0;
+    t += i < n ? partials[i] : 0.0;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
@@ -127,7 +133,6 @@ projgrad_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
     if (threadIdx.x == 0 && status != nullptr) atomicCAS(status, 0, 900);
     return;
   }
-  if (status != nullptr && *reinterpret_cast<volatile int*>(status) != 0) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = blockIdx.x / chunks, chunk = blockIdx.x % chunks;
   const int total_tiles = (tokens + kTileTok - 1) / kTileTok;
@@ -152,6 +157,9 @@ projgrad_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  wait_for_prior_grid();
+  launch_dependents();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && status != nullptr) *status = 0;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -160,7 +168,7 @@ projgrad_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
       bool ok = true;
       for (int i = 0; ok && i < n_tiles; ++i) {
         const int st = i % kStages;
-        if (i >= kStages) ok = mbar_wait(&bars->empty[st], ((i - kStages) / kStages) & 1, abort_flag, status, 701, 32);
+        if (i >= kStages) ok = mbar_wait_clearing(&bars->empty[st], ((i - kStages) / kStages) & 1, abort_flag, status, 701, 32);
         if (!ok) break;
         mbar_arrive_expect_tx(&bars->full[st], kStageBytes);
         tma_load_3d(smem + st * kStageBytes, &map_o, &bars->full[st], 0, (t_begin + i) * kTileTok, bh);
@@ -174,7 +182,7 @@ projgrad_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
       bool ok = true;
       for (int i = 0; ok && i < n_tiles; ++i) {
         const int st = i % kStages;
-        ok = mbar_wait(&bars->full[st], (i / kStages) & 1, abort_flag, status, 702);
+        ok = mbar_wait_clearing(&bars->full[st], (i / kStages) & 1, abort_flag, status, 702);
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
@@ -195,7 +203,7 @@ projgrad_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
     float* dst = partials + (static_cast<size_t>(blockIdx.x) * kHeadDim + row) * kHeadDim;
     bool ok = true;
     if (n_tiles > 0) {
-      ok = mbar_wait(&bars->acc_full, 0, abort_flag, status, 703);
+      ok = mbar_wait_clearing(&bars->acc_full, 0, abort_flag, status, 703);
       tc_fence_after();
     }
     ok = __all_sync(0xFFFFFFFFu, ok);
@@ -230,22 +238,24 @@ projgrad_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
 // dW[h] = sum over batch entries and chunks of the partials, in a fixed order.  One thread per element of dW (a CTA per
 // 256 of them), loads of eight partials in flight ahead of the additions: with one CTA per head the sixteen elements of
 // a thread were summed one after the other, 39 us for 304 partials of 16 heads (5 MB, all in L2).
-__global__ void __launch_bounds__(256) projgrad_reduce_kernel(const float* __restrict__ partials, int batch, int heads,
+__global__ void __launch_bounds__(256) projgrad_reduce_kernel(const float* partials, int batch, int heads,
                                                               int chunks, float* __restrict__ d_w) {
   constexpr int kSlices = kHeadDim * kHeadDim / 256;
   const int h = blockIdx.x / kSlices, e = (blockIdx.x % kSlices) * 256 + threadIdx.x;
   float acc = 0.f;
+  wait_for_prior_grid();
+  launch_dependents();
   for (int b = 0; b < batch; ++b) {
     const float* src = partials + static_cast<size_t>(b * heads + h) * chunks * kHeadDim * kHeadDim + e;
     int c = 0;
     for (; c + 8 <= chunks; c += 8) {
       float v[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = __ldg(src + static_cast<size_t>(c + k) * kHeadDim * kHeadDim);
+      for (int k = 0; k < 8; ++k) v[k] = src[static_cast<size_t>(c + k) * kHeadDim * kHeadDim];
 #pragma unroll
       for (int k = 0; k < 8; ++k) acc += v[k];
     }
-    for (; c < chunks; ++c) acc += __ldg(src + static_cast<size_t>(c) * kHeadDim * kHeadDim);
+    for (; c < chunks; ++c) acc += src[static_cast<size_t>(c) * kHeadDim * kHeadDim];
   }
   d_w[static_cast<size_t>(h) * kHeadDim * kHeadDim + e] = acc;
 }
@@ -269,8 +279,7 @@ size_t train_workspace_bytes(const lite3r_shape& s) {
 }
 
 lite3r_status launch_fill_identity(float* dst, cudaStream_t stream) {
-  fill_identity_kernel<<<(kHeadDim * kHeadDim + 255) / 256, 256, 0, stream>>>(dst);
-  return after_launch();
+  return launch_dependent(fill_identity_kernel, dim3((kHeadDim * kHeadDim + 255) / 256), 256, 0, stream, dst);
 }
 
 lite3r_status launch_mse_distill(const void* student, const void* teacher, int dtype, size_t count, __nv_bfloat16* grad,
@@ -282,14 +291,14 @@ lite3r_status launch_mse_distill(const void* student, const void* teacher, int d
   const int blocks = static_cast<int>(std::min<size_t>(std::min(kMaxMseBlocks, sms * 8), (groups + kMseThreads - 1) / kMseThreads));
   const float grad_scale = static_cast<float>(2.0 / static_cast<double>(count));
   if (dtype == LITE3R_BF16)
-    mse_kernel<<<blocks, kMseThreads, 0, stream>>>(static_cast<const __nv_bfloat16*>(student),
-                                                   static_cast<const __nv_bfloat16*>(teacher), groups, grad_scale, grad, partials);
+    st = launch_dependent(mse_kernel<__nv_bfloat16>, dim3(static_cast<unsigned>(blocks)), kMseThreads, 0, stream,
+                          static_cast<const __nv_bfloat16*>(student), static_cast<const __nv_bfloat16*>(teacher), groups, grad_scale,
+                          grad, partials);
   else
-    mse_kernel<<<blocks, kMseThreads, 0, stream>>>(static_cast<const float*>(student), static_cast<const float*>(teacher),
-                                                   groups, grad_scale, grad, partials);
-  if ((st = after_launch()) != LITE3R_OK) return st;
-  mse_finish_kernel<<<1, kMseThreads, 0, stream>>>(partials, blocks, 1.0 / static_cast<double>(count), loss);
-  return after_launch();
+    st = launch_dependent(mse_kernel<float>, dim3(static_cast<unsigned>(blocks)), kMseThreads, 0, stream,
+                          static_cast<const float*>(student), static_cast<const float*>(teacher), groups, grad_scale, grad, partials);
+  if (st != LITE3R_OK) return st;
+  return launch_dependent(mse_finish_kernel, dim3(1), kMseThreads, 0, stream, partials, blocks, 1.0 / static_cast<double>(count), loss);
 }
 
 lite3r_status launch_proj_lin_backward(const __nv_bfloat16* o_lin, const __nv_bfloat16* d_out, const lite3r_shape& s,
@@ -300,17 +309,18 @@ lite3r_status launch_proj_lin_backward(const __nv_bfloat16* o_lin, const __nv_bf
   const int planes = s.batch * s.heads;
   const int chunks = projgrad_chunks(s, sms);
   const int tiles_per_cta = ceil_div(ceil_div(s.tokens, kTileTok), chunks);
-  alignas(64) CUtensorMap map_o, map_g;
-  if ((st = make_tensor_map_3d(&map_o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o_lin, kHeadDim, s.tokens, planes, kHeadDim,
-                               kTileTok, CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
-  if ((st = make_tensor_map_3d(&map_g, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, d_out, kHeadDim, s.tokens, planes, kHeadDim,
-                               kTileTok, CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
+  const CUtensorMap* const po = make_tensor_map_3d(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o_lin, kHeadDim, s.tokens, planes, kHeadDim,
+                                                   kTileTok, CU_TENSOR_MAP_SWIZZLE_128B);
+  const CUtensorMap* const pg = make_tensor_map_3d(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, d_out, kHeadDim, s.tokens, planes, kHeadDim,
+                                                   kTileTok, CU_TENSOR_MAP_SWIZZLE_128B);
+  if (po == nullptr || pg == nullptr) return LITE3R_ERR_CUDA;
+  const CUtensorMap map_o = *po, map_g = *pg;
   if ((st = ensure_dynamic_smem(projgrad_kernel, static_cast<int>(kSmemBytes))) != LITE3R_OK) return st;
-  projgrad_kernel<<<planes * chunks, kThreads, kSmemBytes, stream>>>(map_o, map_g, s.tokens, chunks, tiles_per_cta, partials,
-                                                                     device_status);
-  if ((st = after_launch()) != LITE3R_OK) return st;
-  projgrad_reduce_kernel<<<s.heads * (kHeadDim * kHeadDim / 256), 256, 0, stream>>>(partials, s.batch, s.heads, chunks, d_w);
-  return after_launch();
+  st = launch_dependent(projgrad_kernel, dim3(static_cast<unsigned>(planes * chunks)), kThreads, static_cast<int>(kSmemBytes), stream,
+                        map_o, map_g, s.tokens, chunks, tiles_per_cta, partials, device_status);
+  if (st != LITE3R_OK) return st;
+  return launch_dependent(projgrad_reduce_kernel, dim3(static_cast<unsigned>(s.heads * (kHeadDim * kHeadDim / 256))), 256, 0, stream,
+                          partials, s.batch, s.heads, chunks, d_w);
 }
 
 }  // namespace lite3r
