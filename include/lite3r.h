@@ -156,6 +156,28 @@ LITE3R_API lite3r_status lite3r_sla_forward(const lite3r_fp8* q, const lite3r_fp
                                  long long out_stride_b, long long out_stride_h, long long out_stride_n,
                                  void* workspace, size_t workspace_bytes, int* device_status, void* stream);
 
+/* One whole step as a single call: quantise Q, K and V (one launch when the sources share a dtype), build the plan
+ * (plan.cls == NULL: inside the forward's workspace), run the forward.  The fields are the arguments of the calls it
+ * stands for, which see the same launches; a caller that runs a step often fills the struct once and pays one call
+ * instead of marshalling some fifty arguments.  All arguments are checked before anything is enqueued. */
+typedef struct {
+  lite3r_shape shape;
+  lite3r_tensor q, k, v;                       /* DEVICE sources */
+  lite3r_fp8 q8, k8, v8;                       /* their quantised form, written (v8.colsum may be NULL) */
+  lite3r_plan plan;                            /* written; the counts are set from the fractions */
+  double crit, neg;
+  lite3r_phi phi;
+  const float* proj;
+  long long proj_head_stride;
+  void* out;
+  lite3r_dtype out_dtype;
+  long long out_stride_b, out_stride_h, out_stride_n;
+  void* workspace;
+  size_t workspace_bytes;
+  int* device_status;
+} lite3r_step;
+LITE3R_API lite3r_status lite3r_sla_step(lite3r_step* step, void* stream);
+
 /* lite3r_sla_forward in two halves, for callers that overlap the block plan with the part of the forward that does
  * not depend on it.  The per-key-block summaries of the linear branch (Algorithm 1's feature map, KV summary and
  * normaliser, with proj folded in) and the fp16 copy of V read only K, V and proj, so

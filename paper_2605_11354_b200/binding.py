@@ -7,6 +7,7 @@ the import of any compute function raises.
 from __future__ import annotations
 
 import ctypes as C
+import itertools
 import os
 from dataclasses import dataclass
 
@@ -43,6 +44,14 @@ class Plan(C.Structure):
                 ("k_marg", C.c_int), ("k_neg", C.c_int)]
 
 
+class Step(C.Structure):
+    _fields_ = [("shape", Shape), ("q", Tensor), ("k", Tensor), ("v", Tensor), ("q8", Fp8), ("k8", Fp8), ("v8", Fp8),
+                ("plan", Plan), ("crit", C.c_double), ("neg", C.c_double), ("phi", C.c_int), ("proj", C.c_void_p),
+                ("proj_head_stride", C.c_longlong), ("out", C.c_void_p), ("out_dtype", C.c_int),
+                ("out_stride_b", C.c_longlong), ("out_stride_h", C.c_longlong), ("out_stride_n", C.c_longlong),
+                ("workspace", C.c_void_p), ("workspace_bytes", C.c_size_t), ("device_status", C.c_void_p)]
+
+
 EXPORTS = ("lite3r_fp8_sizes", "lite3r_plan_sizes", "lite3r_forward_workspace", "lite3r_quantize_fp8",
            "lite3r_sla_plan", "lite3r_sla_forward", "lite3r_status_string", "lite3r_last_cuda_error",
            "lite3r_launch_count", "lite3r_profile_enable", "lite3r_profile_stage_ms",
@@ -50,7 +59,7 @@ EXPORTS = ("lite3r_fp8_sizes", "lite3r_plan_sizes", "lite3r_forward_workspace", 
            "lite3r_sla_forward_begin", "lite3r_sla_forward_finish", "lite3r_forward_workspace_planned",
            "lite3r_workspace_layout", "lite3r_quantize_rows_fp8", "lite3r_linear_fp8", "lite3r_qkv_project_fp8",
            "lite3r_train_workspace", "lite3r_sla_linear_branch", "lite3r_mse_distill", "lite3r_proj_lin_backward",
-           "lite3r_plan_variant", "lite3r_attention_plain_stores")
+           "lite3r_plan_variant", "lite3r_attention_plain_stores", "lite3r_sla_step")
 STATIC_SCRATCH_BYTES = 32 << 20  # LITE3R_STATIC_SCRATCH_BYTES
 
 
@@ -81,6 +90,8 @@ def lib() -> C.CDLL:
                                      C.POINTER(Shape), C.c_double, C.c_double, C.c_int, C.POINTER(Plan), C.c_void_p,
                                      C.c_int, C.c_longlong, C.c_longlong, C.c_longlong, C.c_void_p, C.c_size_t,
                                      C.c_void_p, C.c_void_p]
+    L.lite3r_sla_step.argtypes = [C.c_void_p, C.c_void_p]
+    L.lite3r_sla_step.restype = C.c_int
     L.lite3r_sla_forward_static_scratch.argtypes = [C.POINTER(Fp8), C.POINTER(Fp8), C.POINTER(Fp8), C.c_void_p,
                                                     C.c_longlong, C.POINTER(Shape), C.c_int, C.POINTER(Plan),
                                                     C.c_void_p, C.c_int, C.c_longlong, C.c_longlong, C.c_longlong,
@@ -144,8 +155,9 @@ def _check(status: int, what: str) -> None:
 
 
 def _stream_ptr(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is None:  # the current stream of the current device, without building a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return int(stream.cuda_stream)
 
 
 def selftest_wait_expiry(status: torch.Tensor, limit_ns: int, stream=None) -> None:
@@ -217,19 +229,40 @@ def lite3r_workspace_layout(shape: Shape, crit: float, neg: float, plan_inside: 
 
 
 # ----------------------------------------------------------------------------- device buffers
+_ticks = itertools.count(1)
+_generation = [0]  # changes with every assignment to the buffers below: what was marshalled before that is out of date
+
+
+class _Marshalled:
+    """Buffers whose C struct is kept until one of their fields (or those of another such object) is assigned."""
+
+    _c = None
+
+    def __setattr__(self, name, value):
+        if name != "_c":
+            _generation[0] = next(_ticks)
+        object.__setattr__(self, name, value)
+
+    def c_struct(self):
+        c = self._c
+        if c is None or c[0] != _generation[0]:
+            c = self._c = (_generation[0], self._marshal())
+        return c[1]
+
+
 @dataclass
-class Fp8Tensor:
+class Fp8Tensor(_Marshalled):
     codes: torch.Tensor  # uint8 [B,H,Nb*Bs,D]
     scales: torch.Tensor  # fp32 [B,H,Nb]
     colsum: torch.Tensor | None  # int32 [B,H,Nb,D]; None: the quantiser skips the column sums (only Q and K need them)
 
-    def c_struct(self) -> Fp8:
+    def _marshal(self) -> Fp8:
         return Fp8(self.codes.data_ptr(), self.scales.data_ptr(),
                    self.colsum.data_ptr() if self.colsum is not None else None)
 
 
 @dataclass
-class PlanBuffers:
+class PlanBuffers(_Marshalled):
     cls: torch.Tensor  # int8 [B,H,Nb,Nb]
     crit_idx: torch.Tensor  # int32 [B,H,Nb,k_crit]
     marg_idx: torch.Tensor  # int32 [B,H,Nb,k_marg]
@@ -237,7 +270,7 @@ class PlanBuffers:
     k_marg: int
     k_neg: int
 
-    def c_struct(self) -> Plan:
+    def _marshal(self) -> Plan:
         return Plan(self.cls.data_ptr(), self.crit_idx.data_ptr() if self.k_crit else None,
                     self.marg_idx.data_ptr() if self.k_marg else None, self.k_crit, self.k_marg, self.k_neg)
 
@@ -481,6 +514,36 @@ class SlaForward:
         self.status = torch.zeros(1, dtype=torch.int32, device=self.device)
         self._side = None  # stream of the overlapped first half of the forward, made on first use
         self._graph = None  # (CUDA graph of one whole step, key of the tensors it was captured on)
+        self._step = None  # (key of the tensors and buffers, their marshalled arguments, pointer to those)
+
+    def __setattr__(self, name, value):
+        if not name.startswith("_"):
+            _generation[0] = next(_ticks)  # marshalled arguments hold the engine's buffers and settings
+        object.__setattr__(self, name, value)
+
+    def _run_step(self, q, k, v, proj, stream, out):
+        """quantise + plan + forward through one library call; the arguments are marshalled once per set of tensors."""
+        key = (_generation[0], q.data_ptr(), q.stride(), q.dtype, k.data_ptr(), k.stride(), k.dtype, v.data_ptr(),
+               v.stride(), v.dtype, proj.data_ptr(), proj.stride(), proj.dtype, out.data_ptr(), out.stride(), out.dtype)
+        step = self._step
+        if step is None or step[0] != key:
+            step = self._step = self._marshal_step(key, q, k, v, proj, out)
+        _check(_lib.lite3r_sla_step(step[2], _stream_ptr(stream)), "lite3r_sla_step")
+        return out
+
+    def _marshal_step(self, key, q, k, v, proj, out):
+        if proj.dtype != torch.float32 or not proj.is_cuda or not proj.is_contiguous():
+            raise Lite3rError("lite3r_sla_forward: proj must be a contiguous CUDA float32 tensor")
+        lib()
+        if not self.plan_inside and lite3r_plan_sizes(self.shape, self.crit, self.neg)[3:] != (
+                self.plan.k_crit, self.plan.k_marg, self.plan.k_neg):
+            raise Lite3rError("SlaForward: the plan's buffers were made for other fractions")
+        s = Step(self.shape, *(_source(x, "lite3r_quantize_fp8") for x in (q, k, v)), self.q8.c_struct(), self.k8.c_struct(),
+                 self.v8.c_struct(), Plan() if self.plan_inside else self.plan.c_struct(), self.crit, self.neg, self.phi,
+                 proj.data_ptr(), proj.stride(0) if proj.dim() == 3 else 0, out.data_ptr(),
+                 _check_out(out, "lite3r_sla_forward"), out.stride(0), out.stride(1), out.stride(2), self.workspace.data_ptr(),
+                 self.workspace.numel() * self.workspace.element_size(), self.status.data_ptr())
+        return key, s, C.addressof(s)
 
     def quantize(self, q, k, v, stream=None):
         if q.dtype == k.dtype == v.dtype:
@@ -504,13 +567,8 @@ class SlaForward:
     def run(self, q, k, v, proj, stream=None, out=None, overlap=False):
         """Quantise, plan, forward.  overlap=True runs the plan-independent first half of the forward (summaries, fp16
         V) on a side stream beside the plan kernel; the results are the same."""
-        if self.plan_inside:
-            self.quantize(q, k, v, stream)
-            return self.forward(proj, stream, out)
-        if not overlap or self.plan.k_marg == 0:
-            self.quantize(q, k, v, stream)
-            self.make_plan(stream)
-            return self.forward(proj, stream, out)
+        if self.plan_inside or not overlap or self.plan.k_marg == 0:
+            return self._run_step(q, k, v, proj, stream, self.out if out is None else out)
         main = torch.cuda.current_stream(self.device) if stream is None else stream
         if self._side is None:
             self._side = torch.cuda.Stream(self.device)
@@ -540,8 +598,14 @@ class SlaForward:
             graph = torch.cuda.CUDAGraph()
             capture_stream = torch.cuda.Stream(self.device)
             capture_stream.wait_stream(torch.cuda.current_stream(self.device))
-            with torch.cuda.graph(graph, stream=capture_stream):
-                self.run(q, k, v, proj, out=out, overlap=True)
+            with torch.cuda.stream(capture_stream):
+                # (not torch.cuda.graph: it also collects garbage and empties the allocator's cache, which takes longer
+                # than the capture, now and then half a second, and is of no use to a step that allocates nothing)
+                graph.capture_begin()
+                try:
+                    self.run(q, k, v, proj, out=out, overlap=True)
+                finally:
+                    graph.capture_end()
             torch.cuda.current_stream(self.device).wait_stream(capture_stream)
             self._graph = (graph, key)
         self._graph[0].replay()

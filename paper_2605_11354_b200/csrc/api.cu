@@ -338,7 +338,7 @@ static lite3r_status forward_phases(int phases, const lite3r_fp8* q, const lite3
                                     double crit, double neg, lite3r_phi phi, const lite3r_plan* plan, void* out,
                                     lite3r_dtype out_dtype, long long out_stride_b, long long out_stride_h,
                                     long long out_stride_n, void* workspace, size_t workspace_bytes,
-                                    int* device_status, void* stream, int linear_only = 0) {
+                                    int* device_status, void* stream, int linear_only = 0, bool check_only = false) {
   lite3r_status st = check_shape(shape);
   if (st != LITE3R_OK) return st;
   if ((st = check_fp8(k, true, false)) != LITE3R_OK) return st;
@@ -380,6 +380,7 @@ static lite3r_status forward_phases(int phases, const lite3r_fp8* q, const lite3
   if (workspace == nullptr || !aligned(workspace, 256)) return LITE3R_ERR_INVALID_ARG;
   if (workspace_bytes < forward_workspace_bytes(*shape, c, plan_inside)) return LITE3R_ERR_WORKSPACE;
   if ((st = check_device()) != LITE3R_OK) return st;
+  if (check_only) return LITE3R_OK;
   ForwardArgs a = {};
   if (q != nullptr) a.q = *q;
   a.k = *k;
@@ -411,6 +412,42 @@ lite3r_status lite3r_sla_forward(const lite3r_fp8* q, const lite3r_fp8* k, const
                                  void* workspace, size_t workspace_bytes, int* device_status, void* stream) {
   return forward_phases(3, q, k, v, proj, proj_head_stride, shape, crit, neg, phi, plan, out, out_dtype, out_stride_b,
                         out_stride_h, out_stride_n, workspace, workspace_bytes, device_status, stream);
+}
+
+lite3r_status lite3r_sla_step(lite3r_step* t, void* stream) {
+  if (t == nullptr) return LITE3R_ERR_INVALID_ARG;
+  lite3r_status st = check_shape(&t->shape);
+  if (st != LITE3R_OK) return st;
+  if ((st = check_fractions(t->crit, t->neg)) != LITE3R_OK) return st;
+  const lite3r_tensor* x[3] = {&t->q, &t->k, &t->v};
+  const lite3r_fp8 x8[3] = {t->q8, t->k8, t->v8};
+  for (int n = 0; n < 3; ++n) {
+    if ((st = check_source(x[n])) != LITE3R_OK) return st;
+    if ((st = check_fp8(&x8[n], true, n < 2)) != LITE3R_OK) return st;
+  }
+  const bool plan_inside = t->plan.cls == nullptr;
+  const Counts c = class_counts(ceil_div(t->shape.tokens, t->shape.block), t->crit, t->neg);
+  t->plan.k_crit = c.k_crit;
+  t->plan.k_marg = c.k_marg;
+  t->plan.k_neg = c.k_neg;
+  if (!plan_inside && c.k_crit > 0 && t->plan.crit_idx == nullptr) return LITE3R_ERR_INVALID_ARG;
+  for (int pass = 0; pass < 2; ++pass) {  // checked as a whole before the first launch
+    if (pass == 1) {
+      cudaStream_t cs = static_cast<cudaStream_t>(stream);
+      if (t->q.dtype == t->k.dtype && t->q.dtype == t->v.dtype) {
+        st = launch_quantize(x, x8, 3, t->shape, cs);
+      } else {
+        for (int n = 0; n < 3 && st == LITE3R_OK; ++n) st = launch_quantize(&x[n], &x8[n], 1, t->shape, cs);
+      }
+      if (st != LITE3R_OK) return st;
+      if (!plan_inside && (st = launch_plan(t->q8, t->k8, t->shape, c, t->plan, cs)) != LITE3R_OK) return st;
+    }
+    st = forward_phases(3, &t->q8, &t->k8, &t->v8, t->proj, t->proj_head_stride, &t->shape, t->crit, t->neg, t->phi,
+                        plan_inside ? nullptr : &t->plan, t->out, t->out_dtype, t->out_stride_b, t->out_stride_h,
+                        t->out_stride_n, t->workspace, t->workspace_bytes, t->device_status, stream, 0, pass == 0);
+    if (st != LITE3R_OK) return st;
+  }
+  return LITE3R_OK;
 }
 
 lite3r_status lite3r_sla_forward_begin(const lite3r_fp8* k, const lite3r_fp8* v, const float* proj,
