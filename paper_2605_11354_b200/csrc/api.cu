@@ -164,8 +164,9 @@ const CUtensorMap* cached_map(const MapKey& key) {
 }  // namespace
 
 const CUtensorMap* make_tensor_map_2d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
-                                      uint64_t rows, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle) {
-  return cached_map({base, {inner, rows, 0, 0}, {inner * static_cast<uint64_t>(elem_bytes), 0, 0}, {box_inner, box_rows, 0, 0},
+                                      uint64_t rows, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle,
+                                      uint64_t pitch_bytes) {
+  return cached_map({base, {inner, rows, 0, 0}, {pitch_bytes != 0 ? pitch_bytes : inner * static_cast<uint64_t>(elem_bytes), 0, 0}, {box_inner, box_rows, 0, 0},
                      type, 2, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B});
 }
 

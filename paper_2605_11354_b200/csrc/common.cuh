@@ -156,12 +156,13 @@ lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const flo
 lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls, const lite3r_shape& s, int nb,
                                __nv_bfloat16* g16, float* zeta, int* device_status, bool after_wait, cudaStream_t stream);
 
-// TMA descriptor of a row-major 2-D tensor [rows][inner] (row pitch = inner * elem_bytes, a multiple of 16 bytes)
+// TMA descriptor of a row-major 2-D tensor [rows][inner] (row pitch in bytes, 0: inner * elem_bytes; a multiple of 16)
 // with a box of box_inner x box_rows elements.  The make_tensor_map functions return a descriptor kept by the calling
 // thread (valid until the thread has asked for a few hundred others): descriptors depend on their arguments only, and a
 // caller that runs the same buffers again, or those of many layers in turn, finds them encoded.  NULL: refused.
 const CUtensorMap* make_tensor_map_2d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
-                                      uint64_t rows, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle);
+                                      uint64_t rows, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle,
+                                      uint64_t pitch_bytes = 0);
 // The same for a 3-D tensor [planes][rows][inner] with a box of box_inner x box_rows x 1 (rows past the end of a plane
 // are zero-filled, so a tile never runs into the next plane).
 const CUtensorMap* make_tensor_map_3d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,

@@ -24,29 +24,99 @@ namespace {
 using namespace sm100;
 
 // ------------------------------------------------------------------------------------------------ row quantiser
-__device__ __forceinline__ void load8(const __nv_bfloat16* p, float v[8]) {
-  const uint4 w = *reinterpret_cast<const uint4*>(p);
-  const uint32_t x[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    v[2 * i] = __uint_as_float(x[i] << 16);
-    v[2 * i + 1] = __uint_as_float(x[i] & 0xFFFF0000u);
-  }
-}
-__device__ __forceinline__ void load8(const float* p, float v[8]) {
-  const float4 a = *reinterpret_cast<const float4*>(p);
-  const float4 b = *reinterpret_cast<const float4*>(p + 4);
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
 // e4m3 codes of x / scale (IEEE fp32 division, saturation at +-448, round to nearest even), two values per call
 __device__ __forceinline__ uint32_t quantise_pair(float a, float b, float scale) {
   return __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(a, scale), __fdiv_rn(b, scale)), __NV_SATFINITE, __NV_E4M3);
 }
 
-// One warp per row.  Rows of up to 1024 values are held in registers; longer ones are read twice (maximum, then codes;
-// the second read comes from L1 / L2).
+// Eight values as they lie in memory, their conversion to fp32 and the running maximum of their magnitudes (for bf16 on
+// packed pairs: the maximum of bf16 values is one of them).
 template <typename SrcT>
+struct Eight;
+template <>
+struct Eight<__nv_bfloat16> {
+  uint4 w;
+  using Max = __nv_bfloat162;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) { w = __ldg(reinterpret_cast<const uint4*>(p)); }
+  __device__ __forceinline__ void clear() { w = make_uint4(0u, 0u, 0u, 0u); }
+  static __device__ __forceinline__ Max zero() { return __float2bfloat162_rn(0.f); }
+  __device__ __forceinline__ Max max_with(Max m) const {
+    const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m = __hmax2(m, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[i])));
+    return m;
+  }
+  static __device__ __forceinline__ float top(Max m) { return fmaxf(__low2float(m), __high2float(m)); }
+  __device__ __forceinline__ void values(float v[8]) const {
+    const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      v[2 * i] = __uint_as_float(x[i] << 16);
+      v[2 * i + 1] = __uint_as_float(x[i] & 0xFFFF0000u);
+    }
+  }
+};
+template <>
+struct Eight<float> {
+  float4 a, b;
+  using Max = float;
+  __device__ __forceinline__ void load(const float* p) {
+    a = __ldg(reinterpret_cast<const float4*>(p));
+    b = __ldg(reinterpret_cast<const float4*>(p + 4));
+  }
+  __device__ __forceinline__ void clear() { a = b = make_float4(0.f, 0.f, 0.f, 0.f); }
+  static __device__ __forceinline__ Max zero() { return 0.f; }
+  __device__ __forceinline__ Max max_with(Max m) const {
+    m = fmaxf(fmaxf(m, fabsf(a.x)), fmaxf(fabsf(a.y), fmaxf(fabsf(a.z), fabsf(a.w))));
+    return fmaxf(fmaxf(m, fabsf(b.x)), fmaxf(fabsf(b.y), fmaxf(fabsf(b.z), fabsf(b.w))));
+  }
+  static __device__ __forceinline__ float top(Max m) { return m; }
+  __device__ __forceinline__ void values(float v[8]) const {
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  }
+};
+
+// Codes of eight values of a row with this scale.  x / scale must be the IEEE quotient, but only its e4m3 rounding is
+// kept: the quotient lies between x * r_lo and x * r_hi (r = 1 / scale widened by 2^-20 either way) and rounding is
+// monotone, so equal codes of the two products are the quotient's code; otherwise the eight values are redone with the
+// division.
+struct RowScale {
+  float scale;
+  uint64_t lo2, hi2;
+  __device__ __forceinline__ explicit RowScale(float amax) {
+    scale = __fdiv_rn(__fadd_rn(amax, 1e-8f), 448.0f);
+    const float rcp = __frcp_rn(scale);
+    lo2 = pack_f32x2(rcp * (1.0f - 0x1p-20f), rcp * (1.0f - 0x1p-20f));
+    hi2 = pack_f32x2(rcp * (1.0f + 0x1p-20f), rcp * (1.0f + 0x1p-20f));
+  }
+  __device__ __forceinline__ uint2 codes(const float v[8]) const {
+    const uint64_t neg0 = pack_f32x2(-0.f, -0.f);  // x * r + (-0) is x * r, signed zeros included
+    uint32_t two[4], differ = 0u;
+#pragma unroll
+    for (int c = 0; c < 8; c += 2) {
+      const uint64_t x2 = pack_f32x2(v[c], v[c + 1]);
+      float2 q_lo, q_hi;
+      unpack_f32x2(fma_f32x2(x2, lo2, neg0), q_lo.x, q_lo.y);
+      unpack_f32x2(fma_f32x2(x2, hi2, neg0), q_hi.x, q_hi.y);
+      const uint32_t lo = __nv_cvt_float2_to_fp8x2(q_lo, __NV_SATFINITE, __NV_E4M3);
+      two[c >> 1] = __nv_cvt_float2_to_fp8x2(q_hi, __NV_SATFINITE, __NV_E4M3);
+      differ |= lo ^ two[c >> 1];
+    }
+    if (differ != 0u) {
+#pragma unroll
+      for (int c = 0; c < 8; c += 2) two[c >> 1] = quantise_pair(v[c], v[c + 1], scale);
+    }
+    return make_uint2(two[0] | (two[1] << 16), two[2] | (two[3] << 16));
+  }
+};
+
+// One warp per row.  Rows of up to 256 kSegs values stay in registers as they lie in memory (all requested before the
+// first is used), and bf16 rows of that length are requested one row ahead, so that a warp's loads run under the
+// arithmetic of the row before; longer rows are read twice (maximum, then codes; the second read comes from L1 / L2).
+// Bound by issue slots as much as by HBM (two products and two conversions per pair of values are what the exact
+// rounding costs): 43968 x 1024 bf16 values in 39 us before the loads ran ahead and the maximum went to packed pairs.
+template <typename SrcT, int kSegs>
 __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ x, long long row_stride, int rows, int cols,
                                                        uint8_t* __restrict__ codes, float* __restrict__ scales) {
   wait_for_prior_grid();
@@ -54,107 +124,74 @@ __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ 
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int segs = cols >> 3;
-  for (int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < rows; row += warps) {
-    const SrcT* src = x + static_cast<long long>(row) * row_stride;
-    if (segs <= 4 * 32) {
-      // rows of up to 1024 values stay in registers between the two sweeps (four 8-value segments per lane, all
-      // requested before the first is used): one pass over memory
-      float v[4][8];
+  int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if constexpr (kSegs > 0) {
+    constexpr bool kAhead = sizeof(SrcT) == 2;
+    Eight<SrcT> next[kSegs];
+    auto fetch = [&](int r) {
+      const SrcT* src = x + static_cast<long long>(r) * row_stride + lane * 8;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (lane + 32 * q < segs) {
-          load8(src + (lane + 32 * q) * 8, v[q]);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 8; ++c) v[q][c] = 0.f;
-        }
+      for (int q = 0; q < kSegs; ++q) {
+        if (lane + 32 * q < segs) next[q].load(src + 256 * q);
+        else next[q].clear();
       }
-      float amax = 0.f;
+    };
+    if (row < rows) fetch(row);
+    for (; row < rows; row += warps) {
+      if (!kAhead) fetch(row);
+      Eight<SrcT> cur[kSegs];
+      typename Eight<SrcT>::Max m = Eight<SrcT>::zero();
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int q = 0; q < kSegs; ++q) {
+        cur[q] = next[q];
+        m = cur[q].max_with(m);
+      }
+      if (kAhead && row + warps < rows) fetch(row + warps);
+      const RowScale rs(warp_max(Eight<SrcT>::top(m)));
+      if (lane == 0) scales[row] = rs.scale;
+      uint8_t* dst = codes + static_cast<size_t>(row) * cols + lane * 8;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) amax = fmaxf(amax, fabsf(v[q][c]));
-      amax = warp_max(amax);
-      const float scale = __fdiv_rn(__fadd_rn(amax, 1e-8f), 448.0f);
-      if (lane == 0) scales[row] = scale;
-      uint8_t* dst = codes + static_cast<size_t>(row) * cols;
-      const float rcp = __frcp_rn(scale);
-      const uint64_t r_lo2 = pack_f32x2(rcp * (1.0f - 0x1p-20f), rcp * (1.0f - 0x1p-20f));
-      const uint64_t r_hi2 = pack_f32x2(rcp * (1.0f + 0x1p-20f), rcp * (1.0f + 0x1p-20f));
-      const uint64_t neg0 = pack_f32x2(-0.f, -0.f);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < kSegs; ++q) {
         if (lane + 32 * q >= segs) continue;
-        uint32_t two[4], differ = 0u;
-#pragma unroll
-        for (int c = 0; c < 8; c += 2) {
-          const uint64_t x2 = pack_f32x2(v[q][c], v[q][c + 1]);
-          float2 q_lo, q_hi;
-          unpack_f32x2(fma_f32x2(x2, r_lo2, neg0), q_lo.x, q_lo.y);
-          unpack_f32x2(fma_f32x2(x2, r_hi2, neg0), q_hi.x, q_hi.y);
-          const uint32_t lo = __nv_cvt_float2_to_fp8x2(q_lo, __NV_SATFINITE, __NV_E4M3);
-          two[c >> 1] = __nv_cvt_float2_to_fp8x2(q_hi, __NV_SATFINITE, __NV_E4M3);
-          differ |= lo ^ two[c >> 1];
-        }
-        if (differ != 0u) {  // next to a rounding boundary of the e4m3 grid: redone with the division
-#pragma unroll
-          for (int c = 0; c < 8; c += 2) two[c >> 1] = quantise_pair(v[q][c], v[q][c + 1], scale);
-        }
-        *reinterpret_cast<uint2*>(dst + (lane + 32 * q) * 8) = make_uint2(two[0] | (two[1] << 16), two[2] | (two[3] << 16));
+        float v[8];
+        cur[q].values(v);
+        *reinterpret_cast<uint2*>(dst + 256 * q) = rs.codes(v);
       }
-      continue;
     }
-    float amax = 0.f;
-    for (int s = lane; s < segs; s += 32) {
-      float v[8];
-      load8(src + s * 8, v);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) amax = fmaxf(amax, fabsf(v[c]));
-    }
-    amax = warp_max(amax);
-    const float scale = __fdiv_rn(__fadd_rn(amax, 1e-8f), 448.0f);
-    if (lane == 0) scales[row] = scale;
-    uint8_t* dst = codes + static_cast<size_t>(row) * cols;
-    // x / scale must be the IEEE quotient, but only its e4m3 rounding is kept: the quotient lies between x * r_lo and
-    // x * r_hi (r = 1 / scale widened by 2^-20 either way) and rounding is monotone, so equal codes of the two products
-    // are the quotient's code; otherwise the eight values are redone with the division.
-    const float rcp = __frcp_rn(scale);
-    const uint64_t r_lo2 = pack_f32x2(rcp * (1.0f - 0x1p-20f), rcp * (1.0f - 0x1p-20f));
-    const uint64_t r_hi2 = pack_f32x2(rcp * (1.0f + 0x1p-20f), rcp * (1.0f + 0x1p-20f));
-    const uint64_t neg0 = pack_f32x2(-0.f, -0.f);
-    for (int s = lane; s < segs; s += 32) {
-      float v[8];
-      load8(src + s * 8, v);
-      uint32_t two[4], differ = 0u;
-#pragma unroll
-      for (int c = 0; c < 8; c += 2) {
-        const uint64_t x2 = pack_f32x2(v[c], v[c + 1]);
-        float2 q_lo, q_hi;
-        unpack_f32x2(fma_f32x2(x2, r_lo2, neg0), q_lo.x, q_lo.y);
-        unpack_f32x2(fma_f32x2(x2, r_hi2, neg0), q_hi.x, q_hi.y);
-        const uint32_t lo = __nv_cvt_float2_to_fp8x2(q_lo, __NV_SATFINITE, __NV_E4M3);
-        two[c >> 1] = __nv_cvt_float2_to_fp8x2(q_hi, __NV_SATFINITE, __NV_E4M3);
-        differ |= lo ^ two[c >> 1];
+  } else {
+    for (; row < rows; row += warps) {
+      const SrcT* src = x + static_cast<long long>(row) * row_stride;
+      typename Eight<SrcT>::Max m = Eight<SrcT>::zero();
+      Eight<SrcT> e;
+      for (int s = lane; s < segs; s += 32) {
+        e.load(src + s * 8);
+        m = e.max_with(m);
       }
-      if (differ != 0u) {
-#pragma unroll
-        for (int c = 0; c < 8; c += 2) two[c >> 1] = quantise_pair(v[c], v[c + 1], scale);
+      const RowScale rs(warp_max(Eight<SrcT>::top(m)));
+      if (lane == 0) scales[row] = rs.scale;
+      uint8_t* dst = codes + static_cast<size_t>(row) * cols;
+      for (int s = lane; s < segs; s += 32) {
+        float v[8];
+        e.load(src + s * 8);
+        e.values(v);
+        *reinterpret_cast<uint2*>(dst + s * 8) = rs.codes(v);
       }
-      *reinterpret_cast<uint2*>(dst + s * 8) = make_uint2(two[0] | (two[1] << 16), two[2] | (two[3] << 16));
     }
   }
 }
 
 // ------------------------------------------------------------------------------------------------ GEMM
-constexpr int kStages = 4;
+constexpr int kStages = 3;
 constexpr int kTileM = 128, kTileN = 256, kTileK = 128;  // K in bytes = e4m3 elements
 constexpr int kEpiGroups = kTileN / 64;                   // epilogue warpgroups, one per 64 columns (one head) of the tile
 constexpr int kThreads = 128 + kEpiGroups * 128;          // 4 control warps + the epilogue warpgroups
 constexpr uint32_t kStageBytes = kTileM * kTileK + kTileN * kTileK;  // 48 KB
 constexpr uint32_t kOffB = kTileM * kTileK;
-constexpr uint32_t kOffMisc = kStages * kStageBytes;  // column scales (1 KB), bias (1 KB), reduction slots, column sums
-constexpr uint32_t kOffBar = kOffMisc + 5120;  // + column sums (2 KB)
-constexpr uint32_t kSmemBytes = kOffBar + 256;  // 201984 B: one CTA per SM
+constexpr uint32_t kOffOut = kStages * kStageBytes;   // staged output, 16 KB per epilogue warpgroup (4 KB per warp)
+constexpr uint32_t kOffMisc = kOffOut + kEpiGroups * 16384;  // column scales and bias (two tiles each), reduction slots,
+                                                             // column sums
+constexpr uint32_t kOffBar = kOffMisc + 4096 + 64 + 2048;
+constexpr uint32_t kSmemBytes = kOffBar + 256;  // 219456 B: one CTA per SM
 constexpr uint32_t kAccCols = kTileN;           // one accumulator (128 x 256 fp32)
 constexpr uint32_t kTmemCols = 2 * kAccCols;    // two of them (all of tensor memory): the products of the next tile run
                                                 // under this tile's epilogue
@@ -184,6 +221,12 @@ struct LinearParams {
   int* status;
 };
 
+// Tensor maps of the output: y in boxes of 32 rows x 128 bytes (128B swizzle), or the codes of q, k and v in boxes of 64
+// rows x 64 bytes (64B swizzle).
+struct OutMaps {
+  CUtensorMap m[3];
+};
+
 __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -196,7 +239,7 @@ __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
 // every epilogue and the kernel was bound by the latency of its loads, not by the tensor pipe or the epilogue.
 __global__ void __launch_bounds__(kThreads, 1)
 linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                  const LinearParams p) {
+                  const __grid_constant__ OutMaps maps, const LinearParams p) {
   extern __shared__ __align__(1024) uint8_t smem[];
   Bars* bars = reinterpret_cast<Bars*>(smem + kOffBar);
   volatile int* abort_flag = &bars->abort;
@@ -223,9 +266,8 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     return t;
   };
 
-  float* const s_wscale = reinterpret_cast<float*>(smem + kOffMisc);
-  float* const s_bias = s_wscale + kTileN;
-  float* const s_red = s_bias + kTileN;  // 4 floats per epilogue warpgroup
+  float* const s_wscale = reinterpret_cast<float*>(smem + kOffMisc);  // [2][256] column scales, [2][256] bias
+  float* const s_red = s_wscale + 4 * kTileN;  // 4 floats per epilogue warpgroup
   int* const s_colsum = reinterpret_cast<int*>(s_red + 4 * kEpiGroups);  // 128 ints per epilogue warpgroup
 
   if (threadIdx.x == 0) {
@@ -304,8 +346,7 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const int hh = (warp - 4) >> 2;     // which 64 columns of the tile this warpgroup owns
     const int r = quarter * 32 + lane;  // row of the tile = TMEM lane
     const int tid = threadIdx.x - (4 + hh * 4) * 32;  // thread of the warpgroup
-    float* const wsc = s_wscale + hh * 64;
-    float* const bia = s_bias + hh * 64;
+    uint8_t* const staged = smem + kOffOut + hh * 16384;  // this warpgroup's output on its way to memory
     const int bar_id = 1 + hh;
     bool ok = true;
     int it = 0;
@@ -317,7 +358,10 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const uint32_t acc_addr = tmem + ((static_cast<uint32_t>(quarter) * 32u) << 16) + ab * kAccCols + hh * 64;
     const float sx = row_ok ? __ldg(p.x_scales + row0 + r) : 0.f;
     const int col = ta.col0 + hh * 64;
-    // this warpgroup's 64 column scales and biases (the previous tile's were released by the barrier that ends a tile)
+    // this warpgroup's 64 column scales and biases: two sets by turns, so that this barrier is also what separates the
+    // last reads of a set from its next writes
+    float* const wsc = s_wscale + ab * kTileN + hh * 64;
+    float* const bia = wsc + 2 * kTileN;
     if (tid < 64) {
       wsc[tid] = col + tid < p.d_out ? __ldg(p.w_scales + col + tid) : 0.f;
       bia[tid] = (p.bias != nullptr && col + tid < p.d_out) ? __ldg(p.bias + col + tid) : 0.f;
@@ -328,42 +372,61 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     ok = __all_sync(0xFFFFFFFFu, ok);
     if (!ok) break;
     if (col < p.d_out && !p.fused) {
-      // y = acc * (sx * sw) + b, written row by row (a thread owns 128 contiguous bytes per 32 fp32 columns)
-      uint8_t* const yrow = static_cast<uint8_t*>(p.y) +
-                            static_cast<long long>(row0 + r) * p.y_stride * (p.y_dtype == LITE3R_F32 ? 4 : 2);
+      // y = acc * (sx * sw) + b.  The warp stages its 32 rows, 128 bytes at a time, in the layout the store engine reads
+      // (128B swizzle); rows and columns past the output are clipped by the engine.
+      const bool wide = p.y_dtype == LITE3R_F32;
+      uint8_t* const warp_tile = staged + quarter * 4096;
+      const uint32_t my_row = smem_u32(warp_tile) + lane * 128;
+      const int swz = lane & 7;
 #pragma unroll 1
       for (int cb = 0; cb < 64; cb += 32) {
         uint32_t v[32];
         tmem_ld32(acc_addr + cb, v);
+        if (wide || cb == 0) {  // what was staged here before has been read by the store engine
+          if (lane == 0) bulk_wait_group_read0();
+          __syncwarp();
+        }
         tmem_wait_ld();
         if (cb == 32) {  // the accumulator is in registers: the issuer may reuse it
           tc_fence_before();
           mbar_arrive(&bars->acc_empty[ab]);
         }
-        if (!row_ok) continue;
-        float y[32];
 #pragma unroll
-        for (int c = 0; c < 32; ++c) y[c] = fmaf(__uint_as_float(v[c]), sx * wsc[cb + c], bia[cb + c]);
-        if (p.y_dtype == LITE3R_F32) {
-          float4* dst = reinterpret_cast<float4*>(yrow + static_cast<size_t>(col + cb) * 4);
+        for (int c = 0; c < 32; c += 4) {
+          const float4 sw4 = *reinterpret_cast<const float4*>(wsc + cb + c);
+          const float4 b4 = *reinterpret_cast<const float4*>(bia + cb + c);
+          v[c] = __float_as_uint(fmaf(__uint_as_float(v[c]), sx * sw4.x, b4.x));
+          v[c + 1] = __float_as_uint(fmaf(__uint_as_float(v[c + 1]), sx * sw4.y, b4.y));
+          v[c + 2] = __float_as_uint(fmaf(__uint_as_float(v[c + 2]), sx * sw4.z, b4.z));
+          v[c + 3] = __float_as_uint(fmaf(__uint_as_float(v[c + 3]), sx * sw4.w, b4.w));
+        }
+        if (wide) {
 #pragma unroll
-          for (int c = 0; c < 8; ++c) dst[c] = make_float4(y[4 * c], y[4 * c + 1], y[4 * c + 2], y[4 * c + 3]);
+          for (int c = 0; c < 8; ++c) sts128(my_row + ((c ^ swz) << 4), v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
         } else {
-          uint4* dst = reinterpret_cast<uint4*>(yrow + static_cast<size_t>(col + cb) * 2);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             uint32_t w[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
+              const float y0 = __uint_as_float(v[8 * c + 2 * q]), y1 = __uint_as_float(v[8 * c + 2 * q + 1]);
               if (p.y_dtype == LITE3R_BF16) {
-                __nv_bfloat162 h = __floats2bfloat162_rn(y[8 * c + 2 * q], y[8 * c + 2 * q + 1]);
+                __nv_bfloat162 h = __floats2bfloat162_rn(y0, y1);
                 w[q] = *reinterpret_cast<uint32_t*>(&h);
               } else {
-                __half2 h = __floats2half2_rn(y[8 * c + 2 * q], y[8 * c + 2 * q + 1]);
+                __half2 h = __floats2half2_rn(y0, y1);
                 w[q] = *reinterpret_cast<uint32_t*>(&h);
               }
             }
-            dst[c] = make_uint4(w[0], w[1], w[2], w[3]);
+            sts128(my_row + (((cb / 8 + c) ^ swz) << 4), w[0], w[1], w[2], w[3]);
+          }
+        }
+        if (wide || cb == 32) {
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_2d(&maps.m[0], warp_tile, col + (wide ? cb : 0), row0 + quarter * 32);
+            bulk_commit_group();
           }
         }
       }
@@ -376,6 +439,9 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       const int my_block = r / p.block;                       // token block of the tile this row is in
       const int block_first_warp = my_block * (p.block / 32);  // first warp (0..3) of that block in the warpgroup
       float* const red = s_red + hh * 4;
+      int* const cs = s_colsum + hh * 128;  // column sums [token block of the tile][64]
+      cs[tid] = 0;
+      if (tid == 0) bulk_wait_group_read0();  // the codes of the tile before have left their place
       // pass 1: the row's largest magnitude, then the block's
       // (two columns per instruction: sx * sw and acc * (sx sw) + b as packed fp32 pairs, each lane rounded exactly
       // as the scalar expression would be)
@@ -413,7 +479,8 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       const float r_lo = rcp * (1.0f - 0x1p-20f), r_hi = rcp * (1.0f + 0x1p-20f);
       const uint64_t r_lo2 = pack_f32x2(r_lo, r_lo), r_hi2 = pack_f32x2(r_hi, r_hi);
       const bool want_colsum = p.colsum[part] != nullptr;
-      uint4* const gdst = reinterpret_cast<uint4*>(p.codes[part] + (tile_out * p.block + (r % p.block)) * kHeadDim);
+      const uint32_t my_row = smem_u32(staged) + r * 64;
+      const int swz = (r >> 1) & 3;
 #pragma unroll 1
       for (int cb = 0; cb < 64; cb += 32) {
         uint32_t v[32], packed[8];
@@ -447,44 +514,43 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           }
           packed[c >> 2] = row_ok ? (two[0] | (two[1] << 16)) : 0u;
         }
-        if (block_ok) {  // rows past the sequence end inside an existing block are written as zeros
-          gdst[cb / 16] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-          gdst[cb / 16 + 1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
-        }
+        // rows past the sequence end inside an existing block are written as zeros
+        sts128(my_row + (((cb / 16) ^ swz) << 4), packed[0], packed[1], packed[2], packed[3]);
+        sts128(my_row + (((cb / 16 + 1) ^ swz) << 4), packed[4], packed[5], packed[6], packed[7]);
+      }
+      fence_proxy_async_smem();
+      named_barrier_sync(bar_id, 128);
+      if (tid == 0) {  // two boxes of 64 rows, as far as their blocks exist
+        const int first_row = static_cast<int>((static_cast<size_t>(seq) * p.heads + head) * p.nb * p.block) + tile_in_seq * kTileM;
+        for (int x = 0; x < 2; ++x)
+          if (tile_in_seq * kTileM + x * 64 < p.nb * p.block) tma_store_2d(&maps.m[part], staged + x * 4096, 0, first_row + x * 64);
+        bulk_commit_group();
       }
       if (want_colsum) {
-        // Column sums of the code values (exact integers in units of 2^-9) from the codes the warpgroup has just written
-        // (the barrier orders them; the loads go to L2, past the first-level cache): a thread adds four columns over 16
-        // rows in fp32 (exact: at most 16 x 448 in steps of 2^-9), the eight row groups of the tile meet in shared memory.
-        int* const cs = s_colsum + hh * 128;  // [token block of the tile][64]
-        cs[tid] = 0;
-        named_barrier_sync(bar_id, 128);
-        {
-          const int cg = tid & 15, row_first = (tid >> 4) * 16;
-          const int blk = row_first / p.block;
-          const int tb = tile_in_seq * blocks_in_tile + blk;
-          if (tb < p.nb) {
-            const size_t out_tile = (static_cast<size_t>(seq) * p.heads + head) * p.nb + tb;
-            const uint32_t* src =
-                reinterpret_cast<const uint32_t*>(p.codes[part] + (out_tile * p.block + (row_first % p.block)) * kHeadDim) + cg;
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 4
-            for (int rr = 0; rr < 16; ++rr) {
-              const uint32_t w4 = __ldcg(src + rr * (kHeadDim / 4));
-              const __half2_raw lo = __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(w4 & 0xFFFFu), __NV_E4M3);
-              const __half2_raw hi = __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(w4 >> 16), __NV_E4M3);
-              const float2 f01 = __half22float2(__half2(lo)), f23 = __half22float2(__half2(hi));
-              a0 += f01.x;
-              a1 += f01.y;
-              a2 += f23.x;
-              a3 += f23.y;
-            }
-            int* dst = cs + blk * 64 + cg * 4;
-            atomicAdd(dst, __float2int_rn(a0 * 512.f));
-            atomicAdd(dst + 1, __float2int_rn(a1 * 512.f));
-            atomicAdd(dst + 2, __float2int_rn(a2 * 512.f));
-            atomicAdd(dst + 3, __float2int_rn(a3 * 512.f));
+        // Column sums of the code values (exact integers in units of 2^-9) from the staged codes: a thread adds four columns
+        // over every eighth row in fp32 (exact: at most 8 x 448 in steps of 2^-9), 64 rows at a time, the row groups meet
+        // in shared memory.
+        const int cg = tid & 15;
+#pragma unroll 1
+        for (int x = 0; x < 2; ++x) {
+          float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+          for (int rr = 0; rr < 8; ++rr) {
+            const int row = x * 64 + rr * 8 + (tid >> 4);
+            const uint32_t w4 = *reinterpret_cast<const uint32_t*>(staged + row * 64 + (((cg >> 2) ^ ((row >> 1) & 3)) << 4) + (cg & 3) * 4);
+            const __half2_raw lo = __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(w4 & 0xFFFFu), __NV_E4M3);
+            const __half2_raw hi = __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(w4 >> 16), __NV_E4M3);
+            const float2 f01 = __half22float2(__half2(lo)), f23 = __half22float2(__half2(hi));
+            a0 += f01.x;
+            a1 += f01.y;
+            a2 += f23.x;
+            a3 += f23.y;
           }
+          int* dst = cs + (p.block == 64 ? x * 64 : 0) + cg * 4;
+          atomicAdd(dst, __float2int_rn(a0 * 512.f));
+          atomicAdd(dst + 1, __float2int_rn(a1 * 512.f));
+          atomicAdd(dst + 2, __float2int_rn(a2 * 512.f));
+          atomicAdd(dst + 3, __float2int_rn(a3 * 512.f));
         }
         named_barrier_sync(bar_id, 128);
         if (tid < blocks_in_tile * 64) {
@@ -498,8 +564,8 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       tc_fence_before();
       mbar_arrive(&bars->acc_empty[ab]);  // nothing to do for columns past the output
     }
-    named_barrier_sync(bar_id, 128);  // the column scales, biases and reduction slots are rewritten for the next tile
     }  // tiles
+    bulk_wait_group_read0();  // what is staged stays in place until it has been read
   }
 
   tc_fence_before();
@@ -510,13 +576,19 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   }
 }
 
-lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const LinearParams& p, cudaStream_t stream) {
+lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const CUtensorMap* const (&out)[3], const LinearParams& p,
+                          cudaStream_t stream) {
   const CUtensorMap* const px = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, x_codes, p.d_in, p.rows, kTileK, kTileM,
                                                    CU_TENSOR_MAP_SWIZZLE_128B);
   const CUtensorMap* const pw = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, w_codes, p.d_in, p.d_out, kTileK, kTileN,
                                                    CU_TENSOR_MAP_SWIZZLE_128B);
   if (px == nullptr || pw == nullptr) return LITE3R_ERR_CUDA;
   const CUtensorMap map_x = *px, map_w = *pw;
+  OutMaps maps;
+  for (int i = 0; i < 3; ++i) {
+    if (out[i] == nullptr) return LITE3R_ERR_CUDA;
+    maps.m[i] = *out[i];
+  }
   lite3r_status st;
   if ((st = ensure_dynamic_smem(linear_fp8_kernel, static_cast<int>(kSmemBytes))) != LITE3R_OK) return st;
   const int row_tiles = p.fused ? p.batch * ceil_div(p.tokens, kTileM) : ceil_div(p.rows, kTileM);
@@ -527,23 +599,29 @@ lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const 
   if ((st = sm_count(&sms)) != LITE3R_OK) return st;
   const int grid = q.tiles < sms ? q.tiles : sms;
   return launch_dependent(linear_fp8_kernel, dim3(static_cast<unsigned>(grid)), kThreads, static_cast<int>(kSmemBytes), stream, map_x,
-                          map_w, q);
+                          map_w, maps, q);
+}
+
+template <typename SrcT>
+lite3r_status launch_rowquant_typed(const SrcT* x, long long row_stride, int rows, int cols, uint8_t* codes, float* scales,
+                                    cudaStream_t stream) {
+  int sms = 0;
+  lite3r_status st = sm_count(&sms);
+  if (st != LITE3R_OK) return st;
+  // rows in registers up to 1024 values (512 with half the registers); four or eight resident CTAs per SM walk the rows
+  const int segs = ceil_div(cols, 256);
+  auto* kernel = segs <= 2 ? rowquant_kernel<SrcT, 2> : segs <= 4 ? rowquant_kernel<SrcT, 4> : rowquant_kernel<SrcT, 0>;
+  const int blocks = std::min(ceil_div(rows, 8), sms * 4);
+  return launch_dependent(kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, stream, x, row_stride, rows, cols, codes, scales);
 }
 
 }  // namespace
 
 lite3r_status launch_rowquant(const void* x, int dtype, long long row_stride, int rows, int cols, uint8_t* codes,
                               float* scales, cudaStream_t stream) {
-  int sms = 0;
-  lite3r_status st = sm_count(&sms);
-  if (st != LITE3R_OK) return st;
-  const int blocks = std::min(ceil_div(rows, 8), sms * 8);
-  const dim3 grid(static_cast<unsigned>(blocks));
-  if (dtype == LITE3R_BF16)
-    return launch_dependent(rowquant_kernel<__nv_bfloat16>, grid, 256, 0, stream, static_cast<const __nv_bfloat16*>(x), row_stride,
-                            rows, cols, codes, scales);
-  return launch_dependent(rowquant_kernel<float>, grid, 256, 0, stream, static_cast<const float*>(x), row_stride, rows, cols, codes,
-                          scales);
+  return dtype == LITE3R_BF16
+             ? launch_rowquant_typed(static_cast<const __nv_bfloat16*>(x), row_stride, rows, cols, codes, scales, stream)
+             : launch_rowquant_typed(static_cast<const float*>(x), row_stride, rows, cols, codes, scales, stream);
 }
 
 lite3r_status launch_linear_fp8(const uint8_t* x_codes, const float* x_scales, const uint8_t* w_codes,
@@ -561,7 +639,13 @@ lite3r_status launch_linear_fp8(const uint8_t* x_codes, const float* x_scales, c
   p.y_dtype = y_dtype;
   p.fused = 0;
   p.status = device_status;
-  return launch_gemm(x_codes, w_codes, p, stream);
+  const int elem = y_dtype == LITE3R_F32 ? 4 : 2;
+  const CUtensorMap* const map_y = make_tensor_map_2d(
+      y_dtype == LITE3R_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+      : y_dtype == LITE3R_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                               : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
+      elem, y, d_out, rows, 128 / elem, 32, CU_TENSOR_MAP_SWIZZLE_128B, static_cast<uint64_t>(y_stride) * elem);
+  return launch_gemm(x_codes, w_codes, {map_y, map_y, map_y}, p, stream);
 }
 
 lite3r_status launch_qkv_project(const uint8_t* x_codes, const float* x_scales, const uint8_t* w_codes,
@@ -586,7 +670,11 @@ lite3r_status launch_qkv_project(const uint8_t* x_codes, const float* x_scales, 
     p.colsum[i] = out[i].colsum;
   }
   p.status = device_status;
-  return launch_gemm(x_codes, w_codes, p, stream);
+  const CUtensorMap* maps[3];
+  for (int i = 0; i < 3; ++i)
+    maps[i] = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, out[i].codes, kHeadDim,
+                                 static_cast<uint64_t>(s.batch) * s.heads * p.nb * s.block, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B);
+  return launch_gemm(x_codes, w_codes, maps, p, stream);
 }
 
 }  // namespace lite3r
