@@ -256,11 +256,10 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed cha
 lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls, const lite3r_shape& s, int nb,
                                __nv_bfloat16* g16, float* zeta, int* device_status, bool after_wait, cudaStream_t stream) {
   const uint64_t rows = static_cast<uint64_t>(s.batch) * s.heads * nb;
-  const CUtensorMap* const map = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hws, kSummaryRow, rows, 64, 64,
-                                                    CU_TENSOR_MAP_SWIZZLE_128B);
-  if (map == nullptr) return LITE3R_ERR_CUDA;
-  const CUtensorMap map_s = *map;
-  lite3r_status st;
+  CUtensorMap map_s;
+  lite3r_status st = make_tensor_map_2d(&map_s, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hws, kSummaryRow, rows, 64, 64,
+                                        CU_TENSOR_MAP_SWIZZLE_128B);
+  if (st != LITE3R_OK) return st;
   st = ensure_dynamic_smem(aggregate_mma_kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
   if (rows > 0x7FFFFFFFull - kTileM) return LITE3R_ERR_UNSUPPORTED;

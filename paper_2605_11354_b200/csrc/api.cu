@@ -135,7 +135,8 @@ struct MapSlot {
 };
 constexpr uint32_t kMapSlots = 512, kMapWays = 4;  // per thread; 512 x 256 bytes
 
-const CUtensorMap* cached_map(const MapKey& key) {
+// Copies the descriptor of `key` to *map (a copy, because the next one asked for may take its slot).
+lite3r_status cached_map(CUtensorMap* map, const MapKey& key) {
   thread_local std::unique_ptr<MapSlot[]> slots;
   thread_local uint32_t next_way = 0;
   if (!slots) slots.reset(new MapSlot[kMapSlots]());
@@ -145,9 +146,12 @@ const CUtensorMap* cached_map(const MapKey& key) {
   for (size_t i = 0; i < sizeof(MapKey) / 8; ++i) h = (h ^ words[i]) * 0x9E3779B97F4A7C15ull, h ^= h >> 29;
   MapSlot* const set = slots.get() + (h % (kMapSlots / kMapWays)) * kMapWays;
   for (uint32_t w = 0; w < kMapWays; ++w)
-    if (std::memcmp(&set[w].key, &key, sizeof(MapKey)) == 0) return &set[w].map;
+    if (std::memcmp(&set[w].key, &key, sizeof(MapKey)) == 0) {
+      *map = set[w].map;
+      return LITE3R_OK;
+    }
   EncodeTiledFn fn = encode_fn();
-  if (fn == nullptr) return nullptr;
+  if (fn == nullptr) return LITE3R_ERR_CUDA;
   MapSlot& slot = set[next_way++ % kMapWays];
   slot.key = MapKey{};  // stays invalid if the driver refuses
   const cuuint32_t estr[4] = {1, 1, 1, 1};
@@ -157,30 +161,31 @@ const CUtensorMap* cached_map(const MapKey& key) {
   if (fn(&slot.map, static_cast<CUtensorMapDataType>(key.type), static_cast<cuuint32_t>(key.rank), const_cast<void*>(key.base), dims,
          strides, key.box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, static_cast<CUtensorMapSwizzle>(key.swizzle),
          static_cast<CUtensorMapL2promotion>(key.l2), CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return nullptr;
+    return LITE3R_ERR_CUDA;
   slot.key = key;
-  return &slot.map;
+  *map = slot.map;
+  return LITE3R_OK;
 }
 }  // namespace
 
-const CUtensorMap* make_tensor_map_2d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
+lite3r_status make_tensor_map_2d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
                                       uint64_t rows, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle,
                                       uint64_t pitch_bytes) {
-  return cached_map({base, {inner, rows, 0, 0}, {pitch_bytes != 0 ? pitch_bytes : inner * static_cast<uint64_t>(elem_bytes), 0, 0}, {box_inner, box_rows, 0, 0},
+  return cached_map(map, {base, {inner, rows, 0, 0}, {pitch_bytes != 0 ? pitch_bytes : inner * static_cast<uint64_t>(elem_bytes), 0, 0}, {box_inner, box_rows, 0, 0},
                      type, 2, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B});
 }
 
-const CUtensorMap* make_tensor_map_3d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
+lite3r_status make_tensor_map_3d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
                                       uint64_t rows, uint64_t planes, uint32_t box_inner, uint32_t box_rows,
                                       CUtensorMapSwizzle swizzle) {
   const uint64_t pitch = inner * static_cast<uint64_t>(elem_bytes);
-  return cached_map({base, {inner, rows, planes, 0}, {pitch, pitch * rows, 0}, {box_inner, box_rows, 1, 0}, type, 3, swizzle,
+  return cached_map(map, {base, {inner, rows, planes, 0}, {pitch, pitch * rows, 0}, {box_inner, box_rows, 1, 0}, type, 3, swizzle,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B});
 }
 
-const CUtensorMap* make_tensor_map_4d(CUtensorMapDataType type, const void* base, const uint64_t dims[4],
+lite3r_status make_tensor_map_4d(CUtensorMap* map, CUtensorMapDataType type, const void* base, const uint64_t dims[4],
                                       const uint64_t strides_bytes[3], const uint32_t box[4], CUtensorMapSwizzle swizzle) {
-  return cached_map({base, {dims[0], dims[1], dims[2], dims[3]}, {strides_bytes[0], strides_bytes[1], strides_bytes[2]},
+  return cached_map(map, {base, {dims[0], dims[1], dims[2], dims[3]}, {strides_bytes[0], strides_bytes[1], strides_bytes[2]},
                      {box[0], box[1], box[2], box[3]}, type, 4, swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE});
 }
 

@@ -834,15 +834,12 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   const lite3r_shape& s = a.shape;
   const int nb = ceil_div(s.tokens, BS);
   const uint64_t tiles = static_cast<uint64_t>(s.batch) * s.heads * nb;
-  const CUtensorMap* const ptrs[4] = {
-      make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.q_codes, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B),
-      make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.k_codes, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B),
-      make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, a.v16, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B),
-      make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.g16, 64, tiles * 64, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)};
-  for (const CUtensorMap* m : ptrs)
-    if (m == nullptr) return LITE3R_ERR_CUDA;
-  const CUtensorMap map_q = *ptrs[0], map_k = *ptrs[1], map_v = *ptrs[2], map_g = *ptrs[3];
-  lite3r_status st = LITE3R_OK;
+  lite3r_status st;
+  CUtensorMap map_q, map_k, map_v, map_g, map_o;
+  if ((st = make_tensor_map_2d(&map_q, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.q_codes, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B)) != LITE3R_OK) return st;
+  if ((st = make_tensor_map_2d(&map_k, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, a.k_codes, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B)) != LITE3R_OK) return st;
+  if ((st = make_tensor_map_2d(&map_v, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, a.v16, 64, tiles * BS, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
+  if ((st = make_tensor_map_2d(&map_g, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.g16, 64, tiles * 64, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
   AttnParams p;
   // The output goes through TMA stores when a tiled map can describe it: the token, head and batch dimensions ordered
   // by stride (dimensions of extent 1 last), 16 tokens x 128 bytes per box.  If the driver refuses the map the kernel
@@ -879,14 +876,15 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
       p.dim_batch = i + 1;
     }
   }
-  const CUtensorMap* out_map = nullptr;
+  p.tma_out = 0;
   if (describable && g_plain_stores.load(std::memory_order_relaxed) == 0)
-    out_map = make_tensor_map_4d(a.out_dtype == LITE3R_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                 : a.out_dtype == LITE3R_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
-                                                              : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
-                                 a.out, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
-  p.tma_out = out_map != nullptr ? 1 : 0;
-  const CUtensorMap map_o = out_map != nullptr ? *out_map : map_q;  // any valid map when it is not used
+    p.tma_out = make_tensor_map_4d(&map_o,
+                                   a.out_dtype == LITE3R_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                   : a.out_dtype == LITE3R_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                                : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
+                                   a.out, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) == LITE3R_OK
+                    ? 1 : 0;
+  if (p.tma_out == 0) map_o = map_q;  // any valid map when it is not used
   p.q_scales = a.q_scales;
   p.k_scales = a.k_scales;
   p.crit_idx = a.crit_idx;

@@ -88,6 +88,45 @@ __device__ __forceinline__ void e4m3x4_to_float(uint32_t packed, float out[4]) {
   out[3] = b.y;
 }
 
+// Scale of a tile or row with this largest magnitude.
+__device__ __forceinline__ float e4m3_scale(float amax) { return __fdiv_rn(__fadd_rn(amax, 1e-8f), 448.0f); }
+
+// The e4m3 codes of x / scale, where x / scale is the correctly rounded fp32 quotient (so that codes equal those of a plain
+// fp32 program bit for bit), saturated at +-448 and rounded to nearest even.  The quotient comes from the correctly
+// rounded reciprocal r and two corrections q + (x - q s) r, whose residual a fused multiply-add gives exactly: the first
+// brings the product x r (up to two ulps off) to within one ulp, after which the second is correctly rounded (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990).  Scales are
+// at least 1e-8 / 448, so the residual is exact for every x whose code is not zero.  Five packed multiply-adds per pair;
+// bracketing the quotient between two products and redoing with a division the pairs whose two codes differ took two
+// multiply-adds and two conversions, but one bf16 value in six hundred lies so close to a rounding boundary that a third
+// of all groups of 256 went through the division.
+// Everything is computed for -x / scale, which keeps the sign of a zero through the corrections; flip undoes it.
+struct E4m3Quotient {
+  unsigned long long neg_r2, s2;
+  static constexpr uint32_t kFlip = 0x80808080u;
+  __device__ __forceinline__ explicit E4m3Quotient(float scale) {
+    const float r = -__frcp_rn(scale);
+    asm("mov.b64 %0, {%1, %1};" : "=l"(neg_r2) : "f"(r));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(s2) : "f"(scale));
+  }
+  // two codes (low byte first), sign bits inverted
+  __device__ __forceinline__ uint32_t pair(unsigned long long x2) const {
+    unsigned long long q, e;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(q) : "l"(x2), "l"(neg_r2));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(e) : "l"(q), "l"(s2), "l"(x2));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(e), "l"(neg_r2), "l"(q));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(e) : "l"(q), "l"(s2), "l"(x2));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(e), "l"(neg_r2), "l"(q));
+    float2 y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(y.x), "=f"(y.y) : "l"(q));
+    return __nv_cvt_float2_to_fp8x2(y, __NV_SATFINITE, __NV_E4M3);
+  }
+  // four codes of two pairs
+  __device__ __forceinline__ uint32_t four(unsigned long long a, unsigned long long b) const {
+    return (pair(a) | (pair(b) << 16)) ^ kFlip;
+  }
+};
+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
@@ -157,19 +196,19 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
                                __nv_bfloat16* g16, float* zeta, int* device_status, bool after_wait, cudaStream_t stream);
 
 // TMA descriptor of a row-major 2-D tensor [rows][inner] (row pitch in bytes, 0: inner * elem_bytes; a multiple of 16)
-// with a box of box_inner x box_rows elements.  The make_tensor_map functions return a descriptor kept by the calling
-// thread (valid until the thread has asked for a few hundred others): descriptors depend on their arguments only, and a
-// caller that runs the same buffers again, or those of many layers in turn, finds them encoded.  NULL: refused.
-const CUtensorMap* make_tensor_map_2d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
+// with a box of box_inner x box_rows elements.  The make_tensor_map functions keep what they have encoded (a few hundred
+// descriptors per calling thread): descriptors depend on their arguments only, and a caller that runs the same buffers
+// again, or those of many layers in turn, gets a copy.
+lite3r_status make_tensor_map_2d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
                                       uint64_t rows, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swizzle,
                                       uint64_t pitch_bytes = 0);
 // The same for a 3-D tensor [planes][rows][inner] with a box of box_inner x box_rows x 1 (rows past the end of a plane
 // are zero-filled, so a tile never runs into the next plane).
-const CUtensorMap* make_tensor_map_3d(CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
+lite3r_status make_tensor_map_3d(CUtensorMap* map, CUtensorMapDataType type, int elem_bytes, const void* base, uint64_t inner,
                                       uint64_t rows, uint64_t planes, uint32_t box_inner, uint32_t box_rows,
                                       CUtensorMapSwizzle swizzle);
 // Rank 4, extents dims[0..3], byte strides of dimensions 1..3 (multiples of 16), box of box[0..3] elements.
-const CUtensorMap* make_tensor_map_4d(CUtensorMapDataType type, const void* base, const uint64_t dims[4],
+lite3r_status make_tensor_map_4d(CUtensorMap* map, CUtensorMapDataType type, const void* base, const uint64_t dims[4],
                                       const uint64_t strides_bytes[3], const uint32_t box[4], CUtensorMapSwizzle swizzle);
 
 // The FP8 linear layer in front of the attention (linear.cu).

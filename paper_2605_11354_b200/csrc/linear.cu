@@ -24,11 +24,6 @@ namespace {
 using namespace sm100;
 
 // ------------------------------------------------------------------------------------------------ row quantiser
-// e4m3 codes of x / scale (IEEE fp32 division, saturation at +-448, round to nearest even), two values per call
-__device__ __forceinline__ uint32_t quantise_pair(float a, float b, float scale) {
-  return __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(a, scale), __fdiv_rn(b, scale)), __NV_SATFINITE, __NV_E4M3);
-}
-
 // Eight values as they lie in memory, their conversion to fp32 and the running maximum of their magnitudes (for bf16 on
 // packed pairs: the maximum of bf16 values is one of them).
 template <typename SrcT>
@@ -77,45 +72,23 @@ struct Eight<float> {
   }
 };
 
-// Codes of eight values of a row with this scale.  x / scale must be the IEEE quotient, but only its e4m3 rounding is
-// kept: the quotient lies between x * r_lo and x * r_hi (r = 1 / scale widened by 2^-20 either way) and rounding is
-// monotone, so equal codes of the two products are the quotient's code; otherwise the eight values are redone with the
-// division.
+// Scale of a row and the codes of eight of its values.
 struct RowScale {
   float scale;
-  uint64_t lo2, hi2;
-  __device__ __forceinline__ explicit RowScale(float amax) {
-    scale = __fdiv_rn(__fadd_rn(amax, 1e-8f), 448.0f);
-    const float rcp = __frcp_rn(scale);
-    lo2 = pack_f32x2(rcp * (1.0f - 0x1p-20f), rcp * (1.0f - 0x1p-20f));
-    hi2 = pack_f32x2(rcp * (1.0f + 0x1p-20f), rcp * (1.0f + 0x1p-20f));
-  }
+  E4m3Quotient quotient;
+  __device__ __forceinline__ explicit RowScale(float amax)
+      : scale(e4m3_scale(amax)), quotient(scale) {}
   __device__ __forceinline__ uint2 codes(const float v[8]) const {
-    const uint64_t neg0 = pack_f32x2(-0.f, -0.f);  // x * r + (-0) is x * r, signed zeros included
-    uint32_t two[4], differ = 0u;
-#pragma unroll
-    for (int c = 0; c < 8; c += 2) {
-      const uint64_t x2 = pack_f32x2(v[c], v[c + 1]);
-      float2 q_lo, q_hi;
-      unpack_f32x2(fma_f32x2(x2, lo2, neg0), q_lo.x, q_lo.y);
-      unpack_f32x2(fma_f32x2(x2, hi2, neg0), q_hi.x, q_hi.y);
-      const uint32_t lo = __nv_cvt_float2_to_fp8x2(q_lo, __NV_SATFINITE, __NV_E4M3);
-      two[c >> 1] = __nv_cvt_float2_to_fp8x2(q_hi, __NV_SATFINITE, __NV_E4M3);
-      differ |= lo ^ two[c >> 1];
-    }
-    if (differ != 0u) {
-#pragma unroll
-      for (int c = 0; c < 8; c += 2) two[c >> 1] = quantise_pair(v[c], v[c + 1], scale);
-    }
-    return make_uint2(two[0] | (two[1] << 16), two[2] | (two[3] << 16));
+    return make_uint2(quotient.four(pack_f32x2(v[0], v[1]), pack_f32x2(v[2], v[3])),
+                      quotient.four(pack_f32x2(v[4], v[5]), pack_f32x2(v[6], v[7])));
   }
 };
 
 // One warp per row.  Rows of up to 256 kSegs values stay in registers as they lie in memory (all requested before the
 // first is used), and bf16 rows of that length are requested one row ahead, so that a warp's loads run under the
 // arithmetic of the row before; longer rows are read twice (maximum, then codes; the second read comes from L1 / L2).
-// Bound by issue slots as much as by HBM (two products and two conversions per pair of values are what the exact
-// rounding costs): 43968 x 1024 bf16 values in 39 us before the loads ran ahead and the maximum went to packed pairs.
+// Bound by HBM: 43968 x 1024 bf16 values in 21.5 us (6.3 TB/s of 135 MB; 31 us while a third of the groups of 256 values
+// went through a division).
 template <typename SrcT, int kSegs>
 __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ x, long long row_stride, int rows, int cols,
                                                        uint8_t* __restrict__ codes, float* __restrict__ scales) {
@@ -467,17 +440,13 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       named_barrier_sync(bar_id, 128);
       amax = 0.f;
       for (int wq = 0; wq < p.block / 32; ++wq) amax = fmaxf(amax, red[block_first_warp + wq]);
-      const float scale = __fdiv_rn(__fadd_rn(amax, 1e-8f), 448.0f);
+      const float scale = e4m3_scale(amax);
       const int token_block = tile_in_seq * blocks_in_tile + my_block;
       const bool block_ok = token_block < p.nb;
       const size_t tile_out = (static_cast<size_t>(seq) * p.heads + head) * p.nb + token_block;
       if (block_ok && (r % p.block) == 0) p.scales[part][tile_out] = scale;
-      // pass 2: codes.  x / scale must be the IEEE quotient, but only its e4m3 rounding is kept: the quotient lies
-      // between x * r_lo and x * r_hi (r = 1 / scale widened by 2^-20 either way) and rounding is monotone, so equal
-      // codes of the two products are the quotient's code; otherwise the pair is redone with the division.
-      const float rcp = __frcp_rn(scale);
-      const float r_lo = rcp * (1.0f - 0x1p-20f), r_hi = rcp * (1.0f + 0x1p-20f);
-      const uint64_t r_lo2 = pack_f32x2(r_lo, r_lo), r_hi2 = pack_f32x2(r_hi, r_hi);
+      // pass 2: codes
+      const E4m3Quotient quotient(scale);
       const bool want_colsum = p.colsum[part] != nullptr;
       const uint32_t my_row = smem_u32(staged) + r * 64;
       const int swz = (r >> 1) & 3;
@@ -495,24 +464,12 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           const ulonglong2 sw4 = *reinterpret_cast<const ulonglong2*>(wsc + cb + c);
           const ulonglong2 b4 = *reinterpret_cast<const ulonglong2*>(bia + cb + c);
           const unsigned long long sws[2] = {sw4.x, sw4.y}, bs[2] = {b4.x, b4.y};
-          uint32_t two[2];
+          uint64_t y2[2];
 #pragma unroll
-          for (int h2 = 0; h2 < 2; ++h2) {
-            const uint64_t y2 = fma_f32x2(pack_f32x2(__uint_as_float(v[c + 2 * h2]), __uint_as_float(v[c + 2 * h2 + 1])),
-                                          fma_f32x2(sx2, sws[h2], neg0), bs[h2]);
-            float2 q_lo, q_hi;
-            unpack_f32x2(fma_f32x2(y2, r_lo2, neg0), q_lo.x, q_lo.y);
-            unpack_f32x2(fma_f32x2(y2, r_hi2, neg0), q_hi.x, q_hi.y);
-            const uint32_t lo = __nv_cvt_float2_to_fp8x2(q_lo, __NV_SATFINITE, __NV_E4M3);
-            uint32_t hi = __nv_cvt_float2_to_fp8x2(q_hi, __NV_SATFINITE, __NV_E4M3);
-            if (lo != hi) {
-              float y0, y1;
-              unpack_f32x2(y2, y0, y1);
-              hi = quantise_pair(y0, y1, scale);
-            }
-            two[h2] = hi;
-          }
-          packed[c >> 2] = row_ok ? (two[0] | (two[1] << 16)) : 0u;
+          for (int h2 = 0; h2 < 2; ++h2)
+            y2[h2] = fma_f32x2(pack_f32x2(__uint_as_float(v[c + 2 * h2]), __uint_as_float(v[c + 2 * h2 + 1])),
+                               fma_f32x2(sx2, sws[h2], neg0), bs[h2]);
+          packed[c >> 2] = row_ok ? quotient.four(y2[0], y2[1]) : 0u;
         }
         // rows past the sequence end inside an existing block are written as zeros
         sts128(my_row + (((cb / 16) ^ swz) << 4), packed[0], packed[1], packed[2], packed[3]);
@@ -576,20 +533,14 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   }
 }
 
-lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const CUtensorMap* const (&out)[3], const LinearParams& p,
+lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const OutMaps& maps, const LinearParams& p,
                           cudaStream_t stream) {
-  const CUtensorMap* const px = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, x_codes, p.d_in, p.rows, kTileK, kTileM,
-                                                   CU_TENSOR_MAP_SWIZZLE_128B);
-  const CUtensorMap* const pw = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, w_codes, p.d_in, p.d_out, kTileK, kTileN,
-                                                   CU_TENSOR_MAP_SWIZZLE_128B);
-  if (px == nullptr || pw == nullptr) return LITE3R_ERR_CUDA;
-  const CUtensorMap map_x = *px, map_w = *pw;
-  OutMaps maps;
-  for (int i = 0; i < 3; ++i) {
-    if (out[i] == nullptr) return LITE3R_ERR_CUDA;
-    maps.m[i] = *out[i];
-  }
+  CUtensorMap map_x, map_w;
   lite3r_status st;
+  if ((st = make_tensor_map_2d(&map_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, x_codes, p.d_in, p.rows, kTileK, kTileM,
+                               CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
+  if ((st = make_tensor_map_2d(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, w_codes, p.d_in, p.d_out, kTileK, kTileN,
+                               CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
   if ((st = ensure_dynamic_smem(linear_fp8_kernel, static_cast<int>(kSmemBytes))) != LITE3R_OK) return st;
   const int row_tiles = p.fused ? p.batch * ceil_div(p.tokens, kTileM) : ceil_div(p.rows, kTileM);
   LinearParams q = p;
@@ -640,12 +591,16 @@ lite3r_status launch_linear_fp8(const uint8_t* x_codes, const float* x_scales, c
   p.fused = 0;
   p.status = device_status;
   const int elem = y_dtype == LITE3R_F32 ? 4 : 2;
-  const CUtensorMap* const map_y = make_tensor_map_2d(
-      y_dtype == LITE3R_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-      : y_dtype == LITE3R_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
-                               : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
-      elem, y, d_out, rows, 128 / elem, 32, CU_TENSOR_MAP_SWIZZLE_128B, static_cast<uint64_t>(y_stride) * elem);
-  return launch_gemm(x_codes, w_codes, {map_y, map_y, map_y}, p, stream);
+  OutMaps maps;
+  const lite3r_status st = make_tensor_map_2d(&maps.m[0],
+                                              y_dtype == LITE3R_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                              : y_dtype == LITE3R_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                                       : CU_TENSOR_MAP_DATA_TYPE_FLOAT16,
+                                              elem, y, d_out, rows, 128 / elem, 32, CU_TENSOR_MAP_SWIZZLE_128B,
+                                              static_cast<uint64_t>(y_stride) * elem);
+  if (st != LITE3R_OK) return st;
+  maps.m[1] = maps.m[2] = maps.m[0];
+  return launch_gemm(x_codes, w_codes, maps, p, stream);
 }
 
 lite3r_status launch_qkv_project(const uint8_t* x_codes, const float* x_scales, const uint8_t* w_codes,
@@ -670,10 +625,12 @@ lite3r_status launch_qkv_project(const uint8_t* x_codes, const float* x_scales, 
     p.colsum[i] = out[i].colsum;
   }
   p.status = device_status;
-  const CUtensorMap* maps[3];
+  OutMaps maps;
+  lite3r_status st;
   for (int i = 0; i < 3; ++i)
-    maps[i] = make_tensor_map_2d(CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, out[i].codes, kHeadDim,
-                                 static_cast<uint64_t>(s.batch) * s.heads * p.nb * s.block, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B);
+    if ((st = make_tensor_map_2d(&maps.m[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, out[i].codes, kHeadDim,
+                                 static_cast<uint64_t>(s.batch) * s.heads * p.nb * s.block, 64, 64, CU_TENSOR_MAP_SWIZZLE_64B)) != LITE3R_OK)
+      return st;
   return launch_gemm(x_codes, w_codes, maps, p, stream);
 }
 

@@ -309,12 +309,11 @@ lite3r_status launch_proj_lin_backward(const __nv_bfloat16* o_lin, const __nv_bf
   const int planes = s.batch * s.heads;
   const int chunks = projgrad_chunks(s, sms);
   const int tiles_per_cta = ceil_div(ceil_div(s.tokens, kTileTok), chunks);
-  const CUtensorMap* const po = make_tensor_map_3d(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o_lin, kHeadDim, s.tokens, planes, kHeadDim,
-                                                   kTileTok, CU_TENSOR_MAP_SWIZZLE_128B);
-  const CUtensorMap* const pg = make_tensor_map_3d(CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, d_out, kHeadDim, s.tokens, planes, kHeadDim,
-                                                   kTileTok, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (po == nullptr || pg == nullptr) return LITE3R_ERR_CUDA;
-  const CUtensorMap map_o = *po, map_g = *pg;
+  CUtensorMap map_o, map_g;
+  if ((st = make_tensor_map_3d(&map_o, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o_lin, kHeadDim, s.tokens, planes, kHeadDim, kTileTok,
+                               CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
+  if ((st = make_tensor_map_3d(&map_g, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, d_out, kHeadDim, s.tokens, planes, kHeadDim, kTileTok,
+                               CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
   if ((st = ensure_dynamic_smem(projgrad_kernel, static_cast<int>(kSmemBytes))) != LITE3R_OK) return st;
   st = launch_dependent(projgrad_kernel, dim3(static_cast<unsigned>(planes * chunks)), kThreads, static_cast<int>(kSmemBytes), stream,
                         map_o, map_g, s.tokens, chunks, tiles_per_cta, partials, device_status);

@@ -23,3 +23,18 @@ def test_attention_grids_around_the_number_of_resident_ctas(block, batch, heads,
     again = torch.empty_like(out)
     eng.forward(torch.from_numpy(inputs["proj"]).cuda(), out=again)
     assert torch.equal(again, out)  # whichever CTA computes a tile
+
+
+@pytest.mark.parametrize("block", [64, 128])
+def test_many_buffer_sets_in_turn(block):
+    """Encoded tensor maps are kept for a few hundred buffers: more sets than that, at addresses that come and go, give the
+    same bytes."""
+    wl = small_workload(f"maps{block}", heads=2, tokens=300, block=block)
+    inputs = wk.make_inputs(wl)
+    first, hold = None, []
+    for i in range(400):
+        eng, out = pu.run_gpu(inputs, wl)
+        first = out.clone() if first is None else first
+        assert torch.equal(out, first)
+        if i % 3:
+            hold.append(eng)  # some buffers stay, the others' addresses are taken over
