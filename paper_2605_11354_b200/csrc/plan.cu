@@ -49,6 +49,7 @@ struct Selection {
 };
 
 constexpr int kBuckets = 256;
+constexpr int kRankMax = 64;     // rows of up to this many blocks are ranked by comparing all pairs of entries
 constexpr int kMaxListed = 128;  // candidates of a threshold bucket kept as an index list; fuller buckets are re-scanned
 
 // Position of rank `remaining` (1-based, counted from the top bin down) in a 256-bin histogram: the bin holding it, the
@@ -146,6 +147,51 @@ __device__ void radix_select(Cand cand, int m, int k, unsigned int* hist, int la
   s.take = remaining;
 }
 
+// The same for at most 64 candidates, all of which take part: every candidate is compared with all others (one or two per
+// lane, the others by shuffle), and the key of the one with exactly k - 1 better ones is the threshold.  A threshold
+// bucket usually holds a dozen candidates; the radix select spends some 250 instructions on every digit, and two to
+// four digits, whatever their number.
+template <int kPerLane, class Key>
+__device__ void rank_select_n(Key key_of, int m, int k, int lane, Selection& s) {
+  unsigned long long key[kPerLane];
+  int rank[kPerLane];
+#pragma unroll
+  for (int x = 0; x < kPerLane; ++x) {
+    key[x] = lane + 32 * x < m ? key_of(lane + 32 * x) : 0ull;
+    rank[x] = 0;
+  }
+#pragma unroll
+  for (int y = 0; y < kPerLane; ++y) {
+    const int end = min(m - 32 * y, 32);
+#pragma unroll 1
+    for (int o = 0; o < end; ++o) {
+      const unsigned long long other = __shfl_sync(0xFFFFFFFFu, key[y], o);
+      // an equal key goes first when its candidate does: other >= key, that is other > key - 1 (keys are never 0)
+#pragma unroll
+      for (int x = 0; x < kPerLane; ++x) rank[x] += other > key[x] - (o + 32 * y < lane + 32 * x ? 1 : 0) ? 1 : 0;
+    }
+  }
+  unsigned long long threshold = 0ull;
+#pragma unroll
+  for (int x = 0; x < kPerLane; ++x) {
+    const unsigned hit = __ballot_sync(0xFFFFFFFFu, lane + 32 * x < m && rank[x] == k - 1);
+    if (hit != 0u) threshold = __shfl_sync(0xFFFFFFFFu, key[x], __ffs(hit) - 1);
+  }
+  int above = 0;
+#pragma unroll
+  for (int x = 0; x < kPerLane; ++x) above += __popc(__ballot_sync(0xFFFFFFFFu, lane + 32 * x < m && key[x] > threshold));
+  s.prefix = threshold;
+  s.mask = ~0ull;
+  s.take = k - above;
+}
+template <class Key>
+__device__ void rank_select(Key key_of, int m, int k, int lane, Selection& s) {
+  if (m <= 32)
+    rank_select_n<1>(key_of, m, k, lane, s);
+  else
+    rank_select_n<2>(key_of, m, k, lane, s);
+}
+
 // The k best (largest key, then lowest index) of keys[0..n).  First a histogram over 256 buckets that are linear in
 // the score (bucket(j), any monotone map of the score to 0..255, computed from a single-precision copy): it places
 // the k-th best in one bucket with usually a handful of entries, listed by index (idx, at most kMaxListed) for the
@@ -183,10 +229,14 @@ __device__ Selection select_top(const unsigned long long* keys, Bucket bucket, i
       listed += __popc(b);
     }
     __syncwarp();
-    radix_select([&](int c, unsigned long long& key) {
-      key = keys[idx[c]];
-      return true;
-    }, at.size, remaining, hist, lane, s);
+    if (at.size <= 64) {
+      rank_select([&](int c) { return keys[idx[c]]; }, at.size, remaining, lane, s);
+    } else {
+      radix_select([&](int c, unsigned long long& key) {
+        key = keys[idx[c]];
+        return true;
+      }, at.size, remaining, hist, lane, s);
+    }
   } else {
     radix_select([&](int c, unsigned long long& key) {
       key = keys[c];
@@ -411,8 +461,38 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
   const int i = i0 + warp;
   if (i >= nb) return;
 
-  // Phase B
   const unsigned long long* keys = s_key + static_cast<size_t>(warp) * pitch;
+  if (kDirect && nb <= kRankMax) {
+    // Short rows: the rank of every entry by comparing it with all others (one or two entries per lane, the others read
+    // as broadcasts).  At 22 blocks that is a tenth of what the histogram and the radix select below cost, whose 256
+    // counters alone take longer to clear and scan than the row has entries.
+    unsigned long long key[2];
+    int rank[2] = {0, 0};
+#pragma unroll
+    for (int x = 0; x < 2; ++x) key[x] = lane + 32 * x < nb ? keys[lane + 32 * x] : 0ull;
+    for (int o = 0; o < nb; ++o) {
+      const unsigned long long other = keys[o];
+#pragma unroll
+      for (int x = 0; x < 2; ++x) rank[x] += (other > key[x] || (other == key[x] && o < lane + 32 * x)) ? 1 : 0;
+    }
+    const size_t row = bh_rows + i;
+    int n_crit = 0, n_marg = 0;
+    const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const int j = lane + 32 * x;
+      const int c = j >= nb ? -1 : (rank[x] < k_crit ? 2 : (rank[x] < nb - k_neg ? 1 : 0));
+      if (j < nb) cls[row * nb + j] = static_cast<signed char>(c);
+      const unsigned m_crit = __ballot_sync(0xFFFFFFFFu, c == 2), m_marg = __ballot_sync(0xFFFFFFFFu, c == 1);
+      if (c == 2) crit_idx[row * k_crit + n_crit + __popc(m_crit & below)] = j;
+      if (c == 1 && marg_idx != nullptr) marg_idx[row * k_marg + n_marg + __popc(m_marg & below)] = j;
+      n_crit += __popc(m_crit);
+      n_marg += __popc(m_marg);
+    }
+    return;
+  }
+
+  // Phase B
   unsigned int* hist = s_hist + warp * 2 * kBuckets;  // radix digits; the second half holds the bucket counts
   unsigned int* bucket_hist = hist + kBuckets;
   // Buckets linear in the score between the row's extremes; with fewer than eight rows per CTA (very long
@@ -459,7 +539,9 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
   // Phase C
   const size_t row = bh_rows + i;
   signed char* out_cls = cls + row * nb;
-  int n_crit = 0, n_marg = 0, tie_c = 0, tie_m = 0;
+  int* crit_row = crit_idx + row * k_crit;  // where the row's lists go on
+  int* marg_row = marg_idx != nullptr ? marg_idx + row * k_marg : nullptr;
+  int tie_c = 0, tie_m = 0;
   const unsigned below = (1u << lane) - 1u;
 #pragma unroll 2
   for (int j0 = 0; j0 < nb; j0 += 32) {
@@ -482,38 +564,65 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
     if (in) out_cls[j] = static_cast<signed char>(c);
     const unsigned m_crit = __ballot_sync(0xFFFFFFFFu, c == 2);
     const unsigned m_marg = __ballot_sync(0xFFFFFFFFu, c == 1);
-    if (c == 2) crit_idx[row * k_crit + n_crit + __popc(m_crit & below)] = j;
-    if (c == 1 && marg_idx != nullptr) marg_idx[row * k_marg + n_marg + __popc(m_marg & below)] = j;
-    n_crit += __popc(m_crit);
-    n_marg += __popc(m_marg);
+    if (c == 2) crit_row[__popc(m_crit & below)] = j;
+    crit_row += __popc(m_crit);
+    if (marg_row != nullptr) {
+      if (c == 1) marg_row[__popc(m_marg & below)] = j;
+      marg_row += __popc(m_marg);
+    }
   }
 }
 
+// Two neighbouring column sums times 2^-10 as fp16 pairs hi + lo (22 bits between them).
+__device__ __forceinline__ void split_pair(int v0, int v1, uint32_t& hi, uint32_t& lo) {
+  const float f0 = __int2float_rn(v0) * 0x1p-10f, f1 = __int2float_rn(v1) * 0x1p-10f;
+  const __half2 h = __floats2half2_rn(f0, f1);
+  const float2 back = __half22float2(h);
+  const __half2 l = __floats2half2_rn(f0 - back.x, f1 - back.y);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+__device__ __forceinline__ void mma_m16n8k16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
 // The same plan with the scores kept in shared memory as single-precision values (4 bytes per key instead of an
-// 8-byte ordered key), for long rows: sixteen rows per CTA then fit where eight did, so the column sums of a (b, h)
-// are streamed half as often and twice as many warps hide the latencies of the selection and of the class pass.
-// The ranking stays the exact one.  The single-precision copy is a monotone (weakly order-preserving) image of the
-// exact score and only places a key in one of the 256 buckets; the few keys of a threshold bucket are decided by
-// their exact 64-bit keys, which are recomputed for them from the integer column sums (an int64 dot product, equal
-// to the tensor-core result as long as that is exact, i.e. below 2^53).
-// Warp w of the R = 8 or 16 warps: in phase A row tile w % (R / 8) (eight rows) against every (R / 8)-th group of
-// eight key blocks; in phases B and C row w.
+// 8-byte ordered key): sixteen rows per CTA then fit where eight did, so the column sums of a (b, h) are streamed half as
+// often and twice as many warps hide the latencies of the selection and of the class pass.
+// The ranking stays the exact one.  The single-precision score only gives a key its place on a 16-bit scale between the
+// row's extremes; the few keys near a selection threshold are decided by their exact 64-bit keys, which are recomputed for
+// them from the integer column sums (an int64 dot product, equal to the fp64 tensor-core value as long as that is exact,
+// i.e. below 2^53).
+//   R = 8: the scores are the exact ones (fp64 tensor products), rounded to fp32: near means in the threshold's own place.
+//   R = 16: the scores are approximations from fp16 tensor products of a two-way split of the column sums (hi hi + hi lo
+//     + lo hi, fp32 accumulation), twelve products for 16 x 8 scores where fp64 takes thirty-two of its far slower
+//     ones.  An approximation is off by at most
+//       delta = max_j scale^K_j (224 (2^-17 S + 2^-19) + 2^-25 S),  S = sum_d |colsum^Q_d| 2^-10
+//     (a column sum over its valid tokens is at most 448 in value, so |colsum^K_d| 2^-10 / valid <= 224; the split leaves
+//     out 3 2^-22 of a product and twelve accumulations lose 2^-22 of the sum of magnitudes each, together below 2^-18,
+//     doubled for safety; the last two terms are fp16's smallest step), so near means within 2 delta of the threshold's
+//     place: an entry further above it is certainly selected, one further below certainly not.
+//     16 heads, 2147 blocks: 1210 -> 1005 us with it and the cheaper selections below.
+// Warp w of the R = 8 or 16 warps: in phase A all its rows against every R-th group of eight key blocks; in phases B and
+// C row w.
 template <int R>
 __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restrict__ q_colsum, const int* __restrict__ k_colsum,
                                                                const float* __restrict__ k_scales, int tokens, int block,
                                                                int nb, int k_crit, int k_marg, int k_neg,
                                                                signed char* __restrict__ cls, int* __restrict__ crit_idx,
                                                                int* __restrict__ marg_idx) {
-  constexpr int kRowTiles = R / 8;
-  constexpr int kGroups = R / kRowTiles;  // warps that share a row tile (= 8)
+  constexpr bool kApprox = R == 16;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int pitch = (nb + 3) & ~3;
   float* s_val = reinterpret_cast<float*>(smem_raw);                                              // [R][pitch]
-  unsigned int* s_hist = reinterpret_cast<unsigned int*>(s_val + static_cast<size_t>(R) * pitch);  // [R][2][256]
-  unsigned long long* s_ckey = reinterpret_cast<unsigned long long*>(s_hist + R * 2 * kBuckets);   // [R][2][kMaxListed]
+  unsigned int* s_hist = reinterpret_cast<unsigned int*>(s_val + static_cast<size_t>(R) * pitch);  // [R][256]
+  unsigned long long* s_ckey = reinterpret_cast<unsigned long long*>(s_hist + R * kBuckets);       // [R][2][kMaxListed]
   int* s_q = reinterpret_cast<int*>(s_ckey + R * 2 * kMaxListed);                                  // [R][64]
-  float2* s_range = reinterpret_cast<float2*>(s_q + R * kHeadDim);                                 // [kGroups][R]
-  unsigned short* s_idx = reinterpret_cast<unsigned short*>(s_range + kGroups * R);                // [R][2][kMaxListed]
+  float2* s_range = reinterpret_cast<float2*>(s_q + R * kHeadDim);                                 // [R][R]
+  unsigned short* s_idx = reinterpret_cast<unsigned short*>(s_range + R * R);                      // [R][2][kMaxListed]
+  __shared__ float s_kmax[R];
 
   const int row_tiles = (nb + R - 1) / R;
   const int bh = blockIdx.x / row_tiles;
@@ -533,9 +642,89 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
 
   sm100::wait_for_prior_grid();
   sm100::launch_dependents();
-  {
+  if constexpr (kApprox) {
+    // Phase A, 16 rows x 8 key blocks per warp and step (m16n8k16).  As below, lane (g, t) supplies columns 16 t ..
+    // 16 t + 15 of its rows (rows g and g + 8 for A, key block g of the eight for B), which is one and the same
+    // assignment of columns to k indices on both sides.
+    const int g = lane >> 2, t4 = lane & 3;
+    auto load16 = [&](const int* base, int local, int4 dst[4]) {
+      const int4* src = reinterpret_cast<const int4*>(base + (bh_rows + min(local, nb - 1)) * kHeadDim + 16 * t4);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) dst[q] = __ldg(src + q);
+    };
+    auto split16 = [&](const int4 v[4], uint32_t hi[8], uint32_t lo[8]) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        split_pair(v[q].x, v[q].y, hi[2 * q], lo[2 * q]);
+        split_pair(v[q].z, v[q].w, hi[2 * q + 1], lo[2 * q + 1]);
+      }
+    };
+    uint32_t a_hi[2][8], a_lo[2][8];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      int4 qv[4];
+      load16(q_colsum, i0 + 8 * r + g, qv);
+      split16(qv, a_hi[r], a_lo[r]);
+    }
+    int4 nxt[4];
+    float nxt_ks[2];
+    auto load_scales = [&](int j) {
+#pragma unroll
+      for (int x = 0; x < 2; ++x) nxt_ks[x] = __ldg(k_scales + bh_rows + min(j + x, nb - 1));
+    };
+    load16(k_colsum, warp * 8 + g, nxt);
+    load_scales(warp * 8 + 2 * t4);
+    float lo[2] = {INFINITY, INFINITY}, hi[2] = {-INFINITY, -INFINITY}, kmax = 0.f;
+    const float inv_full = 1.f / static_cast<float>(block);
+    for (int j0 = warp * 8; j0 < nb; j0 += 8 * R) {
+      uint32_t b_hi[8], b_lo[8];
+      split16(nxt, b_hi, b_lo);
+      float factor[2];
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int valid = tokens - (j0 + 2 * t4 + x) * block;
+        factor[x] = valid >= block ? nxt_ks[x] * inv_full : nxt_ks[x] / static_cast<float>(max(valid, 1));
+        kmax = fmaxf(kmax, nxt_ks[x]);
+      }
+      if (j0 + 8 * R < nb) {
+        load16(k_colsum, j0 + 8 * R + g, nxt);
+        load_scales(j0 + 8 * R + 2 * t4);
+      }
+      float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f}, c2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int st = 0; st < 4; ++st) {
+        mma_m16n8k16(c0, a_hi[0][2 * st], a_hi[1][2 * st], a_hi[0][2 * st + 1], a_hi[1][2 * st + 1], b_hi[2 * st], b_hi[2 * st + 1]);
+        mma_m16n8k16(c1, a_hi[0][2 * st], a_hi[1][2 * st], a_hi[0][2 * st + 1], a_hi[1][2 * st + 1], b_lo[2 * st], b_lo[2 * st + 1]);
+        mma_m16n8k16(c2, a_lo[0][2 * st], a_lo[1][2 * st], a_lo[0][2 * st + 1], a_lo[1][2 * st + 1], b_hi[2 * st], b_hi[2 * st + 1]);
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        float* const dst = s_val + static_cast<size_t>(8 * r + g) * pitch + j0 + 2 * t4;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          const float v = (c0[2 * r + x] + (c1[2 * r + x] + c2[2 * r + x])) * factor[x];
+          if (j0 + 2 * t4 + x < nb) {
+            dst[x] = v;
+            lo[r] = fminf(lo[r], v);
+            hi[r] = fmaxf(hi[r], v);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+      for (int o = 1; o <= 2; o <<= 1) {
+        lo[r] = fminf(lo[r], __shfl_xor_sync(0xFFFFFFFFu, lo[r], o));
+        hi[r] = fmaxf(hi[r], __shfl_xor_sync(0xFFFFFFFFu, hi[r], o));
+      }
+      if (t4 == 0) s_range[warp * R + 8 * r + g] = make_float2(lo[r], hi[r]);
+    }
+    kmax = warp_max(kmax);
+    if (lane == 0) s_kmax[warp] = kmax;
+  } else {
     // Phase A: fp64 tensor-core products of the exactly widened int32 column sums (see plan_kernel).
-    const int tile = warp % kRowTiles, grp = warp / kRowTiles;
+    const int grp = warp;
     const int g = lane >> 2, t4 = lane & 3;
     auto widen = [](int v) { return __int2double_rn(v); };  // exact; one instruction
     // `local` is a block index inside the (b, h); past the end the last block is read instead (its products land
@@ -548,7 +737,7 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
     double q_frag[16];
     {
       int4 qv[4];
-      load16(q_colsum, i0 + 8 * tile + g, qv);
+      load16(q_colsum, i0 + g, qv);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         q_frag[4 * q] = widen(qv[q].x);
@@ -566,19 +755,19 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
     load16(k_colsum, grp * 8 + g, nxt);
     load_scales(grp * 8 + 2 * t4, nxt_ks);
     float lo = INFINITY, hi = -INFINITY;
-    float* const my_val = s_val + static_cast<size_t>(8 * tile + g) * pitch;
+    float* const my_val = s_val + static_cast<size_t>(g) * pitch;
     // key blocks in whole blocks of a power-of-two size divide by a multiplication that is exact, so the scale and
     // the division fold into one factor per key block; only the last key block of a sequence can be shorter
     const int last_full = (tokens % block == 0 && block_pow2) ? nb : (block_pow2 ? nb - 1 : 0);  // key blocks below this are whole
 #pragma unroll 2
-    for (int j0 = grp * 8; j0 < nb; j0 += 8 * kGroups) {
+    for (int j0 = grp * 8; j0 < nb; j0 += 8 * R) {
       int4 cur[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) cur[q] = nxt[q];
       const float cur_ks[2] = {nxt_ks[0], nxt_ks[1]};
-      if (j0 + 8 * kGroups < nb) {
-        load16(k_colsum, j0 + 8 * kGroups + g, nxt);
-        load_scales(j0 + 8 * kGroups + 2 * t4, nxt_ks);
+      if (j0 + 8 * R < nb) {
+        load16(k_colsum, j0 + 8 * R + g, nxt);
+        load_scales(j0 + 8 * R + 2 * t4, nxt_ks);
       }
       double c[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
@@ -620,7 +809,7 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
       lo = fminf(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
       hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
     }
-    if (t4 == 0) s_range[grp * R + 8 * tile + g] = make_float2(lo, hi);
+    if (t4 == 0) s_range[grp * R + g] = make_float2(lo, hi);
   }
   __syncthreads();
   const int i = i0 + warp;
@@ -628,11 +817,14 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
 
   // Phase B
   const float* vals = s_val + static_cast<size_t>(warp) * pitch;
-  unsigned int* hist = s_hist + warp * 2 * kBuckets;
-  unsigned int* bucket_hist = hist + kBuckets;
-  float2 range = lane < kGroups ? s_range[lane * R + warp] : make_float2(INFINITY, -INFINITY);
+  // one histogram; the refinement, which needs two, borrows the place of the listed keys, which come after it
+  unsigned int* const hist = s_hist + warp * kBuckets;
+  unsigned int* const bucket_hist = hist;
+  static_assert(kMaxListed * sizeof(unsigned long long) >= kBuckets * sizeof(unsigned int), "borrowed histogram");
+  unsigned int* const second_hist = reinterpret_cast<unsigned int*>(s_ckey + warp * 2 * kMaxListed);
+  float2 range = lane < R ? s_range[lane * R + warp] : make_float2(INFINITY, -INFINITY);
 #pragma unroll
-  for (int o = 1; o < kGroups; o <<= 1) {
+  for (int o = 1; o < R; o <<= 1) {
     range.x = fminf(range.x, __shfl_xor_sync(0xFFFFFFFFu, range.x, o));
     range.y = fmaxf(range.y, __shfl_xor_sync(0xFFFFFFFFu, range.y, o));
   }
@@ -647,7 +839,15 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
   int* const q_row = s_q + warp * kHeadDim;
   q_row[lane] = __ldg(q_colsum + (bh_rows + i) * kHeadDim + lane);
   q_row[lane + 32] = __ldg(q_colsum + (bh_rows + i) * kHeadDim + lane + 32);
+  __syncwarp();
   const int4* const q4 = reinterpret_cast<const int4*>(q_row);
+  int margin = 0;  // places within which an approximate score may be on the wrong side of a threshold
+  if constexpr (kApprox) {
+    const float sum_q = warp_sum((fabsf(static_cast<float>(q_row[lane])) + fabsf(static_cast<float>(q_row[lane + 32]))) * 0x1p-10f);
+    const float k_top = warp_max(lane < R ? s_kmax[lane] : 0.f);
+    const float delta = k_top * (224.f * (0x1p-17f * sum_q + 0x1p-19f) + 0x1p-25f * sum_q);
+    margin = static_cast<int>(fminf(2.f * delta * scale, 65535.f)) + 3;
+  }
   auto exact_key = [&](int j) -> unsigned long long {
     const int4* const k4 = reinterpret_cast<const int4*>(k_colsum + (bh_rows + j) * kHeadDim);
     long long dot = 0;
@@ -672,12 +872,12 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
   // A selection: entries whose place is above t_hi are selected, those inside [t_lo, t_hi] are decided by their exact
   // keys (prefix / mask / take as in Selection), the rest are not.  Each selection leaves the entries of its
   // threshold range (ascending index) and their exact keys behind for the class pass: keys_from 0 = no key needed
-  // (the whole range goes one way), 1 = listed, 2 = recompute (still too many to list after the refinement).
+  // (the whole range goes one way), 1 = listed, 2 = recompute (too many to list).
   // The two selections of a row go through their stages together, so that the refinement and the listing each take
   // one pass over the row for both.
   struct Chosen {
     Selection s;
-    int t_lo, t_hi, keys_from, remaining, size;
+    int k, t_lo, t_hi, keys_from, remaining, size;
     bool refine, list;
   };
   auto begin = [&](int k) -> Chosen {
@@ -687,6 +887,7 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
     r.s.mask = 0ull;
     r.s.take = 0;
     r.s.bucket = 0;
+    r.k = k;
     r.remaining = r.size = 0;
     r.refine = r.list = false;
     if (k <= 0) {
@@ -702,77 +903,111 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
     r.t_hi = r.t_lo + 255;
     r.remaining = k - at.above;
     r.size = at.size;
-    if (r.remaining == r.size)
-      r.s.take = r.size;
-    else if (r.size > kMaxListed)
-      r.refine = true;
-    else
-      r.list = true;
+    r.refine = r.size > kMaxListed / 2;
+    r.list = true;
     return r;
   };
   Chosen cc = begin(k_crit), cm = begin(nb - k_neg);
   if (cc.refine || cm.refine) {  // histograms of the lower eight bits inside the two threshold buckets
 #pragma unroll
     for (int b = 0; b < 8; ++b) {
-      hist[lane + 32 * b] = 0u;
-      bucket_hist[lane + 32 * b] = 0u;  // the first histogram has served both selections
+      hist[lane + 32 * b] = 0u;  // the first histogram has served both selections
+      second_hist[lane + 32 * b] = 0u;
     }
     __syncwarp();
     const int bin_c = cc.refine ? cc.t_lo >> 8 : -1, bin_m = cm.refine ? cm.t_lo >> 8 : -1;
     for (int j = lane; j < nb; j += 32) {
       const int f = fine(j);
       if ((f >> 8) == bin_c) atomicAdd(&hist[f & 255], 1u);
-      if ((f >> 8) == bin_m) atomicAdd(&bucket_hist[f & 255], 1u);
+      if ((f >> 8) == bin_m) atomicAdd(&second_hist[f & 255], 1u);
     }
     __syncwarp();
     auto refined = [&](Chosen& r, const unsigned int* h) {
       if (!r.refine) return;
       const Located at2 = locate(h, r.remaining, lane);
       r.t_lo = r.t_hi = (r.t_lo & ~255) | at2.bin;
-      r.remaining -= at2.above;
-      r.size = at2.size;
-      if (r.remaining == r.size)
-        r.s.take = r.size;
-      else if (r.size <= kMaxListed)
-        r.list = true;
-      else
-        r.keys_from = 2;  // more than kMaxListed entries in one of 65536 places (near-equal scores)
     };
     refined(cc, hist);
-    refined(cm, bucket_hist);
+    refined(cm, second_hist);
     __syncwarp();
+  }
+  for (Chosen* r : {&cc, &cm}) {
+    if (!r->list) continue;
+    r->t_lo = max(r->t_lo - margin, 0);
+    r->t_hi = min(r->t_hi + margin, 65535);
   }
   unsigned long long* const ckey_c = s_ckey + warp * 2 * kMaxListed;
   unsigned long long* const ckey_m = ckey_c + kMaxListed;
   unsigned short* const idx_c = s_idx + warp * 2 * kMaxListed;
   unsigned short* const idx_m = idx_c + kMaxListed;
-  if (cc.list || cm.list) {  // positions of the entries inside the two threshold ranges, ascending
+  if (cc.list || cm.list) {  // positions of the entries inside the two threshold ranges, ascending, and how many are above
     const unsigned below = (1u << lane) - 1u;
-    int listed_c = 0, listed_m = 0;
+    int listed_c = 0, listed_m = 0, above_c = 0, above_m = 0;
     for (int j0 = 0; j0 < nb; j0 += 32) {
       const int j = j0 + lane;
       const int f = j < nb ? fine(j) : -1;
       const bool is_c = cc.list && f >= cc.t_lo && f <= cc.t_hi, is_m = cm.list && f >= cm.t_lo && f <= cm.t_hi;
       const unsigned b_c = __ballot_sync(0xFFFFFFFFu, is_c), b_m = __ballot_sync(0xFFFFFFFFu, is_m);
-      if (is_c) idx_c[listed_c + __popc(b_c & below)] = static_cast<unsigned short>(j);
-      if (is_m) idx_m[listed_m + __popc(b_m & below)] = static_cast<unsigned short>(j);
+      above_c += f > cc.t_hi ? 1 : 0;
+      above_m += f > cm.t_hi ? 1 : 0;
+      const int at_c = listed_c + __popc(b_c & below), at_m = listed_m + __popc(b_m & below);
+      if (is_c && at_c < kMaxListed) idx_c[at_c] = static_cast<unsigned short>(j);
+      if (is_m && at_m < kMaxListed) idx_m[at_m] = static_cast<unsigned short>(j);
       listed_c += __popc(b_c);
       listed_m += __popc(b_m);
     }
+    above_c = __reduce_add_sync(0xFFFFFFFFu, above_c);
+    above_m = __reduce_add_sync(0xFFFFFFFFu, above_m);
     __syncwarp();
-    if (cc.list)
-      for (int c = lane; c < cc.size; c += 32) ckey_c[c] = exact_key(idx_c[c]);
-    if (cm.list)
-      for (int c = lane; c < cm.size; c += 32) ckey_m[c] = exact_key(idx_m[c]);
+    auto settle = [&](Chosen& r, int listed, int above) {
+      if (!r.list) return;
+      r.size = listed;
+      r.remaining = r.k - above;
+      if (r.remaining == 0 || r.remaining == r.size) {  // the whole range goes one way
+        r.s.take = r.remaining;
+        r.list = false;
+      } else if (r.size > kMaxListed) {
+        r.keys_from = 2;
+        r.list = false;
+      }
+    };
+    settle(cc, listed_c, above_c);
+    settle(cm, listed_m, above_m);
+    // Exact keys of the listed entries, eight lanes to an entry (its 256 bytes of column sums read whole; with one entry per
+    // lane every load would touch 32 lines).
+    auto exact_keys = [&](const unsigned short* idx, int size, unsigned long long* ckey) {
+      const int l8 = lane & 7;
+      for (int c0 = 0; c0 < size; c0 += 4) {
+        const int c = c0 + (lane >> 3), j = idx[min(c, size - 1)];
+        const int4* const k4 = reinterpret_cast<const int4*>(k_colsum + (bh_rows + j) * kHeadDim);
+        long long dot = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int4 a = q4[l8 + 8 * h], b = __ldg(k4 + l8 + 8 * h);
+          dot += static_cast<long long>(a.x) * b.x + static_cast<long long>(a.y) * b.y + static_cast<long long>(a.z) * b.z +
+                 static_cast<long long>(a.w) * b.w;
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
+        if (l8 == 0 && c < size)
+          ckey[c] = order_key(ranking_score(static_cast<double>(dot), __ldg(k_scales + bh_rows + j), j));
+      }
+    };
+    if (cc.list) exact_keys(idx_c, cc.size, ckey_c);
+    if (cm.list) exact_keys(idx_m, cm.size, ckey_m);
     __syncwarp();
   }
   auto finish = [&](Chosen& r, const unsigned long long* ckey) {
     if (r.list) {
       r.keys_from = 1;
-      radix_select([&](int c, unsigned long long& key) {
-        key = ckey[c];
-        return true;
-      }, r.size, r.remaining, hist, lane, r.s);
+      if (r.size <= 64) {
+        rank_select([&](int c) { return ckey[c]; }, r.size, r.remaining, lane, r.s);
+      } else {
+        radix_select([&](int c, unsigned long long& key) {
+          key = ckey[c];
+          return true;
+        }, r.size, r.remaining, hist, lane, r.s);
+      }
     } else if (r.keys_from == 2) {  // every pass recomputes the keys it looks at
       const int t_lo = r.t_lo, t_hi = r.t_hi;
       radix_select([&](int c, unsigned long long& key) {
@@ -791,7 +1026,9 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
   // Phase C
   const size_t row = bh_rows + i;
   signed char* out_cls = cls + row * nb;
-  int n_crit = 0, n_marg = 0, tie_c = 0, tie_m = 0, seen_c = 0, seen_m = 0;
+  int* crit_row = crit_idx + row * k_crit;  // where the row's lists go on
+  int* marg_row = marg_idx != nullptr ? marg_idx + row * k_marg : nullptr;
+  int tie_c = 0, tie_m = 0, seen_c = 0, seen_m = 0;
   const unsigned below = (1u << lane) - 1u;
 #pragma unroll 2
   for (int j0 = 0; j0 < nb; j0 += 32) {
@@ -819,17 +1056,19 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
     if (in) out_cls[j] = static_cast<signed char>(c);
     const unsigned m_crit = __ballot_sync(0xFFFFFFFFu, c == 2);
     const unsigned m_marg = __ballot_sync(0xFFFFFFFFu, c == 1);
-    if (c == 2) crit_idx[row * k_crit + n_crit + __popc(m_crit & below)] = j;
-    if (c == 1 && marg_idx != nullptr) marg_idx[row * k_marg + n_marg + __popc(m_marg & below)] = j;
-    n_crit += __popc(m_crit);
-    n_marg += __popc(m_marg);
+    if (c == 2) crit_row[__popc(m_crit & below)] = j;
+    crit_row += __popc(m_crit);
+    if (marg_row != nullptr) {
+      if (c == 1) marg_row[__popc(m_marg & below)] = j;
+      marg_row += __popc(m_marg);
+    }
   }
 }
 
 size_t plan_compact_smem_bytes(int nb, int rows) {
   const size_t pitch = static_cast<size_t>((nb + 3) & ~3);
-  return rows * pitch * 4 + static_cast<size_t>(rows) * 2 * kBuckets * 4 + static_cast<size_t>(rows) * 2 * kMaxListed * 8 +
-         static_cast<size_t>(rows) * kHeadDim * 4 + static_cast<size_t>(8) * rows * sizeof(float2) +
+  return rows * pitch * 4 + static_cast<size_t>(rows) * kBuckets * 4 + static_cast<size_t>(rows) * 2 * kMaxListed * 8 +
+         static_cast<size_t>(rows) * kHeadDim * 4 + static_cast<size_t>(rows) * rows * sizeof(float2) +
          static_cast<size_t>(rows) * 2 * kMaxListed * 2;
 }
 

@@ -3,10 +3,11 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2605_11354_b200 import binding as lt
 from paper_2605_11354_b200 import workloads as wk
 
 import parity_util as pu
-from test_gpu_parity import oracle_subset, small_workload
+from test_gpu_parity import full_parity, oracle_subset, small_workload
 
 pytestmark = pytest.mark.gpu
 
@@ -38,3 +39,39 @@ def test_many_buffer_sets_in_turn(block):
         assert torch.equal(out, first)
         if i % 3:
             hold.append(eng)  # some buffers stay, the others' addresses are taken over
+
+
+@pytest.mark.parametrize("blocks", [1, 32, 33, 64, 65])
+def test_plan_rows_around_the_rank_limit(blocks):
+    """Rows of up to 64 blocks are ranked by comparing all pairs (one or two entries per lane), longer ones selected
+    through histograms."""
+    wl = small_workload(f"rank{blocks}", heads=2, tokens=blocks * 64 - 3, crit=0.2, neg=0.3)
+    full_parity(wl, wk.make_inputs(wl), query_blocks=pu.sample_blocks(wl, [0, 1], 4))
+
+
+@pytest.mark.parametrize("spread", [1e-4, 3e-2])
+@pytest.mark.parametrize("block,blocks", [(64, 150), (128, 131)])
+def test_plan_scores_closer_than_their_approximation(spread, block, blocks):
+    """Sixteen rows per CTA work on approximate scores: key blocks whose exact scores differ by less than the
+    approximation's error have to come out in the exact order all the same."""
+    g = np.random.default_rng(17)
+    wl = small_workload(f"close{blocks}", heads=1, tokens=blocks * block - 5, block=block, crit=0.2, neg=0.5, src_dtype="f32")
+    inputs = wk.make_inputs(wl)
+    for name in ("q", "k"):
+        inputs[name] = (1.0 + spread * g.standard_normal(inputs[name].shape)).astype(np.float32)
+    plans = []
+    try:
+        for variant in (1, 3):
+            lt.lite3r_plan_variant(variant)
+            eng, _ = pu.run_gpu(inputs, wl)
+            plans.append([t.cpu().numpy() for t in (eng.plan.cls, eng.plan.crit_idx, eng.plan.marg_idx)])
+    finally:
+        lt.lite3r_plan_variant(0)
+    assert all(np.array_equal(a, b) for a, b in zip(*plans))
+
+
+@pytest.mark.parametrize("blocks", [64, 65, 128, 129, 193])
+def test_aggregation_inside_one_sequence(blocks):
+    """Key chunks of 64 that end with, before and after the row, row tiles of 128 full and ragged."""
+    wl = small_workload(f"agg{blocks}", heads=3, tokens=blocks * 64, crit=0.05, neg=0.2)
+    full_parity(wl, wk.make_inputs(wl), query_blocks=pu.sample_blocks(wl, [0, 2], 6))
