@@ -584,16 +584,15 @@ class SlaForward:
         return out
 
     def run_graph(self, q, k, v, proj, out=None):
-        """The same step (quantise, plan, forward with the overlapped first half) replayed as one CUDA graph on the
-        current stream: the five kernel launches, the status clear and the stream fork / join of a step then cost one
-        launch on the host, which is a tenth of the step at short sequences.  The graph is captured on first use for
+        """The same step replayed as one CUDA graph on the current stream: its five kernel launches then cost one launch
+        on the host, which is a tenth of the step at short sequences.  The graph is captured on first use for
         these tensors (and again when a tensor's address changes); results are identical to ``run``.  The library
         calls only enqueue work on the stream they are given and allocate nothing, which is what makes them
         capturable; call ``run`` once before (shared-memory limits and tensor maps are set up on first use)."""
         out = self.out if out is None else out
         key = (q.data_ptr(), k.data_ptr(), v.data_ptr(), proj.data_ptr(), out.data_ptr())
         if self._graph is None or self._graph[1] != key:
-            self.run(q, k, v, proj, out=out, overlap=True)  # first-use set-up happens outside the capture
+            self.run(q, k, v, proj, out=out)  # first-use set-up happens outside the capture
             torch.cuda.synchronize(self.device)
             graph = torch.cuda.CUDAGraph()
             capture_stream = torch.cuda.Stream(self.device)
@@ -603,7 +602,7 @@ class SlaForward:
                 # than the capture, now and then half a second, and is of no use to a step that allocates nothing)
                 graph.capture_begin()
                 try:
-                    self.run(q, k, v, proj, out=out, overlap=True)
+                    self.run(q, k, v, proj, out=out)
                 finally:
                     graph.capture_end()
             torch.cuda.current_stream(self.device).wait_stream(capture_stream)

@@ -335,7 +335,7 @@ lite3r_status lite3r_sla_plan(const lite3r_fp8* q, const lite3r_fp8* k, const li
   plan->k_marg = c.k_marg;
   plan->k_neg = c.k_neg;
   if ((st = check_device()) != LITE3R_OK) return st;
-  return launch_plan(*q, *k, *shape, c, *plan, static_cast<cudaStream_t>(stream));
+  return launch_plan(*q, *k, *shape, c, *plan, false, static_cast<cudaStream_t>(stream));
 }
 
 // Shared argument checks and launch of lite3r_sla_forward and its two halves (phases as in launch_forward).
@@ -344,7 +344,8 @@ static lite3r_status forward_phases(int phases, const lite3r_fp8* q, const lite3
                                     double crit, double neg, lite3r_phi phi, const lite3r_plan* plan, void* out,
                                     lite3r_dtype out_dtype, long long out_stride_b, long long out_stride_h,
                                     long long out_stride_n, void* workspace, size_t workspace_bytes,
-                                    int* device_status, void* stream, int linear_only = 0, bool check_only = false) {
+                                    int* device_status, void* stream, int linear_only = 0, bool check_only = false,
+                                    bool chained = false) {
   lite3r_status st = check_shape(shape);
   if (st != LITE3R_OK) return st;
   if ((st = check_fp8(k, true, false)) != LITE3R_OK) return st;
@@ -398,6 +399,7 @@ static lite3r_status forward_phases(int phases, const lite3r_fp8* q, const lite3
   a.plan = effective;
   a.plan_inside = plan_inside ? 1 : 0;
   a.linear_only = linear_only;
+  a.chained = chained;
   a.crit = crit;
   a.neg = neg;
   a.out = out;
@@ -437,23 +439,29 @@ lite3r_status lite3r_sla_step(lite3r_step* t, void* stream) {
   t->plan.k_marg = c.k_marg;
   t->plan.k_neg = c.k_neg;
   if (!plan_inside && c.k_crit > 0 && t->plan.crit_idx == nullptr) return LITE3R_ERR_INVALID_ARG;
-  for (int pass = 0; pass < 2; ++pass) {  // checked as a whole before the first launch
-    if (pass == 1) {
-      cudaStream_t cs = static_cast<cudaStream_t>(stream);
-      if (t->q.dtype == t->k.dtype && t->q.dtype == t->v.dtype) {
-        st = launch_quantize(x, x8, 3, t->shape, cs);
-      } else {
-        for (int n = 0; n < 3 && st == LITE3R_OK; ++n) st = launch_quantize(&x[n], &x8[n], 1, t->shape, cs);
-      }
-      if (st != LITE3R_OK) return st;
-      if (!plan_inside && (st = launch_plan(t->q8, t->k8, t->shape, c, t->plan, cs)) != LITE3R_OK) return st;
-    }
-    st = forward_phases(3, &t->q8, &t->k8, &t->v8, t->proj, t->proj_head_stride, &t->shape, t->crit, t->neg, t->phi,
-                        plan_inside ? nullptr : &t->plan, t->out, t->out_dtype, t->out_stride_b, t->out_stride_h,
-                        t->out_stride_n, t->workspace, t->workspace_bytes, t->device_status, stream, 0, pass == 0);
-    if (st != LITE3R_OK) return st;
+  // phases of the forward as in launch_forward; the whole is checked before the first launch
+  auto forward = [&](int phases, bool check_only) {
+    return forward_phases(phases, &t->q8, &t->k8, &t->v8, t->proj, t->proj_head_stride, &t->shape, t->crit, t->neg, t->phi,
+                          plan_inside ? nullptr : &t->plan, t->out, t->out_dtype, t->out_stride_b, t->out_stride_h,
+                          t->out_stride_n, t->workspace, t->workspace_bytes, t->device_status, stream, 0, check_only, true);
+  };
+  if ((st = forward(3, true)) != LITE3R_OK) return st;
+  cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  if (t->q.dtype == t->k.dtype && t->q.dtype == t->v.dtype) {
+    st = launch_quantize(x, x8, 3, t->shape, cs);
+  } else {
+    for (int n = 0; n < 3 && st == LITE3R_OK; ++n) st = launch_quantize(&x[n], &x8[n], 1, t->shape, cs);
   }
-  return LITE3R_OK;
+  if (st != LITE3R_OK) return st;
+  if (plan_inside) return forward(3, false);
+  if (c.k_marg == 0) {
+    if ((st = launch_plan(t->q8, t->k8, t->shape, c, t->plan, false, cs)) != LITE3R_OK) return st;
+    return forward(3, false);
+  }
+  // the summaries, and beside them the plan
+  if ((st = forward(1, false)) != LITE3R_OK) return st;
+  if ((st = launch_plan(t->q8, t->k8, t->shape, c, t->plan, true, cs)) != LITE3R_OK) return st;
+  return forward(2, false);
 }
 
 lite3r_status lite3r_sla_forward_begin(const lite3r_fp8* k, const lite3r_fp8* v, const float* proj,

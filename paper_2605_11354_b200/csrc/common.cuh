@@ -143,8 +143,9 @@ __device__ __forceinline__ float warp_sum(float v) {
 lite3r_status launch_quantize(const lite3r_tensor* const* x, const lite3r_fp8* out, int count, const lite3r_shape& s,
                               cudaStream_t stream);
 void set_plan_variant(int variant);  // test hook, see lite3r_plan_variant
+// beside_prior: the launch before it in the stream was the summary kernel of the same step, beside which it may run.
 lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r_shape& s, const Counts& c,
-                          const lite3r_plan& plan, cudaStream_t stream);
+                          const lite3r_plan& plan, bool beside_prior, cudaStream_t stream);
 
 struct ForwardArgs {
   lite3r_fp8 q, k, v;
@@ -157,6 +158,7 @@ struct ForwardArgs {
   int out_dtype;
   long long out_stride_b, out_stride_h, out_stride_n;
   int linear_only;      // 1: the sparse branch is left out (the output is the linear branch through proj alone)
+  bool chained;         // the phases follow one another in one stream with nothing but the plan between them
   int plan_inside;      // 1: the plan is built in the workspace from q/k column sums and the fractions below
   double crit, neg;
   void* workspace;

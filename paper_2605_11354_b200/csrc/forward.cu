@@ -110,13 +110,14 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   const Workspace w = carve(a.workspace, s, a.plan.k_crit, a.plan_inside != 0);
   lite3r_status st = LITE3R_OK;
   lite3r_plan plan = a.plan;
-  if (a.plan_inside) {  // the block plan is built first, into the tail of the workspace
+  const Counts counts{plan.k_crit, plan.k_marg, plan.k_neg};
+  if (a.plan_inside) {  // the block plan is built into the tail of the workspace, beside the summaries when there are any
     plan.cls = w.cls;
     plan.crit_idx = w.crit_idx;
     plan.marg_idx = nullptr;
-    const Counts c{plan.k_crit, plan.k_marg, plan.k_neg};
-    if ((st = launch_plan(a.q, a.k, s, c, plan, stream)) != LITE3R_OK) return st;
+    if (counts.k_marg == 0 && (st = launch_plan(a.q, a.k, s, counts, plan, false, stream)) != LITE3R_OK) return st;
   }
+  const bool after_wait = phases != 3 && !a.chained;
   if (phases & 1) profile_mark(0, stream);
   // With a linear branch the summary kernel reads every V row anyway and writes the fp16 operand on the way; the
   // stand-alone pass runs only when there is no linear branch.
@@ -134,14 +135,15 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   if ((phases & 1) && a.plan.k_marg > 0) {
     profile_mark(2, stream);
     st = launch_summary(a.k, a.v, a.proj, a.proj_head_stride, s, a.phi, w.hws, a.plan.k_crit > 0 ? w.v16 : nullptr,
-                        a.device_status, phases != 3, stream);
+                        a.device_status, after_wait, stream);
     if (st != LITE3R_OK) return st;
     profile_mark(3, stream);
   }
   if (!(phases & 2)) return st;
+  if (a.plan_inside && counts.k_marg > 0 && (st = launch_plan(a.q, a.k, s, counts, plan, true, stream)) != LITE3R_OK) return st;
   if (a.plan.k_marg > 0) {
     profile_mark(4, stream);
-    if ((st = launch_aggregate(w.hws, plan.cls, s, nb, w.g16, w.zeta, a.device_status, phases != 3, stream)) != LITE3R_OK) return st;
+    if ((st = launch_aggregate(w.hws, plan.cls, s, nb, w.g16, w.zeta, a.device_status, after_wait, stream)) != LITE3R_OK) return st;
     profile_mark(5, stream);
   }
   AttentionLaunch att;

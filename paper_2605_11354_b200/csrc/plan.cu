@@ -22,6 +22,10 @@
 //     row.  Two selections give the classes: the best k_crit are critical, the best Nb - k_neg are
 //     critical-or-marginal.
 //   Phase C (same warp): class row and ascending index lists, written with ballot prefix sums.
+//
+// late_wait: the launch before this one in the stream (the summaries) neither writes what this kernel reads nor touches
+// what it writes, and has itself waited for everything that does: the two run side by side, and this kernel waits for the
+// other one's completion only before it ends, so that its own completion stands for both.
 #include <atomic>
 
 #include "common.cuh"
@@ -249,7 +253,7 @@ __device__ Selection select_top(const unsigned long long* keys, Bucket bucket, i
 template <int R>
 __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_colsum, const int* __restrict__ k_colsum,
                                                        const float* __restrict__ k_scales, int tokens, int block,
-                                                       int nb, int k_crit, int k_marg, int k_neg,
+                                                       int nb, int k_crit, int k_marg, int k_neg, int late_wait,
                                                        signed char* __restrict__ cls, int* __restrict__ crit_idx,
                                                        int* __restrict__ marg_idx) {
   constexpr int kThreads = R * 32;
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
   const int lane = threadIdx.x & 31;
   const size_t bh_rows = static_cast<size_t>(bh) * nb;
 
-  sm100::wait_for_prior_grid();
+  if (!late_wait) sm100::wait_for_prior_grid();
   sm100::launch_dependents();
   if constexpr (kDirect) {
     // Phase A, R rows x 8 key blocks per warp and step as fp64 tensor-core products (m8n8k4, 16 k-steps over the 64
@@ -489,6 +493,7 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
       n_crit += __popc(m_crit);
       n_marg += __popc(m_marg);
     }
+    if (late_wait) sm100::wait_for_prior_grid();
     return;
   }
 
@@ -571,6 +576,7 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
       marg_row += __popc(m_marg);
     }
   }
+  if (late_wait) sm100::wait_for_prior_grid();
 }
 
 // Two neighbouring column sums times 2^-10 as fp16 pairs hi + lo (22 bits between them).
@@ -610,7 +616,7 @@ __device__ __forceinline__ void mma_m16n8k16(float (&c)[4], uint32_t a0, uint32_
 template <int R>
 __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restrict__ q_colsum, const int* __restrict__ k_colsum,
                                                                const float* __restrict__ k_scales, int tokens, int block,
-                                                               int nb, int k_crit, int k_marg, int k_neg,
+                                                               int nb, int k_crit, int k_marg, int k_neg, int late_wait,
                                                                signed char* __restrict__ cls, int* __restrict__ crit_idx,
                                                                int* __restrict__ marg_idx) {
   constexpr bool kApprox = R == 16;
@@ -640,7 +646,7 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
     return ((valid == block && block_pow2) ? num * inv_block : num / static_cast<double>(valid)) + 0.0;
   };
 
-  sm100::wait_for_prior_grid();
+  if (!late_wait) sm100::wait_for_prior_grid();
   sm100::launch_dependents();
   if constexpr (kApprox) {
     // Phase A, 16 rows x 8 key blocks per warp and step (m16n8k16).  As below, lane (g, t) supplies columns 16 t ..
@@ -1063,6 +1069,7 @@ __global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restr
       marg_row += __popc(m_marg);
     }
   }
+  if (late_wait) sm100::wait_for_prior_grid();
 }
 
 size_t plan_compact_smem_bytes(int nb, int rows) {
@@ -1074,14 +1081,14 @@ size_t plan_compact_smem_bytes(int nb, int rows) {
 
 template <int R>
 lite3r_status launch_compact(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r_shape& s, const Counts& c,
-                             const lite3r_plan& plan, int nb, cudaStream_t stream) {
+                             const lite3r_plan& plan, int nb, int late_wait, cudaStream_t stream) {
   const size_t smem = plan_compact_smem_bytes(nb, R);
   lite3r_status st = ensure_dynamic_smem(plan_compact_kernel<R>, static_cast<int>(smem));
   if (st != LITE3R_OK) return st;
   const int row_tiles = ceil_div(nb, R);
   return launch_dependent(plan_compact_kernel<R>, dim3(static_cast<unsigned>(s.batch * s.heads * row_tiles)), R * 32,
                           static_cast<int>(smem), stream, q.colsum, k.colsum, k.scales, s.tokens, s.block, nb, c.k_crit, c.k_marg,
-                          c.k_neg, plan.cls, plan.crit_idx, plan.marg_idx);
+                          c.k_neg, late_wait, plan.cls, plan.crit_idx, plan.marg_idx);
 }
 
 size_t plan_smem_bytes(int nb, int rows) {
@@ -1096,14 +1103,14 @@ size_t plan_smem_bytes(int nb, int rows) {
 
 template <int R>
 lite3r_status launch_rows(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r_shape& s, const Counts& c,
-                          const lite3r_plan& plan, int nb, cudaStream_t stream) {
+                          const lite3r_plan& plan, int nb, int late_wait, cudaStream_t stream) {
   const size_t smem = plan_smem_bytes(nb, R);
   lite3r_status st = ensure_dynamic_smem(plan_kernel<R>, static_cast<int>(smem));
   if (st != LITE3R_OK) return st;
   const int row_tiles = ceil_div(nb, R);
   return launch_dependent(plan_kernel<R>, dim3(static_cast<unsigned>(s.batch * s.heads * row_tiles)), R * 32,
                           static_cast<int>(smem), stream, q.colsum, k.colsum, k.scales, s.tokens, s.block, nb, c.k_crit, c.k_marg,
-                          c.k_neg, plan.cls, plan.crit_idx, plan.marg_idx);
+                          c.k_neg, late_wait, plan.cls, plan.crit_idx, plan.marg_idx);
 }
 
 }  // namespace
@@ -1113,14 +1120,15 @@ static std::atomic<int> g_plan_variant{0};
 void set_plan_variant(int variant) { g_plan_variant.store(variant, std::memory_order_relaxed); }
 
 lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r_shape& s, const Counts& c,
-                          const lite3r_plan& plan, cudaStream_t stream) {
+                          const lite3r_plan& plan, bool beside_prior, cudaStream_t stream) {
+  const int late_wait = beside_prior ? 1 : 0;
   const int nb = ceil_div(s.tokens, s.block);
   constexpr size_t kLimit = 227 * 1024;
   switch (g_plan_variant.load(std::memory_order_relaxed)) {  // forced by a test; sizes that do not fit are refused
-    case 1: return plan_smem_bytes(nb, 8) <= kLimit ? launch_rows<8>(q, k, s, c, plan, nb, stream) : LITE3R_ERR_UNSUPPORTED;
-    case 2: return plan_compact_smem_bytes(nb, 8) <= kLimit && nb <= 65536 ? launch_compact<8>(q, k, s, c, plan, nb, stream) : LITE3R_ERR_UNSUPPORTED;
-    case 3: return plan_compact_smem_bytes(nb, 16) <= kLimit && nb <= 65536 ? launch_compact<16>(q, k, s, c, plan, nb, stream) : LITE3R_ERR_UNSUPPORTED;
-    case 4: return plan_smem_bytes(nb, 4) <= kLimit ? launch_rows<4>(q, k, s, c, plan, nb, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 1: return plan_smem_bytes(nb, 8) <= kLimit ? launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 2: return plan_compact_smem_bytes(nb, 8) <= kLimit && nb <= 65536 ? launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 3: return plan_compact_smem_bytes(nb, 16) <= kLimit && nb <= 65536 ? launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 4: return plan_smem_bytes(nb, 4) <= kLimit ? launch_rows<4>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
     default: break;
   }
   // Long rows (where the 8-byte keys of eight rows would leave room for a single CTA per SM): single-precision scores in
@@ -1131,14 +1139,14 @@ lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r
   if (st != LITE3R_OK) return st;
   if (plan_smem_bytes(nb, 8) > kLimit / 2 && nb <= 65536) {
     const long long ctas16 = static_cast<long long>(s.batch) * s.heads * ceil_div(nb, 16);
-    if (ctas16 >= 4ll * sms && plan_compact_smem_bytes(nb, 16) <= kLimit) return launch_compact<16>(q, k, s, c, plan, nb, stream);
-    if (plan_compact_smem_bytes(nb, 8) <= kLimit) return launch_compact<8>(q, k, s, c, plan, nb, stream);
+    if (ctas16 >= 4ll * sms && plan_compact_smem_bytes(nb, 16) <= kLimit) return launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream);
+    if (plan_compact_smem_bytes(nb, 8) <= kLimit) return launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream);
   }
   // As many rows per CTA as the row keys allow: the staged key blocks are then shared by more rows.
-  if (plan_smem_bytes(nb, 8) <= kLimit) return launch_rows<8>(q, k, s, c, plan, nb, stream);
-  if (plan_smem_bytes(nb, 4) <= kLimit) return launch_rows<4>(q, k, s, c, plan, nb, stream);
-  if (plan_smem_bytes(nb, 2) <= kLimit) return launch_rows<2>(q, k, s, c, plan, nb, stream);
-  if (plan_smem_bytes(nb, 1) <= kLimit) return launch_rows<1>(q, k, s, c, plan, nb, stream);
+  if (plan_smem_bytes(nb, 8) <= kLimit) return launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream);
+  if (plan_smem_bytes(nb, 4) <= kLimit) return launch_rows<4>(q, k, s, c, plan, nb, late_wait, stream);
+  if (plan_smem_bytes(nb, 2) <= kLimit) return launch_rows<2>(q, k, s, c, plan, nb, late_wait, stream);
+  if (plan_smem_bytes(nb, 1) <= kLimit) return launch_rows<1>(q, k, s, c, plan, nb, late_wait, stream);
   return LITE3R_ERR_UNSUPPORTED;  // more than ~24000 blocks per sequence
 }
 

@@ -41,7 +41,7 @@ def test_many_buffer_sets_in_turn(block):
             hold.append(eng)  # some buffers stay, the others' addresses are taken over
 
 
-@pytest.mark.parametrize("blocks", [1, 32, 33, 64, 65])
+@pytest.mark.parametrize("blocks", [3, 32, 33, 64, 65])
 def test_plan_rows_around_the_rank_limit(blocks):
     """Rows of up to 64 blocks are ranked by comparing all pairs (one or two entries per lane), longer ones selected
     through histograms."""
