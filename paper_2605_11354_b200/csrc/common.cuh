@@ -44,21 +44,30 @@ lite3r_status ensure_dynamic_smem(K* kernel, int bytes) {
 // Enqueues a kernel as a programmatic dependent of the launch before it in the stream: it may start while that one is
 // still running, and waits (griddepcontrol.wait) before it touches anything that one reads or writes.  Every kernel of
 // the library that is launched this way lets its own successor start early as soon as its set-up is done.
+// cluster: CTAs per thread-block cluster.
 template <typename... Params, typename... Args>
-lite3r_status launch_dependent(void (*kernel)(Params...), dim3 grid, int block, int smem_bytes, cudaStream_t stream,
-                               const Args&... args) {
+lite3r_status launch_dependent_cluster(void (*kernel)(Params...), dim3 grid, int block, int smem_bytes, int cluster,
+                                       cudaStream_t stream, const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(static_cast<unsigned>(block));
   cfg.dynamicSmemBytes = static_cast<size_t>(smem_bytes);
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   const lite3r_status st = record_cuda(cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...));
   return st == LITE3R_OK ? after_launch() : st;
+}
+template <typename... Params, typename... Args>
+lite3r_status launch_dependent(void (*kernel)(Params...), dim3 grid, int block, int smem_bytes, cudaStream_t stream,
+                               const Args&... args) {
+  return launch_dependent_cluster(kernel, grid, block, smem_bytes, 1, stream, args...);
 }
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }

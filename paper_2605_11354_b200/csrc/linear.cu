@@ -6,8 +6,10 @@
 //                   sums in the library's own layout, so the separate quantiser pass over Q, K, V disappears.
 //
 // GEMM kernel: persistent CTAs (one per SM) over 128 x 256 output tiles (128 tokens x 256 output columns = four heads
-// of the projection).  Warp 0 = TMA producer (A = activation codes, B = weight codes, both K-major rows of 128 bytes,
-// 128B swizzle, ring of four stages), warp 1 = MMA issuer (four kind::f8f6f4 products of K = 32 per stage into one of
+// of the projection), or pairs of CTAs over tiles of 256 x 256 (cta_group::2 products that read half of the weights from
+// either CTA).  The operand bytes from L2 bound the product: 43968 x 1024 x 1024 took 54.5 us by single CTAs and takes 50 us
+// by pairs, with the tensor pipe busy for 45% of it.  Warp 0 = TMA producer (A = activation codes, B = weight codes, both
+// K-major rows of 128 bytes, 128B swizzle, ring of three or four stages), warp 1 = MMA issuer (four kind::f8f6f4 products of K = 32 per stage into one of
 // two accumulators), warps 4-19 = four epilogue warpgroups, one per 64 columns of the tile (thread = token row = TMEM
 // lane; two passes over the accumulator, maximum then codes, so that a row of 64 values never has to stay in
 // registers).  The products of the next tile run under the epilogue of this one.
@@ -154,23 +156,29 @@ __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ 
 }
 
 // ------------------------------------------------------------------------------------------------ GEMM
-constexpr int kStages = 3;
-constexpr int kTileM = 128, kTileN = 256, kTileK = 128;  // K in bytes = e4m3 elements
+constexpr int kTileM = 128, kTileN = 256, kTileK = 128;  // rows and columns of a CTA's accumulator; K in bytes = e4m3 elements
 constexpr int kEpiGroups = kTileN / 64;                   // epilogue warpgroups, one per 64 columns (one head) of the tile
 constexpr int kThreads = 128 + kEpiGroups * 128;          // 4 control warps + the epilogue warpgroups
-constexpr uint32_t kStageBytes = kTileM * kTileK + kTileN * kTileK;  // 48 KB
-constexpr uint32_t kOffB = kTileM * kTileK;
-constexpr uint32_t kOffOut = kStages * kStageBytes;   // staged output, 16 KB per epilogue warpgroup (4 KB per warp)
-constexpr uint32_t kOffMisc = kOffOut + kEpiGroups * 16384;  // column scales and bias (two tiles each), reduction slots,
-                                                             // column sums
-constexpr uint32_t kOffBar = kOffMisc + 4096 + 64 + 2048;
-constexpr uint32_t kSmemBytes = kOffBar + 256;  // 219456 B: one CTA per SM
 constexpr uint32_t kAccCols = kTileN;           // one accumulator (128 x 256 fp32)
 constexpr uint32_t kTmemCols = 2 * kAccCols;    // two of them (all of tensor memory): the products of the next tile run
                                                 // under this tile's epilogue
+// kPair: two CTAs work on one tile of 256 x 256.  Each loads its own 128 rows of A and one half of B's rows, 32 KB instead
+// of 48 KB per K step and accumulator, since the pair's products read both halves of B from where they lie.
+template <bool kPair>
+struct Layout {
+  static constexpr int kStages = kPair ? 4 : 3;
+  static constexpr int kLoadN = kPair ? kTileN / 2 : kTileN;  // rows of B this CTA loads
+  static constexpr uint32_t kStageBytes = kTileM * kTileK + kLoadN * kTileK;
+  static constexpr uint32_t kOffB = kTileM * kTileK;
+  static constexpr uint32_t kOffOut = kStages * kStageBytes;  // staged output, 16 KB per epilogue warpgroup (4 KB per warp)
+  static constexpr uint32_t kOffMisc = kOffOut + kEpiGroups * 16384;  // column scales and bias (two tiles each), reduction
+                                                                      // slots, column sums
+  static constexpr uint32_t kOffBar = kOffMisc + 4096 + 64 + 2048;
+  static constexpr uint32_t kSmemBytes = kOffBar + 256;  // one CTA per SM
+};
 
 struct Bars {
-  uint64_t full[kStages], empty[kStages];
+  uint64_t full[4], empty[4];
   uint64_t acc_full[2], acc_empty[2];  // accumulator written (issuer -> epilogue) / read out (epilogue -> issuer)
   uint32_t tmem_base;
   int abort;
@@ -210,20 +218,27 @@ __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
 // the accumulators alternate with the CTA's tile count.  The producer and the issuer run ahead into the next tile
 // while the epilogue warps drain the previous accumulator: with one tile per CTA the operand loads stopped during
 // every epilogue and the kernel was bound by the latency of its loads, not by the tensor pipe or the epilogue.
+template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                   const __grid_constant__ OutMaps maps, const LinearParams p) {
+  using L = Layout<kPair>;
+  constexpr int kStages = L::kStages;
+  constexpr uint32_t kStageBytes = L::kStageBytes, kOffB = L::kOffB, kOffOut = L::kOffOut, kOffMisc = L::kOffMisc;
   extern __shared__ __align__(1024) uint8_t smem[];
-  Bars* bars = reinterpret_cast<Bars*>(smem + kOffBar);
+  Bars* bars = reinterpret_cast<Bars*>(smem + L::kOffBar);
   volatile int* abort_flag = &bars->abort;
-  if ((smem_u32(smem) & 1023u) != 0) {
+  if ((smem_u32(smem) & 1023u) != 0) {  // the same in both CTAs of a pair
     if (threadIdx.x == 0 && p.status != nullptr) atomicCAS(p.status, 0, 900);
     return;
   }
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // row tiles never run through a batch boundary in the fused form (a tile belongs to one sequence)
-  const int tiles_per_seq = ((p.fused ? p.tokens : p.rows) + kTileM - 1) / kTileM;
+  constexpr int kCtas = kPair ? 2 : 1;
+  const int tiles_per_seq = ((p.fused ? p.tokens : p.rows) + kCtas * kTileM - 1) / (kCtas * kTileM);
+  const int rank = kPair ? static_cast<int>(cluster_rank()) : 0;
+  const int first_tile = blockIdx.x / kCtas, tile_step = gridDim.x / kCtas;
   const int k_steps = p.d_in / kTileK;
   struct TileAt {
     int seq, tile_in_seq, row0, rows_valid, col0;
@@ -233,8 +248,8 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const int row_tile = tile_id / p.col_tiles;
     t.col0 = (tile_id - row_tile * p.col_tiles) * kTileN;
     t.seq = row_tile / tiles_per_seq;
-    t.tile_in_seq = row_tile - t.seq * tiles_per_seq;
-    t.row0 = p.fused ? t.seq * p.tokens + t.tile_in_seq * kTileM : row_tile * kTileM;
+    t.tile_in_seq = kCtas * (row_tile - t.seq * tiles_per_seq) + rank;  // of 128 rows
+    t.row0 = (p.fused ? t.seq * p.tokens : 0) + t.tile_in_seq * kTileM;
     t.rows_valid = min(kTileM, (p.fused ? p.tokens : p.rows) - t.tile_in_seq * kTileM);
     return t;
   };
@@ -250,16 +265,22 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bars->acc_full[b], 1);
-      mbar_init(&bars->acc_empty[b], kEpiGroups * 128);
+      mbar_init(&bars->acc_empty[b], kCtas * kEpiGroups * 4);  // one arrival per epilogue warp
     }
     bars->abort = 0;
     mbar_fence_init();
   }
   if (warp == 1) {
-    tmem_alloc(&bars->tmem_base, kTmemCols);
-    tmem_relinquish();
+    if constexpr (kPair) {
+      tmem_alloc_pair(&bars->tmem_base, kTmemCols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(&bars->tmem_base, kTmemCols);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
+  if constexpr (kPair) cluster_sync();  // barriers and tensor memory of both CTAs are there
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
@@ -273,27 +294,34 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       tma_prefetch_desc(&map_w);
       bool ok = true;
       int kc = 0;  // K steps issued so far, through all tiles
-      for (int tile_id = blockIdx.x; ok && tile_id < p.tiles; tile_id += gridDim.x) {
+      for (int tile_id = first_tile; ok && tile_id < p.tiles; tile_id += tile_step) {
         const TileAt t = tile_at(tile_id);
         for (int k = 0; ok && k < k_steps; ++k, ++kc) {
           const int st = kc % kStages;
           if (kc >= kStages)
             ok = mbar_wait_clearing(&bars->empty[st], ((kc - kStages) / kStages) & 1, abort_flag, p.status, 601, 32);
           if (!ok) break;
-          mbar_arrive_expect_tx(&bars->full[st], kStageBytes);
-          tma_load_2d(smem + st * kStageBytes, &map_x, &bars->full[st], k * kTileK, t.row0);
-          tma_load_2d(smem + st * kStageBytes + kOffB, &map_w, &bars->full[st], k * kTileK, t.col0);
+          if (rank == 0) mbar_arrive_expect_tx(&bars->full[st], kCtas * kStageBytes);
+          if constexpr (kPair) {  // both CTAs' loads count on the leader's barrier
+            const uint32_t full = cluster_u32(&bars->full[st], 0);
+            tma_load_2d_pair(smem + st * kStageBytes, &map_x, full, k * kTileK, t.row0);
+            tma_load_2d_pair(smem + st * kStageBytes + kOffB, &map_w, full, k * kTileK, t.col0 + rank * L::kLoadN);
+          } else {
+            tma_load_2d(smem + st * kStageBytes, &map_x, &bars->full[st], k * kTileK, t.row0);
+            tma_load_2d(smem + st * kStageBytes + kOffB, &map_w, &bars->full[st], k * kTileK, t.col0);
+          }
         }
       }
+      if (kPair && !ok) __nanosleep(1000000);  // copies under way land before the memory is given up
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc(0, kTileM, kTileN, 0, 0);  // e4m3 x e4m3, both K-major
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t idesc = instr_desc(0, kCtas * kTileM, kTileN, 0, 0);  // e4m3 x e4m3, both K-major
       const uint64_t a_desc0 = smem_desc(smem_u32(smem), 16, 1024, kSwizzle128);
       const uint64_t b_desc0 = smem_desc(smem_u32(smem) + kOffB, 16, 1024, kSwizzle128);
       bool ok = true;
       int kc = 0, it = 0;
-      for (int tile_id = blockIdx.x; ok && tile_id < p.tiles; tile_id += gridDim.x, ++it) {
+      for (int tile_id = first_tile; ok && tile_id < p.tiles; tile_id += tile_step, ++it) {
         const int ab = it & 1;
         // the accumulator was last used two tiles ago: wait until the epilogue warps have read it out
         if (it >= 2) ok = mbar_wait_clearing(&bars->acc_empty[ab], ((it - 2) >> 1) & 1, abort_flag, p.status, 604);
@@ -305,12 +333,19 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           tc_fence_after();
           const uint64_t off = static_cast<uint64_t>((st * kStageBytes) >> 4);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_f8(tmem + ab * kAccCols, a_desc0 + off + ((kk * 32) >> 4), b_desc0 + off + ((kk * 32) >> 4), idesc,
-                   (k > 0 || kk > 0) ? 1u : 0u);
-          mma_commit(&bars->empty[st]);
+          for (int kk = 0; kk < 4; ++kk) {
+            const uint64_t a_desc = a_desc0 + off + ((kk * 32) >> 4), b_desc = b_desc0 + off + ((kk * 32) >> 4);
+            const uint32_t accumulate = (k > 0 || kk > 0) ? 1u : 0u;
+            if constexpr (kPair) mma_f8_pair(tmem + ab * kAccCols, a_desc, b_desc, idesc, accumulate);
+            else mma_f8(tmem + ab * kAccCols, a_desc, b_desc, idesc, accumulate);
+          }
+          if constexpr (kPair) mma_commit_pair(&bars->empty[st]);
+          else mma_commit(&bars->empty[st]);
         }
-        if (ok) mma_commit(&bars->acc_full[ab]);
+        if (ok) {
+          if constexpr (kPair) mma_commit_pair(&bars->acc_full[ab]);
+          else mma_commit(&bars->acc_full[ab]);
+        }
       }
     }
   } else if (warp >= 4) {
@@ -321,9 +356,17 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const int tid = threadIdx.x - (4 + hh * 4) * 32;  // thread of the warpgroup
     uint8_t* const staged = smem + kOffOut + hh * 16384;  // this warpgroup's output on its way to memory
     const int bar_id = 1 + hh;
+    auto acc_read_out = [&](int ab) {  // the issuer waits in the leader
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if constexpr (kPair) mbar_arrive_cluster(cluster_u32(&bars->acc_empty[ab], 0));
+        else mbar_arrive(&bars->acc_empty[ab]);
+      }
+    };
     bool ok = true;
     int it = 0;
-    for (int tile_id = blockIdx.x; ok && tile_id < p.tiles; tile_id += gridDim.x, ++it) {
+    for (int tile_id = first_tile; ok && tile_id < p.tiles; tile_id += tile_step, ++it) {
     const TileAt ta = tile_at(tile_id);
     const int row0 = ta.row0, rows_valid = ta.rows_valid, seq = ta.seq, tile_in_seq = ta.tile_in_seq;
     const int ab = it & 1;
@@ -361,8 +404,7 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         }
         tmem_wait_ld();
         if (cb == 32) {  // the accumulator is in registers: the issuer may reuse it
-          tc_fence_before();
-          mbar_arrive(&bars->acc_empty[ab]);
+          acc_read_out(ab);
         }
 #pragma unroll
         for (int c = 0; c < 32; c += 4) {
@@ -456,8 +498,7 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         tmem_ld32(acc_addr + cb, v);
         tmem_wait_ld();
         if (cb == 32) {  // the accumulator is in registers: the issuer may reuse it
-          tc_fence_before();
-          mbar_arrive(&bars->acc_empty[ab]);
+          acc_read_out(ab);
         }
 #pragma unroll
         for (int c = 0; c < 32; c += 4) {
@@ -518,8 +559,7 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         }
       }
     } else {
-      tc_fence_before();
-      mbar_arrive(&bars->acc_empty[ab]);  // nothing to do for columns past the output
+      acc_read_out(ab);  // nothing to do for columns past the output
     }
     }  // tiles
     bulk_wait_group_read0();  // what is staged stays in place until it has been read
@@ -527,30 +567,49 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 
   tc_fence_before();
   __syncthreads();
+  if constexpr (kPair) cluster_sync();  // neither CTA leaves while the other one's loads, products or arrivals may reach it
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, kTmemCols);
+    if constexpr (kPair) tmem_dealloc_pair(tmem, kTmemCols);
+    else tmem_dealloc(tmem, kTmemCols);
   }
 }
 
-lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const OutMaps& maps, const LinearParams& p,
-                          cudaStream_t stream) {
+int row_tiles(const LinearParams& p, int rows) {
+  return p.fused ? p.batch * ceil_div(p.tokens, rows) : ceil_div(p.rows, rows);
+}
+
+template <bool kPair>
+lite3r_status launch_tiles(const uint8_t* x_codes, const uint8_t* w_codes, const OutMaps& maps, const LinearParams& p, int sms,
+                           cudaStream_t stream) {
+  using L = Layout<kPair>;
+  constexpr int kCtas = kPair ? 2 : 1;
   CUtensorMap map_x, map_w;
   lite3r_status st;
   if ((st = make_tensor_map_2d(&map_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, x_codes, p.d_in, p.rows, kTileK, kTileM,
                                CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
-  if ((st = make_tensor_map_2d(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, w_codes, p.d_in, p.d_out, kTileK, kTileN,
+  if ((st = make_tensor_map_2d(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, w_codes, p.d_in, p.d_out, kTileK, L::kLoadN,
                                CU_TENSOR_MAP_SWIZZLE_128B)) != LITE3R_OK) return st;
-  if ((st = ensure_dynamic_smem(linear_fp8_kernel, static_cast<int>(kSmemBytes))) != LITE3R_OK) return st;
-  const int row_tiles = p.fused ? p.batch * ceil_div(p.tokens, kTileM) : ceil_div(p.rows, kTileM);
+  if ((st = ensure_dynamic_smem(linear_fp8_kernel<kPair>, static_cast<int>(L::kSmemBytes))) != LITE3R_OK) return st;
   LinearParams q = p;
   q.col_tiles = ceil_div(p.d_out, kTileN);
-  q.tiles = q.col_tiles * row_tiles;
+  q.tiles = q.col_tiles * row_tiles(p, kCtas * kTileM);
+  const int grid = kCtas * std::min(q.tiles, sms / kCtas);
+  return launch_dependent_cluster(linear_fp8_kernel<kPair>, dim3(static_cast<unsigned>(grid)), kThreads,
+                                  static_cast<int>(L::kSmemBytes), kCtas, stream, map_x, map_w, maps, q);
+}
+
+// Pairs of CTAs when there is more than one tile of 128 x 256 per SM: a tile's operand bytes, which bound the kernel, are a
+// third fewer.  Up to one tile per SM nothing overlaps and the pair's two hand-shakes are in the way (one frame of the qkv
+// projection, 132 tiles: 13.3 us by single CTAs, 13.8 by pairs).
+lite3r_status launch_gemm(const uint8_t* x_codes, const uint8_t* w_codes, const OutMaps& maps, const LinearParams& p,
+                          cudaStream_t stream) {
   int sms = 0;
-  if ((st = sm_count(&sms)) != LITE3R_OK) return st;
-  const int grid = q.tiles < sms ? q.tiles : sms;
-  return launch_dependent(linear_fp8_kernel, dim3(static_cast<unsigned>(grid)), kThreads, static_cast<int>(kSmemBytes), stream, map_x,
-                          map_w, maps, q);
+  const lite3r_status st = sm_count(&sms);
+  if (st != LITE3R_OK) return st;
+  return static_cast<long long>(ceil_div(p.d_out, kTileN)) * row_tiles(p, kTileM) > sms
+             ? launch_tiles<true>(x_codes, w_codes, maps, p, sms, stream)
+             : launch_tiles<false>(x_codes, w_codes, maps, p, sms, stream);
 }
 
 template <typename SrcT>

@@ -6,6 +6,8 @@ import torch
 from paper_2605_11354_b200 import binding as lt
 from paper_2605_11354_b200 import workloads as wk
 
+from oracle import sla_oracle as orc
+
 import parity_util as pu
 from test_gpu_parity import full_parity, oracle_subset, small_workload
 
@@ -75,3 +77,19 @@ def test_aggregation_inside_one_sequence(blocks):
     """Key chunks of 64 that end with, before and after the row, row tiles of 128 full and ragged."""
     wl = small_workload(f"agg{blocks}", heads=3, tokens=blocks * 64, crit=0.05, neg=0.2)
     full_parity(wl, wk.make_inputs(wl), query_blocks=pu.sample_blocks(wl, [0, 2], 6))
+
+
+@pytest.mark.parametrize("rows,d_out", [(18944, 256), (18945, 256), (9473, 512), (2500, 1984)])
+def test_linear_tiles_around_one_per_sm(rows, d_out):
+    """148 tiles of 128 x 256 are one per SM; from one more on, pairs of CTAs take tiles of 256 x 256: an odd number of row
+    tiles, last tiles of one row, last column tiles of less than half a tile."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn((rows, 256), device="cuda", generator=g)
+    w = torch.randn((d_out, 256), device="cuda", generator=g) / 16
+    (xc, xs), (wc, ws) = lt.lite3r_quantize_rows_fp8(x), lt.lite3r_quantize_rows_fp8(w)
+    y, status = torch.empty((rows, d_out), device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    lt.lite3r_linear_fp8(xc, xs, wc, ws, None, y, status)
+    pick = [0, 1, 127, 128, 255, 256, rows // 2, rows - 2, rows - 1]
+    ref = orc.linear_fp8(*(t.cpu().numpy() for t in (xc[pick], xs.reshape(-1)[pick], wc, ws)))
+    assert status.item() == 0
+    np.testing.assert_allclose(y[pick].cpu().numpy(), ref, rtol=1e-5, atol=1e-5 * np.abs(ref).max())
