@@ -102,37 +102,48 @@ __device__ __forceinline__ float e4m3_scale(float amax) { return __fdiv_rn(__fad
 
 // The e4m3 codes of x / scale, where x / scale is the correctly rounded fp32 quotient (so that codes equal those of a plain
 // fp32 program bit for bit), saturated at +-448 and rounded to nearest even.  The quotient comes from the correctly
-// rounded reciprocal r and two corrections q + (x - q s) r, whose residual a fused multiply-add gives exactly: the first
-// brings the product x r (up to two ulps off) to within one ulp, after which the second is correctly rounded (P. Markstein,
-// "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990).  Scales are
-// at least 1e-8 / 448, so the residual is exact for every x whose code is not zero.  Five packed multiply-adds per pair;
-// bracketing the quotient between two products and redoing with a division the pairs whose two codes differ took two
-// multiply-adds and two conversions, but one bf16 value in six hundred lies so close to a rounding boundary that a third
-// of all groups of 256 went through the division.
+// rounded reciprocal r and corrections q + (x - q s) r, whose residual a fused multiply-add gives exactly (scales are at
+// least 1e-8 / 448, so for every x whose code is not zero).  Two corrections make it correctly rounded: the first brings the
+// product x r to within one ulp, after which the second is (P. Markstein, "Computation of elementary functions on the IBM
+// RISC System/6000 processor", IBM J. Res. Dev. 34, 1990).  One is enough for the code, except for rare scales:
+//   After one correction q = RN(x / s + h) with |h| <= 2^-47 |x / s|, so q and the quotient differ only when x / s lies within
+//   h of the middle M of two neighbouring fp32 values, and their codes only when one of those two is a rounding boundary of
+//   e4m3.  A boundary has at most 5 significant bits, so M as an integer of 25 (at a power of two 26) bits is
+//   m 2^20 +- 1.  With x and s as integers X and S of 24 bits, |X 2^k - M S| (k >= 24) would be below 8.  It is not zero (M is
+//   odd and longer than X), and modulo 2^20 it is +-S: the low 20 bits of S would lie within 8 of 0.  (When they are all
+//   zero, S = t 2^20, |X 2^(k-20) - M t| would be below 1, so zero, which it cannot be.)
+// close says that the scale is one of those (with a margin): the caller then takes the codes with two corrections.  Three
+// packed multiply-adds per pair instead of five.
 // Everything is computed for -x / scale, which keeps the sign of a zero through the corrections; flip undoes it.
 struct E4m3Quotient {
   unsigned long long neg_r2, s2;
+  bool close;
   static constexpr uint32_t kFlip = 0x80808080u;
   __device__ __forceinline__ explicit E4m3Quotient(float scale) {
     const float r = -__frcp_rn(scale);
+    const uint32_t low = __float_as_uint(scale) & 0xFFFFFu;
+    close = low != 0 && ((low + 16u) & 0xFFFFFu) <= 32u;
     asm("mov.b64 %0, {%1, %1};" : "=l"(neg_r2) : "f"(r));
     asm("mov.b64 %0, {%1, %1};" : "=l"(s2) : "f"(scale));
   }
   // two codes (low byte first), sign bits inverted
+  template <bool kTwice>
   __device__ __forceinline__ uint32_t pair(unsigned long long x2) const {
     unsigned long long q, e;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(q) : "l"(x2), "l"(neg_r2));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(e) : "l"(q), "l"(s2), "l"(x2));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(e), "l"(neg_r2), "l"(q));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(e) : "l"(q), "l"(s2), "l"(x2));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(e), "l"(neg_r2), "l"(q));
+#pragma unroll
+    for (int i = 0; i < (kTwice ? 2 : 1); ++i) {
+      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(e) : "l"(q), "l"(s2), "l"(x2));
+      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(e), "l"(neg_r2), "l"(q));
+    }
     float2 y;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(y.x), "=f"(y.y) : "l"(q));
     return __nv_cvt_float2_to_fp8x2(y, __NV_SATFINITE, __NV_E4M3);
   }
-  // four codes of two pairs
+  // four codes of two pairs; kTwice where close
+  template <bool kTwice>
   __device__ __forceinline__ uint32_t four(unsigned long long a, unsigned long long b) const {
-    return (pair(a) | (pair(b) << 16)) ^ kFlip;
+    return (pair<kTwice>(a) | (pair<kTwice>(b) << 16)) ^ kFlip;
   }
 };
 
@@ -140,6 +151,10 @@ __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
   return v;
+}
+// The same for values that are not negative (and not NaN), whose bits are ordered like they are: one instruction.
+__device__ __forceinline__ float warp_max_abs(float v) {
+  return __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(v)));
 }
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

@@ -9,12 +9,16 @@
 // of the projection), or pairs of CTAs over tiles of 256 x 256 (cta_group::2 products that read half of the weights from
 // either CTA).  The operand bytes from L2 bound the product: 43968 x 1024 x 1024 took 54.5 us by single CTAs and takes 50 us
 // by pairs, with the tensor pipe busy for 45% of it.  Warp 0 = TMA producer (A = activation codes, B = weight codes, both
-// K-major rows of 128 bytes, 128B swizzle, ring of three or four stages), warp 1 = MMA issuer (four kind::f8f6f4 products of K = 32 per stage into one of
-// two accumulators), warps 4-19 = four epilogue warpgroups, one per 64 columns of the tile (thread = token row = TMEM
-// lane; two passes over the accumulator, maximum then codes, so that a row of 64 values never has to stay in
-// registers).  The products of the next tile run under the epilogue of this one.
+// K-major rows of 128 bytes, 128B swizzle, ring of three or four stages), warp 1 = MMA issuer (four kind::f8f6f4 products
+// of K = 32 per stage into one of two accumulators), warps 4-19 = four epilogue warpgroups, one per 64 columns of the tile
+// (thread = token row = TMEM lane; two passes over the accumulator so that a row of 64 values never has to stay in
+// registers: the first scales, adds the bias, takes the maximum and writes the values back, the second makes the codes).
+// The products of the next tile run under the epilogue of this one.  With the block quantiser the epilogue is what bounds
+// the kernel: 10992 x 1024 x 3072 in 45 us (49 us while both passes scaled the products and a quotient took two
+// corrections).
 // Every mbarrier wait is bounded; on expiry the CTA sets *device_status and its roles leave their loops.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -80,17 +84,19 @@ struct RowScale {
   E4m3Quotient quotient;
   __device__ __forceinline__ explicit RowScale(float amax)
       : scale(e4m3_scale(amax)), quotient(scale) {}
-  __device__ __forceinline__ uint2 codes(const float v[8]) const {
-    return make_uint2(quotient.four(pack_f32x2(v[0], v[1]), pack_f32x2(v[2], v[3])),
-                      quotient.four(pack_f32x2(v[4], v[5]), pack_f32x2(v[6], v[7])));
+  template <bool kTwice>
+  __device__ __forceinline__ uint2 eight(const float v[8]) const {
+    return make_uint2(quotient.four<kTwice>(pack_f32x2(v[0], v[1]), pack_f32x2(v[2], v[3])),
+                      quotient.four<kTwice>(pack_f32x2(v[4], v[5]), pack_f32x2(v[6], v[7])));
   }
+  __device__ __forceinline__ uint2 codes(const float v[8]) const { return quotient.close ? eight<true>(v) : eight<false>(v); }
 };
 
 // One warp per row.  Rows of up to 256 kSegs values stay in registers as they lie in memory (all requested before the
 // first is used), and bf16 rows of that length are requested one row ahead, so that a warp's loads run under the
 // arithmetic of the row before; longer rows are read twice (maximum, then codes; the second read comes from L1 / L2).
-// Bound by HBM: 43968 x 1024 bf16 values in 21.5 us (6.3 TB/s of 135 MB; 31 us while a third of the groups of 256 values
-// went through a division).
+// Bound by HBM: 43968 x 1024 bf16 values in 18.7 us (135 MB, part of them from L2; 21.5 us with two corrections per
+// quotient, 31 us while a third of the groups of 256 values went through a division).
 template <typename SrcT, int kSegs>
 __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ x, long long row_stride, int rows, int cols,
                                                        uint8_t* __restrict__ codes, float* __restrict__ scales) {
@@ -122,7 +128,7 @@ __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ 
         m = cur[q].max_with(m);
       }
       if (kAhead && row + warps < rows) fetch(row + warps);
-      const RowScale rs(warp_max(Eight<SrcT>::top(m)));
+      const RowScale rs(warp_max_abs(Eight<SrcT>::top(m)));
       if (lane == 0) scales[row] = rs.scale;
       uint8_t* dst = codes + static_cast<size_t>(row) * cols + lane * 8;
 #pragma unroll
@@ -142,7 +148,7 @@ __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ 
         e.load(src + s * 8);
         m = e.max_with(m);
       }
-      const RowScale rs(warp_max(Eight<SrcT>::top(m)));
+      const RowScale rs(warp_max_abs(Eight<SrcT>::top(m)));
       if (lane == 0) scales[row] = rs.scale;
       uint8_t* dst = codes + static_cast<size_t>(row) * cols;
       for (int s = lane; s < segs; s += 32) {
@@ -474,10 +480,15 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           float y0, y1, y2, y3;
           unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), fma_f32x2(sx2, sw4.x, neg0), b4.x), y0, y1);
           unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), fma_f32x2(sx2, sw4.y, neg0), b4.y), y2, y3);
+          v[c] = __float_as_uint(y0);
+          v[c + 1] = __float_as_uint(y1);
+          v[c + 2] = __float_as_uint(y2);
+          v[c + 3] = __float_as_uint(y3);
           amax = fmaxf(amax, fmaxf(fmaxf(fabsf(y0), fabsf(y1)), fmaxf(fabsf(y2), fabsf(y3))));
         }
+        tmem_st32(acc_addr + cb, v);  // the finished values take the products' place
       }
-      amax = warp_max(row_ok ? amax : 0.f);
+      amax = warp_max_abs(row_ok ? amax : 0.f);
       if (lane == 0) red[quarter] = amax;
       named_barrier_sync(bar_id, 128);
       amax = 0.f;
@@ -489,6 +500,7 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       if (block_ok && (r % p.block) == 0) p.scales[part][tile_out] = scale;
       // pass 2: codes
       const E4m3Quotient quotient(scale);
+      tmem_wait_st();
       const bool want_colsum = p.colsum[part] != nullptr;
       const uint32_t my_row = smem_u32(staged) + r * 64;
       const int swz = (r >> 1) & 3;
@@ -500,17 +512,17 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         if (cb == 32) {  // the accumulator is in registers: the issuer may reuse it
           acc_read_out(ab);
         }
+        auto codes_of = [&](auto twice) {
 #pragma unroll
-        for (int c = 0; c < 32; c += 4) {
-          const ulonglong2 sw4 = *reinterpret_cast<const ulonglong2*>(wsc + cb + c);
-          const ulonglong2 b4 = *reinterpret_cast<const ulonglong2*>(bia + cb + c);
-          const unsigned long long sws[2] = {sw4.x, sw4.y}, bs[2] = {b4.x, b4.y};
-          uint64_t y2[2];
+          for (int c = 0; c < 32; c += 4)
+            packed[c >> 2] = quotient.four<decltype(twice)::value>(pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])),
+                                                                   pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])));
+        };
+        if (quotient.close) codes_of(std::true_type());
+        else codes_of(std::false_type());
+        if (!row_ok) {
 #pragma unroll
-          for (int h2 = 0; h2 < 2; ++h2)
-            y2[h2] = fma_f32x2(pack_f32x2(__uint_as_float(v[c + 2 * h2]), __uint_as_float(v[c + 2 * h2 + 1])),
-                               fma_f32x2(sx2, sws[h2], neg0), bs[h2]);
-          packed[c >> 2] = row_ok ? quotient.four(y2[0], y2[1]) : 0u;
+          for (int c = 0; c < 8; ++c) packed[c] = 0u;
         }
         // rows past the sequence end inside an existing block are written as zeros
         sts128(my_row + (((cb / 16) ^ swz) << 4), packed[0], packed[1], packed[2], packed[3]);

@@ -3,14 +3,15 @@
 //
 // One CTA per tile at a time (persistent CTAs of 64 or 128 threads, 64 values per thread).  Tiles travel global ->
 // shared memory by asynchronous 16-byte copies, a few tiles ahead of the one being processed; the tile maximum is
-// reduced through shuffles and shared memory, then every value is divided by the scale (E4m3Quotient: correctly rounded,
-// so the codes equal a plain fp32 program's bit for bit), clamped, cast to e4m3 with round-to-nearest-even and written
+// reduced through shuffles and shared memory, then every value is divided by the scale (E4m3Quotient: as if correctly
+// rounded, so the codes equal a plain fp32 program's bit for bit), clamped, cast to e4m3 with round-to-nearest-even and written
 // with 8-byte stores.  The same pass emits, where asked for, the per-tile column sums of the code values as exact
 // integers (units of 2^-9), which is all the block plan needs.  HBM traffic: 2 (bf16) or 4 (fp32) bytes read and 1 byte
 // written per element; the instruction count per element decides how close the kernel gets to that, hence the packed
-// fp32x2 arithmetic.  Q, K and V of 32 x 16 sequences of 1374 bf16 tokens: 74 us, 5.5 TB/s (100 us with a division behind
-// every bracketed rounding boundary).
+// fp32x2 arithmetic.  Q, K and V of 32 x 16 sequences of 1374 bf16 tokens: 72 us, 5.6 TB/s (100 us with a division behind
+// every bracketed rounding boundary); of four scenes of 16 frames in blocks of 128: 136 us (151 us with two corrections).
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const __grid_constan
     }
     slot = slot + 1 == kDepth ? 0 : slot + 1;
 
-    amax = warp_max(amax);
+    amax = warp_max_abs(amax);
     for (int c = threadIdx.x; c < kHeadDim; c += kThreads) s_col[c] = 0;
     if (kThreads > 32) {
       if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = amax;
@@ -195,26 +196,31 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const __grid_constan
     // per packed-pair instruction, like the two products
     uint64_t sums2[4] = {0ull, 0ull, 0ull, 0ull};
     uint8_t* dst = codes + (static_cast<size_t>(tile) * BS) * kHeadDim + seg * 8;
+    auto codes_of = [&](auto twice) {
 #pragma unroll
-    for (int p = 0; p < kPasses; ++p) {
-      const int row = row0 + p * kRowsPerPass;
-      float* const vp = v[kKeep ? p : 0];
-      if (!kKeep) unpack8(reinterpret_cast<const SrcT*>(mine + p * kThreads * kSegBytes), vp);
-      uint32_t four[2];
+      for (int p = 0; p < kPasses; ++p) {
+        const int row = row0 + p * kRowsPerPass;
+        float* const vp = v[kKeep ? p : 0];
+        if (!kKeep) unpack8(reinterpret_cast<const SrcT*>(mine + p * kThreads * kSegBytes), vp);
+        uint32_t four[2];
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        four[h] = quotient.four(pack_f32x2(vp[4 * h], vp[4 * h + 1]), pack_f32x2(vp[4 * h + 2], vp[4 * h + 3]));
-      if (colsum != nullptr) {
+        for (int h = 0; h < 2; ++h)
+          four[h] = quotient.four<decltype(twice)::value>(pack_f32x2(vp[4 * h], vp[4 * h + 1]),
+                                                          pack_f32x2(vp[4 * h + 2], vp[4 * h + 3]));
+        if (colsum != nullptr) {
 #pragma unroll
-        for (int c = 0; c < 8; c += 2) {
-          const __half2_raw back = __nv_cvt_fp8x2_to_halfraw2(
-              static_cast<__nv_fp8x2_storage_t>((four[c >> 2] >> (8 * (c & 3))) & 0xFFFFu), __NV_E4M3);
-          const float2 f = __half22float2(__half2(back));
-          sums2[c >> 1] = add_f32x2(sums2[c >> 1], pack_f32x2(f.x, f.y));
+          for (int c = 0; c < 8; c += 2) {
+            const __half2_raw back = __nv_cvt_fp8x2_to_halfraw2(
+                static_cast<__nv_fp8x2_storage_t>((four[c >> 2] >> (8 * (c & 3))) & 0xFFFFu), __NV_E4M3);
+            const float2 f = __half22float2(__half2(back));
+            sums2[c >> 1] = add_f32x2(sums2[c >> 1], pack_f32x2(f.x, f.y));
+          }
         }
+        *reinterpret_cast<uint2*>(dst + static_cast<size_t>(row) * kHeadDim) = make_uint2(four[0], four[1]);
       }
-      *reinterpret_cast<uint2*>(dst + static_cast<size_t>(row) * kHeadDim) = make_uint2(four[0], four[1]);
-    }
+    };
+    if (quotient.close) codes_of(std::true_type());
+    else codes_of(std::false_type());
     if (colsum != nullptr) {
       // Column sums over the four row groups of the warp (lanes that differ in bits 3 and 4): each exchange halves
       // the number of columns a lane still carries, so eight columns take six shuffles instead of sixteen.

@@ -93,3 +93,44 @@ def test_linear_tiles_around_one_per_sm(rows, d_out):
     ref = orc.linear_fp8(*(t.cpu().numpy() for t in (xc[pick], xs.reshape(-1)[pick], wc, ws)))
     assert status.item() == 0
     np.testing.assert_allclose(y[pick].cpu().numpy(), ref, rtol=1e-5, atol=1e-5 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("low", [1, 3, -2])
+def test_codes_next_to_rounding_boundaries_at_scales_that_take_a_second_correction(low):
+    """Scales whose last 20 bits are nearly zero: fp32 values whose quotient lies within 2^-46 of the middle of two fp32
+    values next to an e4m3 rounding boundary, in a block tile and in rows."""
+    block = 64
+    tiles = []
+    for t in range(8, 16):
+        scale = np.float32((t << 20) + low) * np.float32(2.0 ** -20)
+        amax = scale * np.float32(448.0)
+        while (amax + np.float32(1e-8)) / np.float32(448.0) > scale:
+            amax = np.nextafter(amax, np.float32(0.0))
+        while (amax + np.float32(1e-8)) / np.float32(448.0) < scale:
+            amax = np.nextafter(amax, np.float32(np.inf))
+        if (amax + np.float32(1e-8)) / np.float32(448.0) != scale:
+            continue  # no largest magnitude gives this scale
+        values = [amax]
+        for m in range(16, 32):
+            for side in (-1, 1):
+                exact = ((m << 20) + side) * ((t << 20) + low)  # the quotient's middle times the scale
+                k = exact.bit_length() - 24
+                for x in (exact >> k, (exact >> k) + 1):
+                    values += [np.float32(np.ldexp(float(x), k - 40 - e)) for e in (-3, 0, 5)]
+        values = [v for v in values if v <= amax]
+        tile = np.resize(np.array(values, dtype=np.float32), block * 64)
+        tile[1::2] *= np.float32(-1.0)
+        tile[0] = amax
+        tiles.append(tile.reshape(block, 64))
+    assert len(tiles) >= 3
+    x = np.stack(tiles).reshape(1, 1, -1, 64)
+    shape = lt.Shape(1, 1, x.shape[2], 64, block)
+    got = lt.alloc_fp8(shape, "cuda")
+    lt.lite3r_quantize_fp8(torch.from_numpy(x).cuda(), shape, got)
+    codes, scales = orc.quantize_fp8_blocks(x, block)
+    assert np.array_equal(got.scales.cpu().numpy().view(np.uint32), scales.view(np.uint32))
+    assert np.array_equal(got.codes.cpu().numpy(), codes)
+    rows = x.reshape(len(tiles), -1)[:, :1024]
+    got_codes, got_scales = lt.lite3r_quantize_rows_fp8(torch.from_numpy(np.ascontiguousarray(rows)).cuda())
+    assert np.array_equal(got_codes.cpu().numpy(), codes.reshape(len(tiles), -1)[:, :1024])
+    assert np.array_equal(got_scales.cpu().numpy().view(np.uint32).ravel(), scales.view(np.uint32).ravel())
