@@ -369,7 +369,7 @@ static lite3r_status forward_phases(int phases, const lite3r_fp8* q, const lite3
       return LITE3R_ERR_INVALID_ARG;
   }
   if (phases & 1) {
-    if (proj == nullptr || !aligned(proj, 16) || proj_head_stride < 0 || (proj_head_stride % 4)) return LITE3R_ERR_INVALID_ARG;
+    if ((proj == nullptr && !linear_only) || !aligned(proj, 16) || proj_head_stride < 0 || (proj_head_stride % 4)) return LITE3R_ERR_INVALID_ARG;
   }
   if (phases & 2) {
     if ((st = check_fp8(q, true, false)) != LITE3R_OK) return st;
@@ -490,7 +490,7 @@ lite3r_status lite3r_train_workspace(const lite3r_shape* shape, double crit, dou
   size_t fwd = 0;
   lite3r_status st = workspace_query(shape, crit, neg, false, &fwd);
   if (st != LITE3R_OK) return st;
-  *bytes = std::max(fwd + kHeadDim * kHeadDim * sizeof(float), train_workspace_bytes(*shape));
+  *bytes = std::max(fwd, train_workspace_bytes(*shape));
   return LITE3R_OK;
 }
 
@@ -503,12 +503,9 @@ lite3r_status lite3r_sla_linear_branch(const lite3r_fp8* q, const lite3r_fp8* k,
   if (st != LITE3R_OK) return st;
   if (plan == nullptr || workspace == nullptr || !aligned(workspace, 256)) return LITE3R_ERR_INVALID_ARG;
   const size_t fwd = forward_workspace_bytes(*shape, Counts{plan->k_crit, plan->k_marg, plan->k_neg});
-  if (workspace_bytes < fwd + kHeadDim * kHeadDim * sizeof(float)) return LITE3R_ERR_WORKSPACE;
-  if ((st = check_device()) != LITE3R_OK) return st;
-  // the projection is left out by running the forward with the identity in its place (exact in every format used)
-  float* identity = reinterpret_cast<float*>(static_cast<char*>(workspace) + fwd);
-  if ((st = launch_fill_identity(identity, static_cast<cudaStream_t>(stream))) != LITE3R_OK) return st;
-  return forward_phases(3, q, k, v, identity, 0, shape, 0.0, 0.0, phi, plan, out, out_dtype, out_stride_b, out_stride_h,
+  if (workspace_bytes < fwd) return LITE3R_ERR_WORKSPACE;
+  // no projection: the forward with the identity in its place (exact in every format used)
+  return forward_phases(3, q, k, v, nullptr, 0, shape, 0.0, 0.0, phi, plan, out, out_dtype, out_stride_b, out_stride_h,
                         out_stride_n, workspace, fwd, device_status, stream, 1);
 }
 

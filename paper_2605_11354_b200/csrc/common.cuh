@@ -249,7 +249,6 @@ lite3r_status launch_qkv_project(const uint8_t* x_codes, const float* x_scales, 
 
 // Training side of the linear-branch projection (train.cu).
 size_t train_workspace_bytes(const lite3r_shape& s);
-lite3r_status launch_fill_identity(float* dst, cudaStream_t stream);
 lite3r_status launch_mse_distill(const void* student, const void* teacher, int dtype, size_t count, __nv_bfloat16* grad,
                                  double* loss, double* partials, cudaStream_t stream);
 lite3r_status launch_proj_lin_backward(const __nv_bfloat16* o_lin, const __nv_bfloat16* d_out, const lite3r_shape& s,

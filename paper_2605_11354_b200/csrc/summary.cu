@@ -50,7 +50,7 @@ struct SummaryParams {
   const float* k_scales;
   const uint8_t* v_codes;
   const float* v_scales;
-  const float* proj;
+  const float* proj;  // NULL: the identity
   long long proj_head_stride;
   int heads, tokens, nb, phi;
   int rounds_per_head, rounds;
@@ -202,7 +202,15 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
         uint8_t* dst = smem + kOffW + e * 128;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const float4 x0 = __ldg(src + 2 * c), x1 = __ldg(src + 2 * c + 1);
+          float4 x0 = {}, x1 = {};
+          if (p.proj != nullptr) {
+            x0 = __ldg(src + 2 * c);
+            x1 = __ldg(src + 2 * c + 1);
+          } else {
+            const int at = e - (half * 32 + c * 8);  // where the one of row e lies in these eight columns
+            x0 = make_float4(at == 0, at == 1, at == 2, at == 3);
+            x1 = make_float4(at == 4, at == 5, at == 6, at == 7);
+          }
           const uint4 v4 = make_uint4(float2_to_half2_bits(x0.x, x0.y), float2_to_half2_bits(x0.z, x0.w),
                                       float2_to_half2_bits(x1.x, x1.y), float2_to_half2_bits(x1.z, x1.w));
           *reinterpret_cast<uint4*>(dst + (((half * 4 + c) ^ (e & 7)) << 4)) = v4;
@@ -354,8 +362,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
           const size_t tile = bh_rows + j;
           const float sv = __ldg(p.v_scales + tile);
           uint32_t hw[32];
-#pragma unroll
           const uint64_t sv2 = pack_f32x2(sv, sv), neg0 = pack_f32x2(-0.f, -0.f);  // x * sv + (-0) is x * sv
+#pragma unroll
           for (int e = 0; e < 32; e += 2) {
             float a0, a1, b0, b1;
             unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(lo[e]), __uint_as_float(lo[e + 1])), sv2, neg0), a0, a1);

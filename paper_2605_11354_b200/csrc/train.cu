@@ -17,14 +17,6 @@ namespace {
 
 using namespace sm100;
 
-// ------------------------------------------------------------------------------------------------ identity (64 x 64)
-__global__ void fill_identity_kernel(float* dst) {
-  wait_for_prior_grid();
-  launch_dependents();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < kHeadDim * kHeadDim) dst[i] = (i / kHeadDim == i % kHeadDim) ? 1.f : 0.f;
-}
-
 // ------------------------------------------------------------------------------------------------ MSE term
 constexpr int kMseThreads = 256;
 constexpr int kMaxMseBlocks = 2048;
@@ -276,10 +268,6 @@ size_t train_workspace_bytes(const lite3r_shape& s) {
   const size_t total_tiles = ceil_div(s.tokens, kTileTok);
   const size_t chunks = std::min<size_t>(total_tiles, std::max<size_t>(1, (2 * 256 + planes - 1) / planes));
   return planes * chunks * kHeadDim * kHeadDim * sizeof(float) + kMaxMseBlocks * sizeof(double) + 1024;
-}
-
-lite3r_status launch_fill_identity(float* dst, cudaStream_t stream) {
-  return launch_dependent(fill_identity_kernel, dim3((kHeadDim * kHeadDim + 255) / 256), 256, 0, stream, dst);
 }
 
 lite3r_status launch_mse_distill(const void* student, const void* teacher, int dtype, size_t count, __nv_bfloat16* grad,
