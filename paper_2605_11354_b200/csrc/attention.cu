@@ -332,10 +332,6 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (kPair) return static_cast<int>((bh_rows + j) * 64);
         return static_cast<int>((bh_rows + j) * 128 + (t & 1) * 64);
       };
-      if (leader && p.steal) {
-        mbar_arrive_expect_tx(&bars->next_full, 16);
-        request_next_cta(answer, &bars->next_full);
-      }
       if (it > 0) {  // the previous tile's last Q K^T and phi(Q) have read the Q tile
         if (steps > 0) ok = wait_all(&bars->s_full[(kc - 1) % kStages], ((kc - 1) / kStages) & 1, 104);
         if (p.k_marg > 0) ok = ok && wait_all(&bars->phi_full, (it - 1) & 1, 105);
@@ -350,6 +346,14 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       int jv[2] = {0, 0};  // key blocks of the V cursor's step
 #pragma unroll 1
       for (int t = 0; t <= steps; ++t) {
+        // The next tile is asked for two steps before the loads of this one end, which covers the answer's latency, and not
+        // earlier: asked for at a tile's start, the tiles left over from the first wave all went to the CTAs that were
+        // first to start, three to an SM, while other SMs ran dry (688 tiles of 69 steps: 248 us per step of two heads of 43968 tokens,
+        // 225 us asked for here).
+        if (t == max(steps - 1, 0) && leader && p.steal) {
+          mbar_arrive_expect_tx(&bars->next_full, 16);
+          request_next_cta(answer, &bars->next_full);
+        }
         int jk[2] = {0, 0};
         if (t < steps) {
           const bool refill = (t & 31) == 0;
