@@ -19,7 +19,7 @@
 // THREE CTAs fit on an SM.  Measured at 10 % of 2147 key blocks: 650 clocks per step and SM (two CTAs with two softmax
 // warpgroups each on alternate steps of one tile, as before: 757).
 // A CTA takes tile after tile: it asks the hardware's work scheduler for a CTA that has not been launched yet and computes
-// that one's tile itself (taken only where the grid is larger than the chip holds).  The next tile's Q, K and V tiles and
+// that one's tile itself (taken only where the grid is larger than the chip holds and a tile has products).  The next tile's Q, K and V tiles and
 // its first scores are then under way while the softmax warps write this tile's output, and what lies between two tiles
 // of a CTA (5.5 k clocks of 13 k: launch, barriers, TMEM allocation, first loads) is paid once.  Barriers are never
 // re-initialised: rings and parities run on a count through all tiles.
@@ -103,7 +103,7 @@ struct AttnParams {
   // output through TMA stores (map_o): position of the token / head / batch dimension among the map's dimensions
   // 1..3 (they are ordered by stride); tma_out = 0: plain stores
   int wait_first;  // the preceding launch must have completed before anything is read
-  int steal;  // more tiles than CTAs fit on the chip: CTAs take over the tiles of CTAs not yet launched
+  int steal;  // more tiles than CTAs fit on the chip: CTAs take over the tiles of CTAs not yet launched (see launch)
   int tma_out, dim_token, dim_head, dim_batch;
   int* status;
 };
@@ -337,7 +337,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (p.k_marg > 0) ok = ok && wait_all(&bars->phi_full, (it - 1) & 1, 105);
         if (!ok) break;
       }
-      if (leader) {
+      if (leader && v_steps > 0) {  // (a tile without products has no reader of Q: the copy could outlive the CTA)
         mbar_arrive_expect_tx(&bars->q_full, 8192);
         for (int x = 0; x < 2; ++x)
           tma_load_2d(smem + kOffQ + x * 4096, &map_q, &bars->q_full, 0,
@@ -911,7 +911,10 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   const int ctas = s.batch * s.heads * p.tiles_per_head;
   int sms = 0;
   if ((st = sm_count(&sms)) != LITE3R_OK) return st;
-  p.steal = ctas > sms * kCtasPerSm ? 1 : 0;
+  // What keeps the producer from running ahead of the softmax warps are the waits for products that read what it loaded.
+  // Without critical and without marginal blocks a tile has none: the output is zeros, every CTA writes its own tile's, and
+  // nothing is taken over (the producer would lap the four slots for tile numbers).
+  p.steal = ctas > sms * kCtasPerSm && (a.k_crit > 0 || a.k_marg > 0) ? 1 : 0;
   // With a linear branch the launch before this one is the aggregation, whose results are needed only at a tile's end: the
   // kernel then runs beside it and waits for its completion itself.  Otherwise it waits before it reads anything.
   p.wait_first = a.overlap_prior ? 0 : 1;

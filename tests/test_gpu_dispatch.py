@@ -28,6 +28,31 @@ def test_attention_grids_around_the_number_of_resident_ctas(block, batch, heads,
     assert torch.equal(again, out)  # whichever CTA computes a tile
 
 
+@pytest.mark.parametrize("crit,neg", [(0.0, 1.0), (1.0, 0.0), (0.4, 0.6)])
+@pytest.mark.parametrize("block,batch,heads,tokens", [(64, 37, 12, 128), (64, 89, 5, 65), (128, 89, 5, 100), (64, 8, 16, 6397)])
+def test_attention_without_products_on_grids_of_any_size(block, batch, heads, tokens, crit, neg):
+    """444, 445, 445 and 6400 attention tiles that have nothing to multiply, in the forward (no critical and no marginal
+    block) and in the linear branch alone (no marginal block, a dense plan among them): zeros in every row."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, k, v = (torch.randn((batch, heads, tokens, 64), device="cuda", generator=g).to(torch.bfloat16) for _ in range(3))
+    proj = torch.randn((heads, 64, 64), device="cuda", generator=g)
+    eng = lt.SlaForward(batch, heads, tokens, block, crit, neg, out_dtype=torch.bfloat16)
+    assert eng.plan.k_marg == 0
+    eng.run(q, k, v, proj)
+    out = torch.full((batch, heads, tokens, 64), float("nan"), device="cuda")
+    if crit == 0.0:
+        eng.run(q, k, v, proj, out=out)
+        torch.cuda.synchronize()
+        assert eng.status.item() == 0 and torch.count_nonzero(out).item() == 0  # (NaN counts as non-zero)
+        out.fill_(float("nan"))
+    nbytes = lt.lite3r_train_workspace(eng.shape, crit, neg)
+    raw = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
+    lt.lite3r_sla_linear_branch(eng.q8, eng.k8, eng.v8, eng.shape, eng.phi, eng.plan, out, raw[(-raw.data_ptr()) % 256:][:nbytes],
+                                eng.status)
+    torch.cuda.synchronize()
+    assert eng.status.item() == 0 and torch.count_nonzero(out).item() == 0
+
+
 @pytest.mark.parametrize("block", [64, 128])
 def test_many_buffer_sets_in_turn(block):
     """Encoded tensor maps are kept for a few hundred buffers: more sets than that, at addresses that come and go, give the
