@@ -314,7 +314,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed cha
 }  // namespace
 
 lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls, const lite3r_shape& s, int nb,
-                               __nv_bfloat16* g16, float* zeta, int* device_status, bool after_wait, cudaStream_t stream) {
+                               __nv_bfloat16* g16, float* zeta, int* device_status, cudaStream_t stream) {
   const uint64_t rows = static_cast<uint64_t>(s.batch) * s.heads * nb;
   CUtensorMap map_s;
   lite3r_status st = make_tensor_map_2d(&map_s, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hws, kSummaryRow, rows, 64, 64,
@@ -350,10 +350,6 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   auto* const kernel = flat ? aggregate_mma_kernel<true> : aggregate_mma_kernel<false>;
   st = ensure_dynamic_smem(kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
-  if (after_wait) {
-    kernel<<<grid, kThreads, kSmemBytes, stream>>>(map_s, cls, nb, total_rows, g16, zeta, device_status);
-    return after_launch();
-  }
   return launch_dependent(kernel, grid, kThreads, static_cast<int>(kSmemBytes), stream, map_s, cls, nb, total_rows, g16, zeta,
                           device_status);
 }

@@ -344,8 +344,7 @@ static lite3r_status forward_phases(int phases, const lite3r_fp8* q, const lite3
                                     double crit, double neg, lite3r_phi phi, const lite3r_plan* plan, void* out,
                                     lite3r_dtype out_dtype, long long out_stride_b, long long out_stride_h,
                                     long long out_stride_n, void* workspace, size_t workspace_bytes,
-                                    int* device_status, void* stream, int linear_only = 0, bool check_only = false,
-                                    bool chained = false) {
+                                    int* device_status, void* stream, int linear_only = 0, bool check_only = false) {
   lite3r_status st = check_shape(shape);
   if (st != LITE3R_OK) return st;
   if ((st = check_fp8(k, true, false)) != LITE3R_OK) return st;
@@ -399,7 +398,6 @@ static lite3r_status forward_phases(int phases, const lite3r_fp8* q, const lite3
   a.plan = effective;
   a.plan_inside = plan_inside ? 1 : 0;
   a.linear_only = linear_only;
-  a.chained = chained;
   a.crit = crit;
   a.neg = neg;
   a.out = out;
@@ -443,7 +441,7 @@ lite3r_status lite3r_sla_step(lite3r_step* t, void* stream) {
   auto forward = [&](int phases, bool check_only) {
     return forward_phases(phases, &t->q8, &t->k8, &t->v8, t->proj, t->proj_head_stride, &t->shape, t->crit, t->neg, t->phi,
                           plan_inside ? nullptr : &t->plan, t->out, t->out_dtype, t->out_stride_b, t->out_stride_h,
-                          t->out_stride_n, t->workspace, t->workspace_bytes, t->device_status, stream, 0, check_only, true);
+                          t->out_stride_n, t->workspace, t->workspace_bytes, t->device_status, stream, 0, check_only);
   };
   if ((st = forward(3, true)) != LITE3R_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);

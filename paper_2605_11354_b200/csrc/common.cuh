@@ -44,6 +44,9 @@ lite3r_status ensure_dynamic_smem(K* kernel, int bytes) {
 // Enqueues a kernel as a programmatic dependent of the launch before it in the stream: it may start while that one is
 // still running, and waits (griddepcontrol.wait) before it touches anything that one reads or writes.  Every kernel of
 // the library that is launched this way lets its own successor start early as soon as its set-up is done.
+// This holds wherever the launch stands: behind an event wait or a copy the stream orders it as an ordinary launch, and
+// captured, the edges from every kernel that it follows, those of a join among them, become programmatic and its wait
+// covers all of them.
 // cluster: CTAs per thread-block cluster.
 template <typename... Params, typename... Args>
 lite3r_status launch_dependent_cluster(void (*kernel)(Params...), dim3 grid, int block, int smem_bytes, int cluster,
@@ -182,7 +185,6 @@ struct ForwardArgs {
   int out_dtype;
   long long out_stride_b, out_stride_h, out_stride_n;
   int linear_only;      // 1: the sparse branch is left out (the output is the linear branch through proj alone)
-  bool chained;         // the phases follow one another in one stream with nothing but the plan between them
   int plan_inside;      // 1: the plan is built in the workspace from q/k column sums and the fractions below
   double crit, neg;
   void* workspace;
@@ -211,15 +213,14 @@ lite3r_status launch_attention(const AttentionLaunch& a, cudaStream_t stream);
 void set_attention_plain_stores(int on);  // test hook, see lite3r_attention_plain_stores
 
 // Per-key-block summaries ((H_j W)^T | z_j) in bf16, one kSummaryRow-wide row per (b, h, key block).
-// Clears *device_status; after_wait as in launch_aggregate.
+// Clears *device_status.
 lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const float* proj, long long proj_head_stride,
                              const lite3r_shape& s, int phi, __nv_bfloat16* hws, __half* v16, int* device_status,
-                             bool after_wait, cudaStream_t stream);
+                             cudaStream_t stream);
 
 // Marginal aggregation G_i = sum over marginal j of the summary rows, as a 0/1-mask GEMM on tensor cores.
-// after_wait: the stream has just waited for an event (the launch is then an ordinary one).
 lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls, const lite3r_shape& s, int nb,
-                               __nv_bfloat16* g16, float* zeta, int* device_status, bool after_wait, cudaStream_t stream);
+                               __nv_bfloat16* g16, float* zeta, int* device_status, cudaStream_t stream);
 
 // TMA descriptor of a row-major 2-D tensor [rows][inner] (row pitch in bytes, 0: inner * elem_bytes; a multiple of 16)
 // with a box of box_inner x box_rows elements.  The make_tensor_map functions keep what they have encoded (a few hundred

@@ -117,7 +117,6 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
     plan.marg_idx = nullptr;
     if (counts.k_marg == 0 && (st = launch_plan(a.q, a.k, s, counts, plan, false, stream)) != LITE3R_OK) return st;
   }
-  const bool after_wait = phases != 3 && !a.chained;
   if (phases & 1) profile_mark(0, stream);
   // With a linear branch the summary kernel reads every V row anyway and writes the fp16 operand on the way; the
   // stand-alone pass runs only when there is no linear branch.
@@ -135,7 +134,7 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   if ((phases & 1) && a.plan.k_marg > 0) {
     profile_mark(2, stream);
     st = launch_summary(a.k, a.v, a.proj, a.proj_head_stride, s, a.phi, w.hws, a.plan.k_crit > 0 ? w.v16 : nullptr,
-                        a.device_status, after_wait, stream);
+                        a.device_status, stream);
     if (st != LITE3R_OK) return st;
     profile_mark(3, stream);
   }
@@ -143,7 +142,7 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   if (a.plan_inside && counts.k_marg > 0 && (st = launch_plan(a.q, a.k, s, counts, plan, true, stream)) != LITE3R_OK) return st;
   if (a.plan.k_marg > 0) {
     profile_mark(4, stream);
-    if ((st = launch_aggregate(w.hws, plan.cls, s, nb, w.g16, w.zeta, a.device_status, after_wait, stream)) != LITE3R_OK) return st;
+    if ((st = launch_aggregate(w.hws, plan.cls, s, nb, w.g16, w.zeta, a.device_status, stream)) != LITE3R_OK) return st;
     profile_mark(5, stream);
   }
   AttentionLaunch att;

@@ -425,14 +425,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
 }
 
 template <int BS>
-lite3r_status launch(const SummaryParams& p, int sm_count, bool after_wait, cudaStream_t stream) {
+lite3r_status launch(const SummaryParams& p, int sm_count, cudaStream_t stream) {
   lite3r_status st = ensure_dynamic_smem(summary_kernel<BS>, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
   const int grid = p.rounds < sm_count * kCtasPerSm ? p.rounds : sm_count * kCtasPerSm;
-  if (after_wait) {
-    summary_kernel<BS><<<grid, kThreads, kSmemBytes, stream>>>(p);
-    return after_launch();
-  }
   return launch_dependent(summary_kernel<BS>, dim3(static_cast<unsigned>(grid)), kThreads, static_cast<int>(kSmemBytes), stream, p);
 }
 
@@ -440,7 +436,7 @@ lite3r_status launch(const SummaryParams& p, int sm_count, bool after_wait, cuda
 
 lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const float* proj, long long proj_head_stride,
                              const lite3r_shape& s, int phi, __nv_bfloat16* hws, __half* v16, int* device_status,
-                             bool after_wait, cudaStream_t stream) {
+                             cudaStream_t stream) {
   SummaryParams p;
   p.k_codes = k.codes;
   p.k_scales = k.scales;
@@ -460,7 +456,7 @@ lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const flo
   int sms = 0;
   lite3r_status st = sm_count(&sms);
   if (st != LITE3R_OK) return st;
-  return s.block == 64 ? launch<64>(p, sms, after_wait, stream) : launch<128>(p, sms, after_wait, stream);
+  return s.block == 64 ? launch<64>(p, sms, stream) : launch<128>(p, sms, stream);
 }
 
 }  // namespace lite3r

@@ -68,6 +68,56 @@ def test_many_buffer_sets_in_turn(block):
             hold.append(eng)  # some buffers stay, the others' addresses are taken over
 
 
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("crit,neg", [(0.1, 0.6), (0.25, 0.75), (0.0, 0.5), (0.0, 1.0)])
+@pytest.mark.parametrize("heads,tokens", [(16, 1374), (1, 30000)])
+def test_calls_behind_event_waits(heads, tokens, crit, neg, captured):
+    """Every kernel is a programmatic dependent, also where its stream has just waited for an event and, captured, where a
+    graph's branches fork and join: two streams share one step (K and V quantised and the first half of the forward on a
+    side stream, the plan on the main one), with summaries longer than the plan and the other way round, and with a copy
+    in front.  What a kernel reads too early holds wrong values here, but no wrong index."""
+    g = torch.Generator(device="cuda").manual_seed(2)
+    sets = [[torch.randn((1, heads, tokens, 64), device="cuda", generator=g).to(torch.bfloat16) for _ in range(3)] for _ in range(2)]
+    proj = torch.randn((heads, 64, 64), device="cuda", generator=g) / 8
+    eng = lt.SlaForward(1, heads, tokens, 64, crit, neg)
+    want = [eng.run(*x, proj).clone() for x in sets]
+    q, k, v = (torch.empty_like(x) for x in sets[0])
+    host = torch.empty_like(q, device="cpu").pin_memory()
+    side = torch.cuda.Stream()
+
+    def step():
+        main = torch.cuda.current_stream()
+        q.copy_(host, non_blocking=True)
+        side.wait_stream(main)
+        lt.lite3r_quantize_fp8(q, eng.shape, eng.q8, main)
+        lt.lite3r_quantize_fp8(k, eng.shape, eng.k8, side)
+        lt.lite3r_quantize_fp8(v, eng.shape, eng.v8, side)
+        main.wait_stream(side)
+        side.wait_stream(main)
+        lt.lite3r_sla_forward_begin(eng.k8, eng.v8, proj, eng.shape, eng.phi, eng.plan, eng.workspace, eng.status, side)
+        eng.make_plan(main)
+        main.wait_stream(side)
+        lt.lite3r_sla_forward_finish(eng.q8, eng.k8, eng.v8, eng.shape, eng.phi, eng.plan, eng.out, eng.workspace, eng.status, main)
+
+    run = step
+    if captured:
+        graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=stream):
+            step()
+        run = graph.replay
+    for i in range(12):
+        for dst, src in zip((host, k, v), sets[i % 2]):
+            dst.copy_(src)
+        for t in (eng.workspace, eng.out.view(torch.uint8), eng.q8.codes, eng.k8.codes, eng.v8.codes):
+            t.fill_(0xEE)
+        eng.plan.cls.zero_()
+        eng.plan.crit_idx.zero_()
+        torch.cuda.synchronize()
+        run()
+        torch.cuda.synchronize()
+        assert eng.status.item() == 0 and torch.equal(eng.out, want[i % 2]), i
+
+
 @pytest.mark.parametrize("blocks", [3, 32, 33, 64, 65])
 def test_plan_rows_around_the_rank_limit(blocks):
     """Rows of up to 64 blocks are ranked by comparing all pairs (one or two entries per lane), longer ones selected
