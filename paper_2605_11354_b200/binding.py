@@ -7,7 +7,6 @@ the import of any compute function raises.
 from __future__ import annotations
 
 import ctypes as C
-import itertools
 import os
 from dataclasses import dataclass
 
@@ -229,40 +228,19 @@ def lite3r_workspace_layout(shape: Shape, crit: float, neg: float, plan_inside: 
 
 
 # ----------------------------------------------------------------------------- device buffers
-_ticks = itertools.count(1)
-_generation = [0]  # changes with every assignment to the buffers below: what was marshalled before that is out of date
-
-
-class _Marshalled:
-    """Buffers whose C struct is kept until one of their fields (or those of another such object) is assigned."""
-
-    _c = None
-
-    def __setattr__(self, name, value):
-        if name != "_c":
-            _generation[0] = next(_ticks)
-        object.__setattr__(self, name, value)
-
-    def c_struct(self):
-        c = self._c
-        if c is None or c[0] != _generation[0]:
-            c = self._c = (_generation[0], self._marshal())
-        return c[1]
-
-
 @dataclass
-class Fp8Tensor(_Marshalled):
+class Fp8Tensor:
     codes: torch.Tensor  # uint8 [B,H,Nb*Bs,D]
     scales: torch.Tensor  # fp32 [B,H,Nb]
     colsum: torch.Tensor | None  # int32 [B,H,Nb,D]; None: the quantiser skips the column sums (only Q and K need them)
 
-    def _marshal(self) -> Fp8:
+    def c_struct(self) -> Fp8:
         return Fp8(self.codes.data_ptr(), self.scales.data_ptr(),
                    self.colsum.data_ptr() if self.colsum is not None else None)
 
 
 @dataclass
-class PlanBuffers(_Marshalled):
+class PlanBuffers:
     cls: torch.Tensor  # int8 [B,H,Nb,Nb]
     crit_idx: torch.Tensor  # int32 [B,H,Nb,k_crit]
     marg_idx: torch.Tensor  # int32 [B,H,Nb,k_marg]
@@ -270,7 +248,7 @@ class PlanBuffers(_Marshalled):
     k_marg: int
     k_neg: int
 
-    def _marshal(self) -> Plan:
+    def c_struct(self) -> Plan:
         return Plan(self.cls.data_ptr(), self.crit_idx.data_ptr() if self.k_crit else None,
                     self.marg_idx.data_ptr() if self.k_marg else None, self.k_crit, self.k_marg, self.k_neg)
 
@@ -516,15 +494,23 @@ class SlaForward:
         self._graph = None  # (CUDA graph of one whole step, key of the tensors it was captured on)
         self._step = None  # (key of the tensors and buffers, their marshalled arguments, pointer to those)
 
-    def __setattr__(self, name, value):
-        if not name.startswith("_"):
-            _generation[0] = next(_ticks)  # marshalled arguments hold the engine's buffers and settings
-        object.__setattr__(self, name, value)
+    def _step_key(self, q, k, v, proj, out):
+        """Everything a step's marshalled arguments or its captured graph hold, read from the tensors and the engine as they
+        are now: a buffer given other storage, a field of the shape or a setting that has changed makes another key."""
+        q8, k8, v8, plan, ws = self.q8, self.k8, self.v8, self.plan, self.workspace
+        qs, ks, vs = q8.colsum, k8.colsum, v8.colsum
+        return (q.data_ptr(), q.stride(), q.dtype, k.data_ptr(), k.stride(), k.dtype, v.data_ptr(), v.stride(), v.dtype,
+                proj.data_ptr(), proj.stride(), proj.dtype, proj.is_contiguous(), out.data_ptr(), out.stride(), out.dtype,
+                q8.codes.data_ptr(), q8.scales.data_ptr(), qs is None or qs.data_ptr(),
+                k8.codes.data_ptr(), k8.scales.data_ptr(), ks is None or ks.data_ptr(),
+                v8.codes.data_ptr(), v8.scales.data_ptr(), vs is None or vs.data_ptr(),
+                plan.cls.data_ptr(), plan.crit_idx.data_ptr(), plan.marg_idx.data_ptr(), plan.k_crit, plan.k_marg, plan.k_neg,
+                ws.data_ptr(), ws.numel(), ws.dtype, self.status.data_ptr(), bytes(self.shape), self.crit, self.neg, self.phi,
+                self.plan_inside)
 
     def _run_step(self, q, k, v, proj, stream, out):
         """quantise + plan + forward through one library call; the arguments are marshalled once per set of tensors."""
-        key = (_generation[0], q.data_ptr(), q.stride(), q.dtype, k.data_ptr(), k.stride(), k.dtype, v.data_ptr(),
-               v.stride(), v.dtype, proj.data_ptr(), proj.stride(), proj.dtype, out.data_ptr(), out.stride(), out.dtype)
+        key = self._step_key(q, k, v, proj, out)
         step = self._step
         if step is None or step[0] != key:
             step = self._step = self._marshal_step(key, q, k, v, proj, out)
@@ -565,8 +551,9 @@ class SlaForward:
         return out
 
     def run(self, q, k, v, proj, stream=None, out=None, overlap=False):
-        """Quantise, plan, forward.  overlap=True runs the plan-independent first half of the forward (summaries, fp16
-        V) on a side stream beside the plan kernel; the results are the same."""
+        """Quantise, plan, forward.  The engine's buffers, shape and settings are taken as they are at each call.
+        overlap=True runs the plan-independent first half of the forward (summaries, fp16 V) on a side stream beside the
+        plan kernel; the results are the same."""
         if self.plan_inside or not overlap or self.plan.k_marg == 0:
             return self._run_step(q, k, v, proj, stream, self.out if out is None else out)
         main = torch.cuda.current_stream(self.device) if stream is None else stream
@@ -586,11 +573,12 @@ class SlaForward:
     def run_graph(self, q, k, v, proj, out=None):
         """The same step replayed as one CUDA graph on the current stream: its five kernel launches then cost one launch
         on the host, which is a tenth of the step at short sequences.  The graph is captured on first use for
-        these tensors (and again when a tensor's address changes); results are identical to ``run``.  The library
-        calls only enqueue work on the stream they are given and allocate nothing, which is what makes them
-        capturable; call ``run`` once before (shared-memory limits and tensor maps are set up on first use)."""
+        these tensors (and again when anything that it holds has changed: a tensor's address, strides or type, a buffer or
+        a setting of the engine); results are identical to ``run``.  The library calls only enqueue work on the stream
+        they are given and allocate nothing, which is what makes them capturable; call ``run`` once before
+        (shared-memory limits and tensor maps are set up on first use)."""
         out = self.out if out is None else out
-        key = (q.data_ptr(), k.data_ptr(), v.data_ptr(), proj.data_ptr(), out.data_ptr())
+        key = self._step_key(q, k, v, proj, out)
         if self._graph is None or self._graph[1] != key:
             self.run(q, k, v, proj, out=out)  # first-use set-up happens outside the capture
             torch.cuda.synchronize(self.device)

@@ -118,6 +118,41 @@ def test_calls_behind_event_waits(heads, tokens, crit, neg, captured):
         assert eng.status.item() == 0 and torch.equal(eng.out, want[i % 2]), i
 
 
+@pytest.mark.parametrize("call", ["run", "run_graph"])
+def test_an_engine_changed_between_two_calls(call):
+    """A step works on the buffers, strides, shape and settings of its call, not on those of the call before."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    B, H, N = 2, 4, 256
+    args = [torch.randn((B, N, H, 64), device="cuda", generator=g) for _ in range(3)]
+    proj = torch.randn((H, 64, 64), device="cuda", generator=g) / 8
+    heads_first = [t.view(B, H, N, 64) for t in args]
+
+    def fresh(x, phi="softmax", batch=B):
+        return lt.SlaForward(batch, H, N, 64, 0.25, 0.25, phi=phi).run(*x, proj)
+
+    eng = lt.SlaForward(B, H, N, 64, 0.25, 0.25)
+    step = lambda x: getattr(eng, call)(*x, proj)  # noqa: E731
+    assert torch.equal(step(heads_first), fresh(heads_first))
+    mixed = [args[0].permute(0, 2, 1, 3), *heads_first[1:]]  # the same address with other strides
+    assert torch.equal(step(mixed), fresh(mixed))
+    held = []
+    for obj, name in ((eng.q8, "codes"), (eng.k8, "scales"), (eng.k8, "colsum"), (eng.v8, "codes"), (eng.plan, "cls"),
+                      (eng.plan, "crit_idx"), (eng, "workspace"), (eng, "out")):
+        t = getattr(obj, name)
+        old, new = t.view(t.shape), torch.zeros_like(t)
+        held.append(old)
+        t.set_(new)
+        assert torch.equal(step(heads_first), fresh(heads_first)), name
+        assert torch.count_nonzero(new) > 0, name  # the step wrote to the new storage
+    eng.phi = lt.PHI_ELU1
+    assert torch.equal(step(heads_first), fresh(heads_first, phi="elu1"))
+    eng.phi = lt.PHI_SOFTMAX
+    eng.shape.batch = 1
+    eng.out.fill_(float("nan"))
+    out = step(heads_first)
+    assert torch.equal(out[:1], fresh([t[:1] for t in heads_first], batch=1)) and torch.isnan(out[1:]).all()
+
+
 @pytest.mark.parametrize("blocks", [3, 32, 33, 64, 65])
 def test_plan_rows_around_the_rank_limit(blocks):
     """Rows of up to 64 blocks are ranked by comparing all pairs (one or two entries per lane), longer ones selected
