@@ -102,9 +102,12 @@ struct AttnParams {
   int heads, tokens, nb, tiles_per_head, k_crit, k_marg, phi, out_dtype;
   // output through TMA stores (map_o): position of the token / head / batch dimension among the map's dimensions
   // 1..3 (they are ordered by stride); tma_out = 0: plain stores
-  int wait_first;  // the preceding launch must have completed before anything is read
-  int steal;  // more tiles than CTAs fit on the chip: CTAs take over the tiles of CTAs not yet launched (see launch)
   int tma_out, dim_token, dim_head, dim_batch;
+  // The preceding launch must have completed before anything is read.  0: it is the aggregation, which writes G and zeta
+  // only; codes, scales, v16 and crit_idx come from launches before it and are read ahead of this kernel's wait on the
+  // word of the aggregation's (sm100.cuh, "reading ahead of the own wait").
+  int wait_first;
+  int steal;  // more tiles than CTAs fit on the chip: CTAs take over the tiles of CTAs not yet launched (see launch)
   int* status;
 };
 

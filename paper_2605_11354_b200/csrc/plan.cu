@@ -25,7 +25,9 @@
 //
 // late_wait: the launch before this one in the stream (the summaries) neither writes what this kernel reads nor touches
 // what it writes, and has itself waited for everything that does: the two run side by side, and this kernel waits for the
-// other one's completion only before it ends, so that its own completion stands for both.
+// other one's completion only before it ends, so that its own completion stands for both.  Until that wait it reads the
+// column sums and scales on the word of the summaries' wait (sm100.cuh, "reading ahead of the own wait"): it may
+// not read anything that the launch before it writes.
 #include <atomic>
 
 #include "common.cuh"

@@ -28,8 +28,17 @@ __device__ __forceinline__ bool elect_one() {
 // programmatic-serialization attribute, may start once every CTA of this grid has got here (or exited).
 // wait_for_prior_grid: blocks until the preceding grid has completed and its writes are visible; a no-op in a kernel
 // that was launched the ordinary way.  A kernel lets its successor start only after its own wait and after its TMEM
-// allocation: at most two launches are then ever under way, no buffer is read (and kept in a first-level cache) by a
-// kernel two launches back while it is rewritten, and a successor's allocation never comes before this kernel's.
+// allocation: at most two launches are then under way, no buffer is read (and kept in a first-level cache) by a kernel two
+// launches back while it is rewritten, and a successor's allocation never comes before this kernel's.  The plan behind the
+// summaries is the exception: it signals at once, so that the aggregation is set up beside both of them, and waits before
+// it ends; the aggregation touches nothing before its own wait.  Every kernel waits before it ends, so that a completed
+// grid stands for all before it.
+// Reading ahead of the own wait: the plan (behind the summaries) and the attention kernel (behind the aggregation) read
+// results of the launch before last ahead of their own wait.  They rest on this: the launch in between, B, signals
+// only after B's wait, so when a CTA of C = B's successor starts, the grids before B have completed and their writes
+// have been performed at device scope (B's wait waited for that); C's grid begins after that with empty first-level
+// caches and finds them in L2.  PTX states the visibility for B alone; for C it is assumed here.  It breaks if B signals before
+// it waits, if a kernel before B ends without having waited, or if C reads ahead anything that B writes.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
