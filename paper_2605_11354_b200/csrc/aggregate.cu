@@ -305,6 +305,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed cha
 
   tc_fence_before();
   __syncthreads();
+  linger_after_abort(abort_flag);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);

@@ -824,6 +824,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   tc_fence_before();
   __syncthreads();
+  linger_after_abort(abort_flag);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_p, kColsP);

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const uint8_t* __restrict__ v
 }
 
 // Self-test of the bounded waits: one thread waits on a barrier that nothing ever arrives on.  The wait must give up
-// after limit_ns, write its code to *status and let the kernel end normally.
+// after limit_ns, write its code to *status and let the kernel end normally, the millisecond for copies under way later.
 __global__ void wait_expiry_probe_kernel(int* status, unsigned long long limit_ns) {
   __shared__ uint64_t bar;
   __shared__ int abort_flag;
@@ -53,6 +53,7 @@ __global__ void wait_expiry_probe_kernel(int* status, unsigned long long limit_n
     abort_flag = 0;
     sm100::mbar_fence_init();
     sm100::mbar_wait(&bar, 0, &abort_flag, status, 999, 0, limit_ns);
+    sm100::linger_after_abort(&abort_flag);
   }
 }
 

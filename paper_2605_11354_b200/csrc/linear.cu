@@ -318,7 +318,6 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           }
         }
       }
-      if (kPair && !ok) __nanosleep(1000000);  // copies under way land before the memory is given up
     }
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
@@ -579,6 +578,7 @@ linear_fp8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 
   tc_fence_before();
   __syncthreads();
+  linger_after_abort(abort_flag);
   if constexpr (kPair) cluster_sync();  // neither CTA leaves while the other one's loads, products or arrivals may reach it
   if (warp == 1) {
     tc_fence_after();

@@ -150,6 +150,16 @@ __device__ __forceinline__ bool mbar_wait_clearing(uint64_t* bar, uint32_t parit
   return false;
 }
 
+// Called by all threads of a CTA after the barrier that ends its roles: when a wait has expired, copies and products may still
+// be under way, and their places in shared and tensor memory are not given up until they have had a millisecond to land.
+// (The role that waits for the prior grid may have left its loop before that wait.)
+__device__ __forceinline__ void linger_after_abort(const volatile int* abort_flag) {
+  if (*abort_flag == 0) return;
+  wait_for_prior_grid();
+  const uint64_t since = global_timer_ns();
+  while (global_timer_ns() - since < 1000000ull) __nanosleep(1000);
+}
+
 // ------------------------------------------------------------------------------------------------ shared memory
 // 16 bytes by 32-bit shared-memory address.
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {

@@ -418,6 +418,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
 
   tc_fence_before();
   __syncthreads();
+  linger_after_abort(abort_flag);
   if (warp == 4) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);

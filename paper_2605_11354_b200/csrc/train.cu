@@ -221,6 +221,7 @@ projgrad_kernel(const __grid_constant__ CUtensorMap map_o, const __grid_constant
   }
   tc_fence_before();
   __syncthreads();
+  linger_after_abort(abort_flag);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);

@@ -380,6 +380,20 @@ def test_device_waits_are_bounded():
     full_parity(wl, wk.make_inputs(wl))
 
 
+def test_an_expired_wait_leaves_time_for_copies_under_way():
+    """After a wait has given up, the kernel keeps its memory for another millisecond (copies may still be landing)."""
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    lt.selftest_wait_expiry(status, 1000)
+    torch.cuda.synchronize()
+    t0.record()
+    lt.selftest_wait_expiry(status, 1000)  # 1 us
+    t1.record()
+    torch.cuda.synchronize()
+    assert int(status.item()) == 999
+    assert t0.elapsed_time(t1) >= 0.95
+
+
 # ------------------------------------------------------------------------------------------------ boundary options
 def bf16_round(x: np.ndarray) -> np.ndarray:
     return wk.round_to_bf16(x.astype(np.float32)).astype(np.float64)
