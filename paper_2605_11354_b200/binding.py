@@ -16,6 +16,7 @@ _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "liblite3r.
 _lib = None
 
 F32, BF16, F16 = 0, 1, 2
+SOURCE_DTYPES = {torch.float32: F32, torch.bfloat16: BF16}
 OUT_DTYPES = {torch.float32: F32, torch.bfloat16: BF16, torch.float16: F16}
 PHI_SOFTMAX, PHI_ELU1 = 0, 1
 PHI_CODES = {"softmax": PHI_SOFTMAX, "elu1": PHI_ELU1}
@@ -233,10 +234,15 @@ class Fp8Tensor:
     codes: torch.Tensor  # uint8 [B,H,Nb*Bs,D]
     scales: torch.Tensor  # fp32 [B,H,Nb]
     colsum: torch.Tensor | None  # int32 [B,H,Nb,D]; None: the quantiser skips the column sums (only Q and K need them)
+    _struct = None, None  # (what the C struct was made from, the struct)
 
     def c_struct(self) -> Fp8:
-        return Fp8(self.codes.data_ptr(), self.scales.data_ptr(),
-                   self.colsum.data_ptr() if self.colsum is not None else None)
+        """The C struct of the buffers as they are now; made anew only when one of their addresses has changed."""
+        colsum = self.colsum
+        key = self.codes.data_ptr(), self.scales.data_ptr(), None if colsum is None else colsum.data_ptr()
+        if self._struct[0] != key:
+            self._struct = key, Fp8(*key)
+        return self._struct[1]
 
 
 @dataclass
@@ -247,10 +253,15 @@ class PlanBuffers:
     k_crit: int
     k_marg: int
     k_neg: int
+    _struct = None, None
 
     def c_struct(self) -> Plan:
-        return Plan(self.cls.data_ptr(), self.crit_idx.data_ptr() if self.k_crit else None,
-                    self.marg_idx.data_ptr() if self.k_marg else None, self.k_crit, self.k_marg, self.k_neg)
+        """As Fp8Tensor.c_struct, for the addresses and the counts."""
+        key = (self.cls.data_ptr(), self.crit_idx.data_ptr() if self.k_crit else None,
+               self.marg_idx.data_ptr() if self.k_marg else None, self.k_crit, self.k_marg, self.k_neg)
+        if self._struct[0] != key:
+            self._struct = key, Plan(*key)
+        return self._struct[1]
 
 
 def alloc_fp8(shape: Shape, device, colsum: bool = True) -> Fp8Tensor:
@@ -275,18 +286,17 @@ def lite3r_quantize_fp8(x: torch.Tensor, shape: Shape, out: Fp8Tensor, stream=No
     """x: CUDA tensor [B,H,N,D] (any b/h/n strides, contiguous D), fp32 or bf16."""
     if not x.is_cuda or x.dim() != 4 or x.stride(3) != 1:
         raise Lite3rError("lite3r_quantize_fp8: x must be a CUDA tensor [B,H,N,D] with contiguous D")
-    dtype = {torch.float32: F32, torch.bfloat16: BF16}.get(x.dtype)
+    dtype = SOURCE_DTYPES.get(x.dtype)
     if dtype is None:
         raise Lite3rError("lite3r_quantize_fp8: dtype must be float32 or bfloat16")
     t = Tensor(x.data_ptr(), dtype, x.stride(0), x.stride(1), x.stride(2))
-    _check(lib().lite3r_quantize_fp8(C.byref(t), C.byref(shape), out.c_struct(), _stream_ptr(stream)),
-           "lite3r_quantize_fp8")
+    _check(lib().lite3r_quantize_fp8(t, shape, out.c_struct(), _stream_ptr(stream)), "lite3r_quantize_fp8")
 
 
 def _source(x: torch.Tensor, what: str) -> Tensor:
     if not x.is_cuda or x.dim() != 4 or x.stride(3) != 1:
         raise Lite3rError(f"{what}: sources must be CUDA tensors [B,H,N,D] with contiguous D")
-    dtype = {torch.float32: F32, torch.bfloat16: BF16}.get(x.dtype)
+    dtype = SOURCE_DTYPES.get(x.dtype)
     if dtype is None:
         raise Lite3rError(f"{what}: dtype must be float32 or bfloat16")
     return Tensor(x.data_ptr(), dtype, x.stride(0), x.stride(1), x.stride(2))
@@ -296,18 +306,20 @@ def lite3r_quantize_fp8_qkv(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, s
                             k_out: Fp8Tensor, v_out: Fp8Tensor, stream=None) -> None:
     """Q, K and V of one attention call quantised by a single launch (same results as three single calls)."""
     tq, tk, tv = (_source(x, "lite3r_quantize_fp8_qkv") for x in (q, k, v))
-    _check(lib().lite3r_quantize_fp8_qkv(C.byref(tq), C.byref(tk), C.byref(tv), C.byref(shape), q_out.c_struct(),
-                                         k_out.c_struct(), v_out.c_struct(), _stream_ptr(stream)),
-           "lite3r_quantize_fp8_qkv")
+    _check(lib().lite3r_quantize_fp8_qkv(tq, tk, tv, shape, q_out.c_struct(), k_out.c_struct(), v_out.c_struct(),
+                                         _stream_ptr(stream)), "lite3r_quantize_fp8_qkv")
 
 
 def lite3r_sla_plan(q: Fp8Tensor, k: Fp8Tensor, shape: Shape, crit: float, neg: float, plan: PlanBuffers,
                     stream=None) -> None:
     p = plan.c_struct()
     qs, ks = q.c_struct(), k.c_struct()
-    _check(lib().lite3r_sla_plan(C.byref(qs), C.byref(ks), C.byref(shape), crit, neg, C.byref(p),
-                                 _stream_ptr(stream)), "lite3r_sla_plan")
-    assert (p.k_crit, p.k_marg, p.k_neg) == (plan.k_crit, plan.k_marg, plan.k_neg)
+    status = lib().lite3r_sla_plan(qs, ks, shape, crit, neg, p, _stream_ptr(stream))
+    same_counts = (p.k_crit, p.k_marg, p.k_neg) == (plan.k_crit, plan.k_marg, plan.k_neg)
+    if not same_counts:
+        plan._struct = None, None  # the library has written its own into it
+    _check(status, "lite3r_sla_plan")
+    assert same_counts
 
 
 def _check_out(out: torch.Tensor, what: str) -> int:
@@ -327,10 +339,9 @@ def lite3r_sla_forward(q: Fp8Tensor, k: Fp8Tensor, v: Fp8Tensor, proj: torch.Ten
     head_stride = proj.stride(0) if proj.dim() == 3 else 0
     p = plan.c_struct() if plan is not None else None
     qs, ks, vs = q.c_struct(), k.c_struct(), v.c_struct()
-    _check(lib().lite3r_sla_forward(C.byref(qs), C.byref(ks), C.byref(vs), proj.data_ptr(), head_stride,
-                                    C.byref(shape), crit, neg, phi, C.byref(p) if p is not None else None,
-                                    out.data_ptr(), out_dtype, out.stride(0), out.stride(1),
-                                    out.stride(2), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
+    _check(lib().lite3r_sla_forward(qs, ks, vs, proj.data_ptr(), head_stride, shape, crit, neg, phi, p, out.data_ptr(),
+                                    out_dtype, out.stride(0), out.stride(1), out.stride(2), workspace.data_ptr(),
+                                    workspace.numel() * workspace.element_size(),
                                     device_status.data_ptr() if device_status is not None else None,
                                     _stream_ptr(stream)), "lite3r_sla_forward")
 
@@ -342,7 +353,7 @@ def lite3r_sla_forward_begin(k: Fp8Tensor, v: Fp8Tensor, proj: torch.Tensor, sha
         raise Lite3rError("lite3r_sla_forward_begin: proj must be a contiguous CUDA float32 tensor")
     head_stride = proj.stride(0) if proj.dim() == 3 else 0
     ks, vs = k.c_struct(), v.c_struct()
-    _check(lib().lite3r_sla_forward_begin(C.byref(ks), C.byref(vs), proj.data_ptr(), head_stride, C.byref(shape), phi,
+    _check(lib().lite3r_sla_forward_begin(ks, vs, proj.data_ptr(), head_stride, shape, phi,
                                           plan.k_crit, plan.k_marg, plan.k_neg, workspace.data_ptr(),
                                           workspace.numel() * workspace.element_size(),
                                           device_status.data_ptr() if device_status is not None else None,
@@ -355,7 +366,7 @@ def lite3r_sla_forward_finish(q: Fp8Tensor, k: Fp8Tensor, v: Fp8Tensor, shape: S
     out_dtype = _check_out(out, "lite3r_sla_forward_finish")
     p = plan.c_struct()
     qs, ks, vs = q.c_struct(), k.c_struct(), v.c_struct()
-    _check(lib().lite3r_sla_forward_finish(C.byref(qs), C.byref(ks), C.byref(vs), C.byref(shape), phi, C.byref(p),
+    _check(lib().lite3r_sla_forward_finish(qs, ks, vs, shape, phi, p,
                                            out.data_ptr(), out_dtype, out.stride(0), out.stride(1), out.stride(2),
                                            workspace.data_ptr(), workspace.numel() * workspace.element_size(),
                                            device_status.data_ptr() if device_status is not None else None,
@@ -377,7 +388,7 @@ def lite3r_sla_forward_static_scratch(q: Fp8Tensor, k: Fp8Tensor, v: Fp8Tensor, 
     p = plan.c_struct()
     qs, ks, vs = q.c_struct(), k.c_struct(), v.c_struct()
     _check(lib().lite3r_sla_forward_static_scratch(
-        C.byref(qs), C.byref(ks), C.byref(vs), proj.data_ptr(), head_stride, C.byref(shape), phi, C.byref(p),
+        qs, ks, vs, proj.data_ptr(), head_stride, shape, phi, p,
         out.data_ptr(), out_dtype, out.stride(0), out.stride(1), out.stride(2),
         device_status.data_ptr() if device_status is not None else None, _stream_ptr(stream)),
         "lite3r_sla_forward_static_scratch")
@@ -389,7 +400,7 @@ def lite3r_quantize_rows_fp8(x: torch.Tensor, stream=None):
     per token for activations, per output row for weights.  Returns (codes uint8 [rows, cols], scales fp32 [rows])."""
     if not x.is_cuda or x.dim() != 2 or x.stride(1) != 1:
         raise Lite3rError("lite3r_quantize_rows_fp8: x must be a CUDA matrix with contiguous columns")
-    dtype = {torch.float32: F32, torch.bfloat16: BF16}.get(x.dtype)
+    dtype = SOURCE_DTYPES.get(x.dtype)
     if dtype is None:
         raise Lite3rError("lite3r_quantize_rows_fp8: dtype must be float32 or bfloat16")
     codes = torch.empty(x.shape, dtype=torch.uint8, device=x.device)
@@ -417,7 +428,7 @@ def lite3r_qkv_project_fp8(x_codes, x_scales, w_codes, w_scales, bias, shape: Sh
     """qkv projection on e4m3 operands with the block quantiser fused into its epilogue: fills the three Fp8Tensors
     the attention calls take.  x_codes [B*N, d_model], w_codes [3*H*64, d_model] ordered (q | k | v) x head x 64."""
     _check(lib().lite3r_qkv_project_fp8(x_codes.data_ptr(), x_scales.data_ptr(), w_codes.data_ptr(), w_scales.data_ptr(),
-                                        bias.data_ptr() if bias is not None else None, C.byref(shape),
+                                        bias.data_ptr() if bias is not None else None, shape,
                                         x_codes.shape[1], q_out.c_struct(), k_out.c_struct(), v_out.c_struct(),
                                         device_status.data_ptr() if device_status is not None else None,
                                         _stream_ptr(stream)), "lite3r_qkv_project_fp8")
@@ -436,7 +447,7 @@ def lite3r_sla_linear_branch(q: Fp8Tensor, k: Fp8Tensor, v: Fp8Tensor, shape: Sh
     out_dtype = _check_out(out, "lite3r_sla_linear_branch")
     p = plan.c_struct()
     qs, ks, vs = q.c_struct(), k.c_struct(), v.c_struct()
-    _check(lib().lite3r_sla_linear_branch(C.byref(qs), C.byref(ks), C.byref(vs), C.byref(shape), phi, C.byref(p),
+    _check(lib().lite3r_sla_linear_branch(qs, ks, vs, shape, phi, p,
                                           out.data_ptr(), out_dtype, out.stride(0), out.stride(1), out.stride(2),
                                           workspace.data_ptr(), workspace.numel() * workspace.element_size(),
                                           device_status.data_ptr() if device_status is not None else None,
@@ -462,7 +473,7 @@ def lite3r_proj_lin_backward(o_lin: torch.Tensor, d_out: torch.Tensor, shape: Sh
     for t in (o_lin, d_out):
         if t.dtype != torch.bfloat16 or not t.is_contiguous():
             raise Lite3rError("lite3r_proj_lin_backward: o_lin and d_out must be contiguous bfloat16")
-    _check(lib().lite3r_proj_lin_backward(o_lin.data_ptr(), d_out.data_ptr(), C.byref(shape), d_proj.data_ptr(),
+    _check(lib().lite3r_proj_lin_backward(o_lin.data_ptr(), d_out.data_ptr(), shape, d_proj.data_ptr(),
                                           workspace.data_ptr(), workspace.numel() * workspace.element_size(),
                                           device_status.data_ptr() if device_status is not None else None,
                                           _stream_ptr(stream)), "lite3r_proj_lin_backward")

@@ -28,6 +28,24 @@ def test_structs_of_buffers_given_other_storage():
             assert getattr(obj.c_struct(), name) == new.data_ptr(), name
 
 
+def test_counts_that_the_library_writes_are_not_kept(monkeypatch):
+    """lite3r_sla_plan writes the counts of its fractions into the struct it is given; a plan made for others stays as it is."""
+    shape = lt.Shape(1, 2, 300, 64, 64)
+    x, plan = lt.alloc_fp8(shape, "cpu"), lt.alloc_plan(shape, 0.25, 0.25, "cpu")
+
+    class Lib:
+        @staticmethod
+        def lite3r_sla_plan(q, k, s, crit, neg, p, stream):
+            p.k_crit += 1
+            return 0
+
+    monkeypatch.setattr(lt, "_lib", Lib)
+    monkeypatch.setattr(lt, "_stream_ptr", lambda stream: 0)
+    with pytest.raises(AssertionError):
+        lt.lite3r_sla_plan(x, x, shape, 0.5, 0.25, plan)
+    assert plan.c_struct().k_crit == plan.k_crit
+
+
 CHANGES = {
     "shape": lambda e: setattr(e.shape, "heads", 1), "crit": lambda e: setattr(e, "crit", 0.5),
     "neg": lambda e: setattr(e, "neg", 0.1), "phi": lambda e: setattr(e, "phi", lt.PHI_ELU1),
