@@ -34,7 +34,7 @@ FP8_OVER_BF16 = 2.0  # nominal dense ratio (4.5 vs 2.25 PFLOP/s)
 # DRAM bytes (read + write) of one launch, keyed by (workload, kernel), from the ncu captures summarised under
 # profiles/; a kernel that changed since its capture has no entry.
 DRAM_BYTES_PER_LAUNCH = {
-    ("vggt8", "attention"): 84932608,
+    ("vggt8", "attention"): 83684864,
     ("vggt8", "plan"): 1494528,
     ("vggt8", "quantize_qkv"): 72801792,
     ("vggt8", "summary"): 23731968,
