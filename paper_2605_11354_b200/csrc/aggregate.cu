@@ -9,8 +9,8 @@
 // and keys are numbered through all (b, h).  Tiles either stay inside one (b, h), or, for short sequences, run through
 // the (b, h) boundaries so that several small problems share a tile (the mask is then block-diagonal); the launcher
 // takes the cheaper tiling.  Per chunk: TMA brings the 64 x 256 slab of summaries (MN-major B operand, four 64-column
-// boxes, 128B swizzle); 128 threads expand the class bytes of their row (fetched a chunk ahead) into the bf16 0/1 A
-// tile (K-major, 128B swizzle) with byte permutes; one thread issues four 128x256x16 MMAs.  Epilogue: the same 128
+// boxes, 128B swizzle); 128 threads expand the class bytes of their row, or sixteen lanes those of a row together
+// (fetched a chunk ahead), into the bf16 0/1 A tile (K-major, 128B swizzle) with byte permutes; one thread issues four 128x256x16 MMAs.  Epilogue: the same 128
 // threads read their accumulator row from TMEM, turn the rows around in shared memory so that stores write whole
 // 128-byte segments, and store the first 4096 columns as bf16 (the attention kernel's B operand) and the last 64
 // (zeta) as fp32.
@@ -325,8 +325,10 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   const int total_rows = static_cast<int>(rows), bh = s.batch * s.heads;
   // Tiles through the (b, h) boundaries pay with a longer reduction (the keys of every (b, h) a tile touches), tiles
   // inside one (b, h) with padding when Nb is not a multiple of 128.  Estimate of either: waves of CTAs (two per SM)
-  // times the cost of a CTA, its set-up and drain counted as three 64-key chunks (at Nb = 172 the two tilings are
-  // measured on a par at about that ratio).
+  // times the cost of a CTA, its set-up and drain counted as three 64-key chunks.  Measured, inside / flat in us: 16 (b, h)
+  // of 129 blocks 19.5 / 17.4, of 172 19.5 / 23.6, of 687 91 / 107; 64 of 64 blocks 23.6 / 19.5, of 86 29.7 / 31.7, of 172
+  // 60.4 / 56.3, of 200 66.6 / 70.7; 512 of 22 blocks 128 / 48, of 64 140 / 106, of 86 179 / 175, of 100 187 / 214.  Of 46
+  // such pairs (2 to 512 (b, h), 5 to 2147 blocks) the estimate misses the faster one twice, by 2 and 4 us.
   int sms = 0;
   if ((st = sm_count(&sms)) != LITE3R_OK) return st;
   constexpr double kFixed = 3.0;

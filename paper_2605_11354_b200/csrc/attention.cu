@@ -11,13 +11,15 @@
 //            to TMEM as packed fp16 (P, 32 columns)
 //   tcgen05  O += P V              kind::f16 with the A operand read from TMEM, V as MN-major B operand from shared
 //                                  memory, one fp32 accumulator in TMEM (64 columns), under the exponentials of step t+1
-// so the softmax warps never wait for a product in the steady state.  The exponential unit is the bound (16 per clock
-// and SM: 512 clocks per step); the products of a step take 384 clocks of tensor pipe at block 64 (M = 64 runs at half
-// rate) and 192 at block 128.  A warp alone needs some 1100 clocks for its 32 x 64 scores (loads, stores and barriers
-// included), so two warps per scheduler are the least that can keep the unit busy and three do it comfortably: S, P and O
-// take 160 TMEM columns, 74 KB of shared memory and 80 registers per thread, and
-// THREE CTAs fit on an SM.  Measured at 10 % of 2147 key blocks: 650 clocks per step and SM (two CTAs with two softmax
-// warpgroups each on alternate steps of one tile, as before: 757).
+// so the softmax warps never wait for a product in the steady state.  The largest unit is the exponential one: 16 per clock
+// and SM, 448 clocks per step with an eighth of the exponentials on the multiply-add pipe; the products of a step take 384
+// clocks of tensor pipe at block 64 (M = 64 runs at half rate) and 192 at block 128.  A warp alone needs some 1100 clocks
+// for its 32 x 64 scores (loads, stores and barriers included), so two warps per scheduler are the least that can keep
+// the unit busy: S, P and O take 160 TMEM columns, 74 KB of shared memory and 80 registers per thread, and THREE CTAs fit
+// on an SM.  Measured at 10 % of 2147 key blocks: 654 clocks per step and SM by the cycle counter (two CTAs with two
+// softmax warpgroups each on alternate steps of one tile, as before: 757).  No unit is saturated (at 5 % of 687 blocks:
+// exponentials 64 %, issue slots 60 %, tensor pipe 54 %): a warp takes maximum, vote and exponentials of a step one after
+// the other, and three warps per scheduler do not fill each other's gaps.
 // A CTA takes tile after tile: it asks the hardware's work scheduler for a CTA that has not been launched yet and computes
 // that one's tile itself (taken only where the grid is larger than the chip holds and a tile has products).  The next tile's Q, K and V tiles and
 // its first scores are then under way while the softmax warps write this tile's output, and what lies between two tiles

@@ -8,7 +8,7 @@
 // GEMM kernel: persistent CTAs (one per SM) over 128 x 256 output tiles (128 tokens x 256 output columns = four heads
 // of the projection), or pairs of CTAs over tiles of 256 x 256 (cta_group::2 products that read half of the weights from
 // either CTA).  The operand bytes from L2 bound the product: 43968 x 1024 x 1024 took 54.5 us by single CTAs and takes 50 us
-// by pairs, with the tensor pipe busy for 45% of it.  Warp 0 = TMA producer (A = activation codes, B = weight codes, both
+// by pairs, with the tensor pipe busy for 46 % of it (in a long run of whole layers, under the power cap at 1.69 GHz, 51 us).  Warp 0 = TMA producer (A = activation codes, B = weight codes, both
 // K-major rows of 128 bytes, 128B swizzle, ring of three or four stages), warp 1 = MMA issuer (four kind::f8f6f4 products
 // of K = 32 per stage into one of two accumulators), warps 4-19 = four epilogue warpgroups, one per 64 columns of the tile
 // (thread = token row = TMEM lane; two passes over the accumulator so that a row of 64 values never has to stay in
@@ -95,8 +95,9 @@ struct RowScale {
 // One warp per row.  Rows of up to 256 kSegs values stay in registers as they lie in memory (all requested before the
 // first is used), and bf16 rows of that length are requested one row ahead, so that a warp's loads run under the
 // arithmetic of the row before; longer rows are read twice (maximum, then codes; the second read comes from L1 / L2).
-// Bound by HBM: 43968 x 1024 bf16 values in 18.7 us (135 MB, part of them from L2; 21.5 us with two corrections per
-// quotient, 31 us while a third of the groups of 256 values went through a division).
+// Bound by HBM: 43968 x 1024 bf16 values (135 MB) in 18.7 us with the input partly in L2 (21.5 us with two corrections per
+// quotient, 31 us while a third of the groups of 256 values went through a division), 29 us after L2 has been flushed, and
+// 32 us, 4.2 TB/s, in a run of layers whose GEMM leaves its 90 MB result in L2.
 template <typename SrcT, int kSegs>
 __global__ void __launch_bounds__(256) rowquant_kernel(const SrcT* __restrict__ x, long long row_stride, int rows, int cols,
                                                        uint8_t* __restrict__ codes, float* __restrict__ scales) {
