@@ -7,8 +7,9 @@
 // roundings separate t_ij from the exact value; the ranking is therefore the exact one except between
 // scores that agree to ~1e-15 relative.  Ranking order: score descending, then key-block index ascending.
 //
-// One CTA of R warps handles R consecutive query blocks (rows) of one (b, h); R = 8 unless the row keys of a very
-// long sequence do not fit in shared memory.
+// plan_kernel (rows of up to 80 blocks, and those too long for plan_compact_kernel): one CTA of R warps handles R
+// consecutive query blocks (rows) of one (b, h); R = 8 unless the row keys of a very long sequence do not fit in shared
+// memory.
 //   Phase A (whole CTA): the scores of the R rows against all key blocks, kept in shared memory as order-preserving
 //     64-bit keys.  R = 8: fp64 tensor-core products (m8n8k4) fed with the int32 column sums straight from global
 //     memory, no staging and no barrier.  R < 8: 64 key blocks at a time staged in shared memory as doubles; a lane
@@ -29,6 +30,7 @@
 // column sums and scales on the word of the summaries' wait (sm100.cuh, "reading ahead of the own wait"): it may
 // not read anything that the launch before it writes.
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -590,495 +592,679 @@ __device__ __forceinline__ void split_pair(int v0, int v1, uint32_t& hi, uint32_
   hi = *reinterpret_cast<const uint32_t*>(&h);
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
-__device__ __forceinline__ void mma_m16n8k16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+__device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
+__device__ __forceinline__ uint32_t as_word(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
+// Two neighbouring column sums times `mult` (together below 449 * 2^16) as fp16 pairs hi + mid in units of 2^16: hi the
+// nearest integer, mid the next eight bits, what is left out at most 2^-9.  Integer bits are put under the exponent of a
+// power of two (1024 + n is exact in fp16 for n < 1024) and the offset is taken off again: no conversion instruction.
+__device__ __forceinline__ void digits_pair(int v0, int v1, int mult, uint32_t& hi, uint32_t& mid) {
+  constexpr uint32_t kBias = (0x6600u << 16) + 0x8080u;  // 1536.0 over the upper half; 128.5 steps of mid
+  const uint32_t w0 = static_cast<uint32_t>(v0 * mult) + kBias, w1 = static_cast<uint32_t>(v1 * mult) + kBias;
+  const uint32_t m = (__byte_perm(w0, w1, 0x5511) & 0x00FF00FFu) | 0x64006400u;  // 1024 + (0..255)
+  hi = as_word(__hadd2(as_half2(__byte_perm(w0, w1, 0x7632)), as_half2(0xE600E600u)));          // - 1536
+  mid = as_word(__hfma2(as_half2(m), as_half2(0x1C001C00u), as_half2(0xC480C480u)));            // / 256 - 4.5
+}
+__device__ __forceinline__ void mma_m16n8k16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+               : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
-// The same plan with the scores kept in shared memory as single-precision values (4 bytes per key instead of an
-// 8-byte ordered key): sixteen rows per CTA then fit where eight did, so the column sums of a (b, h) are streamed half as
-// often and twice as many warps hide the latencies of the selection and of the class pass.
-// The ranking stays the exact one.  The single-precision score only gives a key its place on a 16-bit scale between the
-// row's extremes; the few keys near a selection threshold are decided by their exact 64-bit keys, which are recomputed for
-// them from the integer column sums (an int64 dot product, equal to the fp64 tensor-core value as long as that is exact,
-// i.e. below 2^53).
-//   R = 8: the scores are the exact ones (fp64 tensor products), rounded to fp32: near means in the threshold's own place.
-//   R = 16: the scores are approximations from fp16 tensor products of a two-way split of the column sums (hi hi + hi lo
-//     + lo hi, fp32 accumulation), twelve products for 16 x 8 scores where fp64 takes thirty-two of its far slower
-//     ones.  An approximation is off by at most
-//       delta = max_j scale^K_j (224 (2^-17 S + 2^-19) + 2^-25 S),  S = sum_d |colsum^Q_d| 2^-10
-//     (a column sum over its valid tokens is at most 448 in value, so |colsum^K_d| 2^-10 / valid <= 224; the split leaves
-//     out 3 2^-22 of a product and twelve accumulations lose 2^-22 of the sum of magnitudes each, together below 2^-18,
-//     doubled for safety; the last two terms are fp16's smallest step), so near means within 2 delta of the threshold's
-//     place: an entry further above it is certainly selected, one further below certainly not.
-//     16 heads, 2147 blocks: 1210 -> 1005 us with it and the cheaper selections below.
-// Warp w of the R = 8 or 16 warps: in phase A all its rows against every R-th group of eight key blocks; in phases B and
-// C row w.
+// Places: what a score becomes in shared memory, two bytes instead of an eight-byte key.  The row's scores lie within
+// +-448 S max_j scale^K_j with S = sum_d |colsum^Q_d| 2^-10; this interval is mapped linearly to the integers
+// kPlaceLow .. kPlaceHigh.  All of them are bit patterns of normal, finite fp16 numbers, which are ordered like the
+// integers, so one instruction compares two of them; an entry past the row's end holds a NaN, which fails every comparison.
+constexpr int kPlaceMid = 16024, kPlaceSpan = 14990, kPlaceLow = 1024, kPlaceHigh = 31030;
+constexpr int kNever = 0x7C00, kTopPlace = 0x7BFF;  // above every place; place of an entry found to be critical
+constexpr int kListed = 64;                         // entries of a threshold range that are decided from a list
+constexpr int kFewListed = 14;                      // with more than this in its bucket the range is narrowed first
+
+// Pitch of a row of places: 16-byte aligned, and eight rows on different banks for 4-byte accesses (an odd multiple of 16
+// bytes).
+__host__ __device__ constexpr int place_pitch(int nb) { return (((nb + 7) >> 3) | 1) << 3; }
+
+// Bits 0..7: which of the eight halves of four mask words (0xFFFF or 0 each) are set.
+__device__ __forceinline__ uint32_t mask_bits(uint32_t m0, uint32_t m1, uint32_t m2, uint32_t m3) {
+  const uint32_t x = (m0 & 0x00020001u) | (m1 & 0x00080004u) | (m2 & 0x00200010u) | (m3 & 0x00800040u);
+  return (x | (x >> 16)) & 0xFFu;
+}
+
+// Without a branch: counts one in shared memory where flag holds; *dst++ = v where flag != 0.
+__device__ __forceinline__ void count_if(uint32_t counter, bool flag) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p red.shared.add.u32 [%0], 1;\n\t}" ::"r"(counter), "r"(flag ? 1u : 0u) : "memory");
+}
+__device__ __forceinline__ void append_if(int*& dst, int v, uint32_t flag) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.global.u32 [%0], %1;\n\t@p add.s64 %0, %0, 4;\n\t}"
+               : "+l"(dst) : "r"(v), "r"(flag) : "memory");
+}
+
+// The same plan for rows of more than kRankMax blocks: approximate scores as 16-bit places in shared memory, exact keys
+// only for the few entries that the approximation leaves undecided at a selection threshold.
+//   Phase A (whole CTA, R = 16 or 8 rows): fp16 tensor products (m16n8k16) of the query sums split in two (hi + lo, 22 bits)
+//     and the key sums' upper 18 bits as two digits (hi + mid): hi hi + hi mid + lo hi.  A key block of `valid` tokens
+//     has |colsum| <= 448 512 valid, so colsum * mult with mult = floor(128 / valid) fills the digits' range in short
+//     last blocks too.  What is left out, per unit of S (khat up to 448): the key digits' rest 2^-9, lo mid 2^-12,
+//     the query's rest 448 2^-22, twelve fp32 accumulations 12 * 448 * 2^-22, the scalings 448 3 2^-24: together below
+//     0.004, and at most twice that in a last block whose sums reach only half the range.  In places: 0.004 *
+//     14990 / 448 = 0.14 (0.27), plus 0.5 for the rounding to an integer.  Places of two entries that differ by two or
+//     more are therefore in the order of the exact scores, and the k-th largest place is within 0.77 of that of the
+//     k-th largest score: an entry two places above the k-th largest place is selected, one two below is not, and only
+//     those within one place (`margin`) need their exact 64-bit keys, recomputed from the integer column sums (an
+//     int64 dot product, equal to the fp64 tensor-core value as long as that is exact, i.e. below 2^53).
+//     Rows without such an interval (all sums zero, a scale that is not finite) leave everything undecided.
+//   Phase B (one warp per row): the bucket of a 256-bucket histogram between the row's extremes that holds the k-th
+//     largest place; when it is too full, a second histogram inside that bucket, one counter per place; then the entries of
+//     the bucket and a margin on both sides as a list (up to kListed, in any order), ranked by comparing all pairs, first
+//     by place, then, inside the margin, by exact key and index.  Longer lists (ties, rows without places) go to the radix
+//     select, which recomputes keys pass by pass.  What was decided is written back over the places, so that the class of
+//     every entry is a comparison with two thresholds.
+//   Phase C (same warp): eight entries per lane and turn: class bytes (stored as aligned 8-byte words, shifted over from the
+//     neighbouring lane where the row's address is not a multiple of eight) and the ascending lists, whose positions
+//     come from one warp scan of the lanes' counts.
+// Bound by instruction issue: 9.0 k instructions per row of 2147 blocks, half of the issue slots or more taken.  Single-precision
+// scores read four bytes at a time, with ballots for every 32 entries, took 17 k and, at four bytes an entry, room for one
+// CTA per SM instead of two: 16 heads of 2147 blocks 1005 -> 460 us, of 687 blocks (with 64-bit keys before) 108 -> 61 us.
 template <int R>
-__global__ void __launch_bounds__(R * 32) plan_compact_kernel(const int* __restrict__ q_colsum, const int* __restrict__ k_colsum,
-                                                               const float* __restrict__ k_scales, int tokens, int block,
-                                                               int nb, int k_crit, int k_marg, int k_neg, int late_wait,
-                                                               signed char* __restrict__ cls, int* __restrict__ crit_idx,
-                                                               int* __restrict__ marg_idx) {
-  constexpr bool kApprox = R == 16;
+__global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int* __restrict__ q_colsum, const int* __restrict__ k_colsum,
+                                                                       const float* __restrict__ k_scales, int tokens, int block,
+                                                                       int nb, int k_crit, int k_marg, int k_neg, int late_wait, int mult_last, float factor_last,
+                                                                       signed char* __restrict__ cls, int* __restrict__ crit_idx,
+                                                                       int* __restrict__ marg_idx) {
+  static_assert(R == 8 || R == 16, "rows of one tensor product");
+  static_assert(kBuckets * 4 >= 2 * kListed * 8 && R * kBuckets * 4 >= 4096, "undecided entries and query operands take the histograms' place");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int pitch = (nb + 3) & ~3;
-  float* s_val = reinterpret_cast<float*>(smem_raw);                                              // [R][pitch]
-  unsigned int* s_hist = reinterpret_cast<unsigned int*>(s_val + static_cast<size_t>(R) * pitch);  // [R][256]
-  unsigned long long* s_ckey = reinterpret_cast<unsigned long long*>(s_hist + R * kBuckets);       // [R][2][kMaxListed]
-  int* s_q = reinterpret_cast<int*>(s_ckey + R * 2 * kMaxListed);                                  // [R][64]
-  float2* s_range = reinterpret_cast<float2*>(s_q + R * kHeadDim);                                 // [R][R]
-  unsigned short* s_idx = reinterpret_cast<unsigned short*>(s_range + R * R);                      // [R][2][kMaxListed]
-  __shared__ float s_kmax[R];
+  const int pitch = place_pitch(nb);
+  unsigned short* s_place = reinterpret_cast<unsigned short*>(smem_raw);                              // [R][pitch]
+  unsigned int* s_hist = reinterpret_cast<unsigned int*>(s_place + static_cast<size_t>(R) * pitch);   // [R][kBuckets]
+  uint4* s_a = reinterpret_cast<uint4*>(s_hist);  // [2][4][32] query operands (hi, lo) of phase A, ahead of the histograms
+  unsigned int* s_list = s_hist + R * kBuckets;                                                          // [R][2][kListed]
+  int* s_q = reinterpret_cast<int*>(s_list + R * 2 * kListed);                                        // [R][64]
+  unsigned int* s_range = reinterpret_cast<unsigned int*>(s_q + R * kHeadDim);                        // [R][R] lowest | highest << 16
+  __shared__ float s_sum[R];
+  __shared__ unsigned s_kmax[R];
 
   const int row_tiles = (nb + R - 1) / R;
   const int bh = blockIdx.x / row_tiles;
   const int i0 = (blockIdx.x % row_tiles) * R;
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);  // (known to be the same in all lanes)
   const int lane = threadIdx.x & 31;
   const size_t bh_rows = static_cast<size_t>(bh) * nb;
-  const bool block_pow2 = (block & (block - 1)) == 0;
-  const double inv_block = 1.0 / static_cast<double>(block);
-
-  // the ranking score from an exact dot product (same expression in phase A and for the recomputed keys)
-  auto ranking_score = [&](double dot, float ks, int j) {
-    const int valid = min(block, tokens - j * block);
-    const double num = dot * static_cast<double>(ks);
-    return ((valid == block && block_pow2) ? num * inv_block : num / static_cast<double>(valid)) + 0.0;
-  };
+  const int g = lane >> 2, t4 = lane & 3;
 
   if (!late_wait) sm100::wait_for_prior_grid();
   sm100::launch_dependents();
-  if constexpr (kApprox) {
-    // Phase A, 16 rows x 8 key blocks per warp and step (m16n8k16).  As below, lane (g, t) supplies columns 16 t ..
-    // 16 t + 15 of its rows (rows g and g + 8 for A, key block g of the eight for B), which is one and the same
-    // assignment of columns to k indices on both sides.
-    const int g = lane >> 2, t4 = lane & 3;
-    auto load16 = [&](const int* base, int local, int4 dst[4]) {
-      const int4* src = reinterpret_cast<const int4*>(base + (bh_rows + min(local, nb - 1)) * kHeadDim + 16 * t4);
+
+  // ---- Phase A
+  // Lane (g, t) supplies columns 16 t .. 16 t + 15 of its rows (rows g and g + 8 for A, key block g of the warp's eight for
+  // B), one and the same assignment of columns to k indices on both sides.  Key sums come straight from global memory
+  // (L2) one step ahead; past the end the last block is read instead.
+  int4 nxt[4];
+  float nxt_ks[2];
+  auto load_keys = [&](int j0) {
+    const int4* src = reinterpret_cast<const int4*>(k_colsum + (bh_rows + min(j0 + g, nb - 1)) * kHeadDim + 16 * t4);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) dst[q] = __ldg(src + q);
-    };
-    auto split16 = [&](const int4 v[4], uint32_t hi[8], uint32_t lo[8]) {
+    for (int q = 0; q < 4; ++q) nxt[q] = __ldg(src + q);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) nxt_ks[x] = __ldg(k_scales + bh_rows + min(j0 + 2 * t4 + x, nb - 1));
+  };
+  load_keys(warp * 8);
+  {
+    const int2 qv = __ldg(reinterpret_cast<const int2*>(q_colsum + (bh_rows + min(i0 + warp, nb - 1)) * kHeadDim) + lane);
+    *reinterpret_cast<int2*>(s_q + warp * kHeadDim + 2 * lane) = qv;
+    const unsigned sum_q = __reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(abs(qv.x)) + static_cast<unsigned>(abs(qv.y)));
+    unsigned kmax = 0u;  // bits of the largest scale: scales are not negative, and what is not a number counts as the largest
+    for (int j = warp * 32; j < nb; j += R * 32) kmax = max(kmax, __float_as_uint(__ldg(k_scales + bh_rows + min(j + lane, nb - 1))));
+    kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
+    if (lane == 0) {
+      s_sum[warp] = static_cast<float>(sum_q) * 0x1p-10f;
+      s_kmax[warp] = kmax;
+    }
+    if (warp < 4) {  // operands of k-step `warp`
+      uint4 hi = make_uint4(0u, 0u, 0u, 0u), lo = hi;
+      auto load_row = [&](int r) {
+        return __ldg(reinterpret_cast<const int4*>(q_colsum + (bh_rows + min(i0 + r, nb - 1)) * kHeadDim + 16 * t4) + warp);
+      };
+      const int4 v = load_row(g);
+      split_pair(v.x, v.y, hi.x, lo.x);
+      split_pair(v.z, v.w, hi.z, lo.z);
+      if constexpr (R == 16) {
+        const int4 v8 = load_row(g + 8);
+        split_pair(v8.x, v8.y, hi.y, lo.y);
+        split_pair(v8.z, v8.w, hi.w, lo.w);
+      }
+      s_a[warp * 32 + lane] = hi;
+      s_a[(4 + warp) * 32 + lane] = lo;
+    }
+  }
+  __syncthreads();
+  const float k_top = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, lane < R ? s_kmax[lane] : 0u));
+  // places per unit of a row's score; 0: the row has no places
+  auto places_per_unit = [&](int r) {
+    const float reach = 448.f * s_sum[r] * k_top;
+    return reach > 0.f && reach < 0x1p126f ? __fdividef(static_cast<float>(kPlaceSpan), reach) : 0.f;
+  };
+  {
+    constexpr int kHalves = R / 8;
+    float unit[kHalves];
+    uint32_t lo2[kHalves], hi2[kHalves];
+#pragma unroll
+    for (int r = 0; r < kHalves; ++r) {
+      unit[r] = places_per_unit(8 * r + g);
+      lo2[r] = 0x7BFF7BFFu;
+      hi2[r] = 0u;
+    }
+    const int mult_full = 128 / block;
+    // one step of eight key blocks; `edge`: the last block or what lies behind it is among them
+    auto step = [&](int j0, auto edge) {
+      constexpr bool kEdge = decltype(edge)::value;
+      const int mult = kEdge && j0 + g >= nb - 1 ? mult_last : mult_full;
+      uint32_t b_hi[8], b_mid[8];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        split_pair(v[q].x, v[q].y, hi[2 * q], lo[2 * q]);
-        split_pair(v[q].z, v[q].w, hi[2 * q + 1], lo[2 * q + 1]);
+        digits_pair(nxt[q].x, nxt[q].y, mult, b_hi[2 * q], b_mid[2 * q]);
+        digits_pair(nxt[q].z, nxt[q].w, mult, b_hi[2 * q + 1], b_mid[2 * q + 1]);
       }
-    };
-    uint32_t a_hi[2][8], a_lo[2][8];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      int4 qv[4];
-      load16(q_colsum, i0 + 8 * r + g, qv);
-      split16(qv, a_hi[r], a_lo[r]);
-    }
-    int4 nxt[4];
-    float nxt_ks[2];
-    auto load_scales = [&](int j) {
-#pragma unroll
-      for (int x = 0; x < 2; ++x) nxt_ks[x] = __ldg(k_scales + bh_rows + min(j + x, nb - 1));
-    };
-    load16(k_colsum, warp * 8 + g, nxt);
-    load_scales(warp * 8 + 2 * t4);
-    float lo[2] = {INFINITY, INFINITY}, hi[2] = {-INFINITY, -INFINITY}, kmax = 0.f;
-    const float inv_full = 1.f / static_cast<float>(block);
-    for (int j0 = warp * 8; j0 < nb; j0 += 8 * R) {
-      uint32_t b_hi[8], b_lo[8];
-      split16(nxt, b_hi, b_lo);
-      float factor[2];
-#pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        const int valid = tokens - (j0 + 2 * t4 + x) * block;
-        factor[x] = valid >= block ? nxt_ks[x] * inv_full : nxt_ks[x] / static_cast<float>(max(valid, 1));
-        kmax = fmaxf(kmax, nxt_ks[x]);
+      const int j = j0 + 2 * t4;
+      float factor[2] = {nxt_ks[0], nxt_ks[1]};
+      if constexpr (kEdge) {
+        if (j >= nb - 1) factor[0] *= factor_last;
+        if (j + 1 >= nb - 1) factor[1] *= factor_last;
+      } else {
+        if (j0 + 8 * R < nb) load_keys(j0 + 8 * R);
       }
-      if (j0 + 8 * R < nb) {
-        load16(k_colsum, j0 + 8 * R + g, nxt);
-        load_scales(j0 + 8 * R + 2 * t4);
-      }
-      float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f}, c2[4] = {0.f, 0.f, 0.f, 0.f};
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int st = 0; st < 4; ++st) {
-        mma_m16n8k16(c0, a_hi[0][2 * st], a_hi[1][2 * st], a_hi[0][2 * st + 1], a_hi[1][2 * st + 1], b_hi[2 * st], b_hi[2 * st + 1]);
-        mma_m16n8k16(c1, a_hi[0][2 * st], a_hi[1][2 * st], a_hi[0][2 * st + 1], a_hi[1][2 * st + 1], b_lo[2 * st], b_lo[2 * st + 1]);
-        mma_m16n8k16(c2, a_lo[0][2 * st], a_lo[1][2 * st], a_lo[0][2 * st + 1], a_lo[1][2 * st + 1], b_hi[2 * st], b_hi[2 * st + 1]);
+        const uint4 a_hi = s_a[st * 32 + lane], a_lo = s_a[(4 + st) * 32 + lane];
+        mma_m16n8k16(c, a_hi, b_hi[2 * st], b_hi[2 * st + 1]);
+        mma_m16n8k16(c, a_hi, b_mid[2 * st], b_mid[2 * st + 1]);
+        mma_m16n8k16(c, a_lo, b_hi[2 * st], b_hi[2 * st + 1]);
       }
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        float* const dst = s_val + static_cast<size_t>(8 * r + g) * pitch + j0 + 2 * t4;
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-          const float v = (c0[2 * r + x] + (c1[2 * r + x] + c2[2 * r + x])) * factor[x];
-          if (j0 + 2 * t4 + x < nb) {
-            dst[x] = v;
-            lo[r] = fminf(lo[r], v);
-            hi[r] = fmaxf(hi[r], v);
-          }
+      for (int r = 0; r < kHalves; ++r) {
+        // 1.5 * 2^23 leaves the rounded place in the low mantissa bits
+        const float at0 = fmaf(c[2 * r], factor[0] * unit[r], 12582912.f + kPlaceMid);
+        const float at1 = fmaf(c[2 * r + 1], factor[1] * unit[r], 12582912.f + kPlaceMid);
+        uint32_t both = __byte_perm(__float_as_uint(at0), __float_as_uint(at1), 0x5410);
+        // (sums that no quantiser has written could lead anywhere: every place has to be one)
+        both = as_word(__hmin2(__hmax2(as_half2(both), as_half2(kPlaceLow * 0x10001u)), as_half2(kPlaceHigh * 0x10001u)));
+        if constexpr (kEdge) {
+          if (j + 1 >= nb) both |= j >= nb ? 0xFFFFFFFFu : 0xFFFF0000u;
         }
+        *reinterpret_cast<uint32_t*>(s_place + static_cast<size_t>(8 * r + g) * pitch + j) = both;
+        lo2[r] = as_word(__hmin2(as_half2(lo2[r]), as_half2(both)));
+        hi2[r] = as_word(__hmax2(as_half2(hi2[r]), as_half2(both)));
       }
-    }
+    };
+    int j0 = warp * 8;
+    for (; j0 + 8 < nb; j0 += 8 * R) step(j0, std::false_type{});
+    if (j0 < nb) step(j0, std::true_type{});
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    for (int r = 0; r < kHalves; ++r) {
 #pragma unroll
       for (int o = 1; o <= 2; o <<= 1) {
-        lo[r] = fminf(lo[r], __shfl_xor_sync(0xFFFFFFFFu, lo[r], o));
-        hi[r] = fmaxf(hi[r], __shfl_xor_sync(0xFFFFFFFFu, hi[r], o));
+        lo2[r] = as_word(__hmin2(as_half2(lo2[r]), as_half2(__shfl_xor_sync(0xFFFFFFFFu, lo2[r], o))));
+        hi2[r] = as_word(__hmax2(as_half2(hi2[r]), as_half2(__shfl_xor_sync(0xFFFFFFFFu, hi2[r], o))));
       }
-      if (t4 == 0) s_range[warp * R + 8 * r + g] = make_float2(lo[r], hi[r]);
+      if (t4 == 0) s_range[warp * R + 8 * r + g] = min(lo2[r] & 0xFFFFu, lo2[r] >> 16) | (max(hi2[r] & 0xFFFFu, hi2[r] >> 16) << 16);
     }
-    kmax = warp_max(kmax);
-    if (lane == 0) s_kmax[warp] = kmax;
-  } else {
-    // Phase A: fp64 tensor-core products of the exactly widened int32 column sums (see plan_kernel).
-    const int grp = warp;
-    const int g = lane >> 2, t4 = lane & 3;
-    auto widen = [](int v) { return __int2double_rn(v); };  // exact; one instruction
-    // `local` is a block index inside the (b, h); past the end the last block is read instead (its products land
-    // in rows or columns that are never stored), which keeps the loads free of predicates and zero fills
-    auto load16 = [&](const int* base, int local, int4 dst[4]) {
-      const int4* src = reinterpret_cast<const int4*>(base + (bh_rows + min(local, nb - 1)) * kHeadDim + 16 * t4);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) dst[q] = __ldg(src + q);
-    };
-    double q_frag[16];
-    {
-      int4 qv[4];
-      load16(q_colsum, i0 + g, qv);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        q_frag[4 * q] = widen(qv[q].x);
-        q_frag[4 * q + 1] = widen(qv[q].y);
-        q_frag[4 * q + 2] = widen(qv[q].z);
-        q_frag[4 * q + 3] = widen(qv[q].w);
-      }
-    }
-    auto load_scales = [&](int j, float dst[2]) {
-#pragma unroll
-      for (int x = 0; x < 2; ++x) dst[x] = __ldg(k_scales + bh_rows + min(j + x, nb - 1));
-    };
-    int4 nxt[4];
-    float nxt_ks[2];
-    load16(k_colsum, grp * 8 + g, nxt);
-    load_scales(grp * 8 + 2 * t4, nxt_ks);
-    float lo = INFINITY, hi = -INFINITY;
-    float* const my_val = s_val + static_cast<size_t>(g) * pitch;
-    // key blocks in whole blocks of a power-of-two size divide by a multiplication that is exact, so the scale and
-    // the division fold into one factor per key block; only the last key block of a sequence can be shorter
-    const int last_full = (tokens % block == 0 && block_pow2) ? nb : (block_pow2 ? nb - 1 : 0);  // key blocks below this are whole
-#pragma unroll 2
-    for (int j0 = grp * 8; j0 < nb; j0 += 8 * R) {
-      int4 cur[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) cur[q] = nxt[q];
-      const float cur_ks[2] = {nxt_ks[0], nxt_ks[1]};
-      if (j0 + 8 * R < nb) {
-        load16(k_colsum, j0 + 8 * R + g, nxt);
-        load_scales(j0 + 8 * R + 2 * t4, nxt_ks);
-      }
-      double c[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int vals[4] = {cur[q].x, cur[q].y, cur[q].z, cur[q].w};
-#pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          const int st = 4 * q + y;
-          const double bv = widen(vals[y]);
-          asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-                       : "+d"(c[st & 1][0]), "+d"(c[st & 1][1])
-                       : "d"(q_frag[st]), "d"(bv));
-        }
-      }
-      if (j0 + 8 <= last_full) {  // all eight key blocks of the step exist and are whole (warp-uniform)
-        float tf[2];
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-          tf[x] = static_cast<float>((c[0][x] + c[1][x]) * (static_cast<double>(cur_ks[x]) * inv_block) + 0.0);
-          lo = fminf(lo, tf[x]);
-          hi = fmaxf(hi, tf[x]);
-        }
-        *reinterpret_cast<float2*>(my_val + j0 + 2 * t4) = make_float2(tf[0], tf[1]);
-      } else {
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-          const int j = j0 + 2 * t4 + x;
-          if (j < nb) {
-            const float tf = static_cast<float>(ranking_score(c[0][x] + c[1][x], cur_ks[x], j));
-            my_val[j] = tf;
-            lo = fminf(lo, tf);
-            hi = fmaxf(hi, tf);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int o = 1; o <= 2; o <<= 1) {
-      lo = fminf(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
-      hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
-    }
-    if (t4 == 0) s_range[grp * R + g] = make_float2(lo, hi);
   }
+  const bool no_places = places_per_unit(warp) == 0.f;
   __syncthreads();
   const int i = i0 + warp;
   if (i >= nb) return;
 
-  // Phase B
-  const float* vals = s_val + static_cast<size_t>(warp) * pitch;
-  // one histogram; the refinement, which needs two, borrows the place of the listed keys, which come after it
+  // ---- Phase B
+  unsigned short* const row = s_place + static_cast<size_t>(warp) * pitch;
+  const uint4* const row8 = reinterpret_cast<const uint4*>(row);  // eight places
+  const int chunks = (nb + 7) >> 3;
   unsigned int* const hist = s_hist + warp * kBuckets;
-  unsigned int* const bucket_hist = hist;
-  static_assert(kMaxListed * sizeof(unsigned long long) >= kBuckets * sizeof(unsigned int), "borrowed histogram");
-  unsigned int* const second_hist = reinterpret_cast<unsigned int*>(s_ckey + warp * 2 * kMaxListed);
-  float2 range = lane < R ? s_range[lane * R + warp] : make_float2(INFINITY, -INFINITY);
-#pragma unroll
-  for (int o = 1; o < R; o <<= 1) {
-    range.x = fminf(range.x, __shfl_xor_sync(0xFFFFFFFFu, range.x, o));
-    range.y = fmaxf(range.y, __shfl_xor_sync(0xFFFFFFFFu, range.y, o));
-  }
-  const float lo = __shfl_sync(0xFFFFFFFFu, range.x, 0), hi = __shfl_sync(0xFFFFFFFFu, range.y, 0);
-  // A key's place between the row's extremes on a 16-bit scale; its upper eight bits are the bucket of the first
-  // histogram, the lower eight refine a bucket that turns out too full to list.  Both are monotone in the score.
-  const float scale = hi > lo ? 65535.5f / (hi - lo) : 0.f;
-  // computed once, in the histogram pass, and left in place of the score (which nothing needs after that)
-  int* const places = reinterpret_cast<int*>(s_val + static_cast<size_t>(warp) * pitch);
-  auto fine = [&](int j) -> int { return places[j]; };
-  // exact 64-bit key of entry j of this row (the row's own column sums wait in shared memory)
-  int* const q_row = s_q + warp * kHeadDim;
-  q_row[lane] = __ldg(q_colsum + (bh_rows + i) * kHeadDim + lane);
-  q_row[lane + 32] = __ldg(q_colsum + (bh_rows + i) * kHeadDim + lane + 32);
-  __syncwarp();
-  const int4* const q4 = reinterpret_cast<const int4*>(q_row);
-  int margin = 0;  // places within which an approximate score may be on the wrong side of a threshold
-  if constexpr (kApprox) {
-    const float sum_q = warp_sum((fabsf(static_cast<float>(q_row[lane])) + fabsf(static_cast<float>(q_row[lane + 32]))) * 0x1p-10f);
-    const float k_top = warp_max(lane < R ? s_kmax[lane] : 0.f);
-    const float delta = k_top * (224.f * (0x1p-17f * sum_q + 0x1p-19f) + 0x1p-25f * sum_q);
-    margin = static_cast<int>(fminf(2.f * delta * scale, 65535.f)) + 3;
-  }
-  auto exact_key = [&](int j) -> unsigned long long {
+  unsigned int* const list_c = s_list + warp * 2 * kListed;  // index | place << 16 | selected << 31
+  unsigned int* const list_m = list_c + kListed;
+  const int4* const q4 = reinterpret_cast<const int4*>(s_q + warp * kHeadDim);
+  const int margin = no_places ? 0x7FFF : 1;
+  const double inv_block = 1.0 / static_cast<double>(block);
+  const unsigned below = (1u << lane) - 1u;
+  const unsigned range = lane < R ? s_range[lane * R + warp] : 0x0000FFFFu;
+  const int low = static_cast<int>(__reduce_min_sync(0xFFFFFFFFu, range & 0xFFFFu)), high = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, range >> 16));
+
+  // the ranking score from an exact dot product (same expression as in plan_kernel)
+  auto exact_order_key = [&](long long dot, int j) -> unsigned long long {
+    const int valid = min(block, tokens - j * block);
+    const double num = static_cast<double>(dot) * static_cast<double>(__ldg(k_scales + bh_rows + j));
+    return order_key((valid == block ? num * inv_block : num / static_cast<double>(valid)) + 0.0);  // block is a power of two
+  };
+  auto dot4 = [](const int4& a, const int4& b) -> long long {
+    return static_cast<long long>(a.x) * b.x + static_cast<long long>(a.y) * b.y + static_cast<long long>(a.z) * b.z +
+           static_cast<long long>(a.w) * b.w;
+  };
+  auto exact_key = [&](int j) -> unsigned long long {  // of entry j, by one lane
     const int4* const k4 = reinterpret_cast<const int4*>(k_colsum + (bh_rows + j) * kHeadDim);
     long long dot = 0;
-#pragma unroll
-    for (int d = 0; d < kHeadDim / 4; ++d) {
-      const int4 a = q4[d], b = __ldg(k4 + d);
-      dot += static_cast<long long>(a.x) * b.x + static_cast<long long>(a.y) * b.y + static_cast<long long>(a.z) * b.z +
-             static_cast<long long>(a.w) * b.w;
-    }
-    return order_key(ranking_score(static_cast<double>(dot), __ldg(k_scales + bh_rows + j), j));
+#pragma unroll 4
+    for (int d = 0; d < kHeadDim / 4; ++d) dot += dot4(q4[d], __ldg(k4 + d));
+    return exact_order_key(dot, j);
   };
+
+  auto half_of = [](const uint4& v, int x) -> int {
+    const uint32_t w = x < 2 ? v.x : (x < 4 ? v.y : (x < 6 ? v.z : v.w));
+    return static_cast<int>((x & 1) ? w >> 16 : w & 0xFFFFu);
+  };
+  // The passes over a row are loops of the whole warp (a lane past the end has eight entries that fail every comparison):
+  // lanes that leave a loop early, or take a branch of their own, would run what follows separately.
+  auto chunk = [&](int c) -> uint4 { return c < chunks ? row8[c] : make_uint4(~0u, ~0u, ~0u, ~0u); };
+  auto clear_hist = [&]() {
+    __syncwarp();
 #pragma unroll
-  for (int b = 0; b < 8; ++b) bucket_hist[lane + 32 * b] = 0u;
-  __syncwarp();
-  for (int j = lane; j < nb; j += 32) {
-    const int f = min(65535, max(0, __float2int_rz((vals[j] - lo) * scale)));
-    places[j] = f;
-    atomicAdd(&bucket_hist[f >> 8], 1u);
+    for (int x = 0; x < 2; ++x) reinterpret_cast<uint4*>(hist)[lane + 32 * x] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+  };
+  // The eight neighbouring counters of a lane and how many entries the lanes before it have (in its group of `width` lanes).
+  auto levels_of = [&](int width, int (&count)[8], int& before, int& after) {
+    const uint4 a = reinterpret_cast<const uint4*>(hist)[2 * lane], b = reinterpret_cast<const uint4*>(hist)[2 * lane + 1];
+    count[0] = a.x, count[1] = a.y, count[2] = a.z, count[3] = a.w;
+    count[4] = b.x, count[5] = b.y, count[6] = b.z, count[7] = b.w;
+    int total = 0;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) total += count[x];
+    after = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xFFFFFFFFu, after, o, width);
+      if (o < width && (lane & (width - 1)) >= o) after += up;
+    }
+    before = after - total;
+  };
+  // If the k-th entry is in one of the lane's counters: entries before that counter, its size and its number among the
+  // lane's, packed (rows have fewer than 2^14 entries).
+  auto level_at = [](const int (&count)[8], int before, int k) -> unsigned {
+    unsigned found = 0u;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      if (before < k) found = static_cast<unsigned>(before) << 17 | static_cast<unsigned>(count[x]) << 3 | static_cast<unsigned>(x);
+      before += count[x];
+    }
+    return found;
+  };
+  // first histogram: 256 buckets of 2^shift places, from the highest place down (the places span less than 2^15: shift <= 7)
+  const int shift = max(24 - __clz(high - low), 0);
+  const uint32_t counters = sm100::smem_u32(hist);
+  clear_hist();
+  for (int c0 = 0; c0 < chunks; c0 += 32) {
+    const uint4 v = chunk(c0 + lane);
+    if (8 * c0 + 256 <= nb) {
+#pragma unroll
+      for (int x = 0; x < 8; ++x) atomicAdd(&hist[(high - half_of(v, x)) >> shift], 1u);
+    } else {  // (what lies past the end is above the highest place)
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+        count_if(counters + (((high - half_of(v, x)) >> shift) << 2), half_of(v, x) <= high);
+    }
   }
   __syncwarp();
 
-  // A selection: entries whose place is above t_hi are selected, those inside [t_lo, t_hi] are decided by their exact
-  // keys (prefix / mask / take as in Selection), the rest are not.  Each selection leaves the entries of its
-  // threshold range (ascending index) and their exact keys behind for the class pass: keys_from 0 = no key needed
-  // (the whole range goes one way), 1 = listed, 2 = recompute (too many to list).
-  // The two selections of a row go through their stages together, so that the refinement and the listing each take
-  // one pass over the row for both.
+  // A selection: entries whose place is above t_hi are selected, those in [t_lo, t_hi] are decided one by one (from a list
+  // or, `recompute`, by passes over the row), the rest are not.
   struct Chosen {
-    Selection s;
-    int k, t_lo, t_hi, keys_from, remaining, size;
-    bool refine, list;
+    int k, t_lo, t_hi;
+    int above, bucket_hi;  // entries with a place above bucket_hi
+    bool open, recompute;  // something is to be decided; too many entries for a list
+    Selection s;           // (recompute)
   };
   auto begin = [&](int k) -> Chosen {
     Chosen r;
-    r.keys_from = 0;
-    r.s.prefix = 0ull;
-    r.s.mask = 0ull;
-    r.s.take = 0;
-    r.s.bucket = 0;
     r.k = k;
-    r.remaining = r.size = 0;
-    r.refine = r.list = false;
-    if (k <= 0) {
-      r.t_lo = r.t_hi = 65536;
-      return r;
-    }
-    if (k >= nb) {
-      r.t_lo = r.t_hi = -1;
-      return r;
-    }
-    const Located at = locate(bucket_hist, k, lane);
-    r.t_lo = at.bin << 8;
-    r.t_hi = r.t_lo + 255;
-    r.remaining = k - at.above;
-    r.size = at.size;
-    r.refine = r.size > kMaxListed / 2;
-    r.list = true;
+    r.open = k > 0 && k < nb;
+    r.recompute = false;
+    r.above = r.bucket_hi = 0;
+    r.t_lo = k <= 0 ? kNever : 0;  // an empty interval above or below all places
+    r.t_hi = r.t_lo - 1;
     return r;
   };
   Chosen cc = begin(k_crit), cm = begin(nb - k_neg);
-  if (cc.refine || cm.refine) {  // histograms of the lower eight bits inside the two threshold buckets
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      hist[lane + 32 * b] = 0u;  // the first histogram has served both selections
-      second_hist[lane + 32 * b] = 0u;
-    }
-    __syncwarp();
-    const int bin_c = cc.refine ? cc.t_lo >> 8 : -1, bin_m = cm.refine ? cm.t_lo >> 8 : -1;
-    for (int j = lane; j < nb; j += 32) {
-      const int f = fine(j);
-      if ((f >> 8) == bin_c) atomicAdd(&hist[f & 255], 1u);
-      if ((f >> 8) == bin_m) atomicAdd(&second_hist[f & 255], 1u);
-    }
-    __syncwarp();
-    auto refined = [&](Chosen& r, const unsigned int* h) {
-      if (!r.refine) return;
-      const Located at2 = locate(h, r.remaining, lane);
-      r.t_lo = r.t_hi = (r.t_lo & ~255) | at2.bin;
+  {
+    int count[8], before, after, size_c = 0, size_m = 0;
+    levels_of(32, count, before, after);
+    auto find = [&](Chosen& r) -> int {
+      const int src = __ffs(static_cast<int>(__ballot_sync(0xFFFFFFFFu, before < r.k && r.k <= after))) - 1;
+      const unsigned found = __shfl_sync(0xFFFFFFFFu, level_at(count, before, r.k), src);
+      r.t_hi = high - ((8 * src + static_cast<int>(found & 7u)) << shift);
+      r.t_lo = r.t_hi - (1 << shift) + 1;
+      r.above = static_cast<int>(found >> 17);
+      return static_cast<int>((found >> 3) & 0x3FFFu);
     };
-    refined(cc, hist);
-    refined(cm, second_hist);
-    __syncwarp();
-  }
-  for (Chosen* r : {&cc, &cm}) {
-    if (!r->list) continue;
-    r->t_lo = max(r->t_lo - margin, 0);
-    r->t_hi = min(r->t_hi + margin, 65535);
-  }
-  unsigned long long* const ckey_c = s_ckey + warp * 2 * kMaxListed;
-  unsigned long long* const ckey_m = ckey_c + kMaxListed;
-  unsigned short* const idx_c = s_idx + warp * 2 * kMaxListed;
-  unsigned short* const idx_m = idx_c + kMaxListed;
-  if (cc.list || cm.list) {  // positions of the entries inside the two threshold ranges, ascending, and how many are above
-    const unsigned below = (1u << lane) - 1u;
-    int listed_c = 0, listed_m = 0, above_c = 0, above_m = 0;
-    for (int j0 = 0; j0 < nb; j0 += 32) {
-      const int j = j0 + lane;
-      const int f = j < nb ? fine(j) : -1;
-      const bool is_c = cc.list && f >= cc.t_lo && f <= cc.t_hi, is_m = cm.list && f >= cm.t_lo && f <= cm.t_hi;
-      const unsigned b_c = __ballot_sync(0xFFFFFFFFu, is_c), b_m = __ballot_sync(0xFFFFFFFFu, is_m);
-      above_c += f > cc.t_hi ? 1 : 0;
-      above_m += f > cm.t_hi ? 1 : 0;
-      const int at_c = listed_c + __popc(b_c & below), at_m = listed_m + __popc(b_m & below);
-      if (is_c && at_c < kMaxListed) idx_c[at_c] = static_cast<unsigned short>(j);
-      if (is_m && at_m < kMaxListed) idx_m[at_m] = static_cast<unsigned short>(j);
-      listed_c += __popc(b_c);
-      listed_m += __popc(b_m);
-    }
-    above_c = __reduce_add_sync(0xFFFFFFFFu, above_c);
-    above_m = __reduce_add_sync(0xFFFFFFFFu, above_m);
-    __syncwarp();
-    auto settle = [&](Chosen& r, int listed, int above) {
-      if (!r.list) return;
-      r.size = listed;
-      r.remaining = r.k - above;
-      if (r.remaining == 0 || r.remaining == r.size) {  // the whole range goes one way
-        r.s.take = r.remaining;
-        r.list = false;
-      } else if (r.size > kMaxListed) {
-        r.keys_from = 2;
-        r.list = false;
-      }
-    };
-    settle(cc, listed_c, above_c);
-    settle(cm, listed_m, above_m);
-    // Exact keys of the listed entries, eight lanes to an entry (its 256 bytes of column sums read whole; with one entry per
-    // lane every load would touch 32 lines).
-    auto exact_keys = [&](const unsigned short* idx, int size, unsigned long long* ckey) {
-      const int l8 = lane & 7;
-      for (int c0 = 0; c0 < size; c0 += 4) {
-        const int c = c0 + (lane >> 3), j = idx[min(c, size - 1)];
-        const int4* const k4 = reinterpret_cast<const int4*>(k_colsum + (bh_rows + j) * kHeadDim);
-        long long dot = 0;
+    if (cc.open) size_c = find(cc);
+    if (cm.open) size_m = find(cm);
+    // Too many entries: a second histogram inside the two buckets, a counter for each of their (at most 128) places.
+    if (shift > 0 && max(size_c, size_m) > kFewListed) {
+      const int width = 1 << shift;
+      const int top_c = cc.open ? cc.t_hi : -1, top_m = cm.open ? cm.t_hi : -1;  // (no place is within `width` below -1)
+      clear_hist();
+      for (int c0 = 0; c0 < chunks; c0 += 32) {
+        const uint4 v = chunk(c0 + lane);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int4 a = q4[l8 + 8 * h], b = __ldg(k4 + l8 + 8 * h);
-          dot += static_cast<long long>(a.x) * b.x + static_cast<long long>(a.y) * b.y + static_cast<long long>(a.z) * b.z +
-                 static_cast<long long>(a.w) * b.w;
+        for (int x = 0; x < 8; ++x) {
+          const int p = half_of(v, x);
+          const unsigned at_c = static_cast<unsigned>(top_c - p), at_m = static_cast<unsigned>(top_m - p);
+          count_if(counters + (at_c << 2), at_c < static_cast<unsigned>(width));
+          count_if(counters + 512 + (at_m << 2), at_m < static_cast<unsigned>(width));
         }
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
-        if (l8 == 0 && c < size)
-          ckey[c] = order_key(ranking_score(static_cast<double>(dot), __ldg(k_scales + bh_rows + j), j));
       }
-    };
-    if (cc.list) exact_keys(idx_c, cc.size, ckey_c);
-    if (cm.list) exact_keys(idx_m, cm.size, ckey_m);
+      __syncwarp();
+      int count2[8], before2, after2;
+      levels_of(16, count2, before2, after2);  // lanes 0-15: the first selection's counters, 16-31 the second's
+      const int k = lane < 16 ? cc.k - cc.above : cm.k - cm.above;
+      const unsigned found = level_at(count2, before2, k);
+      const unsigned where = __ballot_sync(0xFFFFFFFFu, before2 < k && k <= after2);
+      auto enter = [&](Chosen& r, int base) {
+        if (!r.open) return;
+        const int src = __ffs(static_cast<int>((where >> base) & 0xFFFFu)) - 1;
+        const unsigned f = __shfl_sync(0xFFFFFFFFu, found, base + src);
+        r.t_hi -= 8 * src + static_cast<int>(f & 7u);
+        r.t_lo = r.t_hi;
+        r.above += static_cast<int>(f >> 17);
+      };
+      enter(cc, 0);
+      enter(cm, 16);
+    }
+  }
+  __syncwarp();
+  for (Chosen* r : {&cc, &cm}) {
+    if (!r->open) continue;
+    r->bucket_hi = r->t_hi;
+    r->t_lo = max(r->t_lo - margin, 1);
+    r->t_hi = min(r->t_hi + margin, kTopPlace - 1);
+    if (no_places) {
+      r->above = 0;
+      r->bucket_hi = r->t_hi;
+    }
+  }
+
+  if (cc.open || cm.open) {  // the entries of the two ranges, in any order
+    if (lane < 2) hist[lane] = 0u;
+    __syncwarp();
+    auto twice = [](int place) { return as_half2(static_cast<uint32_t>(place) * 0x10001u); };
+    const __half2 lo_c = twice(cc.t_lo), end_c = twice(cc.t_hi + 1), lo_m = twice(cm.t_lo), end_m = twice(cm.t_hi + 1);
+    for (int c0 = 0; c0 < chunks; c0 += 32) {
+      const uint4 v = chunk(c0 + lane);
+      const uint32_t words[4] = {v.x, v.y, v.z, v.w};
+      uint32_t in_c[4], in_m[4];
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        in_c[w] = __hge2_mask(as_half2(words[w]), lo_c) & ~__hge2_mask(as_half2(words[w]), end_c);
+        in_m[w] = __hge2_mask(as_half2(words[w]), lo_m) & ~__hge2_mask(as_half2(words[w]), end_m);
+      }
+      uint32_t bits = mask_bits(in_c[0], in_c[1], in_c[2], in_c[3]) | mask_bits(in_m[0], in_m[1], in_m[2], in_m[3]) << 8;
+      while (__any_sync(0xFFFFFFFFu, bits != 0u)) {
+        if (bits != 0u) {
+          const int b = __ffs(static_cast<int>(bits)) - 1, j = 8 * (c0 + lane) + (b & 7), which = b >> 3;
+          bits &= bits - 1u;
+          const unsigned at = atomicAdd(hist + which, 1u);
+          if (at < static_cast<unsigned>(kListed)) list_c[which * kListed + at] = (static_cast<unsigned>(row[j]) << 16) | static_cast<unsigned>(j);
+        }
+        __syncwarp();
+      }
+    }
     __syncwarp();
   }
-  auto finish = [&](Chosen& r, const unsigned long long* ckey) {
-    if (r.list) {
-      r.keys_from = 1;
-      if (r.size <= 64) {
-        rank_select([&](int c) { return ckey[c]; }, r.size, r.remaining, lane, r.s);
-      } else {
-        radix_select([&](int c, unsigned long long& key) {
-          key = ckey[c];
-          return true;
-        }, r.size, r.remaining, hist, lane, r.s);
+  const int n_c = cc.open ? static_cast<int>(hist[0]) : 0, n_m = cm.open ? static_cast<int>(hist[1]) : 0;
+  __syncwarp();
+  cc.recompute = n_c > kListed;
+  cm.recompute = n_m > kListed;
+
+  // Decides the listed entries of both selections side by side, kPer entries per lane: first those of the critical list,
+  // then those of the other.  The selected ones are marked (bit 31).
+  unsigned long long* const u_key = reinterpret_cast<unsigned long long*>(hist);        // [2 kListed], over the histogram
+  const int m_c = cc.recompute ? 0 : n_c, m_m = cm.recompute ? 0 : n_m;
+  auto decide = [&](auto per) {
+    constexpr int kPer = decltype(per)::value;
+    // the lists are read four entries at a time, the shorter one as far as the longer one goes
+    const int end = (max(m_c, m_m) + 3) & ~3;
+    for (int o = 0; o < end; o += 32) {
+      const int at = o + lane;
+      if (at >= m_c && at < end) list_c[at] = 0u;
+      if (at >= m_m && at < end) list_m[at] = 0u;
+    }
+    __syncwarp();
+    unsigned e[kPer];
+    int place[kPer], rank[kPer];
+    bool in[kPer], of_m[kPer];
+    const unsigned int* own[kPer];
+    struct Two {
+      int c, m;
+    };
+    auto tally = [&](const bool (&flag)[kPer]) {  // how many entries of either list have the flag
+      Two n = {0, 0};
+#pragma unroll
+      for (int x = 0; x < kPer; ++x) {
+        n.c += __popc(__ballot_sync(0xFFFFFFFFu, flag[x] && !of_m[x]));
+        n.m += __popc(__ballot_sync(0xFFFFFFFFu, flag[x] && of_m[x]));
       }
-    } else if (r.keys_from == 2) {  // every pass recomputes the keys it looks at
-      const int t_lo = r.t_lo, t_hi = r.t_hi;
+      return n;
+    };
+    bool flag[kPer];
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+      const int at = lane + 32 * x;
+      of_m[x] = at >= m_c;
+      in[x] = at < m_c + m_m;
+      own[x] = of_m[x] ? list_m : list_c;
+      e[x] = in[x] ? own[x][of_m[x] ? at - m_c : at] : 0u;
+      place[x] = static_cast<int>(e[x] >> 16);
+      rank[x] = 0;
+      flag[x] = in[x] && place[x] > (of_m[x] ? cm.bucket_hi : cc.bucket_hi);
+    }
+    // how many of the listed are selected: the margin took in some that are counted as above the bucket
+    Two need = tally(flag);
+    need.c += cc.k - cc.above;
+    need.m += cm.k - cm.above;
+    for (int o = 0; o < end; o += 4) {
+#pragma unroll
+      for (int x = 0; x < kPer; ++x) {
+        const uint4 v = *reinterpret_cast<const uint4*>(own[x] + o);
+        rank[x] += (v.x > e[x] ? 1 : 0) + (v.y > e[x] ? 1 : 0) + (v.z > e[x] ? 1 : 0) + (v.w > e[x] ? 1 : 0);
+      }
+    }
+    Two kth = {0, 0};
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+      const int hit = in[x] && rank[x] == (of_m[x] ? need.m : need.c) - 1 ? place[x] : 0;
+      kth.c = max(kth.c, of_m[x] ? 0 : hit);
+      kth.m = max(kth.m, of_m[x] ? hit : 0);
+    }
+    kth.c = __reduce_max_sync(0xFFFFFFFFu, kth.c);
+    kth.m = __reduce_max_sync(0xFFFFFFFFu, kth.m);
+    bool sel[kPer], und[kPer];
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+      const int d = place[x] - (of_m[x] ? kth.m : kth.c);
+      sel[x] = in[x] && d > margin;
+      und[x] = in[x] && d >= -margin && !sel[x];
+    }
+    const Two sure = tally(sel), open = tally(und);
+    need.c -= sure.c;
+    need.m -= sure.m;
+    const bool exact_c = need.c != open.c, exact_m = need.m != open.m;  // else all that are open are selected
+    if (exact_c || exact_m) {
+      // exact keys of the open entries, eight lanes to an entry (its 256 bytes of column sums read whole)
+      const int l8 = lane & 7;
+#pragma unroll
+      for (int x = 0; x < kPer; ++x) {
+        unsigned todo = __ballot_sync(0xFFFFFFFFu, und[x] && (of_m[x] ? exact_m : exact_c));
+        while (todo != 0u) {
+          // the first four of those left, one for each group of eight lanes
+          const unsigned t1 = todo & (todo - 1u), t2 = t1 & (t1 - 1u), t3 = t2 & (t2 - 1u);
+          const unsigned mine = lane < 8 ? todo : (lane < 16 ? t1 : (lane < 24 ? t2 : t3));
+          const int src = __ffs(static_cast<int>(mine != 0u ? mine : todo)) - 1;
+          const int j = static_cast<int>(__shfl_sync(0xFFFFFFFFu, e[x], src) & 0xFFFFu);
+          const int4* const k4 = reinterpret_cast<const int4*>(k_colsum + (bh_rows + j) * kHeadDim);
+          long long dot = dot4(q4[l8], __ldg(k4 + l8)) + dot4(q4[l8 + 8], __ldg(k4 + l8 + 8));
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
+          if (l8 == 0) u_key[32 * x + src] = exact_order_key(dot, j);
+          todo = t3 & (t3 - 1u);
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int x = 0; x < kPer; ++x) {
+        const bool exact = und[x] && (of_m[x] ? exact_m : exact_c);
+        const unsigned long long key = exact ? u_key[32 * x + lane] : 0ull;
+        int better = 0;
+#pragma unroll
+        for (int y = 0; y < kPer; ++y) {
+          unsigned others = __ballot_sync(0xFFFFFFFFu, und[y] && (of_m[y] ? exact_m : exact_c));
+          const unsigned theirs = __ballot_sync(0xFFFFFFFFu, of_m[y]);
+          for (; others != 0u; others &= others - 1u) {
+            const int src = __ffs(static_cast<int>(others)) - 1;
+            const unsigned j = __shfl_sync(0xFFFFFFFFu, e[y], src) & 0xFFFFu;
+            const unsigned long long other = u_key[32 * y + src];
+            if (((theirs >> src) & 1u) == (of_m[x] ? 1u : 0u) && (other > key || (other == key && j < (e[x] & 0xFFFFu)))) ++better;
+          }
+        }
+        if (und[x]) sel[x] = !exact || better < (of_m[x] ? need.m : need.c);
+      }
+    } else {
+#pragma unroll
+      for (int x = 0; x < kPer; ++x) sel[x] = sel[x] || und[x];
+    }
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+      const int at = of_m[x] ? kListed + lane + 32 * x - m_c : lane + 32 * x;
+      if (sel[x]) list_c[at] = e[x] | 0x80000000u;
+    }
+    __syncwarp();
+  };
+  __syncwarp();
+  if (m_c + m_m > 64)
+    decide(std::integral_constant<int, 4>{});
+  else if (m_c + m_m > 32)
+    decide(std::integral_constant<int, 2>{});
+  else if (m_c + m_m > 0)
+    decide(std::integral_constant<int, 1>{});
+
+  // Thresholds of the class pass: place >= thr_c is critical, else place >= thr_m marginal.  What was decided is written
+  // over the places: kTopPlace for critical, `mark` = thr_c - 1 for marginal, 0 for negligible.  No other entry holds
+  // `mark`: as the upper end of the critical range its entries have all been decided.
+  const int thr_c = cc.t_hi + 1, mark = max(thr_c - 1, 0), thr_m = min(cm.t_hi + 1, mark);
+  if (cc.recompute || cm.recompute) {
+    auto resolve = [&](Chosen& r) {
+      if (!r.recompute) return;
+      int above = 0;
+      for (int j = lane; j < nb; j += 32) above += static_cast<int>(row[j]) > r.t_hi ? 1 : 0;
+      above = __reduce_add_sync(0xFFFFFFFFu, above);
       radix_select([&](int c, unsigned long long& key) {
-        const int f = fine(c);
-        if (f < t_lo || f > t_hi) return false;
+        const int f = row[c];
+        if (f < r.t_lo || f > r.t_hi) return false;
         key = exact_key(c);
         return true;
-      }, nb, r.remaining, hist, lane, r.s);
-    }
-  };
-  finish(cc, ckey_c);
-  finish(cm, ckey_m);
-  const Selection sc = cc.s, sm = cm.s;
-  const int from_c = cc.keys_from, from_m = cm.keys_from;
-
-  // Phase C
-  const size_t row = bh_rows + i;
-  signed char* out_cls = cls + row * nb;
-  int* crit_row = crit_idx + row * k_crit;  // where the row's lists go on
-  int* marg_row = marg_idx != nullptr ? marg_idx + row * k_marg : nullptr;
-  int tie_c = 0, tie_m = 0, seen_c = 0, seen_m = 0;
-  const unsigned below = (1u << lane) - 1u;
-#pragma unroll 2
-  for (int j0 = 0; j0 < nb; j0 += 32) {
-    const int j = j0 + lane;
-    const bool in = j < nb;
-    const int f = in ? fine(j) : -2;
-    bool sel_c = in && f > cc.t_hi, sel_m = in && f > cm.t_hi;
-    const bool at_c = f >= cc.t_lo && f <= cc.t_hi, at_m = f >= cm.t_lo && f <= cm.t_hi;
-    if (__any_sync(0xFFFFFFFFu, at_c || at_m)) {
-      // the entries of a threshold bucket come by in the order in which the selection listed them
-      const unsigned b_at_c = __ballot_sync(0xFFFFFFFFu, at_c), b_at_m = __ballot_sync(0xFFFFFFFFu, at_m);
-      unsigned long long kc = 0ull, km = 0ull;
-      if (at_c && from_c != 0) kc = (from_c == 1 ? ckey_c[seen_c + __popc(b_at_c & below)] : exact_key(j)) & sc.mask;
-      if (at_m && from_m != 0) km = (from_m == 1 ? ckey_m[seen_m + __popc(b_at_m & below)] : exact_key(j)) & sm.mask;
-      seen_c += __popc(b_at_c);
-      seen_m += __popc(b_at_m);
-      const bool eq_c = at_c && kc == sc.prefix, eq_m = at_m && km == sm.prefix;
+      }, nb, r.k - above, hist, lane, r.s);
+    };
+    resolve(cc);
+    resolve(cm);
+    int tie_c = 0, tie_m = 0;
+    for (int j0 = 0; j0 < nb; j0 += 32) {
+      const int j = j0 + lane;
+      const int f = j < nb ? row[j] : -2;
+      const bool range_m = f >= cm.t_lo && f <= cm.t_hi;
+      const bool at_c = cc.recompute && f >= cc.t_lo && f <= cc.t_hi, at_m = cm.recompute && range_m;
+      const unsigned long long key = at_c || at_m ? exact_key(j) : 0ull;
+      const unsigned long long kc = key & cc.s.mask, km = key & cm.s.mask;
+      const bool eq_c = at_c && kc == cc.s.prefix, eq_m = at_m && km == cm.s.prefix;
       const unsigned b_eq_c = __ballot_sync(0xFFFFFFFFu, eq_c), b_eq_m = __ballot_sync(0xFFFFFFFFu, eq_m);
-      sel_c = sel_c || (at_c && kc > sc.prefix) || (eq_c && tie_c + __popc(b_eq_c & below) < sc.take);
-      sel_m = sel_m || (at_m && km > sm.prefix) || (eq_m && tie_m + __popc(b_eq_m & below) < sm.take);
+      const bool sel_c = at_c && (kc > cc.s.prefix || (eq_c && tie_c + __popc(b_eq_c & below) < cc.s.take));
+      const bool sel_m = at_m && (km > cm.s.prefix || (eq_m && tie_m + __popc(b_eq_m & below) < cm.s.take));
       tie_c += __popc(b_eq_c);
       tie_m += __popc(b_eq_m);
+      if (sel_c)
+        row[j] = kTopPlace;
+      else if (at_m)
+        row[j] = static_cast<unsigned short>(sel_m ? mark : 0);
+      else if (at_c && !range_m)
+        row[j] = static_cast<unsigned short>(mark);
     }
-    const int c = !in ? -1 : (sel_c ? 2 : (sel_m ? 1 : 0));
-    if (in) out_cls[j] = static_cast<signed char>(c);
-    const unsigned m_crit = __ballot_sync(0xFFFFFFFFu, c == 2);
-    const unsigned m_marg = __ballot_sync(0xFFFFFFFFu, c == 1);
-    if (c == 2) crit_row[__popc(m_crit & below)] = j;
-    crit_row += __popc(m_crit);
+    __syncwarp();
+  }
+  // the marginal list first: an entry of both lists that is not critical keeps what that one says
+  for (int o = 0; o < m_m; o += 32) {
+    const unsigned e = o + lane < m_m ? list_m[o + lane] : 0u;
+    if (o + lane < m_m && row[e & 0xFFFFu] != kTopPlace) row[e & 0xFFFFu] = static_cast<unsigned short>((e >> 31) != 0u ? mark : 0);
+  }
+  __syncwarp();
+  for (int o = 0; o < m_c; o += 32) {
+    const unsigned e = o + lane < m_c ? list_c[o + lane] : 0u;
+    const bool top = (e >> 31) != 0u;
+    if (top || (o + lane < m_c && static_cast<int>(e >> 16) > cm.t_hi)) row[e & 0xFFFFu] = static_cast<unsigned short>(top ? kTopPlace : mark);
+  }
+  __syncwarp();
+
+  // ---- Phase C
+  const size_t out_row = bh_rows + i;
+  signed char* const out_cls = cls + out_row * nb;
+  const int ahead = static_cast<int>(reinterpret_cast<uintptr_t>(out_cls) & 7u);  // bytes of the first word that are not ours
+  int* crit_row = crit_idx + out_row * k_crit;
+  int* marg_row = marg_idx != nullptr ? marg_idx + out_row * k_marg : nullptr;
+  const __half2 thr_c2 = as_half2(static_cast<uint32_t>(thr_c) * 0x10001u), thr_m2 = as_half2(static_cast<uint32_t>(thr_m) * 0x10001u);
+  const int words = (nb + ahead + 7) >> 3;
+  uint2 saved = make_uint2(0u, 0u);
+  for (int c0 = 0; c0 < words; c0 += 32) {
+    const int c = c0 + lane;
+    const uint4 v = chunk(c);
+    const uint32_t pairs[4] = {v.x, v.y, v.z, v.w};
+    uint32_t top[4], mid[4], two[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      top[w] = __hge2_mask(as_half2(pairs[w]), thr_c2);
+      mid[w] = __hge2_mask(as_half2(pairs[w]), thr_m2) & ~top[w];
+      two[w] = (top[w] & 0x00020002u) | (mid[w] & 0x00010001u);
+    }
+    const uint2 own = make_uint2(__byte_perm(two[0], two[1], 0x6420), __byte_perm(two[2], two[3], 0x6420));
+    // word c of the row's 8-byte words: the last `ahead` bytes of the entries before, the first of the lane's own
+    const uint2 left = make_uint2(__shfl_sync(0xFFFFFFFFu, own.x, lane - 1), __shfl_sync(0xFFFFFFFFu, own.y, lane - 1));
+    const uint2 prev = lane == 0 ? saved : left;
+    saved = left;
+    const int from = 8 - ahead;
+    const uint32_t x0 = from >= 8 ? own.x : (from >= 4 ? prev.y : prev.x);
+    const uint32_t x1 = from >= 8 ? own.y : (from >= 4 ? own.x : prev.y);
+    const uint32_t x2 = from >= 4 ? own.y : own.x;
+    const uint2 word = make_uint2(__funnelshift_r(x0, x1, 8 * (from & 3)), __funnelshift_r(x1, x2, 8 * (from & 3)));
+    const int j = 8 * c - ahead;  // entry of the word's first byte
+    const bool whole = j >= 0 && j + 8 <= nb;
+    if (whole) *reinterpret_cast<uint2*>(out_cls + j) = word;
+    for (unsigned part = __ballot_sync(0xFFFFFFFFu, !whole && c < words); part != 0u; part &= part - 1u) {  // first and last word of the row
+      const int src = __ffs(static_cast<int>(part)) - 1, jb = 8 * (c0 + src) - ahead + lane;
+      const uint32_t w0 = __shfl_sync(0xFFFFFFFFu, word.x, src), w1 = __shfl_sync(0xFFFFFFFFu, word.y, src);
+      if (lane < 8 && jb >= 0 && jb < nb) out_cls[jb] = static_cast<signed char>((lane < 4 ? w0 : w1) >> (8 * (lane & 3)));
+    }
+    const uint32_t bits_c = mask_bits(top[0], top[1], top[2], top[3]), bits_m = mask_bits(mid[0], mid[1], mid[2], mid[3]);
+    const int count = __popc(bits_c) | (__popc(bits_m) << 16);
+    int incl = count;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    const int excl = incl - count;
+    int* dst = crit_row + (excl & 0xFFFF);
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+      append_if(dst, 8 * c + x, bits_c & (1u << x));
+    crit_row += total & 0xFFFF;
     if (marg_row != nullptr) {
-      if (c == 1) marg_row[__popc(m_marg & below)] = j;
-      marg_row += __popc(m_marg);
+      dst = marg_row + (excl >> 16);
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+        append_if(dst, 8 * c + x, bits_m & (1u << x));
+      marg_row += total >> 16;
     }
   }
   if (late_wait) sm100::wait_for_prior_grid();
 }
 
+constexpr int kMostBlocks = 16383;  // (counts are packed into 14 bits)
 size_t plan_compact_smem_bytes(int nb, int rows) {
-  const size_t pitch = static_cast<size_t>((nb + 3) & ~3);
-  return rows * pitch * 4 + static_cast<size_t>(rows) * kBuckets * 4 + static_cast<size_t>(rows) * 2 * kMaxListed * 8 +
-         static_cast<size_t>(rows) * kHeadDim * 4 + static_cast<size_t>(rows) * rows * sizeof(float2) +
-         static_cast<size_t>(rows) * 2 * kMaxListed * 2;
+  return static_cast<size_t>(rows) * (place_pitch(nb) * 2 + kBuckets * 4 + 2 * kListed * 4 + kHeadDim * 4 + rows * 4);
 }
 
 template <int R>
@@ -1088,9 +1274,11 @@ lite3r_status launch_compact(const lite3r_fp8& q, const lite3r_fp8& k, const lit
   lite3r_status st = ensure_dynamic_smem(plan_compact_kernel<R>, static_cast<int>(smem));
   if (st != LITE3R_OK) return st;
   const int row_tiles = ceil_div(nb, R);
+  const int valid_last = s.tokens - (nb - 1) * s.block, mult_last = 128 / valid_last;
+  const float factor_last = 128.f / static_cast<float>(valid_last * mult_last);
   return launch_dependent(plan_compact_kernel<R>, dim3(static_cast<unsigned>(s.batch * s.heads * row_tiles)), R * 32,
                           static_cast<int>(smem), stream, q.colsum, k.colsum, k.scales, s.tokens, s.block, nb, c.k_crit, c.k_marg,
-                          c.k_neg, late_wait, plan.cls, plan.crit_idx, plan.marg_idx);
+                          c.k_neg, late_wait, mult_last, factor_last, plan.cls, plan.crit_idx, plan.marg_idx);
 }
 
 size_t plan_smem_bytes(int nb, int rows) {
@@ -1125,24 +1313,22 @@ lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r
                           const lite3r_plan& plan, bool beside_prior, cudaStream_t stream) {
   const int late_wait = beside_prior ? 1 : 0;
   const int nb = ceil_div(s.tokens, s.block);
-  constexpr size_t kLimit = 227 * 1024;
+  constexpr size_t kLimit = 227 * 1024, kCompactLimit = kLimit - 256;  // (that kernel has static shared memory, too)
   switch (g_plan_variant.load(std::memory_order_relaxed)) {  // forced by a test; sizes that do not fit are refused
     case 1: return plan_smem_bytes(nb, 8) <= kLimit ? launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
-    case 2: return plan_compact_smem_bytes(nb, 8) <= kLimit && nb <= 65536 ? launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
-    case 3: return plan_compact_smem_bytes(nb, 16) <= kLimit && nb <= 65536 ? launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 2: return plan_compact_smem_bytes(nb, 8) <= kCompactLimit && nb <= kMostBlocks ? launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 3: return plan_compact_smem_bytes(nb, 16) <= kCompactLimit && nb <= kMostBlocks ? launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
     case 4: return plan_smem_bytes(nb, 4) <= kLimit ? launch_rows<4>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
     default: break;
   }
-  // Long rows (where the 8-byte keys of eight rows would leave room for a single CTA per SM): single-precision scores in
-  // shared memory, sixteen rows per CTA when that still leaves every SM several CTAs to work on, else eight (index
-  // lists hold 16-bit positions: rows of up to 65536 blocks).
-  int sms = 0;
-  lite3r_status st = sm_count(&sms);
-  if (st != LITE3R_OK) return st;
-  if (plan_smem_bytes(nb, 8) > kLimit / 2 && nb <= 65536) {
-    const long long ctas16 = static_cast<long long>(s.batch) * s.heads * ceil_div(nb, 16);
-    if (ctas16 >= 4ll * sms && plan_compact_smem_bytes(nb, 16) <= kLimit) return launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream);
-    if (plan_compact_smem_bytes(nb, 8) <= kLimit) return launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream);
+  // Rows of more than 80 blocks: approximate scores as 16-bit places.  Its fixed part is larger than that of the 64-bit keys
+  // (16 heads of 65 blocks: 9.1 against 8.3 us), the share of every entry smaller: 512 heads of 86 blocks 92.5 against 97.0
+  // us, 64 of 172 28 against 38.6, 16 of 687 61 against 108.  Sixteen rows per CTA wherever they fit (some 6300 blocks;
+  // two heads of 2147 blocks, where eight rows would be twice as many CTAs: 75 against 105 us), else eight.
+  constexpr int kShortRow = 80;
+  if (nb > kShortRow && nb <= kMostBlocks) {
+    if (plan_compact_smem_bytes(nb, 16) <= kCompactLimit) return launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream);
+    if (plan_compact_smem_bytes(nb, 8) <= kCompactLimit) return launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream);
   }
   // As many rows per CTA as the row keys allow: the staged key blocks are then shared by more rows.
   if (plan_smem_bytes(nb, 8) <= kLimit) return launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream);

@@ -182,6 +182,31 @@ def test_plan_scores_closer_than_their_approximation(spread, block, blocks):
     assert all(np.array_equal(a, b) for a, b in zip(*plans))
 
 
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("blocks", [81, 96, 97, 255, 256, 257, 513])
+def test_plan_from_places_equals_plan_from_exact_keys(blocks, block):
+    """Rows from the shortest that the approximate scores serve, around whole and ragged groups of 8 and 256 entries, a
+    last block of one token, rows without a single place (queries of zero), lists that are empty, full, or share their
+    threshold: the same plan bit for bit as from 64-bit keys of every entry."""
+    g = np.random.default_rng(blocks)
+    wl = small_workload(f"places{blocks}", heads=3, tokens=(blocks - 1) * block + 1, block=block, src_dtype="f32")
+    inputs = wk.make_inputs(wl)
+    inputs["q"][:, 0, 2 * block:3 * block] = 0.0
+    inputs["k"][:, 1] *= np.exp(2.0 * g.standard_normal((1, wl.tokens, 1))).astype(np.float32)  # key blocks of very different scale
+    inputs["k"][:, 2, block:2 * block] = inputs["k"][:, 2, :block]
+    try:
+        for crit, neg in ((0.1, 0.6), (0.0, 0.4), (0.3, 0.7), (0.05, 0.0), (1.0, 0.0), (0.0, 1.0)):
+            plans = []
+            for variant in (1, 0, 2):
+                lt.lite3r_plan_variant(variant)
+                eng, _ = pu.run_gpu(inputs, wl, crit=crit, neg=neg)
+                plans.append([t.cpu().numpy() for t in (eng.plan.cls, eng.plan.crit_idx, eng.plan.marg_idx)])
+            for other in plans[1:]:
+                assert all(np.array_equal(a, b) for a, b in zip(plans[0], other)), (crit, neg)
+    finally:
+        lt.lite3r_plan_variant(0)
+
+
 @pytest.mark.parametrize("blocks", [64, 65, 128, 129, 193])
 def test_aggregation_inside_one_sequence(blocks):
     """Key chunks of 64 that end with, before and after the row, row tiles of 128 full and ragged."""
