@@ -64,6 +64,12 @@ constexpr int kStages = 2;  // K ring and V ring
 constexpr uint32_t kColsS = 64, kColsO = 64, kColsP = 32;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleThreshold = 8.0f;  // lazy rescale: keep the old reference until it is beaten by 2^8
+// A step in which no score of the row can beat the reference by more than 2^15 needs no maximum: probabilities of up to 2^15
+// are fp16 numbers of full precision (the largest is 2^16 - 32).  The kernel is bound by what the softmax warps issue (copies
+// that leave out the exponentials, the maxima or the sums of a step are 13-20, 7-10 and 3 % faster, one with a quarter of the
+// P V products 1-3 %).  16 heads of 10992 / 43968 tokens, 4 x 16 of 21984 in blocks of 128, 4 of 137400: 92.5 / 518 / 826 /
+// 2292 us with a maximum in every step, 86.4 / 486 / 778 / 2166 us with it only where this bound does not do.
+constexpr float kHeadroom = 15.0f;
 constexpr float kNoMax = -1.0e30f;    // reference maximum of a row that has seen no valid key yet
 constexpr int kScalSlots = 4;
 
@@ -97,6 +103,7 @@ static_assert(sizeof(Bars) <= 256, "barrier block");
 struct AttnParams {
   const float* q_scales;
   const float* k_scales;
+  const float* k_norms;  // largest norm of a key block's rows, in units of the codes (NULL: not known)
   const int* crit_idx;  // [B*H*Nb][k_crit]
   const float* zeta;    // [B*H*Nb][64]
   void* out;
@@ -315,7 +322,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // Key blocks and their scales are fetched 32 steps at a time, lane l holding those of step 32 c + l, and handed
     // to the issuing lane by a shuffle: no global load sits in the per-step path.
     int jl[2] = {0, 0};
-    float sl[2] = {0.f, 0.f};
+    float sl[2] = {0.f, 0.f}, nl[2] = {INFINITY, INFINITY};  // scale; scale times largest norm
     float sq[2] = {0.f, 0.f};
     // The K cursor runs one step ahead of the V cursor (Q K^T of step t+1 is issued under the exponentials of step t, before
     // P V of step t): the events the two wait for alternate in time in exactly this order, so blocking waits lose nothing.
@@ -381,6 +388,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           // when Q K^T of entry n + 2 has completed and with it the softmax threads' reads of entry n.
           if (refill) {
             for (int hf = 0; hf < kHalves; ++hf) sl[hf] = ldg_pinned(p.k_scales + bh_rows + jl[hf]);
+            if (p.k_norms != nullptr)
+              for (int hf = 0; hf < kHalves; ++hf) nl[hf] = ldg_pinned(p.k_norms + bh_rows + jl[hf]) * sl[hf];
             if (t == 0)
               for (int hf = 0; hf < kHalves; ++hf) sq[hf] = ldg_pinned(p.q_scales + bh_rows + tile.i_q[hf]) * (kLog2e * 0.125f);
           }
@@ -388,9 +397,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const float skf = __shfl_sync(0xFFFFFFFFu, sl[hf], t & 31);
             int valid = p.tokens - jk[hf] * BS - (kPair ? 0 : (t & 1) * kStepKeys);
             valid = max(0, min(kStepKeys, valid));
+            // second word: the factor times the largest norm, rounded up to a multiple of 2^7 steps of the last place (infinity
+            // where it is not known), and in these seven bits the number of valid keys
+            const float reach = sq[hf] * __shfl_sync(0xFFFFFFFFu, nl[hf], t & 31);
+            const uint32_t reach_bits = reach < 1.0e30f ? (__float_as_uint(reach) + 0x7Fu) & ~0x7Fu : 0x7F800000u;
             if (leader)
               sts_volatile_v2(smem_u32(smem + kOffScal) + (kc % kScalSlots) * 16 + hf * 8, __float_as_uint(sq[hf] * skf),
-                              static_cast<uint32_t>(valid));
+                              reach_bits | static_cast<uint32_t>(valid));
           }
           if (leader) mbar_arrive(&bars->k_full[st]);
           ++kc;
@@ -569,6 +582,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // The query row comes from the Q tile in shared memory (64-byte rows, 64B swizzle: 16-byte chunk c of row r sits at
     // chunk c ^ ((r >> 1) & 3)).  The loops over chunks are not unrolled: the kernel's code has to stay within the
     // instruction cache.
+    float q_norm = INFINITY;  // norm of the query row in units of the codes (not known without a linear branch)
     if (p.k_marg > 0) {
       const float sq = __ldg(p.q_scales + bh_rows + iq);
       if (!(ok = mbar_wait_far(&bars->q_full, it & 1, abort_flag, p.status, 307))) break;
@@ -598,6 +612,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         shift = mxq * cq;  // sq > 0 commutes with max
       }
+      uint64_t squares[2] = {0ull, 0ull};  // bit pattern of (0.f, 0.f)
 #pragma unroll 1
       for (int c4 = 0; c4 < 4; ++c4) {
         const uint4 raw = lds128(q_row + ((c4 ^ qswz) << 4));
@@ -610,6 +625,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
           for (int y = 0; y < 4; y += 2) {
             float e0, e1;
+            const uint64_t pair = pack_f32x2(fv[y], fv[y + 1]);
+            squares[y >> 1] = fma_f32x2(pair, pair, squares[y >> 1]);
             if (phi_softmax) {  // the softmax normaliser cancels in the ratio
               e0 = ex2(fmaf(fv[y], cq, -shift));
               e1 = ex2(fmaf(fv[y + 1], cq, -shift));
@@ -623,6 +640,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         sts128(phi_row + (((c4 * 2) ^ swz) << 4), pk8[0], pk8[1], pk8[2], pk8[3]);
         sts128(phi_row + (((c4 * 2 + 1) ^ swz) << 4), pk8[4], pk8[5], pk8[6], pk8[7]);
       }
+      float sq0, sq1;
+      unpack_f32x2(add_f32x2(squares[0], squares[1]), sq0, sq1);
+      q_norm = sqrtf(sq0 + sq1);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->phi_full);
@@ -640,7 +660,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // the step's scalars, left by the producer before it completed the K stage
       const uint2 scal = lds_volatile_v2(scal_slot + (kc % kScalSlots) * 16);
       const float c = __uint_as_float(scal.x);
-      const int valid = static_cast<int>(scal.y);
+      const int valid = static_cast<int>(scal.y & 0x7Fu);
       tmem_wait_ld();
       // the whole row of scores is in registers: the issuer may overwrite S with step t+1 right away
       tc_fence_before();
@@ -653,29 +673,34 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (32 + k >= valid) xb[k] = 0xFF800000u;
         }
       }
-      // row maximum of the raw scores (c > 0 commutes with max), eight independent chains; a step without any valid key
-      // (second half of a short last block) leaves the reference where it is
-      float mx[8];
+      // |q . k| <= |q| |k| bounds the step's scores (its rounding is far below what 2^15 leaves to the largest fp16 number).
+      // Queries and keys of ordinary size pass it in all but the first steps of a tile (91 % of the steps at 22 key blocks,
+      // 99.9 % at 687), which then go without the maximum, its vote and the wait for both.
+      if (!__all_sync(0xFFFFFFFFu, q_norm * __uint_as_float(scal.y) <= m_ref + kHeadroom)) {
+        // row maximum of the raw scores (c > 0 commutes with max), eight independent chains; a step without any valid key
+        // (second half of a short last block) leaves the reference where it is
+        float mx[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) mx[q] = fmaxf(__uint_as_float(xa[q]), __uint_as_float(xb[q]));
+        for (int q = 0; q < 8; ++q) mx[q] = fmaxf(__uint_as_float(xa[q]), __uint_as_float(xb[q]));
 #pragma unroll
-      for (int k = 8; k < 32; k += 8) {
+        for (int k = 8; k < 32; k += 8) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) mx[q] = max3(mx[q], __uint_as_float(xa[k + q]), __uint_as_float(xb[k + q]));
-      }
-      const float top = fmaxf(max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7])) * c, kNoMax);
-      // lazy rescale: the reference of a row moves only when it is beaten by 2^8 (and in the first step)
-      if (__any_sync(0xFFFFFFFFu, top > m_ref + kRescaleThreshold)) {
-        const float m_new = top > m_ref + kRescaleThreshold ? top : m_ref;
-        const float alpha = ex2(m_ref - m_new);
-        l *= alpha;
-        m_ref = m_new;
-        if (t > 0) {
-          // O is being accumulated into by the P V product of step t-1: wait for it first
-          const int u = vc + t - 1;
-          if (!(ok = mbar_wait_far(&bars->v_done[u % kStages], (u / kStages) & 1, abort_flag, p.status, 303))) break;
-          tc_fence_after();
-          rescale_accumulator(o_addr, alpha);
+          for (int q = 0; q < 8; ++q) mx[q] = max3(mx[q], __uint_as_float(xa[k + q]), __uint_as_float(xb[k + q]));
+        }
+        const float top = fmaxf(max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7])) * c, kNoMax);
+        // lazy rescale: the reference of a row moves only when it is beaten by 2^8 (and in the first step)
+        if (__any_sync(0xFFFFFFFFu, top > m_ref + kRescaleThreshold)) {
+          const float m_new = top > m_ref + kRescaleThreshold ? top : m_ref;
+          const float alpha = ex2(m_ref - m_new);
+          l *= alpha;
+          m_ref = m_new;
+          if (t > 0) {
+            // O is being accumulated into by the P V product of step t-1: wait for it first
+            const int u = vc + t - 1;
+            if (!(ok = mbar_wait_far(&bars->v_done[u % kStages], (u / kStages) & 1, abort_flag, p.status, 303))) break;
+            tc_fence_after();
+            rescale_accumulator(o_addr, alpha);
+          }
         }
       }
       uint32_t packed[32];
@@ -897,6 +922,7 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   if (p.tma_out == 0) map_o = map_q;  // any valid map when it is not used
   p.q_scales = a.q_scales;
   p.k_scales = a.k_scales;
+  p.k_norms = a.k_norms;
   p.crit_idx = a.crit_idx;
   p.zeta = a.zeta;
   p.out = a.out;

@@ -198,6 +198,7 @@ struct AttentionLaunch {
   const float* q_scales;
   const float* k_scales;
   const float* v_scales;
+  const float* k_norms;       // [tiles] largest norm of a key block's rows in units of the codes; NULL: not known
   const __half* v16;          // [tiles*Bs][64] dequantised V as fp16
   const __nv_bfloat16* g16;   // [tiles][64][64] aggregated projected summaries, [e][d]
   const float* zeta;          // [tiles][64]
@@ -215,7 +216,7 @@ void set_attention_plain_stores(int on);  // test hook, see lite3r_attention_pla
 // Per-key-block summaries ((H_j W)^T | z_j) in bf16, one kSummaryRow-wide row per (b, h, key block).
 // Clears *device_status.
 lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const float* proj, long long proj_head_stride,
-                             const lite3r_shape& s, int phi, __nv_bfloat16* hws, __half* v16, int* device_status,
+                             const lite3r_shape& s, int phi, __nv_bfloat16* hws, __half* v16, float* k_norms, int* device_status,
                              cudaStream_t stream);
 
 // Marginal aggregation G_i = sum over marginal j of the summary rows, as a 0/1-mask GEMM on tensor cores.

@@ -64,6 +64,7 @@ struct Workspace {
   __nv_bfloat16* g16;  // [tiles][64][64] aggregated summaries, [e][d]
   float* zeta;         // [tiles][64]
   __half* v16;         // [tiles*Bs][64]  dequantised V as fp16
+  float* k_norms;      // [tiles]         largest norm of a key block's rows, in units of the codes
   signed char* cls;    // [tiles][Nb]     block classes, only when the plan is built inside the workspace
   int* crit_idx;       // [tiles][k_crit] critical lists, likewise
   size_t bytes;
@@ -88,6 +89,7 @@ Workspace carve(void* base, const lite3r_shape& s, int k_crit = 0, bool plan_ins
   w.zeta = reinterpret_cast<float*>(take(tiles * kHeadDim * sizeof(float)));
   w.offsets[3] = off;
   w.v16 = reinterpret_cast<__half*>(take(tiles * s.block * kHeadDim * sizeof(__half)));
+  w.k_norms = reinterpret_cast<float*>(take(tiles * sizeof(float)));
   w.cls = nullptr;
   w.crit_idx = nullptr;
   w.offsets[4] = w.offsets[5] = off;
@@ -135,7 +137,7 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   if ((phases & 1) && a.plan.k_marg > 0) {
     profile_mark(2, stream);
     st = launch_summary(a.k, a.v, a.proj, a.proj_head_stride, s, a.phi, w.hws, a.plan.k_crit > 0 ? w.v16 : nullptr,
-                        a.device_status, stream);
+                        a.plan.k_crit > 0 ? w.k_norms : nullptr, a.device_status, stream);
     if (st != LITE3R_OK) return st;
     profile_mark(3, stream);
   }
@@ -154,6 +156,7 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   att.k_scales = a.k.scales;
   att.v_scales = a.v.scales;
   att.v16 = w.v16;
+  att.k_norms = a.plan.k_marg > 0 ? w.k_norms : nullptr;  // (from the summary kernel)
   att.g16 = w.g16;
   att.zeta = w.zeta;
   att.crit_idx = plan.crit_idx;

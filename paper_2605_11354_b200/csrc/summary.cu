@@ -14,7 +14,9 @@
 // their K row, apply the feature map, and write phi and the V code values to shared memory in the operands' swizzled
 // layouts; one thread of a fifth warp issues the MMAs; the compute threads then move H from TMEM to shared memory
 // (scaled, fp16), and finally (H W)^T from TMEM to global memory (rows parked in shared memory first, so that stores
-// write whole 128-byte rows).  Next to a sparse branch the kernel also writes the dequantised V rows it has just read
+// write whole 128-byte rows).  Next to a sparse branch it writes the largest norm of a block's key rows, with which the
+// attention kernel bounds its scores (43968 / 4 x 21984 tokens: 70.5 -> 72.6 / 115.9 -> 119.3 us, a tenth of what that
+// saves), and the dequantised V rows it has just read
 // (fp16, the attention kernel's P V operand), which saves a pass of its own over V.  Rounds of one CTA are serial; four CTAs per SM
 // overlap their phases.  Every barrier wait is bounded.
 #include "common.cuh"
@@ -43,7 +45,10 @@ struct Bars {
   uint64_t ab_full, h_done, h_full, hw_done;
   uint32_t tmem_base;
   int abort;
+  uint32_t norm2[4];  // per warp: bits of the largest squared norm of its key rows
 };
+
+static_assert(sizeof(Bars) <= kSmemBytes - kOffBar, "barrier block");
 
 struct SummaryParams {
   const uint8_t* k_codes;
@@ -55,6 +60,7 @@ struct SummaryParams {
   int heads, tokens, nb, phi;
   int rounds_per_head, rounds;
   __nv_bfloat16* hws;
+  float* k_norms;  // when not NULL: also writes the largest norm of the block's key rows, in units of the codes
   __half* v16;  // when not NULL: also writes the dequantised V rows (code value x block scale, fp16) read on the way
   int* status;
 };
@@ -233,6 +239,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
         const int j = j0 + tile_tok;
         const int valid = j < p.nb ? min(BS, p.tokens - j * BS) : 0;
         uint32_t pw[32], vw[32];
+        uint64_t squares[4] = {0ull, 0ull, 0ull, 0ull};  // bit pattern of (0.f, 0.f)
         if (s < valid) {
           const size_t tile = bh_rows + j;
           const uint4* ksrc = reinterpret_cast<const uint4*>(p.k_codes + (tile * BS + s) * kHeadDim);
@@ -269,6 +276,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
               x[c * 16 + q * 4 + 2] = hi.x;
               x[c * 16 + q * 4 + 3] = hi.y;
             }
+          }
+          if (p.k_norms != nullptr) {
+#pragma unroll
+            for (int d = 0; d < 64; d += 2) squares[(d >> 1) & 3] = fma_f32x2(pack_f32x2(x[d], x[d + 1]), pack_f32x2(x[d], x[d + 1]), squares[(d >> 1) & 3]);
           }
           if (p.phi == LITE3R_PHI_SOFTMAX) {
             // Any common shift of the exponents cancels in the ratio.  448 * scale bounds every component of the block,
@@ -322,6 +333,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
           store_row_swizzled(smem + kOffV, t, vw);
         }
         store_row_swizzled(smem + kOffA, t, pw);
+        if (p.k_norms != nullptr) {
+          float n0, n1;
+          unpack_f32x2(add_f32x2(add_f32x2(squares[0], squares[1]), add_f32x2(squares[2], squares[3])), n0, n1);
+          const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(n0 + n1));  // (not negative: ordered like the bits)
+          if (lane == 0) bars->norm2[warp] = top;
+        }
         if (p.v16 != nullptr && j < p.nb) {
           // The attention kernel's P V operand (code value x block scale as fp16, the stand-alone pass's arithmetic),
           // from the rows this warp has just put into the V operand tile (zeros past the end of the sequence): read
@@ -351,6 +368,15 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
       // H row: TMEM -> scaled fp16 -> B operand of MMA 2; z row -> global
       if (!(ok = mbar_wait_clearing(&bars->h_done, ph, abort_flag, p.status, 503))) break;
       tc_fence_after();
+      // (all warps have left their largest norms before the products that have just completed; they leave the next round's only
+      // after every thread has arrived below)
+      uint32_t top2 = 0u;
+      const bool stores_norm = p.k_norms != nullptr && t < kTilesPerRound && j0 + t < p.nb;
+      if (stores_norm) {
+        constexpr int kWarps = BS / 32;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) top2 = max(top2, bars->norm2[t * kWarps + w]);
+      }
       {
         uint32_t lo[32], hi[32];
         tmem_ld32(lane_addr + kColH, lo);
@@ -376,6 +402,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) summary_kernel(const Sum
       }
       fence_proxy_async_smem();
       mbar_arrive(&bars->h_full);
+      if (stores_norm) p.k_norms[bh_rows + j0 + t] = sqrtf(__uint_as_float(top2));
 
       // (H W)^T row e': TMEM -> bf16 -> global
       if (!(ok = mbar_wait_clearing(&bars->hw_done, ph, abort_flag, p.status, 504))) break;
@@ -436,8 +463,8 @@ lite3r_status launch(const SummaryParams& p, int sm_count, cudaStream_t stream) 
 }  // namespace
 
 lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const float* proj, long long proj_head_stride,
-                             const lite3r_shape& s, int phi, __nv_bfloat16* hws, __half* v16, int* device_status,
-                             cudaStream_t stream) {
+                             const lite3r_shape& s, int phi, __nv_bfloat16* hws, __half* v16, float* k_norms,
+                             int* device_status, cudaStream_t stream) {
   SummaryParams p;
   p.k_codes = k.codes;
   p.k_scales = k.scales;
@@ -453,6 +480,7 @@ lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const flo
   p.rounds = s.batch * s.heads * p.rounds_per_head;
   p.hws = hws;
   p.v16 = v16;
+  p.k_norms = k_norms;
   p.status = device_status;
   int sms = 0;
   lite3r_status st = sm_count(&sms);

@@ -271,3 +271,21 @@ def test_codes_next_to_rounding_boundaries_at_scales_that_take_a_second_correcti
     got_codes, got_scales = lt.lite3r_quantize_rows_fp8(torch.from_numpy(np.ascontiguousarray(rows)).cuda())
     assert np.array_equal(got_codes.cpu().numpy(), codes.reshape(len(tiles), -1)[:, :1024])
     assert np.array_equal(got_scales.cpu().numpy().view(np.uint32).ravel(), scales.view(np.uint32).ravel())
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("climb", [7.9, 8.1, 14.8, 15.2, 15.95, 16.1, 40.0])
+def test_attention_with_and_without_a_row_maximum(climb, block):
+    """A step whose scores cannot beat the row's reference by more than 2^15 (norm of the query times largest norm of the key
+    block) goes without a maximum.  Query and key rows share a direction, so that the bound is nearly reached: a second
+    critical block 2^climb above the first, on both sides of the rescale threshold (8), of the bound (15) and of the
+    largest fp16 number (16); a ragged last block."""
+    g = np.random.default_rng(block)
+    wl = small_workload(f"climb{climb}", heads=2, tokens=8 * block - 9, block=block, crit=0.5, neg=0.25, src_dtype="f32")
+    inputs = wk.make_inputs(wl)
+    top = 1.0 + climb / np.log2(np.e)
+    level = np.repeat(np.array([1.0, top, top - 0.5, 0.9, 0.2, 0.1, -0.1, -0.2]), block)[:wl.tokens]
+    for name, along in (("q", 8.0), ("k", level[None, None, :, None])):
+        inputs[name] = (along / 8.0 + 0.02 * g.standard_normal(inputs[name].shape)).astype(np.float32)
+    eng, _ = full_parity(wl, inputs)
+    assert (eng.plan.crit_idx.cpu().numpy() == np.arange(4)).all()
