@@ -71,7 +71,7 @@ constexpr float kRescaleThreshold = 8.0f;  // lazy rescale: keep the old referen
 // 2292 us with a maximum in every step, 86.4 / 486 / 778 / 2166 us with it only where this bound does not do.
 constexpr float kHeadroom = 15.0f;
 constexpr float kNoMax = -1.0e30f;    // reference maximum of a row that has seen no valid key yet
-constexpr int kScalSlots = 4;
+constexpr int kScalSlots = 64;
 
 // shared-memory map (bytes from a 1024-aligned base); a step's tiles take half a stage at block 128 (one key block's)
 constexpr uint32_t kStageK = 8192, kStageV = 16384;
@@ -84,7 +84,7 @@ constexpr uint32_t kOffZeta = kOffPhi + 16384;           // zeta_i of the linear
 constexpr uint32_t kOffScal = kOffZeta + 1024;           // per step and query block: {exponent factor, valid keys}
 constexpr uint32_t kOffNext = kOffScal + kScalSlots * 16;  // answer of the work scheduler (16 B), tile numbers (4 x 4 B)
 constexpr uint32_t kOffBar = kOffNext + 32;
-constexpr uint32_t kSmemBytes = kOffBar + 256;           // three CTAs per SM: 3 * (75104 + 1024 reserved) <= 233472
+constexpr uint32_t kSmemBytes = kOffBar + 256;           // three CTAs per SM: 3 * (76064 + 1024 reserved) <= 233472
 constexpr int kTileSlots = 4;
 
 struct Bars {
@@ -197,15 +197,17 @@ __device__ __forceinline__ void exp2_pair_fma(uint64_t a2, float& p0, float& p1)
 }
 
 // exp2 of 32 scaled scores, packed to fp16 pairs; adds them to two running pairs of sums.  Arguments and sums run on
-// pairs of columns (packed fp32x2 fma / add).  Every eighth pair goes to the multiply-add units (2 % faster at 16 heads of
-// 10992 tokens and 1 % at 137400 than none; every fourth costs more instructions than it saves and is slower than none).
+// pairs of columns (packed fp32x2 fma / add).  Every eighth pair goes to the multiply-add units at block 64, every fifth at
+// block 128, where the products leave the tensor pipe idle for longer (16 heads of 43968 tokens in blocks of 64: none 514 us,
+// every 16th 494, eighth 486, fifth 500, fourth 500; 4 x 16 of 21984 in blocks of 128: 811, 789, 776, 764, 764).
+template <int kPolyEvery>
 __device__ __forceinline__ void exp_half_row(const uint32_t (&x)[32], uint64_t c2, uint64_t shift2, uint32_t* packed,
                                              uint64_t (&sum2)[2]) {
 #pragma unroll
   for (int k = 0; k < 32; k += 2) {
     const uint64_t a2 = fma_f32x2(pack_f32x2(__uint_as_float(x[k]), __uint_as_float(x[k + 1])), c2, shift2);
     float p0, p1;
-    if (((k >> 1) & 7) == 7) {
+    if ((k >> 1) % kPolyEvery == kPolyEvery - 1) {
       exp2_pair_fma(a2, p0, p1);
     } else {
       float a0, a1;
@@ -246,6 +248,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr int kHalves = kPair ? 2 : 1;             // independent M=64 problems per CTA
   constexpr int kStepsPerBlock = BS / kStepKeys;     // 1 or 2
   constexpr int kM = kPair ? 64 : 128;
+  constexpr int kPolyEvery = kPair ? 8 : 5;  // pairs of exponentials per one on the multiply-add units (see exp_half_row)
   constexpr uint32_t kTxK = kHalves * 4096, kTxV = kHalves * 8192;  // bytes of a step's tiles
 
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -322,8 +325,6 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // Key blocks and their scales are fetched 32 steps at a time, lane l holding those of step 32 c + l, and handed
     // to the issuing lane by a shuffle: no global load sits in the per-step path.
     int jl[2] = {0, 0};
-    float sl[2] = {0.f, 0.f}, nl[2] = {INFINITY, INFINITY};  // scale; scale times largest norm
-    float sq[2] = {0.f, 0.f};
     // The K cursor runs one step ahead of the V cursor (Q K^T of step t+1 is issued under the exponentials of step t, before
     // P V of step t): the events the two wait for alternate in time in exactly this order, so blocking waits lose nothing.
     bool ok = true;
@@ -383,27 +384,24 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             for (int hf = 0; hf < kHalves; ++hf)
               tma_load_2d(smem + kOffK + st * kStageK + hf * 4096, &map_k, &bars->k_full[st], 0, tile_row(t, jk[hf]));
           }
-          // The step's scalars for the softmax threads, on their way while the tiles travel: the factor that turns a raw
-          // score into a base-2 exponent and the number of valid keys.  The slot of entry n is rewritten for entry n + 4,
-          // when Q K^T of entry n + 2 has completed and with it the softmax threads' reads of entry n.
+          // The steps' scalars for the softmax threads, made when their key blocks are fetched, lane l those of the l-th step,
+          // while the tiles travel.  Slots are those of the ring entries: the 32 written here are at most entries kc .. kc + 31,
+          // and those that may still be read kc - 2 and kc - 1.
           if (refill) {
-            for (int hf = 0; hf < kHalves; ++hf) sl[hf] = ldg_pinned(p.k_scales + bh_rows + jl[hf]);
-            if (p.k_norms != nullptr)
-              for (int hf = 0; hf < kHalves; ++hf) nl[hf] = ldg_pinned(p.k_norms + bh_rows + jl[hf]) * sl[hf];
-            if (t == 0)
-              for (int hf = 0; hf < kHalves; ++hf) sq[hf] = ldg_pinned(p.q_scales + bh_rows + tile.i_q[hf]) * (kLog2e * 0.125f);
-          }
-          for (int hf = 0; hf < kHalves; ++hf) {
-            const float skf = __shfl_sync(0xFFFFFFFFu, sl[hf], t & 31);
-            int valid = p.tokens - jk[hf] * BS - (kPair ? 0 : (t & 1) * kStepKeys);
-            valid = max(0, min(kStepKeys, valid));
-            // second word: the factor times the largest norm, rounded up to a multiple of 2^7 steps of the last place (infinity
-            // where it is not known), and in these seven bits the number of valid keys
-            const float reach = sq[hf] * __shfl_sync(0xFFFFFFFFu, nl[hf], t & 31);
-            const uint32_t reach_bits = reach < 1.0e30f ? (__float_as_uint(reach) + 0x7Fu) & ~0x7Fu : 0x7F800000u;
-            if (leader)
-              sts_volatile_v2(smem_u32(smem + kOffScal) + (kc % kScalSlots) * 16 + hf * 8, __float_as_uint(sq[hf] * skf),
-                              reach_bits | static_cast<uint32_t>(valid));
+            for (int hf = 0; hf < kHalves; ++hf) {
+              const float sk = ldg_pinned(p.k_scales + bh_rows + jl[hf]);
+              const float c = ldg_pinned(p.q_scales + bh_rows + tile.i_q[hf]) * (kLog2e * 0.125f) * sk;  // raw score -> base-2 exponent
+              int valid = p.tokens - jl[hf] * BS - (kPair ? 0 : ((t + lane) & 1) * kStepKeys);
+              valid = max(0, min(kStepKeys, valid));
+              // second word: the factor times the largest norm, rounded up to a multiple of 2^7 steps of the last place (infinity
+              // where it is not known), and in these seven bits the number of valid keys
+              const float reach = p.k_norms != nullptr ? c * ldg_pinned(p.k_norms + bh_rows + jl[hf]) : INFINITY;
+              const uint32_t reach_bits = reach < 1.0e30f ? (__float_as_uint(reach) + 0x7Fu) & ~0x7Fu : 0x7F800000u;
+              if (t + lane < steps)
+                sts_volatile_v2(smem_u32(smem + kOffScal) + ((kc + lane) % kScalSlots) * 16 + hf * 8, __float_as_uint(c),
+                                reach_bits | static_cast<uint32_t>(valid));
+            }
+            __syncwarp();
           }
           if (leader) mbar_arrive(&bars->k_full[st]);
           ++kc;
@@ -707,8 +705,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       {
         const uint64_t c2 = pack_f32x2(c, c), shift2 = pack_f32x2(-m_ref, -m_ref);
         uint64_t sum2[2] = {0ull, 0ull};  // bit pattern of (0.f, 0.f)
-        exp_half_row(xa, c2, shift2, packed, sum2);
-        exp_half_row(xb, c2, shift2, packed + 16, sum2);
+        exp_half_row<kPolyEvery>(xa, c2, shift2, packed, sum2);
+        exp_half_row<kPolyEvery>(xb, c2, shift2, packed + 16, sum2);
         float s0, s1;
         unpack_f32x2(add_f32x2(sum2[0], sum2[1]), s0, s1);
         l += s0 + s1;
