@@ -5,15 +5,23 @@
 // accumulation is fp32 in TMEM, so this equals the gather-and-add of the summaries while reading each summary once per
 // 128 query blocks instead of once per query block.
 //
-// One CTA computes a 128 (rows) x 256 (summary columns) tile; the reduction runs over key blocks in chunks of 64.  Rows
-// and keys are numbered through all (b, h).  Tiles either stay inside one (b, h), or, for short sequences, run through
-// the (b, h) boundaries so that several small problems share a tile (the mask is then block-diagonal); the launcher
-// takes the cheaper tiling.  Per chunk: TMA brings the 64 x 256 slab of summaries (MN-major B operand, four 64-column
-// boxes, 128B swizzle); 128 threads expand the class bytes of their row, or sixteen lanes those of a row together
-// (fetched a chunk ahead), into the bf16 0/1 A tile (K-major, 128B swizzle) with byte permutes; one thread issues four 128x256x16 MMAs.  Epilogue: the same 128
-// threads read their accumulator row from TMEM, turn the rows around in shared memory so that stores write whole
-// 128-byte segments, and store the first 4096 columns as bf16 (the attention kernel's B operand) and the last 64
-// (zeta) as fp32.
+// A tile is 128 (rows) x 256 (summary columns; the last column tile is the 64 of zeta); the reduction runs over key blocks
+// in chunks of 64.  Rows and keys are numbered through all (b, h).  Tiles either stay inside one (b, h), or, for short
+// sequences, run through the (b, h) boundaries so that several small problems share a tile (the mask is then
+// block-diagonal); the launcher takes the cheaper tiling.
+//
+// Persistent CTAs, one per SM, walk the tiles (the column tiles of a row tile are neighbours, so that the CTAs running at any
+// time share class rows and summaries in L2).  The ring of four chunks runs on through the tiles and the two accumulators
+// alternate, so that loads, mask tiles and products of the next tile run under the stores of this one.  Warp 0 brings the
+// 64 x 256 slab of summaries by TMA (MN-major B operand, four 64-column boxes, 128B swizzle); warp 1 issues four
+// 128x256x16 MMAs per chunk; two warpgroups, each taking every other chunk, expand the class bytes into the bf16 0/1 A tile
+// (K-major, 128B swizzle), eight lanes to a row; two more, one per accumulator, read their rows from TMEM, turn them around
+// in shared memory so that stores write whole 128-byte segments, and store the first 4096 columns as bf16 (the attention
+// kernel's B operand) and the last 64 (zeta) as fp32.
+// Bound by shared memory: a chunk's products read 48 KB of operands in 512 clocks of tensor pipe, TMA writes 32 KB and the
+// masks 16 KB beside them.  Against two CTAs per SM of one tile each, which set up, filled their ring and drained one
+// after the other: 512 (b, h) of 22 / 86 blocks 49.6 / 177 -> 41.4 / 119 us, 64 of 172 62 -> 43.5 us, 16 of 172 / 687 / 2147
+// blocks 20.8 / 92 / 551 -> 18.8 / 80 / 548 us (4 of 2147, 7.8 tiles per SM: 140 -> 148 us).
 #include <algorithm>
 
 #include "common.cuh"
@@ -25,62 +33,98 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kStages = 2;  // 96 KB of operand stages: two CTAs per SM, one's epilogue overlaps the other's main loop
-constexpr int kThreads = 192;
+constexpr int kStages = 4;
 constexpr int kTileM = 128, kTileN = 256, kChunk = 64;
+constexpr int kColTiles = (kSummaryRow + kTileN - 1) / kTileN;
+constexpr int kBuilders = 2;    // warpgroups that expand masks (warps 4-11)
+constexpr int kDrainers = 2;    // warpgroups that store results, one per accumulator (warps 12-19)
+constexpr int kThreads = 128 + (kBuilders + kDrainers) * 128;
 constexpr uint32_t kABytes = kTileM * kChunk * 2;   // 16 KB
 constexpr uint32_t kBBytes = kChunk * kTileN * 2;   // 32 KB
 constexpr uint32_t kOffA = 0;
 constexpr uint32_t kOffB = kStages * kABytes;
-constexpr uint32_t kOffBar = kOffB + kStages * kBBytes;
-constexpr uint32_t kSmemBytes = kOffBar + 128;
-constexpr uint32_t kTmemCols = 256;
+constexpr uint32_t kOffOut = kOffB + kStages * kBBytes;  // 4 KB per storing warp
+constexpr uint32_t kOffBar = kOffOut + kDrainers * 4 * 4096;
+constexpr uint32_t kSmemBytes = kOffBar + 192;
+constexpr uint32_t kTmemCols = 2 * kTileN;
 
 struct Bars {
-  uint64_t a_full[kStages], b_full[kStages], empty[kStages], acc_full;
+  uint64_t a_full[kStages], b_full[kStages], empty[kStages];
+  uint64_t acc_full[2], acc_empty[2];
   uint32_t tmem_base;
   int abort;
 };
+static_assert(sizeof(Bars) <= 192, "barrier block");
+
+struct AggregateParams {
+  const signed char* cls;
+  int nb, total_rows;
+  int row_tiles;  // of one (b, h), or (flat) of all rows
+  float inverse;  // of row_tiles, or (flat) of nb
+  int tiles;      // row tiles times column tiles, of all (b, h)
+  __nv_bfloat16* g16;
+  float* zeta;
+  int* status;
+};
+
+// Rows and keys are numbered through all (b, h): row R = (b h) Nb + i, key (b h) Nb + j, the row numbers of the class
+// matrix, the summaries and the outputs.  A tile is 128 consecutive rows and reduces over the keys of the (b, h) it
+// touches.
+struct Tile {
+  int col, row0, row_limit, key0, chunks;
+};
+// n / d for n / d below 2^22 (a float quotient is then off by at most one).
+__device__ __forceinline__ int divide(int n, int d, float inverse) {
+  int q = static_cast<int>(static_cast<float>(n) * inverse);
+  const int rest = n - q * d;
+  q += rest >= d ? 1 : 0;
+  return rest < 0 ? q - 1 : q;
+}
+template <bool kFlat>
+__device__ __forceinline__ Tile tile_at(const AggregateParams& p, int id) {
+  Tile t;
+  const int rt = id / kColTiles;
+  t.col = id - rt * kColTiles;
+  int key_end;
+  if (kFlat) {
+    t.row0 = rt * kTileM;
+    t.row_limit = p.total_rows;
+    t.key0 = divide(t.row0, p.nb, p.inverse) * p.nb;
+    key_end = divide(min(t.row0 + kTileM, p.total_rows) - 1, p.nb, p.inverse) * p.nb + p.nb;
+  } else {
+    const int bh = divide(rt, p.row_tiles, p.inverse);
+    t.key0 = bh * p.nb;
+    key_end = t.key0 + p.nb;
+    t.row0 = t.key0 + (rt - bh * p.row_tiles) * kTileM;
+    t.row_limit = key_end;
+  }
+  t.chunks = (key_end - t.key0 + kChunk - 1) / kChunk;
+  return t;
+}
 
 template <bool kFlat>
-__global__ void __launch_bounds__(kThreads, 2)
-aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed char* __restrict__ cls, int nb,
-                     int total_rows, __nv_bfloat16* __restrict__ g16, float* __restrict__ zeta, int* status) {
+__global__ void __launch_bounds__(kThreads, 1)
+aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateParams p) {
   extern __shared__ __align__(1024) uint8_t smem[];
   Bars* bars = reinterpret_cast<Bars*>(smem + kOffBar);
   volatile int* abort_flag = &bars->abort;
   if ((smem_u32(smem) & 1023u) != 0) {
-    if (threadIdx.x == 0 && status != nullptr) atomicCAS(status, 0, 901);
+    if (threadIdx.x == 0 && p.status != nullptr) atomicCAS(p.status, 0, 901);
     return;
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_tile = blockIdx.x;           // 0..16, 256 summary columns each (the last one holds zeta)
-  // Rows and keys are numbered through all (b, h): row R = (b h) Nb + i, key (b h) Nb + j, the row numbers of the class
-  // matrix, the summaries and the outputs.  A tile is 128 consecutive rows and reduces over the keys of the (b, h) it
-  // touches.  Long sequences: the tile stays inside one (b, h) (grid z).  Short ones (flat): tiles run through the
-  // (b, h) boundaries, so several small problems share one tile instead of each padding its own; the mask is then
-  // block-diagonal, a row only ever selecting keys of its own (b, h).
-  int row0, row_limit, key0, key_end;
-  if (kFlat) {
-    row0 = blockIdx.y * kTileM;
-    row_limit = total_rows;
-    key0 = (row0 / nb) * nb;
-    key_end = (min(row0 + kTileM, total_rows) - 1) / nb * nb + nb;
-  } else {
-    key0 = blockIdx.z * nb;
-    key_end = key0 + nb;
-    row0 = key0 + blockIdx.y * kTileM;
-    row_limit = key_end;
-  }
-  const int chunks = (key_end - key0 + kChunk - 1) / kChunk;
+  const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int step = static_cast<int>(gridDim.x);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(&bars->a_full[s], 128);
+      mbar_init(&bars->a_full[s], 4);  // one arrival per warp
       mbar_init(&bars->b_full[s], 1);
       mbar_init(&bars->empty[s], 1);
     }
-    mbar_init(&bars->acc_full, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&bars->acc_full[b], 1);
+      mbar_init(&bars->acc_empty[b], 4);
+    }
     bars->abort = 0;
     mbar_fence_init();
   }
@@ -101,174 +145,201 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed cha
   if (warp == 0) {
     if (lane == 0) {
       tma_prefetch_desc(&map_s);
-      for (int c = 0; c < chunks; ++c) {
-        const int st = c % kStages;
-        if (!mbar_wait(&bars->empty[st], ((c / kStages) & 1) ^ 1, abort_flag, status, 401)) break;
-        mbar_arrive_expect_tx(&bars->b_full[st], kBBytes);
-        const int row = key0 + c * kChunk;
-        for (int q = 0; q < 4; ++q)  // columns past 4160 and rows past the tensor are zero-filled by TMA
-          tma_load_2d(smem + kOffB + st * kBBytes + q * 8192, &map_s, &bars->b_full[st], n_tile * kTileN + q * 64, row);
+      bool ok = true;
+      int kc = 0;  // chunks so far, through all tiles
+      for (int id = blockIdx.x; ok && id < p.tiles; id += step) {
+        const Tile t = tile_at<kFlat>(p, id);
+        const int boxes = t.col == kColTiles - 1 ? 1 : kTileN / 64;
+        for (int c = 0; c < t.chunks; ++c, ++kc) {
+          const int st = kc % kStages;
+          if (!(ok = mbar_wait(&bars->empty[st], ((kc / kStages) & 1) ^ 1, abort_flag, p.status, 401))) break;
+          mbar_arrive_expect_tx(&bars->b_full[st], boxes * 8192);
+          for (int q = 0; q < boxes; ++q)  // rows past the tensor are zero-filled by TMA
+            tma_load_2d(smem + kOffB + st * kBBytes + q * 8192, &map_s, &bars->b_full[st], t.col * kTileN + q * 64, t.key0 + c * kChunk);
+        }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc(1, kTileM, kTileN, 0, 1);  // bf16, A K-major, B MN-major
+      constexpr uint32_t idesc_all = instr_desc(1, kTileM, kTileN, 0, 1);  // bf16, A K-major, B MN-major
+      constexpr uint32_t idesc_zeta = instr_desc(1, kTileM, 64, 0, 1);
       const uint32_t a_addr = smem_u32(smem + kOffA), b_addr = smem_u32(smem + kOffB);
       bool ok = true;
-      for (int c = 0; c < chunks && ok; ++c) {
-        const int st = c % kStages;
-        const uint32_t par = (c / kStages) & 1;
-        ok = mbar_wait(&bars->a_full[st], par, abort_flag, status, 402) &&
-             mbar_wait(&bars->b_full[st], par, abort_flag, status, 403);
-        if (!ok) break;
+      int kc = 0, it = 0;
+      for (int id = blockIdx.x; ok && id < p.tiles; id += step, ++it) {
+        const Tile t = tile_at<kFlat>(p, id);
+        const uint32_t idesc = t.col == kColTiles - 1 ? idesc_zeta : idesc_all;
+        const uint32_t acc = tmem + (it & 1) * kTileN;
+        if (!(ok = mbar_wait(&bars->acc_empty[it & 1], ((it >> 1) & 1) ^ 1, abort_flag, p.status, 406))) break;
         tc_fence_after();
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t a = smem_desc(a_addr + st * kABytes + kk * 32, 16, 1024, kSwizzle128);
-          const uint64_t b = smem_desc(b_addr + st * kBBytes + kk * 2048, 8192, 1024, kSwizzle128);
-          mma_f16(tmem, a, b, idesc, (c > 0 || kk > 0) ? 1u : 0u);
-        }
-        mma_commit(&bars->empty[st]);
-      }
-      if (ok) mma_commit(&bars->acc_full);
-    }
-  } else {
-    const int quarter = warp & 3;
-    const int r = quarter * 32 + lane;  // accumulator row = TMEM lane = row row0 + r
-    const int row = row0 + r;
-    const bool row_ok = row < row_limit;
-    const int own0 = row_ok ? row / nb * nb : 0;  // first key of this row's (b, h)
-    const signed char* row_ptr = cls + static_cast<size_t>(row_ok ? row : 0) * nb;
-    bool ok = true;
-    // Chunk c covers keys key0 + 64 c ..; of those, positions p_lo .. p_hi - 1 belong to this row's (b, h) and have a
-    // class byte, at row_ptr + (key - own0).  The bytes travel as the aligned 32-bit words that hold them (rows start
-    // at any byte; words without an in-range byte are not read), fetched one chunk ahead, so that the latency hides
-    // behind the wait for the stage and the expansion.
-    auto fetch = [&](int c, uint32_t w[17]) {
-      const int j0 = key0 + c * kChunk - own0;  // class-byte index of position 0: negative before the row's keys
-      const int p_lo = max(0, -j0), p_hi = min(kChunk, nb - j0);
-      const intptr_t addr = reinterpret_cast<intptr_t>(row_ptr) + j0;
-      const uint32_t* wp = reinterpret_cast<const uint32_t*>(addr & ~intptr_t(3));
-      const int a = static_cast<int>(addr & 3);  // word k holds positions 4 k - a .. 4 k - a + 3
-      const int k_lo = (p_lo + a) >> 2;          // first and one-past-last word with an in-range byte
-      const int k_n = (row_ok && c < chunks) ? ((p_hi + a + 3) >> 2) - k_lo : 0;
-#pragma unroll
-      for (int k = 0; k < 17; ++k) w[k] = static_cast<unsigned>(k - k_lo) < static_cast<unsigned>(max(k_n, 0)) ? __ldg(wp + k) : 0u;
-    };
-    auto realign = [&](int c, const uint32_t (&w)[17], uint32_t (&m)[16]) {
-      const int j0 = key0 + c * kChunk - own0;
-      const int p_lo = max(0, -j0), p_hi = min(kChunk, nb - j0);
-      const uint32_t shift = static_cast<uint32_t>((reinterpret_cast<intptr_t>(row_ptr) + j0) & 3) * 8u;
-      // realigned class bytes; bit 0 of a class (0 negligible, 1 marginal, 2 critical) says "marginal"
-#pragma unroll
-      for (int k = 0; k < 16; ++k) m[k] = __funnelshift_r(w[k], w[k + 1], shift) & 0x01010101u;
-      if (p_lo > 0 || p_hi < kChunk) {  // positions outside the row's keys hold other rows' bytes
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          const int lo = min(max(p_lo - 4 * k, 0), 4), hi = min(max(p_hi - 4 * k, 0), 4);  // bytes lo .. hi - 1 stay
-          const uint32_t keep = lo < hi ? (0xFFFFFFFFu >> (32 - 8 * hi)) & (0xFFFFFFFFu << (8 * lo)) : 0u;
-          m[k] &= keep;
-        }
-      }
-    };
-    auto expand = [&](int st, const uint32_t (&m)[16]) {
-      uint8_t* arow = smem + kOffA + st * kABytes + r * 128;
-#pragma unroll
-      for (int ch = 0; ch < 8; ++ch) {  // 8 mask entries (two class words) per 16-byte chunk
-        // bytes (b0 b1 b2 b3) of 0/1 -> bf16 pairs: (b0 | b1 << 16) * 0x3F80 has 1.0 where the byte is 1
-        const uint32_t lo = m[2 * ch], hi = m[2 * ch + 1];
-        const uint32_t o0 = __byte_perm(lo, 0u, 0x4140) * 0x3F80u, o1 = __byte_perm(lo, 0u, 0x4342) * 0x3F80u;
-        const uint32_t o2 = __byte_perm(hi, 0u, 0x4140) * 0x3F80u, o3 = __byte_perm(hi, 0u, 0x4342) * 0x3F80u;
-        *reinterpret_cast<uint4*>(arow + ((ch ^ (r & 7)) << 4)) = make_uint4(o0, o1, o2, o3);
-      }
-    };
-    uint32_t w[17];
-    if constexpr (kFlat) {
-      fetch(0, w);
-      for (int c = 0; c < chunks; ++c) {
-        const int st = c % kStages;
-        uint32_t m[16];
-        realign(c, w, m);
-        fetch(c + 1, w);
-        if (!(ok = mbar_wait(&bars->empty[st], ((c / kStages) & 1) ^ 1, abort_flag, status, 404))) break;
-        expand(st, m);
-        fence_proxy_async_smem();
-        mbar_arrive(&bars->a_full[st]);
-      }
-    } else {
-      // Inside one (b, h) every chunk but the last holds 64 keys of every row.  Sixteen lanes then take the sixteen groups
-      // of four keys of one row: a load reads two rows' 64 bytes instead of touching 32 lines (what a chunk otherwise waits
-      // for: 17 loads of one word per row and thread take the first-level cache three times as long as the product
-      // takes the tensor pipe), and a store writes two whole 128-byte operand rows.  The words of the next chunk are
-      // requested before this one's are expanded, those of the last chunk, one row per thread as above, before the first.
-      // 16 heads, 2147 blocks: 697 -> 570 us.
-      const int whole = (nb - 1) / kChunk;  // chunks that end before the row's last key
-      fetch(whole, w);
-      const int sub = lane >> 4, kg = lane & 15;
-      const int first = quarter * 32 + sub;  // rows first, first + 2, ... of the tile
-      const char* const base = reinterpret_cast<const char*>(cls) + static_cast<size_t>(key0) * nb + 4 * kg;
-      const int top = row_limit - key0 - 1;  // rows past the (b, h) read its last row; their sums are not stored
-      auto fetch2 = [&](int c, uint32_t (&w0)[16], uint32_t (&w1)[16]) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const char* const p = base + static_cast<size_t>(min(row0 - key0 + first + 2 * i, top)) * nb + c * kChunk;
-          const uint32_t* const wp = reinterpret_cast<const uint32_t*>(reinterpret_cast<intptr_t>(p) & ~intptr_t(3));
-          w0[i] = __ldg(wp);
-          w1[i] = __ldg(wp + 1);  // (a row that starts on a word does not need it; it still lies inside the array)
-        }
-      };
-      uint32_t w0[16], w1[16];
-      if (whole > 0) fetch2(0, w0, w1);
-      for (int c = 0; c < chunks; ++c) {
-        const int st = c % kStages;
-        uint32_t m[16];
-        if (c < whole) {
-          // byte address of row first + 2 i modulo 4, times 8: the shift that realigns its words
-          const uint32_t shift0 = (static_cast<uint32_t>(reinterpret_cast<intptr_t>(base)) + static_cast<uint32_t>(nb) * (row0 - key0 + first)) * 8u;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) m[i] = __funnelshift_r(w0[i], w1[i], shift0 + 16u * i * static_cast<uint32_t>(nb)) & 0x01010101u;
-          if (c + 1 < whole) fetch2(c + 1, w0, w1);
-        } else {
-          realign(c, w, m);
-        }
-        if (!(ok = mbar_wait(&bars->empty[st], ((c / kStages) & 1) ^ 1, abort_flag, status, 404))) break;
-        if (c < whole) {
-          const uint32_t a_row = smem_u32(smem + kOffA) + st * kABytes + first * 128 + (kg & 1) * 8;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const uint32_t o0 = __byte_perm(m[i], 0u, 0x4140) * 0x3F80u, o1 = __byte_perm(m[i], 0u, 0x4342) * 0x3F80u;
-            const uint32_t at = a_row + i * 256 + (((kg >> 1) ^ ((2 * i + sub) & 7)) << 4);
-            asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at), "r"(o0), "r"(o1) : "memory");
+        for (int c = 0; c < t.chunks; ++c, ++kc) {
+          const int st = kc % kStages;
+          const uint32_t par = (kc / kStages) & 1;
+          ok = mbar_wait(&bars->b_full[st], par, abort_flag, p.status, 403) &&
+               mbar_wait(&bars->a_full[st], par, abort_flag, p.status, 402);
+          if (!ok) break;
+          tc_fence_after();
+          for (int kk = 0; kk < 4; ++kk) {
+            const uint64_t a = smem_desc(a_addr + st * kABytes + kk * 32, 16, 1024, kSwizzle128);
+            const uint64_t b = smem_desc(b_addr + st * kBBytes + kk * 2048, 8192, 1024, kSwizzle128);
+            mma_f16(acc, a, b, idesc, (c > 0 || kk > 0) ? 1u : 0u);
           }
-        } else {
-          expand(st, m);
+          mma_commit(&bars->empty[st]);
         }
-        fence_proxy_async_smem();
-        mbar_arrive(&bars->a_full[st]);
+        if (ok) mma_commit(&bars->acc_full[it & 1]);
       }
     }
-    if (ok && (ok = mbar_wait(&bars->acc_full, 0, abort_flag, status, 405))) {
-      tc_fence_after();
-      const uint32_t lane_addr = tmem + ((static_cast<uint32_t>(quarter) * 32u) << 16);
-      // A thread owns one accumulator row, so direct stores would touch 32 different lines per instruction.  Each
-      // warp turns its 32 rows x 128 bytes (64 bf16 columns) around in shared memory (the operand stages are free:
-      // every MMA has completed) and stores whole 128-byte row segments, four rows per instruction.
-      uint8_t* const stage = smem + quarter * 4096;
-#pragma unroll 1
-      for (int pp = 0; pp < kTileN / 64; ++pp) {
-        const int n = n_tile * kTileN + pp * 64;
-        if (n >= kSummaryRow) break;
-        if (n < kHeadDim * kHeadDim) {
-          uint32_t pk[32];
+  } else if (warp >= 4 && warp < 4 + 4 * kBuilders) {
+    // Eight lanes take the eight groups of eight keys of one row, a warp four rows at a time, eight times.  The class bytes
+    // of a group travel as the three aligned words that hold them (rows start at any byte), requested a chunk of the
+    // warpgroup's ahead, so that the latency hides behind the wait for the stage and the expansion: loads read whole
+    // 64-byte rows, stores write whole 128-byte operand rows.
+    const int group = (warp - 4) >> 2, quarter = warp & 3;
+    const int first = quarter * 32 + (lane >> 3);  // rows first, first + 4, ... of the tile
+    const int kg = lane & 7;
+    // the warpgroup's position: tile, its chunk, chunks so far
+    struct At {
+      Tile t;
+      int id, c, kc, own;  // own (flat): first key of the (b, h) of row `first`
+    };
+    auto enter = [&](At& at) {
+      at.t = tile_at<kFlat>(p, at.id);
+      at.own = kFlat ? divide(min(at.t.row0 + first, p.total_rows - 1), p.nb, p.inverse) * p.nb : at.t.key0;
+    };
+    auto settle = [&](At& at) {  // carries a chunk number past the tile's end over to the next tiles
+      while (at.id < p.tiles && at.c >= at.t.chunks) {
+        at.c -= at.t.chunks;
+        at.id += step;
+        if (at.id < p.tiles) enter(at);
+      }
+    };
+    // Calls fn(i, row, own) for the lane's eight rows: row (clamped to the tile's last) and first key of its (b, h).
+    auto each_row = [&](const At& at, auto fn) {
+      int own = at.own;
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            uint32_t v[32];
-            tmem_ld32(lane_addr + pp * 64 + half * 32, v);
+      for (int i = 0; i < 8; ++i) {
+        const int row = min(at.t.row0 + first + 4 * i, at.t.row_limit - 1);
+        if constexpr (kFlat) {
+          if (p.nb >= 4)
+            own += row - own >= p.nb ? p.nb : 0;
+          else
+            own = divide(row, p.nb, p.inverse) * p.nb;
+        }
+        fn(i, row, own);
+      }
+    };
+    // Whether every position of the chunk is a key of every row, and of none its last (a word behind it is then still
+    // inside the class matrix).
+    auto whole = [&](const At& at) { return !kFlat && (at.c + 1) * kChunk < p.nb; };
+    const intptr_t cls0 = reinterpret_cast<intptr_t>(p.cls);
+    auto fetch = [&](const At& at, uint32_t (&w)[8][3]) {
+      if (at.id >= p.tiles) return;
+      const int key = at.t.key0 + at.c * kChunk + 8 * kg;  // the group's first
+      if (whole(at)) {
+        each_row(at, [&](int i, int row, int own) {
+          const uint32_t* const wp = reinterpret_cast<const uint32_t*>((cls0 + static_cast<long long>(row) * p.nb + (key - own)) & ~intptr_t(3));
+#pragma unroll
+          for (int k = 0; k < 3; ++k) w[i][k] = static_cast<uint32_t>(ldg_pinned(reinterpret_cast<const int*>(wp + k)));
+        });
+      } else {
+        each_row(at, [&](int i, int row, int own) {
+          const intptr_t addr = cls0 + static_cast<long long>(row) * p.nb + (key - own);
+          const uint32_t* const wp = reinterpret_cast<const uint32_t*>(addr & ~intptr_t(3));
+          const int at0 = key - own - static_cast<int>(addr & 3);  // key number in its row of the first word's first byte
+#pragma unroll
+          for (int k = 0; k < 3; ++k)  // words without a byte of the row are not read
+            w[i][k] = at0 + 4 * k + 3 >= 0 && at0 + 4 * k < p.nb ? static_cast<uint32_t>(ldg_pinned(reinterpret_cast<const int*>(wp + k))) : 0u;
+        });
+      }
+    };
+    // A class byte (0 negligible, 1 marginal, 2 critical) picks the two bytes of its bf16 mask entry (0x3F80 for 1) from a
+    // table: b0 + 256 b1 times 0x11 are the four nibbles b0, b0, b1, b1 of a byte permutation's selector.
+    auto expand = [&](uint32_t bytes, uint32_t& o0, uint32_t& o1) {
+      const uint32_t sel = bytes * 0x11u + 0x40404040u;
+      o0 = __byte_perm(0x00008000u, 0x00003F00u, sel);
+      o1 = __byte_perm(0x00008000u, 0x00003F00u, sel >> 16);
+    };
+    // the group's eight class bytes of each row; zero outside the row's keys, where the words hold other rows' bytes
+    auto realign = [&](const At& at, const uint32_t (&w)[8][3], uint32_t (&m)[8][2]) {
+      const int key = at.t.key0 + at.c * kChunk + 8 * kg;
+      const bool all = whole(at);
+      each_row(at, [&](int i, int row, int own) {
+        const uint32_t shift = (static_cast<uint32_t>(cls0) + static_cast<uint32_t>(row) * static_cast<uint32_t>(p.nb) + static_cast<uint32_t>(key - own)) * 8u;
+        m[i][0] = __funnelshift_r(w[i][0], w[i][1], shift);  // (of the shift the lower five bits count)
+        m[i][1] = __funnelshift_r(w[i][1], w[i][2], shift);
+        if (!all) {
+          const int j = key - own;
+          const int from = min(max(-j, 0), 8), to = min(max(p.nb - j, 0), 8);  // bytes from .. to - 1 stay
+          const uint64_t keep = from < to ? (~0ull >> (64 - 8 * to)) & (~0ull << (8 * from)) : 0ull;
+          m[i][0] &= static_cast<uint32_t>(keep);
+          m[i][1] &= static_cast<uint32_t>(keep >> 32);
+        }
+      });
+    };
+    At at;
+    at.id = blockIdx.x;
+    at.c = at.kc = group;
+    if (at.id < p.tiles) enter(at);
+    settle(at);
+    uint32_t w[8][3];
+    fetch(at, w);
+    while (at.id < p.tiles) {
+      uint32_t m[8][2];
+      realign(at, w, m);
+      const int st = at.kc % kStages;
+      const uint32_t parity = ((at.kc / kStages) & 1) ^ 1;
+      at.c += kBuilders;
+      at.kc += kBuilders;
+      settle(at);
+      fetch(at, w);  // the warpgroup's next chunk
+      if (!mbar_wait(&bars->empty[st], parity, abort_flag, p.status, 404)) break;
+      const uint32_t base = smem_u32(smem + kOffA) + st * kABytes + first * 128;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        uint32_t o[4];
+        expand(m[i][0], o[0], o[1]);
+        expand(m[i][1], o[2], o[3]);
+        sts128(base + i * 512 + ((kg ^ ((first + 4 * i) & 7)) << 4), o[0], o[1], o[2], o[3]);
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->a_full[st]);
+    }
+  } else if (warp >= 4 + 4 * kBuilders) {
+    const int which = (warp - 4 - 4 * kBuilders) >> 2;  // accumulator
+    const int quarter = warp & 3;
+    const uint32_t lane_addr = tmem + which * kTileN + ((static_cast<uint32_t>(quarter) * 32u) << 16);
+    // A thread owns one accumulator row, so direct stores would touch 32 different lines per instruction.  Each
+    // warp turns its 32 rows x 128 bytes (64 bf16 columns) around in shared memory and stores whole 128-byte row
+    // segments, four rows per instruction.
+    uint8_t* const stage = smem + kOffOut + (warp - 4 - 4 * kBuilders) * 4096;
+    int n = 0;  // tiles of this accumulator so far
+    for (int id = blockIdx.x + which * step; id < p.tiles; id += 2 * step, ++n) {
+      const Tile t = tile_at<kFlat>(p, id);
+      if (!mbar_wait(&bars->acc_full[which], n & 1, abort_flag, p.status, 405)) break;
+      tc_fence_after();
+      const int row_w = t.row0 + quarter * 32;  // the warp's first row
+      if (t.col < kColTiles - 1) {
+#pragma unroll 1
+        for (int pp = 0; pp < kTileN / 64; ++pp) {
+          uint32_t pk[32];
+          {
+            uint32_t v0[32], v1[32];
+            tmem_ld32(lane_addr + pp * 64, v0);
+            tmem_ld32(lane_addr + pp * 64 + 32, v1);
             tmem_wait_ld();
 #pragma unroll
             for (int x = 0; x < 16; ++x) {
-              __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[2 * x]), __uint_as_float(v[2 * x + 1]));
-              pk[half * 16 + x] = *reinterpret_cast<uint32_t*>(&h);
+              __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v0[2 * x]), __uint_as_float(v0[2 * x + 1]));
+              pk[x] = *reinterpret_cast<uint32_t*>(&h);
+              h = __floats2bfloat162_rn(__uint_as_float(v1[2 * x]), __uint_as_float(v1[2 * x + 1]));
+              pk[16 + x] = *reinterpret_cast<uint32_t*>(&h);
             }
+          }
+          if (pp == kTileN / 64 - 1) {  // the accumulator has been read
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->acc_empty[which]);
           }
 #pragma unroll
           for (int ch = 0; ch < 8; ++ch)
@@ -276,27 +347,31 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const signed cha
                 make_uint4(pk[4 * ch], pk[4 * ch + 1], pk[4 * ch + 2], pk[4 * ch + 3]);
           __syncwarp();
           const int ch = lane & 7;
+          __nv_bfloat16* const dst = p.g16 + static_cast<size_t>(row_w) * (kHeadDim * kHeadDim) + t.col * kTileN + pp * 64 + ch * 8;
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
             const int rr = 4 * k + (lane >> 3);
-            const int ir = row0 + quarter * 32 + rr;
             const uint4 val = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((ch ^ (rr & 7)) << 4));
-            if (ir < row_limit)
-              *reinterpret_cast<uint4*>(g16 + static_cast<size_t>(ir) * kHeadDim * kHeadDim + n + ch * 8) = val;
+            if (row_w + rr < t.row_limit) *reinterpret_cast<uint4*>(dst + static_cast<size_t>(rr) * (kHeadDim * kHeadDim)) = val;
           }
           __syncwarp();
-        } else {
+        }
+      } else {
+        uint32_t v0[32], v1[32];
+        tmem_ld32(lane_addr, v0);
+        tmem_ld32(lane_addr + 32, v1);
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->acc_empty[which]);
+        if (row_w + lane < t.row_limit) {
+          float4* dst = reinterpret_cast<float4*>(p.zeta + static_cast<size_t>(row_w + lane) * kHeadDim);
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            uint32_t v[32];
-            tmem_ld32(lane_addr + pp * 64 + half * 32, v);
-            tmem_wait_ld();
-            if (!row_ok) continue;
-            float4* dst = reinterpret_cast<float4*>(zeta + static_cast<size_t>(row) * kHeadDim + (n - kHeadDim * kHeadDim) + half * 32);
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              dst[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                                   __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+          for (int q = 0; q < 8; ++q) {
+            dst[q] = make_float4(__uint_as_float(v0[4 * q]), __uint_as_float(v0[4 * q + 1]), __uint_as_float(v0[4 * q + 2]),
+                                 __uint_as_float(v0[4 * q + 3]));
+            dst[8 + q] = make_float4(__uint_as_float(v1[4 * q]), __uint_as_float(v1[4 * q + 1]), __uint_as_float(v1[4 * q + 2]),
+                                     __uint_as_float(v1[4 * q + 3]));
           }
         }
       }
@@ -323,20 +398,18 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   if (st != LITE3R_OK) return st;
   if (rows > 0x7FFFFFFFull - kTileM) return LITE3R_ERR_UNSUPPORTED;
   const int total_rows = static_cast<int>(rows), bh = s.batch * s.heads;
-  // Tiles through the (b, h) boundaries pay with a longer reduction (the keys of every (b, h) a tile touches), tiles
-  // inside one (b, h) with padding when Nb is not a multiple of 128.  Estimate of either: waves of CTAs (two per SM)
-  // times the cost of a CTA, its set-up and drain counted as three 64-key chunks.  Measured, inside / flat in us: 16 (b, h)
-  // of 129 blocks 19.5 / 17.4, of 172 19.5 / 23.6, of 687 91 / 107; 64 of 64 blocks 23.6 / 19.5, of 86 29.7 / 31.7, of 172
-  // 60.4 / 56.3, of 200 66.6 / 70.7; 512 of 22 blocks 128 / 48, of 64 140 / 106, of 86 179 / 175, of 100 187 / 214.  Of 46
-  // such pairs (2 to 512 (b, h), 5 to 2147 blocks) the estimate misses the faster one twice, by 2 and 4 us.
   int sms = 0;
   if ((st = sm_count(&sms)) != LITE3R_OK) return st;
-  constexpr double kFixed = 3.0;
-  const long long slots = 2ll * sms, col_tiles = ceil_div(kSummaryRow, kTileN);
-  const long long ctas_inside = col_tiles * bh * ceil_div(nb, kTileM);
-  // (a chunk inside one (b, h), whose mask tiles are read sixteen lanes to a row, takes four fifths of a flat one's time)
-  const double time_inside = static_cast<double>((ctas_inside + slots - 1) / slots) * (kFixed + 0.8 * ceil_div(nb, kChunk));
+  // Tiles through the (b, h) boundaries pay with a longer reduction (the keys of every (b, h) a tile touches) and with masks
+  // that have to be cut to every row's own keys, tiles inside one (b, h) with padding when Nb is not a multiple of 128.
+  // Estimate of either, in half microseconds: rounds of one tile per SM times the cost of a tile, 1.6 + one per chunk of 64
+  // keys inside a (b, h), 2.8 + 1.5 per chunk through the boundaries.  Measured, inside / flat in us: 16 (b, h) of 22 blocks
+  // 10.8 / 12.8, of 172 18.8 / 27.0, of 687 80 / 121; 64 of 64 blocks 18.9 / 20.9, of 172 43.5 / 57.8; 512 of 22 blocks 76 / 41,
+  // of 64 97 / 97, of 86 119 / 154.
   const long long row_tiles = ceil_div(total_rows, kTileM);
+  const long long tiles_inside = static_cast<long long>(kColTiles) * bh * ceil_div(nb, kTileM), tiles_flat = kColTiles * row_tiles;
+  if (tiles_inside > 0x7FFFFFFFll - 2 * sms || tiles_flat > 0x7FFFFFFFll - 2 * sms) return LITE3R_ERR_UNSUPPORTED;
+  const double time_inside = static_cast<double>((tiles_inside + sms - 1) / sms) * (1.6 + ceil_div(nb, kChunk));
   // chunks of a flat tile: one (b, h) when it starts and ends in the same one, else every (b, h) it touches
   double flat_chunks = 0.0;
   const long long probe = std::min<long long>(row_tiles, 4096);  // the pattern repeats; a prefix is representative
@@ -346,15 +419,23 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
     flat_chunks += ceil_div(k1 - k0, kChunk);
   }
   flat_chunks /= static_cast<double>(probe);
-  const long long ctas_flat = col_tiles * row_tiles;
-  const double time_flat = static_cast<double>((ctas_flat + slots - 1) / slots) * (kFixed + flat_chunks);
-  const int flat = time_flat < time_inside ? 1 : 0;
-  const dim3 grid(ceil_div(kSummaryRow, kTileN), flat ? ceil_div(total_rows, kTileM) : ceil_div(nb, kTileM), flat ? 1 : bh);
+  const double time_flat = static_cast<double>((tiles_flat + sms - 1) / sms) * (2.8 + 1.5 * flat_chunks);
+  const bool flat = time_flat < time_inside;
+  AggregateParams p;
+  p.cls = cls;
+  p.nb = nb;
+  p.total_rows = total_rows;
+  p.row_tiles = flat ? static_cast<int>(row_tiles) : ceil_div(nb, kTileM);
+  p.inverse = 1.f / static_cast<float>(flat ? nb : p.row_tiles);
+  p.tiles = static_cast<int>(flat ? tiles_flat : tiles_inside);
+  p.g16 = g16;
+  p.zeta = zeta;
+  p.status = device_status;
   auto* const kernel = flat ? aggregate_mma_kernel<true> : aggregate_mma_kernel<false>;
   st = ensure_dynamic_smem(kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
-  return launch_dependent(kernel, grid, kThreads, static_cast<int>(kSmemBytes), stream, map_s, cls, nb, total_rows, g16, zeta,
-                          device_status);
+  return launch_dependent(kernel, dim3(static_cast<unsigned>(std::min(p.tiles, sms))), kThreads, static_cast<int>(kSmemBytes), stream,
+                          map_s, p);
 }
 
 }  // namespace lite3r

@@ -214,6 +214,16 @@ def test_aggregation_inside_one_sequence(blocks):
     full_parity(wl, wk.make_inputs(wl), query_blocks=pu.sample_blocks(wl, [0, 2], 6))
 
 
+@pytest.mark.parametrize("batch,heads,blocks", [(40, 5, 1), (67, 3, 2), (50, 4, 3), (31, 7, 5), (40, 11, 21), (3, 2, 260)])
+def test_aggregation_tiles_of_persistent_ctas(batch, heads, blocks):
+    """Row tiles that run through many sequences of one to five key blocks (also fewer than four, where a step of four rows
+    skips whole sequences), and several tiles per CTA, inside a sequence and through the boundaries: ring and accumulators
+    go round."""
+    wl = small_workload(f"aggp{blocks}", batch=batch, heads=heads, tokens=blocks * 64 - 7, crit=0.0 if blocks == 1 else 0.2,
+                        neg=0.0 if blocks < 3 else 0.3)
+    full_parity(wl, wk.make_inputs(wl), query_blocks=pu.sample_blocks(wl, [0, heads - 1], min(150, batch * blocks)))
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("rows,d_in,d_out", [(18944, 256, 256), (18945, 256, 256), (9473, 1024, 512), (2500, 1152, 1984)])
 def test_linear_tiles_around_one_per_sm(rows, d_in, d_out, dtype):
