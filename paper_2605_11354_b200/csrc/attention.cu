@@ -626,8 +626,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const uint64_t pair = pack_f32x2(fv[y], fv[y + 1]);
             squares[y >> 1] = fma_f32x2(pair, pair, squares[y >> 1]);
             if (phi_softmax) {  // the softmax normaliser cancels in the ratio
-              e0 = ex2(fmaf(fv[y], cq, -shift));
-              e1 = ex2(fmaf(fv[y + 1], cq, -shift));
+              unpack_f32x2(fma_f32x2(pair, pack_f32x2(cq, cq), pack_f32x2(-shift, -shift)), e0, e1);
+              e0 = ex2(e0);
+              e1 = ex2(e1);
             } else {
               e0 = fv[y] > 0.f ? fmaf(fv[y], sq, 1.f) : ex2(fv[y] * cq);
               e1 = fv[y + 1] > 0.f ? fmaf(fv[y + 1], sq, 1.f) : ex2(fv[y + 1] * cq);
@@ -729,7 +730,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (p.k_marg > 0) {
       if (!(ok = mbar_wait_far(&bars->v_full[v_last % kStages], (v_last / kStages) & 1, abort_flag, p.status, 308))) break;
       const uint32_t zeta = smem_u32(smem + kOffZeta) + (it & 1) * 512 + hf * 256;
-      float den4[4] = {0.f, 0.f, 0.f, 0.f};
+      uint64_t den2[2] = {0ull, 0ull};  // bit pattern of (0.f, 0.f)
 #pragma unroll 1
       for (int c8 = 0; c8 < 8; ++c8) {  // 16-byte chunks of eight components
         const uint4 rw = lds128(phi_row + ((c8 ^ swz) << 4));
@@ -737,13 +738,16 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
           const uint4 z = lds128(zeta + c8 * 32 + half * 16);
-          den4[0] = fmaf(__uint_as_float(words[2 * half] << 16), __uint_as_float(z.x), den4[0]);
-          den4[1] = fmaf(__uint_as_float(words[2 * half] & 0xFFFF0000u), __uint_as_float(z.y), den4[1]);
-          den4[2] = fmaf(__uint_as_float(words[2 * half + 1] << 16), __uint_as_float(z.z), den4[2]);
-          den4[3] = fmaf(__uint_as_float(words[2 * half + 1] & 0xFFFF0000u), __uint_as_float(z.w), den4[3]);
+          den2[0] = fma_f32x2(pack_f32x2(__uint_as_float(words[2 * half] << 16), __uint_as_float(words[2 * half] & 0xFFFF0000u)),
+                              pack_f32x2(__uint_as_float(z.x), __uint_as_float(z.y)), den2[0]);
+          den2[1] = fma_f32x2(pack_f32x2(__uint_as_float(words[2 * half + 1] << 16), __uint_as_float(words[2 * half + 1] & 0xFFFF0000u)),
+                              pack_f32x2(__uint_as_float(z.z), __uint_as_float(z.w)), den2[1]);
         }
       }
-      den = (den4[0] + den4[1]) + (den4[2] + den4[3]);
+      float d0, d1, d2, d3;
+      unpack_f32x2(den2[0], d0, d1);
+      unpack_f32x2(den2[1], d2, d3);
+      den = (d0 + d1) + (d2 + d3);
       // (the last P V product is the one before)
       if (steps > 0 && !(ok = mbar_wait_far(&bars->v_done[(v_last - 1) % kStages], ((v_last - 1) / kStages) & 1, abort_flag, p.status, 304))) break;
     }
@@ -778,11 +782,21 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->s_free);
       }
-      // (without a critical block O, without a linear branch its product was never written)
+      if (steps == 0 || p.k_marg == 0) {  // without a critical block O, without a linear branch its product was never written
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const float o = steps > 0 ? __uint_as_float(v[k]) : 0.f, lin = p.k_marg > 0 ? __uint_as_float(u[k]) : 0.f;
-        v[k] = __float_as_uint(fmaf(lin, l_scale, o * inv_l));
+        for (int k = 0; k < 32; ++k) {
+          if (steps == 0) v[k] = 0u;
+          if (p.k_marg == 0) u[k] = 0u;
+        }
+      }
+      const uint64_t inv2 = pack_f32x2(inv_l, inv_l), lin2 = pack_f32x2(l_scale, l_scale);
+#pragma unroll
+      for (int k = 0; k < 32; k += 2) {
+        const uint64_t o = mul_f32x2(pack_f32x2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])), inv2);
+        float y0, y1;
+        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(u[k]), __uint_as_float(u[k + 1])), lin2, o), y0, y1);
+        v[k] = __float_as_uint(y0);
+        v[k + 1] = __float_as_uint(y1);
       }
       if (wide) {
 #pragma unroll
