@@ -390,7 +390,8 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
 }  // namespace
 
 lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls, const lite3r_shape& s, int nb,
-                               __nv_bfloat16* g16, float* zeta, int* device_status, cudaStream_t stream) {
+                               int attention_ctas, int steps, __nv_bfloat16* g16, float* zeta, int* device_status,
+                               cudaStream_t stream) {
   const uint64_t rows = static_cast<uint64_t>(s.batch) * s.heads * nb;
   CUtensorMap map_s;
   lite3r_status st = make_tensor_map_2d(&map_s, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hws, kSummaryRow, rows, 64, 64,
@@ -409,7 +410,6 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   const long long row_tiles = ceil_div(total_rows, kTileM);
   const long long tiles_inside = static_cast<long long>(kColTiles) * bh * ceil_div(nb, kTileM), tiles_flat = kColTiles * row_tiles;
   if (tiles_inside > 0x7FFFFFFFll - 2 * sms || tiles_flat > 0x7FFFFFFFll - 2 * sms) return LITE3R_ERR_UNSUPPORTED;
-  const double time_inside = static_cast<double>((tiles_inside + sms - 1) / sms) * (1.6 + ceil_div(nb, kChunk));
   // chunks of a flat tile: one (b, h) when it starts and ends in the same one, else every (b, h) it touches
   double flat_chunks = 0.0;
   const long long probe = std::min<long long>(row_tiles, 4096);  // the pattern repeats; a prefix is representative
@@ -419,8 +419,19 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
     flat_chunks += ceil_div(k1 - k0, kChunk);
   }
   flat_chunks /= static_cast<double>(probe);
-  const double time_flat = static_cast<double>((tiles_flat + sms - 1) / sms) * (2.8 + 1.5 * flat_chunks);
-  const bool flat = time_flat < time_inside;
+  auto rounds = [](long long tiles, long long ctas) { return static_cast<double>((tiles + ctas - 1) / ctas); };
+  auto time_on = [&](long long ctas, bool flat) {
+    return flat ? rounds(tiles_flat, ctas) * (2.8 + 1.5 * flat_chunks) : rounds(tiles_inside, ctas) * (1.6 + ceil_div(nb, kChunk));
+  };
+  // A CTA of this kernel fills its SM.  Where the whole attention grid finds room on the SMs that are left, it goes through its
+  // critical blocks (1.4 half microseconds a step) meanwhile: that many SMs are left to it if the aggregation on the others
+  // takes a microsecond less than on all of them and those steps together.  16 heads of 1374 tokens (176 attention CTAs of six steps): a whole
+  // pass 31.6 -> 27.4 us.
+  long long ctas = sms;
+  const long long spare = sms - ceil_div(attention_ctas, kAttentionCtasPerSm);
+  auto best_on = [&](long long n) { return std::min(time_on(n, true), time_on(n, false)); };
+  if (steps > 0 && spare > 0 && best_on(spare) + 2.0 < best_on(sms) + 1.4 * steps) ctas = spare;
+  const bool flat = time_on(ctas, true) < time_on(ctas, false);
   AggregateParams p;
   p.cls = cls;
   p.nb = nb;
@@ -434,7 +445,7 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   auto* const kernel = flat ? aggregate_mma_kernel<true> : aggregate_mma_kernel<false>;
   st = ensure_dynamic_smem(kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
-  return launch_dependent(kernel, dim3(static_cast<unsigned>(std::min(p.tiles, sms))), kThreads, static_cast<int>(kSmemBytes), stream,
+  return launch_dependent(kernel, dim3(static_cast<unsigned>(std::min<long long>(p.tiles, ctas))), kThreads, static_cast<int>(kSmemBytes), stream,
                           map_s, p);
 }
 

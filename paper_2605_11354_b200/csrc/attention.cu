@@ -53,7 +53,7 @@ using namespace sm100;
 constexpr int kCtrlWarps = 4;
 constexpr int kSoftmaxWarps = 4;
 constexpr int kThreads = (kCtrlWarps + kSoftmaxWarps) * 32;
-constexpr int kCtasPerSm = 3;
+constexpr int kCtasPerSm = kAttentionCtasPerSm;
 constexpr int kCtrlRegs = 48, kSoftmaxRegs = 112;  // 128 * 48 + 128 * 112 = 256 * 80, the launch allocation
 constexpr int kStepKeys = 64;
 constexpr int kStages = 2;  // K ring and V ring

@@ -220,8 +220,12 @@ lite3r_status launch_summary(const lite3r_fp8& k, const lite3r_fp8& v, const flo
                              cudaStream_t stream);
 
 // Marginal aggregation G_i = sum over marginal j of the summary rows, as a 0/1-mask GEMM on tensor cores.
+// attention_ctas, steps: CTAs of the attention kernel that runs beside it and the steps each makes before it needs the sums
+// (0: it does not run beside).
 lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls, const lite3r_shape& s, int nb,
-                               __nv_bfloat16* g16, float* zeta, int* device_status, cudaStream_t stream);
+                               int attention_ctas, int steps, __nv_bfloat16* g16, float* zeta, int* device_status,
+                               cudaStream_t stream);
+constexpr int kAttentionCtasPerSm = 3;
 
 // TMA descriptor of a row-major 2-D tensor [rows][inner] (row pitch in bytes, 0: inner * elem_bytes; a multiple of 16)
 // with a box of box_inner x box_rows elements.  The make_tensor_map functions keep what they have encoded (a few hundred

@@ -145,7 +145,9 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   if (a.plan_inside && counts.k_marg > 0 && (st = launch_plan(a.q, a.k, s, counts, plan, true, stream)) != LITE3R_OK) return st;
   if (a.plan.k_marg > 0) {
     profile_mark(4, stream);
-    if ((st = launch_aggregate(w.hws, plan.cls, s, nb, w.g16, w.zeta, a.device_status, stream)) != LITE3R_OK) return st;
+    const int attention_ctas = s.batch * s.heads * (BS == 64 ? (nb + 1) / 2 : nb);
+    const int steps = a.linear_only || profile_enabled() ? 0 : a.plan.k_crit * (BS / 64);
+    if ((st = launch_aggregate(w.hws, plan.cls, s, nb, attention_ctas, steps, w.g16, w.zeta, a.device_status, stream)) != LITE3R_OK) return st;
     profile_mark(5, stream);
   }
   AttentionLaunch att;

@@ -224,6 +224,26 @@ def test_aggregation_tiles_of_persistent_ctas(batch, heads, blocks):
     full_parity(wl, wk.make_inputs(wl), query_blocks=pu.sample_blocks(wl, [0, heads - 1], min(150, batch * blocks)))
 
 
+@pytest.mark.parametrize("batch,heads,tokens,block,crit", [(1, 16, 1374, 64, 0.25), (3, 5, 3001, 128, 0.15), (1, 16, 832, 64, 0.1),
+                                                           (1, 12, 1374, 128, 0.25), (2, 16, 1374, 64, 0.25), (1, 4, 12016, 64, 0.15)])
+def test_aggregation_beside_the_attention_kernel(batch, heads, tokens, block, crit):
+    """Attention grids that fit on the SMs a narrower aggregation leaves free, and grids that do not: the same output as with
+    the aggregation on all SMs (which is what it gets while stage times are taken)."""
+    wl = small_workload("beside", batch=batch, heads=heads, tokens=tokens, block=block, crit=crit, neg=0.5)
+    inputs = wk.make_inputs(wl)
+    eng, out = pu.run_gpu(inputs, wl)
+    again = torch.empty_like(out)
+    lt.profile_enable(True)
+    try:
+        eng.forward(torch.from_numpy(inputs["proj"]).cuda(), out=again)
+    finally:
+        lt.profile_enable(False)
+    assert int(eng.status.item()) == 0
+    for _ in range(3):
+        eng.forward(torch.from_numpy(inputs["proj"]).cuda(), out=out)
+        assert torch.equal(out, again)
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("rows,d_in,d_out", [(18944, 256, 256), (18945, 256, 256), (9473, 1024, 512), (2500, 1152, 1984)])
 def test_linear_tiles_around_one_per_sm(rows, d_in, d_out, dtype):
