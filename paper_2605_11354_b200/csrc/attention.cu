@@ -293,6 +293,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     bars->abort = 0;
     mbar_fence_init();
   }
+  if (warp == 3 && lane == 0) {  // fetched while barriers and tensor memory are set up
+    tma_prefetch_desc(&map_q);
+    tma_prefetch_desc(&map_k);
+    tma_prefetch_desc(&map_v);
+    tma_prefetch_desc(&map_g);
+    tma_prefetch_desc(&map_o);
+  }
   if (warp == 1) {
     tmem_alloc(&bars->tmem_p, kColsP);
     tmem_alloc(&bars->tmem_s, kColsS);
