@@ -424,13 +424,21 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
     return flat ? rounds(tiles_flat, ctas) * (2.8 + 1.5 * flat_chunks) : rounds(tiles_inside, ctas) * (1.6 + ceil_div(nb, kChunk));
   };
   // A CTA of this kernel fills its SM.  Where the whole attention grid finds room on the SMs that are left, it goes through its
-  // critical blocks (1.4 half microseconds a step) meanwhile: that many SMs are left to it if the aggregation on the others
-  // takes a microsecond less than on all of them and those steps together.  16 heads of 1374 tokens (176 attention CTAs of six steps): a whole
-  // pass 31.6 -> 27.4 us.
+  // critical blocks meanwhile: that many SMs are left to it if the longer of the two is then at least a microsecond shorter than
+  // one after the other on all SMs.  A step of the attention kernel takes 1.4 / 1.65 / 2 half microseconds with one / two / three
+  // of its CTAs on an SM.  16 heads of 1374 tokens (176 attention CTAs of six steps): a whole pass 31.5 -> 27.3 us; 15 of 3001 in
+  // blocks of 128 43.6 -> 40.6 us.
   long long ctas = sms;
   const long long spare = sms - ceil_div(attention_ctas, kAttentionCtasPerSm);
-  auto best_on = [&](long long n) { return std::min(time_on(n, true), time_on(n, false)); };
-  if (steps > 0 && spare > 0 && best_on(spare) + 2.0 < best_on(sms) + 1.4 * steps) ctas = spare;
+  if (steps > 0 && spare > 0) {
+    auto best_on = [&](long long n) { return std::min(time_on(n, true), time_on(n, false)); };
+    auto steps_on = [&](long long n) {
+      const long long per_sm = (attention_ctas + n - 1) / n;
+      return steps * (per_sm <= 1 ? 1.4 : per_sm == 2 ? 1.65 : 2.0);
+    };
+    const long long taken = std::min(spare, time_on(spare, true) < time_on(spare, false) ? tiles_flat : tiles_inside);
+    if (std::max(best_on(spare), steps_on(sms - taken)) + 2.0 < best_on(sms) + steps_on(sms)) ctas = spare;
+  }
   const bool flat = time_on(ctas, true) < time_on(ctas, false);
   AggregateParams p;
   p.cls = cls;
