@@ -16,10 +16,9 @@
 // clocks of tensor pipe at block 64 (M = 64 runs at half rate) and 192 at block 128.  A warp alone needs some 1100 clocks
 // for its 32 x 64 scores (loads, stores and barriers included), so two warps per scheduler are the least that can keep
 // the unit busy: S, P and O take 160 TMEM columns, 74 KB of shared memory and 80 registers per thread, and THREE CTAs fit
-// on an SM.  Measured at 10 % of 2147 key blocks: 654 clocks per step and SM by the cycle counter (two CTAs with two
-// softmax warpgroups each on alternate steps of one tile, as before: 757).  No unit is saturated (at 5 % of 687 blocks:
-// exponentials 64 %, issue slots 60 %, tensor pipe 54 %): a warp takes maximum, vote and exponentials of a step one after
-// the other, and three warps per scheduler do not fill each other's gaps.
+// on an SM (two CTAs with two softmax warpgroups each on alternate steps of one tile: 757 clocks per step and SM at 10 % of
+// 2147 key blocks, three CTAs 654 with a maximum in every step).  No unit is saturated; what the softmax warps issue decides
+// (see kHeadroom).
 // A CTA takes tile after tile: it asks the hardware's work scheduler for a CTA that has not been launched yet and computes
 // that one's tile itself (taken only where the grid is larger than the chip holds and a tile has products).  The next tile's Q, K and V tiles and
 // its first scores are then under way while the softmax warps write this tile's output, and what lies between two tiles
@@ -81,7 +80,7 @@ constexpr uint32_t kOffV = kOffK + kStages * kStageK;
 constexpr uint32_t kOffPhi = kOffV + kStages * kStageV;  // phi(Q) as bf16 A operand of the linear product (16 KB); after
                                                          // that product the output rows, each warp in its own rows' place
 constexpr uint32_t kOffZeta = kOffPhi + 16384;           // zeta_i of the linear branch (256 B per query block), two tiles
-constexpr uint32_t kOffScal = kOffZeta + 1024;           // per step and query block: {exponent factor, valid keys}
+constexpr uint32_t kOffScal = kOffZeta + 1024;           // per ring entry and query block: {exponent factor, bound and valid keys}
 constexpr uint32_t kOffNext = kOffScal + kScalSlots * 16;  // answer of the work scheduler (16 B), tile numbers (4 x 4 B)
 constexpr uint32_t kOffBar = kOffNext + 32;
 constexpr uint32_t kSmemBytes = kOffBar + 256;           // three CTAs per SM: 3 * (76064 + 1024 reserved) <= 233472
