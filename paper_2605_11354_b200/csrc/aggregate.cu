@@ -102,7 +102,10 @@ __device__ __forceinline__ Tile tile_at(const AggregateParams& p, int id) {
   return t;
 }
 
-template <bool kFlat>
+// kShare: the mask warpgroups share every chunk's rows instead of taking every other chunk, which gets a tile under way sooner but
+// pays each chunk's waits twice: for grids whose CTAs have one tile each (16 heads of 832 tokens 24.3 -> 23.4 us a pass; 16 heads
+// of 687 blocks, eleven tiles to a CTA, 80 -> 99 us alone).
+template <bool kFlat, bool kShare>
 __global__ void __launch_bounds__(kThreads, 1)
 aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateParams p) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -117,7 +120,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(&bars->a_full[s], 4);  // one arrival per warp
+      mbar_init(&bars->a_full[s], kShare ? 4 * kBuilders : 4);  // one arrival per warp
       mbar_init(&bars->b_full[s], 1);
       mbar_init(&bars->empty[s], 1);
     }
@@ -190,12 +193,14 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
       }
     }
   } else if (warp >= 4 && warp < 4 + 4 * kBuilders) {
-    // Eight lanes take the eight groups of eight keys of one row, a warp four rows at a time, eight times.  The class bytes
-    // of a group travel as the three aligned words that hold them (rows start at any byte), requested a chunk of the
-    // warpgroup's ahead, so that the latency hides behind the wait for the stage and the expansion: loads read whole
+    // Eight lanes take the eight groups of eight keys of one row, a warp four rows at a time, eight times (sharing: four
+    // times).  The class bytes of a group travel as the three aligned words that hold them (rows start at any byte), requested a chunk of
+    // the warpgroup's ahead, so that the latency hides behind the wait for the stage and the expansion: loads read whole
     // 64-byte rows, stores write whole 128-byte operand rows.
+    constexpr int kRows = kShare ? kTileM / (16 * kBuilders) : kTileM / 16;  // of a lane
+    constexpr int kStride = kShare ? 1 : kBuilders;                           // chunks from one of the warpgroup's to its next
     const int group = (warp - 4) >> 2, quarter = warp & 3;
-    const int first = quarter * 32 + (lane >> 3);  // rows first, first + 4, ... of the tile
+    const int first = ((kShare ? group * 4 : 0) + quarter) * 4 * kRows + (lane >> 3);  // rows first, first + 4, ... of the tile
     const int kg = lane & 7;
     // the warpgroup's position: tile, its chunk, chunks so far
     struct At {
@@ -213,11 +218,11 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
         if (at.id < p.tiles) enter(at);
       }
     };
-    // Calls fn(i, row, own) for the lane's eight rows: row (clamped to the tile's last) and first key of its (b, h).
+    // Calls fn(i, row, own) for the lane's rows: row (clamped to the tile's last) and first key of its (b, h).
     auto each_row = [&](const At& at, auto fn) {
       int own = at.own;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < kRows; ++i) {
         const int row = min(at.t.row0 + first + 4 * i, at.t.row_limit - 1);
         if constexpr (kFlat) {
           if (p.nb >= 4)
@@ -232,7 +237,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
     // inside the class matrix).
     auto whole = [&](const At& at) { return !kFlat && (at.c + 1) * kChunk < p.nb; };
     const intptr_t cls0 = reinterpret_cast<intptr_t>(p.cls);
-    auto fetch = [&](const At& at, uint32_t (&w)[8][3]) {
+    auto fetch = [&](const At& at, uint32_t (&w)[kRows][3]) {
       if (at.id >= p.tiles) return;
       const int key = at.t.key0 + at.c * kChunk + 8 * kg;  // the group's first
       if (whole(at)) {
@@ -260,7 +265,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
       o1 = __byte_perm(0x00008000u, 0x00003F00u, sel >> 16);
     };
     // the group's eight class bytes of each row; zero outside the row's keys, where the words hold other rows' bytes
-    auto realign = [&](const At& at, const uint32_t (&w)[8][3], uint32_t (&m)[8][2]) {
+    auto realign = [&](const At& at, const uint32_t (&w)[kRows][3], uint32_t (&m)[kRows][2]) {
       const int key = at.t.key0 + at.c * kChunk + 8 * kg;
       const bool all = whole(at);
       each_row(at, [&](int i, int row, int own) {
@@ -278,24 +283,24 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
     };
     At at;
     at.id = blockIdx.x;
-    at.c = at.kc = group;
+    at.c = at.kc = kShare ? 0 : group;
     if (at.id < p.tiles) enter(at);
     settle(at);
-    uint32_t w[8][3];
+    uint32_t w[kRows][3];
     fetch(at, w);
     while (at.id < p.tiles) {
-      uint32_t m[8][2];
+      uint32_t m[kRows][2];
       realign(at, w, m);
       const int st = at.kc % kStages;
       const uint32_t parity = ((at.kc / kStages) & 1) ^ 1;
-      at.c += kBuilders;
-      at.kc += kBuilders;
+      at.c += kStride;
+      at.kc += kStride;
       settle(at);
       fetch(at, w);  // the warpgroup's next chunk
       if (!mbar_wait(&bars->empty[st], parity, abort_flag, p.status, 404)) break;
       const uint32_t base = smem_u32(smem + kOffA) + st * kABytes + first * 128;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < kRows; ++i) {
         uint32_t o[4];
         expand(m[i][0], o[0], o[1]);
         expand(m[i][1], o[2], o[3]);
@@ -450,7 +455,9 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   p.g16 = g16;
   p.zeta = zeta;
   p.status = device_status;
-  auto* const kernel = flat ? aggregate_mma_kernel<true> : aggregate_mma_kernel<false>;
+  const bool share = p.tiles <= ctas;
+  auto* const kernel = flat ? (share ? aggregate_mma_kernel<true, true> : aggregate_mma_kernel<true, false>)
+                            : (share ? aggregate_mma_kernel<false, true> : aggregate_mma_kernel<false, false>);
   st = ensure_dynamic_smem(kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
   return launch_dependent(kernel, dim3(static_cast<unsigned>(std::min<long long>(p.tiles, ctas))), kThreads, static_cast<int>(kSmemBytes), stream,
