@@ -19,7 +19,7 @@
 // in shared memory so that stores write whole 128-byte segments, and store the first 4096 columns as bf16 (the attention
 // kernel's B operand) and the last 64 (zeta) as fp32.
 // Bound by shared memory: a chunk's products read 48 KB of operands in 512 clocks of tensor pipe, TMA writes 32 KB and the
-// masks 16 KB beside them.  Against two CTAs per SM of one tile each, which set up, filled their ring and drained one
+// masks 16 KB beside them.  Where a CTA has one tile it is a chain instead: masks, products, stores (see kOne).  Against two CTAs per SM of one tile each, which set up, filled their ring and drained one
 // after the other: 512 (b, h) of 22 / 86 blocks 49.6 / 177 -> 41.4 / 119 us, 64 of 172 62 -> 43.5 us, 16 of 172 / 687 / 2147
 // blocks 20.8 / 92 / 551 -> 18.8 / 80 / 548 us (4 of 2147, 7.8 tiles per SM: 140 -> 148 us).
 #include <algorithm>
@@ -102,10 +102,15 @@ __device__ __forceinline__ Tile tile_at(const AggregateParams& p, int id) {
   return t;
 }
 
-// kShare: the mask warpgroups share every chunk's rows instead of taking every other chunk, which gets a tile under way sooner but
-// pays each chunk's waits twice: for grids whose CTAs have one tile each (16 heads of 832 tokens 24.3 -> 23.4 us a pass; 16 heads
-// of 687 blocks, eleven tiles to a CTA, 80 -> 99 us alone).
-template <bool kFlat, bool kShare>
+// kOne: every CTA has one tile, and what counts is how soon its products can start.
+//   Inside a (b, h) the mask warpgroups then share every chunk's rows instead of taking every other chunk, which pays each
+//   chunk's waits twice (16 heads of 687 blocks, eleven tiles to a CTA, 80 -> 99 us alone).
+//   Through the boundaries, where a tile's keys fit into the ring, all its masks are made at once: operand tiles zeroed ahead
+//   of the wait for the plan, then a one written for every marginal entry of the tile's 128 Nb class bytes, which lie one after
+//   the other, four to a thread and turn.  Kernel alone, chunk by chunk / at once in us: 20 (b, h) of 15 blocks 8.3 / 6.2, 64 of
+//   8 7.6 / 5.7, 64 of 15 9.1 / 6.6, 32 of 22 8.6 / 6.3 (the last mask was ready 5100 clocks after the plan, products and stores
+//   take 4000 more); a whole pass of 4 x 5 (b, h) of 900 tokens 25.0 -> 21.6 us, of 2 x 16 of 1374 40.0 -> 37.5.
+template <bool kFlat, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1)
 aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateParams p) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -117,10 +122,12 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
   }
   const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int step = static_cast<int>(gridDim.x);
+  constexpr bool kAtOnce = kFlat && kOne, kShare = !kFlat && kOne;
+  constexpr int kAtOnceThreads = (kBuilders + kDrainers) * 128;  // (the storing warps have nothing else to do yet)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(&bars->a_full[s], kShare ? 4 * kBuilders : 4);  // one arrival per warp
+      mbar_init(&bars->a_full[s], kAtOnce ? kAtOnceThreads / 32 : kShare ? 4 * kBuilders : 4);  // one arrival per warp
       mbar_init(&bars->b_full[s], 1);
       mbar_init(&bars->empty[s], 1);
     }
@@ -135,6 +142,10 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
     tmem_alloc(&bars->tmem_base, kTmemCols);
     tmem_relinquish();
   }
+  if (kAtOnce && warp >= 4) {
+    const uint32_t bytes = tile_at<kFlat>(p, blockIdx.x).chunks * kABytes;
+    for (uint32_t at = (threadIdx.x - 128) * 16; at < bytes; at += kAtOnceThreads * 16) sts128(smem_u32(smem + kOffA) + at, 0u, 0u, 0u, 0u);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -145,6 +156,42 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
   // itself before it reads G and zeta).
   sm100::launch_dependents();
 
+  if (kAtOnce && warp >= 4) {
+    // The class bytes of the tile's rows, in the aligned words that hold them, two words to a thread and turn.
+    const Tile t = tile_at<kFlat>(p, blockIdx.x);
+    const char* const first = reinterpret_cast<const char*>(p.cls) + static_cast<long long>(t.row0) * p.nb;
+    const int ahead = static_cast<int>(reinterpret_cast<intptr_t>(first) & 3);  // bytes of the first word before the tile's
+    const int bytes = (min(t.row0 + kTileM, t.row_limit) - t.row0) * p.nb;
+    const int words = (ahead + bytes + 3) >> 2;
+    const int* const src = reinterpret_cast<const int*>(first - ahead);
+    const int own0 = t.row0 - t.key0;  // row 0 of the tile inside its (b, h)
+    for (int w = threadIdx.x - 128; w < words; w += 2 * kAtOnceThreads) {
+      uint32_t four[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) four[k] = w + k * kAtOnceThreads < words ? static_cast<uint32_t>(ldg_pinned(src + w + k * kAtOnceThreads)) : 0u;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int e0 = 4 * (w + k * kAtOnceThreads) - ahead;  // entry of the word's first byte
+        int row = divide(max(e0, 0), p.nb, p.inverse), col = e0 - row * p.nb;
+        int own = divide(own0 + row, p.nb, p.inverse) * p.nb;  // first key of the row's (b, h), from the tile's
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          if (((four[k] >> (8 * b)) & 0xFFu) == 1u && e0 + b >= 0 && e0 + b < bytes) {
+            const int key = own + col;
+            sts16(smem_u32(smem + kOffA) + (key >> 6) * kABytes + row * 128 + ((((key >> 3) & 7) ^ (row & 7)) << 4) + (key & 7) * 2, 0x3F80u);
+          }
+          if (++col == p.nb) {
+            col = 0;
+            ++row;
+            own += own0 + row == own + p.nb ? p.nb : 0;
+          }
+        }
+      }
+    }
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bars->a_full[0]);
+  }
   if (warp == 0) {
     if (lane == 0) {
       tma_prefetch_desc(&map_s);
@@ -179,7 +226,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
           const int st = kc % kStages;
           const uint32_t par = (kc / kStages) & 1;
           ok = mbar_wait(&bars->b_full[st], par, abort_flag, p.status, 403) &&
-               mbar_wait(&bars->a_full[st], par, abort_flag, p.status, 402);
+               mbar_wait(&bars->a_full[kAtOnce ? 0 : st], par, abort_flag, p.status, 402);
           if (!ok) break;
           tc_fence_after();
           for (int kk = 0; kk < 4; ++kk) {
@@ -192,7 +239,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
         if (ok) mma_commit(&bars->acc_full[it & 1]);
       }
     }
-  } else if (warp >= 4 && warp < 4 + 4 * kBuilders) {
+  } else if (!kAtOnce && warp >= 4 && warp < 4 + 4 * kBuilders) {
     // Eight lanes take the eight groups of eight keys of one row, a warp four rows at a time, eight times (sharing: four
     // times).  The class bytes of a group travel as the three aligned words that hold them (rows start at any byte), requested a chunk of
     // the warpgroup's ahead, so that the latency hides behind the wait for the stage and the expansion: loads read whole
@@ -409,23 +456,28 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   // Tiles through the (b, h) boundaries pay with a longer reduction (the keys of every (b, h) a tile touches) and with masks
   // that have to be cut to every row's own keys, tiles inside one (b, h) with padding when Nb is not a multiple of 128.
   // Estimate of either, in half microseconds: rounds of one tile per SM times the cost of a tile, 1.6 + one per chunk of 64
-  // keys inside a (b, h), 2.8 + 1.5 per chunk through the boundaries.  Measured, inside / flat in us: 16 (b, h) of 22 blocks
-  // 10.8 / 12.8, of 172 18.8 / 27.0, of 687 80 / 121; 64 of 64 blocks 18.9 / 20.9, of 172 43.5 / 57.8; 512 of 22 blocks 76 / 41,
-  // of 64 97 / 97, of 86 119 / 154.
+  // keys inside a (b, h), 2.8 + 1.5 per chunk through the boundaries; where one round does and the masks are made at once,
+  // 1.2 + 1.4 per chunk + one per 32 blocks of a row (its class bytes).  Measured, inside / flat in us: 16 (b, h) of 172 blocks
+  // 14.5 / 21.7, of 687 80 / 121; 64 of 64 blocks 18.9 / 20.9, of 172 43.5 / 57.8; 512 of 22 blocks 71 / 37, of 64 97 / 97, of 86
+  // 119 / 154; with the masks at once 4 (b, h) of 22 blocks 4.7 / 5.6, 10 of 15 5.6 / 6.2, 15 of 64 6.5 / 6.9, 16 of 22 6.3 / 6.2,
+  // 12 of 32 6.2 / 5.9, 20 of 15 7.3 / 6.2, 32 of 22 8.5 / 6.3, 64 of 8 12.8 / 5.7.
   const long long row_tiles = ceil_div(total_rows, kTileM);
   const long long tiles_inside = static_cast<long long>(kColTiles) * bh * ceil_div(nb, kTileM), tiles_flat = kColTiles * row_tiles;
   if (tiles_inside > 0x7FFFFFFFll - 2 * sms || tiles_flat > 0x7FFFFFFFll - 2 * sms) return LITE3R_ERR_UNSUPPORTED;
   // chunks of a flat tile: one (b, h) when it starts and ends in the same one, else every (b, h) it touches
   double flat_chunks = 0.0;
+  int most_chunks = 0;
   const long long probe = std::min<long long>(row_tiles, 4096);  // the pattern repeats; a prefix is representative
   for (long long t = 0; t < probe; ++t) {
     const int r0 = static_cast<int>(t) * kTileM;
     const int k0 = r0 / nb * nb, k1 = (std::min(r0 + kTileM, total_rows) - 1) / nb * nb + nb;
     flat_chunks += ceil_div(k1 - k0, kChunk);
+    most_chunks = std::max(most_chunks, ceil_div(k1 - k0, kChunk));
   }
   flat_chunks /= static_cast<double>(probe);
   auto rounds = [](long long tiles, long long ctas) { return static_cast<double>((tiles + ctas - 1) / ctas); };
   auto time_on = [&](long long ctas, bool flat) {
+    if (flat && tiles_flat <= ctas && most_chunks <= kStages) return 1.2 + 1.4 * most_chunks + nb / 32.0;
     return flat ? rounds(tiles_flat, ctas) * (2.8 + 1.5 * flat_chunks) : rounds(tiles_inside, ctas) * (1.6 + ceil_div(nb, kChunk));
   };
   // A CTA of this kernel fills its SM.  Where the whole attention grid finds room on the SMs that are left, it goes through its
@@ -455,9 +507,9 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   p.g16 = g16;
   p.zeta = zeta;
   p.status = device_status;
-  const bool share = p.tiles <= ctas;
-  auto* const kernel = flat ? (share ? aggregate_mma_kernel<true, true> : aggregate_mma_kernel<true, false>)
-                            : (share ? aggregate_mma_kernel<false, true> : aggregate_mma_kernel<false, false>);
+  const bool one = p.tiles <= ctas;
+  auto* const kernel = flat ? (one && most_chunks <= kStages ? aggregate_mma_kernel<true, true> : aggregate_mma_kernel<true, false>)
+                            : (one ? aggregate_mma_kernel<false, true> : aggregate_mma_kernel<false, false>);
   st = ensure_dynamic_smem(kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
   return launch_dependent(kernel, dim3(static_cast<unsigned>(std::min<long long>(p.tiles, ctas))), kThreads, static_cast<int>(kSmemBytes), stream,

@@ -224,6 +224,24 @@ def test_aggregation_tiles_of_persistent_ctas(batch, heads, blocks):
     full_parity(wl, wk.make_inputs(wl), query_blocks=pu.sample_blocks(wl, [0, heads - 1], min(150, batch * blocks)))
 
 
+@pytest.mark.parametrize("batch,heads,blocks", [(3, 43, 1), (32, 32, 1), (23, 3, 5), (16, 4, 15), (28, 1, 36), (9, 3, 37), (6, 19, 9)])
+def test_aggregation_tiles_whose_masks_are_made_at_once(batch, heads, blocks):
+    """One tile per CTA through the (b, h) boundaries: 129 rows, 1024 rows (the most that are one tile per SM), rows that start at
+    every byte of a word, tiles that begin and end inside a sequence, and 1026 rows, where the tiles are two to a CTA again.
+    The same output from class bytes at odd addresses."""
+    wl = small_workload(f"once{blocks}", batch=batch, heads=heads, tokens=blocks * 64 - 7, crit=0.0 if blocks == 1 else 0.2,
+                        neg=0.0 if blocks < 3 else 0.3)
+    inputs = wk.make_inputs(wl)
+    eng, out = full_parity(wl, inputs, query_blocks=pu.sample_blocks(wl, [0, heads - 1], min(60, batch * blocks)))
+    proj, want, cls = torch.from_numpy(inputs["proj"]).cuda(), out.clone(), eng.plan.cls
+    for shift in (1, 2, 3):
+        raw = torch.ones(cls.numel() + 8, dtype=torch.int8, device="cuda")  # marginal all round
+        eng.plan.cls = raw[shift:shift + cls.numel()].view(cls.shape)
+        eng.plan.cls.copy_(cls)
+        assert torch.equal(eng.forward(proj, out=torch.empty_like(out)), want), shift
+    assert int(eng.status.item()) == 0
+
+
 @pytest.mark.parametrize("batch,heads,tokens,block,crit", [(1, 16, 1374, 64, 0.25), (3, 5, 3001, 128, 0.15), (1, 16, 832, 64, 0.1),
                                                            (1, 12, 1374, 128, 0.25), (2, 16, 1374, 64, 0.25), (1, 4, 12016, 64, 0.15)])
 def test_aggregation_beside_the_attention_kernel(batch, heads, tokens, block, crit):
