@@ -399,10 +399,12 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               const float c = ldg_pinned(p.q_scales + bh_rows + tile.i_q[hf]) * (kLog2e * 0.125f) * sk;  // raw score -> base-2 exponent
               int valid = p.tokens - jl[hf] * BS - (kPair ? 0 : ((t + lane) & 1) * kStepKeys);
               valid = max(0, min(kStepKeys, valid));
-              // second word: the factor times the largest norm, rounded up to a multiple of 2^7 steps of the last place (infinity
-              // where it is not known), and in these seven bits the number of valid keys
+              // second word: the factor times the largest norm, raised by 2^7 steps of the last place or more to a multiple of
+              // that many (infinity where it is not known), and in these seven bits the number of valid keys.  With u = 2^-24 the
+              // norms may be 9.5 u (query: 17 roundings under the root, and the root's) and 6 u (key: 10) too small, this
+              // product 1 u, and a score 64 u too large; what is added is 128 u or more.
               const float reach = p.k_norms != nullptr ? c * ldg_pinned(p.k_norms + bh_rows + jl[hf]) : INFINITY;
-              const uint32_t reach_bits = reach < 1.0e30f ? (__float_as_uint(reach) + 0x7Fu) & ~0x7Fu : 0x7F800000u;
+              const uint32_t reach_bits = reach < 1.0e30f ? (__float_as_uint(reach) + 0xFFu) & ~0x7Fu : 0x7F800000u;
               if (t + lane < steps)
                 sts_volatile_v2(smem_u32(smem + kOffScal) + ((kc + lane) % kScalSlots) * 16 + hf * 8, __float_as_uint(c),
                                 reach_bits | static_cast<uint32_t>(valid));
@@ -678,10 +680,12 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (32 + k >= valid) xb[k] = 0xFF800000u;
         }
       }
-      // |q . k| <= |q| |k| bounds the step's scores (its rounding is far below what 2^15 leaves to the largest fp16 number).
+      // |q . k| <= |q| |k| bounds the step's scores, also as computed: the second word allows for the roundings before, and the
+      // product and the sum here are rounded to the safe side (references beyond 2^24 are further apart than what 2^15 leaves
+      // to the largest fp16 number).
       // Queries and keys of ordinary size pass it in all but the first steps of a tile (91 % of the steps at 22 key blocks,
       // 99.9 % at 687), which then go without the maximum, its vote and the wait for both.
-      if (!__all_sync(0xFFFFFFFFu, q_norm * __uint_as_float(scal.y) <= m_ref + kHeadroom)) {
+      if (!__all_sync(0xFFFFFFFFu, __fmul_ru(q_norm, __uint_as_float(scal.y)) <= __fadd_rd(m_ref, kHeadroom))) {
         // row maximum of the raw scores (c > 0 commutes with max), eight independent chains; a step without any valid key
         // (second half of a short last block) leaves the reference where it is
         float mx[8];

@@ -337,3 +337,33 @@ def test_attention_with_and_without_a_row_maximum(climb, block):
         inputs[name] = (along / 8.0 + 0.02 * g.standard_normal(inputs[name].shape)).astype(np.float32)
     eng, _ = full_parity(wl, inputs)
     assert (eng.plan.crit_idx.cpu().numpy() == np.arange(4)).all()
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("ones,first,last", [(42, 0x41F0F633, 0x41F0F63C), (23, 0x42DC3CE9, 0x42DC3CEE), (39, 0x4317517A, 0x4317517C)])
+def test_attention_bound_is_not_rounded_below_the_scores(ones, first, last, block):
+    """Scores of 3e7 to 2e8 (base 2), where neighbouring fp32 numbers are 2 to 16 apart.  The last block's single key lies 2^16
+    or more above the reference, past the largest fp16 number, but with these scales the norms' product, rounded to nearest,
+    is not above the reference plus 15: taken for the bound, the probability is infinite.  All values are one, so every
+    softmax gives one."""
+    eng = lt.SlaForward(1, 1, 2 * block + 1, block, 2 / 3, 0.0)
+    assert (eng.plan.k_crit, eng.plan.k_marg) == (2, 1)
+    row = torch.zeros(64, dtype=torch.uint8, device="cuda")
+    row[:ones] = 0x7E  # 448
+    for t in (eng.q8, eng.k8, eng.v8):
+        t.codes.zero_()
+        t.scales.fill_(1.0)
+    eng.q8.codes[0, 0, :2 * block + 1] = row
+    eng.q8.scales.fill_(0.75)
+    eng.k8.codes[0, 0, :block] = row
+    eng.k8.codes[0, 0, 2 * block] = row
+    bits = torch.tensor([first, 0x3F800000, last], dtype=torch.int32, device="cuda")
+    eng.k8.scales[0, 0] = bits.view(torch.float32)
+    eng.v8.codes[0, 0, :2 * block + 1] = 0x38  # 1
+    eng.plan.cls[0, 0] = torch.tensor([2, 1, 2], dtype=torch.int8)
+    eng.plan.crit_idx[0, 0] = torch.tensor([0, 2], dtype=torch.int32)
+    eng.plan.marg_idx[0, 0] = 1
+    out = eng.forward(torch.zeros((1, 64, 64), device="cuda"))
+    assert int(eng.status.item()) == 0
+    # probabilities are rounded to fp16 in the product and not in the sum: 2^-11
+    torch.testing.assert_close(out, torch.ones_like(out), rtol=2.0 ** -10, atol=0.0)
