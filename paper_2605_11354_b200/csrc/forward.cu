@@ -121,10 +121,10 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
     if (counts.k_marg == 0 && (st = launch_plan(a.q, a.k, s, counts, plan, false, stream)) != LITE3R_OK) return st;
   }
   if (phases & 1) profile_mark(0, stream);
-  // With a linear branch the summary kernel reads every V row anyway and writes the fp16 operand on the way; the
-  // stand-alone pass runs only when there is no linear branch.
-  const bool v16_from_summary = a.plan.k_marg > 0;
-  if ((phases & 1) && a.plan.k_crit > 0 && !v16_from_summary && !a.linear_only) {
+  // The sparse branch's operands.  With a linear branch the summary kernel reads every K and V row anyway, writes the fp16
+  // operand on the way and the norms that bound the scores; the stand-alone pass runs only when there is no linear branch.
+  const bool sparse = a.plan.k_crit > 0 && !a.linear_only;
+  if ((phases & 1) && sparse && a.plan.k_marg == 0) {
     const size_t words = static_cast<size_t>(rows) * BS * kHeadDim / 16;  // 16 codes per thread and pass
     int sms = 0;
     if ((st = sm_count(&sms)) != LITE3R_OK) return st;
@@ -136,8 +136,8 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   }
   if ((phases & 1) && a.plan.k_marg > 0) {
     profile_mark(2, stream);
-    st = launch_summary(a.k, a.v, a.proj, a.proj_head_stride, s, a.phi, w.hws, a.plan.k_crit > 0 ? w.v16 : nullptr,
-                        a.plan.k_crit > 0 ? w.k_norms : nullptr, a.device_status, stream);
+    st = launch_summary(a.k, a.v, a.proj, a.proj_head_stride, s, a.phi, w.hws, sparse ? w.v16 : nullptr,
+                        sparse ? w.k_norms : nullptr, a.device_status, stream);
     if (st != LITE3R_OK) return st;
     profile_mark(3, stream);
   }
@@ -158,7 +158,7 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   att.k_scales = a.k.scales;
   att.v_scales = a.v.scales;
   att.v16 = w.v16;
-  att.k_norms = a.plan.k_marg > 0 ? w.k_norms : nullptr;  // (from the summary kernel)
+  att.k_norms = sparse && a.plan.k_marg > 0 ? w.k_norms : nullptr;  // (from the summary kernel)
   att.g16 = w.g16;
   att.zeta = w.zeta;
   att.crit_idx = plan.crit_idx;

@@ -38,6 +38,23 @@ def test_linear_branch_alone(block, phi, tokens):
     assert rel <= pu.REL_L2_TOL and mx <= pu.MAX_ABS_TOL
 
 
+@pytest.mark.parametrize("block", [64, 128])
+def test_linear_branch_alone_writes_nothing_of_the_sparse_branch(block):
+    """The fp16 values and the key norms are operands of the sparse branch: their part of the workspace stays as it was."""
+    wl = small_workload(f"olin-stores-{block}", tokens=1000, block=block, heads=2, batch=2)
+    eng, _ = pu.run_gpu(wk.make_inputs(wl), wl)
+    ws = aligned_bytes(lt.lite3r_train_workspace(eng.shape, wl.crit, wl.neg))
+    ws.fill_(0xEE)
+    offsets = lt.lite3r_workspace_layout(eng.shape, wl.crit, wl.neg)
+    o_lin = torch.empty((wl.batch, wl.heads, wl.tokens, 64), device="cuda")
+    lt.lite3r_sla_linear_branch(eng.q8, eng.k8, eng.v8, eng.shape, eng.phi, eng.plan, o_lin, ws, eng.status)
+    torch.cuda.synchronize()
+    assert int(eng.status.item()) == 0
+    assert eng.plan.k_crit > 0 and offsets[4] > offsets[3]
+    assert (ws[offsets[3]:offsets[4]] == 0xEE).all()
+    assert not (ws[offsets[0]:offsets[1]] == 0xEE).all()
+
+
 @pytest.mark.parametrize("dtype,count", [(torch.float32, 8 * 12345), (torch.bfloat16, 8 * 70001), (torch.float32, 8)])
 def test_mse_distillation_term(dtype, count):
     g = np.random.default_rng(7)
