@@ -20,7 +20,10 @@ LITE3R_API lite3r_status lite3r_selftest_wait_expiry(int* device_status, unsigne
 
 /* Stage timing for benchmarks.  After lite3r_profile_enable(1) (call it with the device current; it creates CUDA
  * events, no device memory), every lite3r_sla_forward brackets its four stages -- V operand preparation, key-block
- * summaries, marginal aggregation, attention -- with event records on the call's stream.  lite3r_profile_stage_ms
+ * summaries, marginal aggregation, attention -- with event records on the call's stream.  The launches are those of any
+ * other call, but each stage waits for the end of the one before: what normally overlaps (the attention kernel's critical
+ * blocks run beside the aggregation, for which a small call's aggregation gets fewer SMs) shows one after the other, so that
+ * the stages of a small call add up to more than the call takes.  lite3r_profile_stage_ms
  * waits for the last forward's events (the only blocking call of the library) and writes the four durations in
  * milliseconds to ms (HOST, 4 floats; a stage that did not run reports 0).  Not thread-safe; meant for one
  * benchmarking thread. */

@@ -146,7 +146,8 @@ lite3r_status run_forward(const ForwardArgs& a, int phases, cudaStream_t stream)
   if (a.plan.k_marg > 0) {
     profile_mark(4, stream);
     const int attention_ctas = s.batch * s.heads * (BS == 64 ? (nb + 1) / 2 : nb);
-    const int steps = a.linear_only || profile_enabled() ? 0 : a.plan.k_crit * (BS / 64);
+    // (the same grid while stage times are taken, although nothing then runs beside it: they are times of these launches)
+    const int steps = sparse ? a.plan.k_crit * (BS / 64) : 0;
     if ((st = launch_aggregate(w.hws, plan.cls, s, nb, attention_ctas, steps, w.g16, w.zeta, a.device_status, stream)) != LITE3R_OK) return st;
     profile_mark(5, stream);
   }

@@ -1,4 +1,6 @@
 """Edges of the size rules by which the library picks a kernel variant or the shape of a launch, against the oracle."""
+import json
+
 import numpy as np
 import pytest
 import torch
@@ -245,21 +247,56 @@ def test_aggregation_tiles_whose_masks_are_made_at_once(batch, heads, blocks):
 @pytest.mark.parametrize("batch,heads,tokens,block,crit", [(1, 16, 1374, 64, 0.25), (3, 5, 3001, 128, 0.15), (1, 16, 832, 64, 0.1),
                                                            (1, 12, 1374, 128, 0.25), (2, 16, 1374, 64, 0.25), (1, 4, 12016, 64, 0.15)])
 def test_aggregation_beside_the_attention_kernel(batch, heads, tokens, block, crit):
-    """Attention grids that fit on the SMs a narrower aggregation leaves free, and grids that do not: the same output as with
-    the aggregation on all SMs (which is what it gets while stage times are taken)."""
+    """Attention grids that fit on the SMs a narrower aggregation leaves free, and grids that do not: the same output every
+    time, and the same sums over the marginal blocks as from a plan without critical blocks, whose aggregation gets all SMs."""
     wl = small_workload("beside", batch=batch, heads=heads, tokens=tokens, block=block, crit=crit, neg=0.5)
     inputs = wk.make_inputs(wl)
     eng, out = pu.run_gpu(inputs, wl)
-    again = torch.empty_like(out)
+    want = out.clone()
+    offsets = lt.lite3r_workspace_layout(eng.shape, wl.crit, wl.neg)
+    sums = eng.workspace[offsets[1]:offsets[3]]
+    proj = torch.from_numpy(inputs["proj"]).cuda()
+    for _ in range(3):
+        sums.fill_(0xEE)
+        eng.forward(proj, out=out)
+        assert torch.equal(out, want)
+    beside = sums.clone()
+    plan = eng.plan
+    plan.k_crit, plan.k_neg = 0, plan.k_crit + plan.k_neg
+    sums.fill_(0xEE)
+    lt.lite3r_sla_forward(eng.q8, eng.k8, eng.v8, proj, eng.shape, eng.phi, plan, out, eng.workspace, eng.status)
+    assert int(eng.status.item()) == 0
+    assert torch.equal(sums, beside)
+
+
+@pytest.mark.parametrize("batch,heads,tokens,block,crit", [(1, 16, 1374, 64, 0.25), (3, 5, 3001, 128, 0.15), (1, 2, 512, 64, 0.25)])
+def test_stage_times_are_those_of_the_launches_of_any_call(batch, heads, tokens, block, crit, tmp_path):
+    """Grid, block and shared memory of every kernel of a forward, without and with stage times."""
+    eng = lt.SlaForward(batch, heads, tokens, block, crit, 0.5)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    q, k, v = (torch.randn((batch, heads, tokens, 64), device="cuda", generator=g) for _ in range(3))
+    proj = torch.randn((heads, 64, 64), device="cuda", generator=g)
+    eng.run(q, k, v, proj)
+    torch.cuda.synchronize()
+
+    def launches(name):
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            eng.forward(proj)
+            torch.cuda.synchronize()
+        prof.export_chrome_trace(str(tmp_path / name))
+        events = json.loads((tmp_path / name).read_text())["traceEvents"]
+        return [(e["name"], e["args"]["grid"], e["args"]["block"], e["args"]["shared memory"])
+                for e in sorted(events, key=lambda e: e.get("ts", 0)) if e.get("cat") == "kernel"]
+
+    if not launches("first.json"):
+        pytest.skip("the profiler records no launches here")
+    plain = launches("plain.json")
     lt.profile_enable(True)
     try:
-        eng.forward(torch.from_numpy(inputs["proj"]).cuda(), out=again)
+        timed = launches("timed.json")
     finally:
         lt.profile_enable(False)
-    assert int(eng.status.item()) == 0
-    for _ in range(3):
-        eng.forward(torch.from_numpy(inputs["proj"]).cuda(), out=out)
-        assert torch.equal(out, again)
+    assert len(plain) == 3 and timed == plain
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
