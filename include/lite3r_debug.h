@@ -36,8 +36,8 @@ LITE3R_API long long lite3r_launch_count(void);
 /* Test hook: which of its kernels lite3r_sla_plan (and a forward that builds its own plan) uses.  0 = chosen by the
  * size of the problem (the default); 1 = eight rows per CTA with 64-bit keys in shared memory (what short rows get); 2 / 3 =
  * eight / sixteen rows per CTA with approximate scores as 16-bit places in shared memory and exact keys recomputed for the
- * entries that these leave undecided (what all but short rows get); 4 = four rows per CTA with staged column sums (what
- * rows too long for the others get).  Every variant gives the same plan; a forced variant that does not fit the shape makes the plan call
+ * entries that these leave undecided (what all but short rows get); 4 = one row per CTA with staged column sums (what rows
+ * too long for the others get).  Every variant gives the same plan; a forced variant that does not fit the shape makes the plan call
  * return LITE3R_ERR_UNSUPPORTED.  Process-wide. */
 LITE3R_API lite3r_status lite3r_plan_variant(int variant);
 

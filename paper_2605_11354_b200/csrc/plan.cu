@@ -7,13 +7,11 @@
 // roundings separate t_ij from the exact value; the ranking is therefore the exact one except between
 // scores that agree to ~1e-15 relative.  Ranking order: score descending, then key-block index ascending.
 //
-// plan_kernel (rows of up to 80 blocks, and those too long for plan_compact_kernel): one CTA of R warps handles R
-// consecutive query blocks (rows) of one (b, h); R = 8 unless the row keys of a very long sequence do not fit in shared
-// memory.
+// plan_kernel: one CTA of R warps handles R consecutive query blocks (rows) of one (b, h); R = 8 for rows of up to 80
+// blocks, R = 1 for those too long for plan_compact_kernel.
 //   Phase A (whole CTA): the scores of the R rows against all key blocks, kept in shared memory as order-preserving
 //     64-bit keys.  R = 8: fp64 tensor-core products (m8n8k4) fed with the int32 column sums straight from global
-//     memory, no staging and no barrier.  R < 8: 64 key blocks at a time staged in shared memory as doubles; a lane
-//     owns one key block and R/4 rows, so every staged value feeds several fp64 FMAs.
+//     memory, no staging and no barrier.  R = 1: 32 key blocks at a time staged in shared memory as doubles, one to a lane.
 //   Phase B (one warp per row): "the k best of the row".  A histogram over 256 buckets that are linear in the score
 //     places the k-th best in a bucket of usually a handful of keys; those are listed by index and a
 //     most-significant-digit-first radix select over their 64-bit keys (8-bit digits placed at the highest bit on
@@ -39,7 +37,8 @@ namespace lite3r {
 
 namespace {
 
-constexpr int kChunk = 64;          // key blocks staged per pass (upper bound; the used part is keys_per_warp * R)
+constexpr int kStaged = 32;           // key blocks staged per pass (R = 1)
+constexpr int kLongestRow = 24316;    // blocks; longer sequences are refused
 constexpr int kPitch = kHeadDim + 4;  // staged row pitch in doubles: 16-byte aligned rows; 8-byte reads of four consecutive
                                       // values from four (eight) rows and 16-byte reads of eight rows fall on different banks
 
@@ -263,11 +262,7 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
   constexpr int kThreads = R * 32;
   constexpr bool kDirect = R >= 8;                // column sums straight from global memory into the fp64 MMA
   constexpr int kTiles = kDirect ? R / 8 : 1;     // 8-row MMA tiles per warp
-  constexpr int kGroups = R >= 4 ? 4 : R;        // (staged path) row groups inside a warp
-  constexpr int kRowsPerLane = R / kGroups;       // (staged path) rows whose score one lane accumulates
-  constexpr int kKeysPerWarp = 32 / kGroups;
-  constexpr int kStep = kKeysPerWarp * R;         // (staged path) key blocks per staged pass (<= kChunk)
-  static_assert(kDirect || kStep <= kChunk, "staging buffer too small");
+  static_assert(kDirect || R == 1, "one row per CTA, or whole 8-row tiles");
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int pitch = (nb + 1) & ~1;  // key-row pitch: keeps everything behind the keys 16-byte aligned
@@ -401,67 +396,49 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
       if (t4 == 0) s_range[warp * R + 8 * m + g] = make_float2(lo[m], hi[m]);
     }
   } else {
-    // Phase A for sequences too long for eight rows of keys per CTA: the column sums of kStep key blocks at a time
-    // are staged in shared memory as doubles (fetched with 16-byte loads one pass ahead); a lane owns one key block
-    // and R / 4 rows, so every staged value feeds several fp64 FMAs.  Both staged arrays use a row pitch of 68
-    // doubles, which keeps the 16-byte reads of the key rows and of the row groups of a warp on different banks.
-    double* s_q = reinterpret_cast<double*>(s_idx + R * 2 * kMaxListed);  // [R][kPitch]
-    double* s_k = s_q + R * kPitch;                             // [kChunk][kPitch]
-    for (int t = threadIdx.x; t < R * kHeadDim; t += kThreads) {
-      const int r = t / kHeadDim, d = t % kHeadDim;
-      s_q[r * kPitch + d] = (i0 + r < nb) ? static_cast<double>(q_colsum[(bh_rows + i0 + r) * kHeadDim + d]) : 0.0;
-    }
-    constexpr int kLoads = kStep * (kHeadDim / 4) / kThreads;  // int4 loads per thread and pass
-    const int kl = lane % kKeysPerWarp, rg = lane / kKeysPerWarp;
-    const int jj = warp * kKeysPerWarp + kl;
+    // Phase A for one very long row: the column sums of 32 key blocks at a time are staged in shared memory as doubles
+    // (fetched with 16-byte loads one pass ahead), and a lane takes one of them.  The pitch of 68 doubles keeps the
+    // 16-byte reads of eight staged rows on different banks.
+    double* s_q = reinterpret_cast<double*>(s_idx + R * 2 * kMaxListed);  // [kPitch]
+    double* s_k = s_q + kPitch;                                           // [kStaged][kPitch]
+    for (int d = lane; d < kHeadDim; d += 32) s_q[d] = static_cast<double>(q_colsum[(bh_rows + i0) * kHeadDim + d]);
+    constexpr int kLoads = kStaged * (kHeadDim / 4) / kThreads;  // int4 loads per thread and pass
     int4 pre[kLoads];
     auto prefetch = [&](int j0) {
       const int4* src = reinterpret_cast<const int4*>(k_colsum + (bh_rows + j0) * kHeadDim);
-      const int n4 = min(kStep, nb - j0) * (kHeadDim / 4);
+      const int n4 = min(kStaged, nb - j0) * (kHeadDim / 4);
 #pragma unroll
       for (int q = 0; q < kLoads; ++q) {
-        const int v = threadIdx.x + q * kThreads;
+        const int v = lane + q * kThreads;
         pre[q] = v < n4 ? __ldg(src + v) : make_int4(0, 0, 0, 0);
       }
     };
     prefetch(0);
-    for (int j0 = 0; j0 < nb; j0 += kStep) {
+    for (int j0 = 0; j0 < nb; j0 += kStaged) {
       __syncthreads();
-      const int nj = min(kStep, nb - j0);
 #pragma unroll
       for (int q = 0; q < kLoads; ++q) {
-        const int v = threadIdx.x + q * kThreads;
+        const int v = lane + q * kThreads;
         double* dst = s_k + (v / (kHeadDim / 4)) * kPitch + (v % (kHeadDim / 4)) * 4;
         *reinterpret_cast<double2*>(dst) = make_double2(static_cast<double>(pre[q].x), static_cast<double>(pre[q].y));
         *reinterpret_cast<double2*>(dst + 2) = make_double2(static_cast<double>(pre[q].z), static_cast<double>(pre[q].w));
       }
-      if (j0 + kStep < nb) prefetch(j0 + kStep);
+      if (j0 + kStaged < nb) prefetch(j0 + kStaged);
       __syncthreads();
-      if (jj < nj) {
-        const double2* kr = reinterpret_cast<const double2*>(s_k + jj * kPitch);
-        const double2* qr = reinterpret_cast<const double2*>(s_q + rg * kRowsPerLane * kPitch);
-        double acc[kRowsPerLane];
-#pragma unroll
-        for (int x = 0; x < kRowsPerLane; ++x) acc[x] = 0.0;
+      const int j = j0 + lane;
+      if (j < nb) {
+        const double2* kr = reinterpret_cast<const double2*>(s_k + lane * kPitch);
+        const double2* qr = reinterpret_cast<const double2*>(s_q);
+        double acc = 0.0;
 #pragma unroll 8
         for (int d2 = 0; d2 < kHeadDim / 2; ++d2) {
-          const double2 kv = kr[d2];
-#pragma unroll
-          for (int x = 0; x < kRowsPerLane; ++x) {
-            const double2 qv = qr[x * (kPitch / 2) + d2];
-            acc[x] = fma(qv.x, kv.x, acc[x]);
-            acc[x] = fma(qv.y, kv.y, acc[x]);
-          }
+          const double2 kv = kr[d2], qv = qr[d2];
+          acc = fma(qv.x, kv.x, acc);
+          acc = fma(qv.y, kv.y, acc);
         }
-        const int j = j0 + jj;
         const int valid = min(block, tokens - j * block);
-        const double ks = static_cast<double>(k_scales[bh_rows + j]);
-        const double n_valid = static_cast<double>(valid);
-#pragma unroll
-        for (int x = 0; x < kRowsPerLane; ++x) {
-          const double t = acc[x] * ks / n_valid + 0.0;
-          s_key[static_cast<size_t>(rg * kRowsPerLane + x) * pitch + j] = order_key(t);
-        }
+        const double t = acc * static_cast<double>(k_scales[bh_rows + j]) / static_cast<double>(valid) + 0.0;
+        s_key[j] = order_key(t);
       }
     }
   }
@@ -504,9 +481,8 @@ __global__ void __launch_bounds__(R * 32) plan_kernel(const int* __restrict__ q_
   // Phase B
   unsigned int* hist = s_hist + warp * 2 * kBuckets;  // radix digits; the second half holds the bucket counts
   unsigned int* bucket_hist = hist + kBuckets;
-  // Buckets linear in the score between the row's extremes; with fewer than eight rows per CTA (very long
-  // sequences) there is no single-precision copy and every key falls into bucket 0, which leaves the whole
-  // selection to the radix select.
+  // Buckets linear in the score between the row's extremes; with one row per CTA (very long sequences) there are no bucket
+  // bytes and every key falls into bucket 0, which leaves the whole selection to the radix select.
   float lo = 0.f, scale = 0.f;
   unsigned char* bkt = s_bkt + static_cast<size_t>(warp) * pitch;
   if constexpr (kDirect) {
@@ -1285,10 +1261,10 @@ size_t plan_smem_bytes(int nb, int rows) {
   const size_t pitch = static_cast<size_t>((nb + 1) & ~1);
   const size_t common = rows * pitch * 8 + static_cast<size_t>(rows) * 2 * kBuckets * 4 +
                         static_cast<size_t>(rows) * 2 * kMaxListed * 2;  // keys, two histograms, two index lists
-  // eight rows or more: score ranges and one bucket byte per key (the column sums come straight from global memory);
-  // fewer rows: the staged column sums as doubles
-  if (rows >= 8) return common + static_cast<size_t>(rows) * rows * sizeof(float2) + rows * pitch;
-  return common + static_cast<size_t>(rows) * kPitch * 8 + static_cast<size_t>(kChunk) * kPitch * 8;
+  // eight rows: score ranges and one bucket byte per key (the column sums come straight from global memory); one row: the
+  // staged column sums as doubles
+  if (rows == 8) return common + static_cast<size_t>(rows) * rows * sizeof(float2) + rows * pitch;
+  return common + (1 + kStaged) * static_cast<size_t>(kPitch) * 8;
 }
 
 template <int R>
@@ -1318,7 +1294,7 @@ lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r
     case 1: return plan_smem_bytes(nb, 8) <= kLimit ? launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
     case 2: return plan_compact_smem_bytes(nb, 8) <= kCompactLimit && nb <= kMostBlocks ? launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
     case 3: return plan_compact_smem_bytes(nb, 16) <= kCompactLimit && nb <= kMostBlocks ? launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
-    case 4: return plan_smem_bytes(nb, 4) <= kLimit ? launch_rows<4>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 4: return nb <= kLongestRow ? launch_rows<1>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
     default: break;
   }
   // Rows of more than 80 blocks: approximate scores as 16-bit places.  Its fixed part is larger than that of the 64-bit keys
@@ -1330,12 +1306,9 @@ lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r
     if (plan_compact_smem_bytes(nb, 16) <= kCompactLimit) return launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream);
     if (plan_compact_smem_bytes(nb, 8) <= kCompactLimit) return launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream);
   }
-  // As many rows per CTA as the row keys allow: the staged key blocks are then shared by more rows.
-  if (plan_smem_bytes(nb, 8) <= kLimit) return launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream);
-  if (plan_smem_bytes(nb, 4) <= kLimit) return launch_rows<4>(q, k, s, c, plan, nb, late_wait, stream);
-  if (plan_smem_bytes(nb, 2) <= kLimit) return launch_rows<2>(q, k, s, c, plan, nb, late_wait, stream);
-  if (plan_smem_bytes(nb, 1) <= kLimit) return launch_rows<1>(q, k, s, c, plan, nb, late_wait, stream);
-  return LITE3R_ERR_UNSUPPORTED;  // more than ~24000 blocks per sequence
+  if (nb <= kShortRow) return launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream);
+  if (nb <= kLongestRow) return launch_rows<1>(q, k, s, c, plan, nb, late_wait, stream);  // (from some 13600 blocks on)
+  return LITE3R_ERR_UNSUPPORTED;
 }
 
 }  // namespace lite3r

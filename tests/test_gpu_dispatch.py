@@ -16,6 +16,22 @@ from test_gpu_parity import full_parity, oracle_subset, small_workload
 pytestmark = pytest.mark.gpu
 
 
+def launches(call, tmp_path):
+    """Name, grid, block and shared memory of the kernels that call() launches, in their order."""
+    def record():
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            call()
+            torch.cuda.synchronize()
+        prof.export_chrome_trace(str(tmp_path / "trace.json"))
+        events = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
+        return [(e["name"], e["args"]["grid"], e["args"]["block"], e["args"]["shared memory"])
+                for e in sorted(events, key=lambda e: e.get("ts", 0)) if e.get("cat") == "kernel"]
+
+    if not record():
+        pytest.skip("the profiler records no launches here")
+    return record()
+
+
 @pytest.mark.parametrize("block,batch,heads,tokens", [(64, 37, 12, 128), (64, 89, 5, 65), (64, 23, 29, 200), (128, 89, 5, 100)])
 def test_attention_grids_around_the_number_of_resident_ctas(block, batch, heads, tokens):
     """444, 445, 1334 and 445 attention tiles: three per SM are resident, from one more on CTAs take over tiles."""
@@ -209,6 +225,39 @@ def test_plan_from_places_equals_plan_from_exact_keys(blocks, block):
         lt.lite3r_plan_variant(0)
 
 
+@pytest.mark.parametrize("blocks", [13592, 13593])
+def test_plan_of_the_longest_rows(blocks, tmp_path):
+    """The longest row that fits as 16-bit places and the first that gets one row per CTA (from there on the kernel that the
+    hook forces as variant 4): classes and lists of sampled rows from exact scores."""
+    tokens, kc = blocks * 64 - 5, round(0.002 * blocks)
+    shape = lt.Shape(1, 1, tokens, 64, 64)
+    g = torch.Generator(device="cuda").manual_seed(blocks)
+    q8, k8 = lt.alloc_fp8(shape, "cuda"), lt.alloc_fp8(shape, "cuda")
+    for out in (q8, k8):
+        lt.lite3r_quantize_fp8(torch.randn((1, 1, tokens, 64), device="cuda", generator=g, dtype=torch.bfloat16), shape, out)
+    k8.colsum[0, 0, 7] = k8.colsum[0, 0, 3]  # a tie
+    k8.scales[0, 0, 7] = k8.scales[0, 0, 3]
+    plan = lt.alloc_plan(shape, 0.002, 0.99, "cuda")
+    calls = []
+    try:
+        for variant in (0, 4):
+            lt.lite3r_plan_variant(variant)
+            plan.cls.fill_(-1)
+            calls.append(launches(lambda: lt.lite3r_sla_plan(q8, k8, shape, 0.002, 0.99, plan), tmp_path))
+            rows = torch.tensor([0, 1, blocks // 2, blocks - 2, blocks - 1], device="cuda")
+            valid = torch.full((blocks,), 64.0, device="cuda", dtype=torch.float64)
+            valid[-1] = 59.0
+            scores = q8.colsum[0, 0, rows].double() @ k8.colsum[0, 0].double().T * (k8.scales[0, 0].double() / valid)
+            rank = torch.argsort(torch.argsort(-scores, dim=1, stable=True), dim=1)
+            want = torch.where(rank < plan.k_crit, 2, torch.where(rank < blocks - plan.k_neg, 1, 0)).to(torch.int8)
+            assert plan.k_crit == kc and torch.equal(plan.cls[0, 0, rows], want)
+            assert torch.equal(plan.crit_idx[0, 0, rows].long(), (want == 2).nonzero()[:, 1].view(len(rows), -1))
+            assert torch.equal(plan.marg_idx[0, 0, rows].long(), (want == 1).nonzero()[:, 1].view(len(rows), -1))
+    finally:
+        lt.lite3r_plan_variant(0)
+    assert (calls[0] == calls[1]) == (blocks > 13592)
+
+
 @pytest.mark.parametrize("blocks", [64, 65, 128, 129, 193])
 def test_aggregation_inside_one_sequence(blocks):
     """Key chunks of 64 that end with, before and after the row, row tiles of 128 full and ragged."""
@@ -279,21 +328,10 @@ def test_stage_times_are_those_of_the_launches_of_any_call(batch, heads, tokens,
     eng.run(q, k, v, proj)
     torch.cuda.synchronize()
 
-    def launches(name):
-        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-            eng.forward(proj)
-            torch.cuda.synchronize()
-        prof.export_chrome_trace(str(tmp_path / name))
-        events = json.loads((tmp_path / name).read_text())["traceEvents"]
-        return [(e["name"], e["args"]["grid"], e["args"]["block"], e["args"]["shared memory"])
-                for e in sorted(events, key=lambda e: e.get("ts", 0)) if e.get("cat") == "kernel"]
-
-    if not launches("first.json"):
-        pytest.skip("the profiler records no launches here")
-    plain = launches("plain.json")
+    plain = launches(lambda: eng.forward(proj), tmp_path)
     lt.profile_enable(True)
     try:
-        timed = launches("timed.json")
+        timed = launches(lambda: eng.forward(proj), tmp_path)
     finally:
         lt.profile_enable(False)
     assert len(plain) == 3 and timed == plain
