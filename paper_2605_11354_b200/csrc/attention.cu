@@ -174,8 +174,8 @@ static __device__ __noinline__ void rescale_accumulator(uint32_t o_addr, float a
 // 2^a for a pair of arguments on the fused-multiply-add units: a = n + f with n = round(a) (adding 1.5 * 2^23 leaves n in
 // the low mantissa bits) and |f| <= 1/2, 2^f by a degree-5 polynomial (minimax in the relative error by a Remez
 // exchange; 2.1e-7 in fp32 arithmetic over all of [-1/2, 1/2], the size of the hardware approximation's own error),
-// n added to the exponent field.  Arguments are at most the rescale threshold; from below they are clamped to stay inside
-// the exponent range (a value that small is zero as a probability).
+// n added to the exponent field.  Arguments are at most 15 (kHeadroom) and a rounding; from below they are clamped to stay
+// inside the exponent range (a value that small is zero as a probability).
 __device__ __forceinline__ void exp2_pair_fma(uint64_t a2, float& p0, float& p1) {
   float a0, a1;
   unpack_f32x2(a2, a0, a1);

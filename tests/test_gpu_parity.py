@@ -202,9 +202,8 @@ def test_all_scores_tied_in_a_long_row():
 
 
 def test_plan_of_a_very_long_sequence():
-    """3000 blocks: the 64-bit row keys of eight query blocks no longer fit in shared memory, so the plan runs on the
-    kernel that keeps single-precision scores and recomputes the exact keys at the selection thresholds.  Quantiser
-    and plan are compared in full, the output on a few sampled query blocks."""
+    """3000 blocks, more than any benchmark configuration: approximate scores as 16-bit places, exact keys recomputed at
+    the selection thresholds.  Quantiser and plan are compared in full, the output on a few sampled query blocks."""
     wl = small_workload("long", tokens=3000 * 64 - 17, heads=1, src_dtype="bf16", crit=0.01, neg=0.95)
     inputs = wk.make_inputs(wl)
     full_parity(wl, inputs, query_blocks=pu.sample_blocks(wl, [0], 6, seed=5))
@@ -230,10 +229,11 @@ def plan_only(inputs, wl, crit=None, neg=None):
 
 @pytest.mark.parametrize("variant", [1, 2, 3, 4])
 def test_every_plan_kernel_on_ties_and_near_ties(variant, plan_variant):
-    """The four plan kernels (64-bit keys, single-precision scores with 8 or 16 rows per CTA, staged column sums) must
-    give the oracle's plan bit for bit on the cases that separate them: exact ties (duplicated key blocks), rows
+    """The four plan kernels (64-bit keys, 16-bit places with 8 or 16 rows per CTA, one row per CTA from staged column
+    sums) must give the oracle's plan bit for bit on the cases that separate them: exact ties (duplicated key blocks), rows
     whose scores are all equal (every entry in one place of the selection histogram: the keys are recomputed pass by
-    pass), a crowded histogram bucket that only the refinement separates, ragged last blocks, and empty classes."""
+    pass), a crowded histogram bucket, which the 16-bit places have to divide further, ragged last blocks, and empty
+    classes."""
     plan_variant(variant)
     # duplicated key blocks in a ragged sequence of 300 blocks
     wl = small_workload(f"var{variant}-ties", tokens=300 * 64 - 21, heads=2, src_dtype="f32", crit=0.1, neg=0.45)
@@ -255,7 +255,7 @@ def test_every_plan_kernel_on_ties_and_near_ties(variant, plan_variant):
     assert np.array_equal(eng.plan.cls.cpu().numpy(), ref["cls"])
     # a crowded bucket: 390 key blocks with scores within 5 % of each other and ten a hundred times larger, which
     # stretch the histogram's range so that the 390 share one of its 256 buckets (far more than the candidate list
-    # keeps) and only the 16-bit refinement separates them
+    # keeps): a second histogram, one counter per place, narrows the range, exact keys decide inside it
     g = np.random.default_rng(variant)
     inputs["q"][:] = 1.0
     level = (1.0 + 0.05 * g.uniform(-1.0, 1.0, 400)).astype(np.float32)
