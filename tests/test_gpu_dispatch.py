@@ -1,6 +1,4 @@
 """Edges of the size rules by which the library picks a kernel variant or the shape of a launch, against the oracle."""
-import json
-
 import numpy as np
 import pytest
 import torch
@@ -16,20 +14,26 @@ from test_gpu_parity import full_parity, oracle_subset, small_workload
 pytestmark = pytest.mark.gpu
 
 
-def launches(call, tmp_path):
-    """Name, grid, block and shared memory of the kernels that call() launches, in their order."""
-    def record():
-        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-            call()
-            torch.cuda.synchronize()
-        prof.export_chrome_trace(str(tmp_path / "trace.json"))
-        events = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
-        return [(e["name"], e["args"]["grid"], e["args"]["block"], e["args"]["shared memory"])
-                for e in sorted(events, key=lambda e: e.get("ts", 0)) if e.get("cat") == "kernel"]
+def launches(call):
+    """Name, grid, block and shared memory of the kernels that call() launches, from a captured graph of it."""
+    from cuda.bindings import driver
 
-    if not record():
-        pytest.skip("the profiler records no launches here")
-    return record()
+    def ok(result):
+        assert result[0] == driver.CUresult.CUDA_SUCCESS, result[0]
+        return result[1] if len(result) == 2 else result[1:]
+
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    count = ok(driver.cuGraphGetNodes(raw))[1]
+    found = []
+    for node in ok(driver.cuGraphGetNodes(raw, count))[0]:
+        if ok(driver.cuGraphNodeGetType(node)) == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            p = ok(driver.cuGraphKernelNodeGetParams(node))
+            name = ok(driver.cuFuncGetName(p.func) if int(p.func) else driver.cuKernelGetName(p.kern)).decode()
+            found.append((name, (p.gridDimX, p.gridDimY, p.gridDimZ), p.blockDimX, p.sharedMemBytes))
+    return sorted(found)
 
 
 @pytest.mark.parametrize("block,batch,heads,tokens", [(64, 37, 12, 128), (64, 89, 5, 65), (64, 23, 29, 200), (128, 89, 5, 100)])
@@ -226,7 +230,7 @@ def test_plan_from_places_equals_plan_from_exact_keys(blocks, block):
 
 
 @pytest.mark.parametrize("blocks", [13592, 13593])
-def test_plan_of_the_longest_rows(blocks, tmp_path):
+def test_plan_of_the_longest_rows(blocks):
     """The longest row that fits as 16-bit places and the first that gets one row per CTA (from there on the kernel that the
     hook forces as variant 4): classes and lists of sampled rows from exact scores."""
     tokens, kc = blocks * 64 - 5, round(0.002 * blocks)
@@ -243,7 +247,8 @@ def test_plan_of_the_longest_rows(blocks, tmp_path):
         for variant in (0, 4):
             lt.lite3r_plan_variant(variant)
             plan.cls.fill_(-1)
-            calls.append(launches(lambda: lt.lite3r_sla_plan(q8, k8, shape, 0.002, 0.99, plan), tmp_path))
+            lt.lite3r_sla_plan(q8, k8, shape, 0.002, 0.99, plan)
+            calls.append(launches(lambda: lt.lite3r_sla_plan(q8, k8, shape, 0.002, 0.99, plan)))
             rows = torch.tensor([0, 1, blocks // 2, blocks - 2, blocks - 1], device="cuda")
             valid = torch.full((blocks,), 64.0, device="cuda", dtype=torch.float64)
             valid[-1] = 59.0
@@ -319,7 +324,7 @@ def test_aggregation_beside_the_attention_kernel(batch, heads, tokens, block, cr
 
 
 @pytest.mark.parametrize("batch,heads,tokens,block,crit", [(1, 16, 1374, 64, 0.25), (3, 5, 3001, 128, 0.15), (1, 2, 512, 64, 0.25)])
-def test_stage_times_are_those_of_the_launches_of_any_call(batch, heads, tokens, block, crit, tmp_path):
+def test_stage_times_are_those_of_the_launches_of_any_call(batch, heads, tokens, block, crit):
     """Grid, block and shared memory of every kernel of a forward, without and with stage times."""
     eng = lt.SlaForward(batch, heads, tokens, block, crit, 0.5)
     g = torch.Generator(device="cuda").manual_seed(4)
@@ -328,10 +333,10 @@ def test_stage_times_are_those_of_the_launches_of_any_call(batch, heads, tokens,
     eng.run(q, k, v, proj)
     torch.cuda.synchronize()
 
-    plain = launches(lambda: eng.forward(proj), tmp_path)
+    plain = launches(lambda: eng.forward(proj))
     lt.profile_enable(True)
     try:
-        timed = launches(lambda: eng.forward(proj), tmp_path)
+        timed = launches(lambda: eng.forward(proj))
     finally:
         lt.profile_enable(False)
     assert len(plain) == 3 and timed == plain
