@@ -480,23 +480,36 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
     if (flat && tiles_flat <= ctas && most_chunks <= kStages) return 1.2 + 1.4 * most_chunks + nb / 32.0;
     return flat ? rounds(tiles_flat, ctas) * (2.8 + 1.5 * flat_chunks) : rounds(tiles_inside, ctas) * (1.6 + ceil_div(nb, kChunk));
   };
-  // A CTA of this kernel fills its SM.  Where the whole attention grid finds room on the SMs that are left, it goes through its
-  // critical blocks meanwhile: that many SMs are left to it if the longer of the two is then at least a microsecond shorter than
-  // one after the other on all SMs.  A step of the attention kernel takes 1.4 / 1.65 / 2 half microseconds with one / two / three
-  // of its CTAs on an SM.  16 heads of 1374 tokens (176 attention CTAs of six steps): a whole pass 31.5 -> 27.3 us; 15 of 3001 in
-  // blocks of 128 43.6 -> 40.6 us.
-  long long ctas = sms;
+  // A CTA of this kernel fills its SM.  Where the whole attention grid finds room on the SMs that are left, it runs beside this
+  // one up to the end of its critical blocks, and what counts is the longer of the two instead of their sum.  That part of the
+  // attention kernel takes 4.5 half microseconds (launch, set-up, phi(Q)) and 1.4 / 1.65 / 2 per step with one / two / three of its CTAs
+  // on an SM.  Both tilings are tried on all SMs, and on those that three attention CTAs to an SM leave (taken when that is a
+  // microsecond shorter).  A whole pass, all SMs and no room / as chosen here in us: 16 heads of 1374 tokens 31.5 / 26.0,
+  // 15 of 3001 in blocks of 128 43.6 / 40.6; tiles inside the (b, h) without / through the boundaries with room: 8 heads of 629
+  // tokens 22.6 / 20.5, of 1374 28.4 / 22.6, of 3000 28.0 / 24.9, 16 of 832 24.9 / 21.9.
+  struct Choice {
+    bool flat;
+    long long ctas;
+    double own, both;
+  };
+  auto choice = [&](bool flat, long long ctas) {
+    const double own = time_on(ctas, flat);
+    const long long left = sms - std::min(ctas, flat ? tiles_flat : tiles_inside);
+    const bool beside = left * kAttentionCtasPerSm >= attention_ctas;
+    const long long per_sm = beside ? (attention_ctas + left - 1) / left : kAttentionCtasPerSm;
+    const double other = steps == 0 ? 0.0 : 4.5 + steps * (per_sm <= 1 ? 1.4 : per_sm == 2 ? 1.65 : 2.0);
+    return Choice{flat, ctas, own, beside ? std::max(own, other) : own + other};
+  };
+  Choice best = choice(false, sms);
+  const Choice through = choice(true, sms);
+  if (through.both < best.both || (through.both == best.both && through.own < best.own)) best = through;
   const long long spare = sms - ceil_div(attention_ctas, kAttentionCtasPerSm);
   if (steps > 0 && spare > 0) {
-    auto best_on = [&](long long n) { return std::min(time_on(n, true), time_on(n, false)); };
-    auto steps_on = [&](long long n) {
-      const long long per_sm = (attention_ctas + n - 1) / n;
-      return steps * (per_sm <= 1 ? 1.4 : per_sm == 2 ? 1.65 : 2.0);
-    };
-    const long long taken = std::min(spare, time_on(spare, true) < time_on(spare, false) ? tiles_flat : tiles_inside);
-    if (std::max(best_on(spare), steps_on(sms - taken)) + 2.0 < best_on(sms) + steps_on(sms)) ctas = spare;
+    for (const Choice& c : {choice(false, spare), choice(true, spare)})
+      if (c.both + 2.0 < best.both) best = c;
   }
-  const bool flat = time_on(ctas, true) < time_on(ctas, false);
+  const bool flat = best.flat;
+  const long long ctas = best.ctas;
   AggregateParams p;
   p.cls = cls;
   p.nb = nb;

@@ -299,7 +299,8 @@ def test_aggregation_tiles_whose_masks_are_made_at_once(batch, heads, blocks):
 
 
 @pytest.mark.parametrize("batch,heads,tokens,block,crit", [(1, 16, 1374, 64, 0.25), (3, 5, 3001, 128, 0.15), (1, 16, 832, 64, 0.1),
-                                                           (1, 12, 1374, 128, 0.25), (2, 16, 1374, 64, 0.25), (1, 4, 12016, 64, 0.15)])
+                                                           (1, 12, 1374, 128, 0.25), (2, 16, 1374, 64, 0.25), (1, 4, 12016, 64, 0.15),
+                                                           (1, 8, 629, 64, 0.15), (1, 8, 3000, 64, 0.05), (1, 8, 4122, 64, 0.1)])
 def test_aggregation_beside_the_attention_kernel(batch, heads, tokens, block, crit):
     """Attention grids that fit on the SMs a narrower aggregation leaves free, and grids that do not: the same output every
     time, and the same sums over the marginal blocks as from a plan without critical blocks, whose aggregation gets all SMs."""
@@ -340,6 +341,22 @@ def test_stage_times_are_those_of_the_launches_of_any_call(batch, heads, tokens,
     finally:
         lt.profile_enable(False)
     assert len(plain) == 3 and timed == plain
+
+
+@pytest.mark.parametrize("heads,tokens,crit", [(8, 629, 0.15), (8, 1374, 0.25), (16, 832, 0.1), (8, 3000, 0.05)])
+def test_aggregation_leaves_room_for_the_attention_grid(heads, tokens, crit):
+    """Where one round of tiles through the (b, h) boundaries leaves SMs on which the whole attention grid fits, three CTAs to
+    an SM, the aggregation takes no more than that, although tiles inside the (b, h) are shorter for themselves."""
+    eng = lt.SlaForward(1, heads, tokens, 64, crit, 0.6)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    q, k, v = (torch.randn((1, heads, tokens, 64), device="cuda", generator=g) for _ in range(3))
+    proj = torch.randn((heads, 64, 64), device="cuda", generator=g)
+    eng.run(q, k, v, proj)
+    grids = {name: grid[0] for name, grid, *_ in launches(lambda: eng.forward(proj))}
+    aggregation, = (n for name, n in grids.items() if "aggregate" in name)
+    attention, = (n for name, n in grids.items() if "attention" in name)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert attention <= 3 * (sms - aggregation)
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
