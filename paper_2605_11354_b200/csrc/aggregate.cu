@@ -62,6 +62,7 @@ struct AggregateParams {
   int row_tiles;  // of one (b, h), or (flat) of all rows
   float inverse;  // of row_tiles, or (flat) of nb
   int tiles;      // row tiles times column tiles, of all (b, h)
+  int cols;       // (masks at once) column tiles of a CTA
   __nv_bfloat16* g16;
   float* zeta;
   int* status;
@@ -102,14 +103,17 @@ __device__ __forceinline__ Tile tile_at(const AggregateParams& p, int id) {
   return t;
 }
 
-// kOne: every CTA has one tile, and what counts is how soon its products can start.
+// kOne: every CTA has one tile (masks at once: one or two), and what counts is how soon its products can start.
 //   Inside a (b, h) the mask warpgroups then share every chunk's rows instead of taking every other chunk, which pays each
 //   chunk's waits twice (16 heads of 687 blocks, eleven tiles to a CTA, 80 -> 99 us alone).
 //   Through the boundaries, where a tile's keys fit into the ring, all its masks are made at once: operand tiles zeroed ahead
 //   of the wait for the plan, then a one written for every marginal entry of the tile's 128 Nb class bytes, which lie one after
 //   the other, four to a thread and turn.  Kernel alone, chunk by chunk / at once in us: 20 (b, h) of 15 blocks 8.3 / 6.2, 64 of
 //   8 7.6 / 5.7, 64 of 15 9.1 / 6.6, 32 of 22 8.6 / 6.3 (the last mask was ready 5100 clocks after the plan, products and stores
-//   take 4000 more); a whole pass of 4 x 5 (b, h) of 900 tokens 25.0 -> 21.6 us, of 2 x 16 of 1374 40.0 -> 37.5.
+//   take 4000 more); a whole pass of 4 x 5 (b, h) of 900 tokens 25.0 -> 21.6 us, of 2 x 16 of 1374 40.0 -> 37.5.  A CTA can
+//   take two neighbouring column tiles of a row tile with the same masks, one per accumulator: where one each would be more than
+//   one per SM (64 (b, h) of 22 blocks, 187 tiles: 17.5 -> 8.2 us from the end of the plan, a pass 71.5 -> 64.1), and where the SMs
+//   left over are worth more to the attention kernel.
 template <bool kFlat, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1)
 aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateParams p) {
@@ -121,8 +125,15 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
     return;
   }
   const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const int step = static_cast<int>(gridDim.x);
   constexpr bool kAtOnce = kFlat && kOne, kShare = !kFlat && kOne;
+  // the CTA's tiles: first, first + step, ... below last
+  int first_tile = blockIdx.x, last_tile = p.tiles, step = gridDim.x;
+  if (kAtOnce) {
+    const int groups = (kColTiles + p.cols - 1) / p.cols, rt = first_tile / groups;
+    first_tile = rt * kColTiles + (first_tile - rt * groups) * p.cols;
+    last_tile = min(first_tile + p.cols, (rt + 1) * kColTiles);
+    step = 1;
+  }
   constexpr int kAtOnceThreads = (kBuilders + kDrainers) * 128;  // (the storing warps have nothing else to do yet)
 
   if (threadIdx.x == 0) {
@@ -143,7 +154,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
     tmem_relinquish();
   }
   if (kAtOnce && warp >= 4) {
-    const uint32_t bytes = tile_at<kFlat>(p, blockIdx.x).chunks * kABytes;
+    const uint32_t bytes = tile_at<kFlat>(p, first_tile).chunks * kABytes;
     for (uint32_t at = (threadIdx.x - 128) * 16; at < bytes; at += kAtOnceThreads * 16) sts128(smem_u32(smem + kOffA) + at, 0u, 0u, 0u, 0u);
   }
   tc_fence_before();
@@ -158,7 +169,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
 
   if (kAtOnce && warp >= 4) {
     // The class bytes of the tile's rows, in the aligned words that hold them, two words to a thread and turn.
-    const Tile t = tile_at<kFlat>(p, blockIdx.x);
+    const Tile t = tile_at<kFlat>(p, first_tile);
     const char* const first = reinterpret_cast<const char*>(p.cls) + static_cast<long long>(t.row0) * p.nb;
     const int ahead = static_cast<int>(reinterpret_cast<intptr_t>(first) & 3);  // bytes of the first word before the tile's
     const int bytes = (min(t.row0 + kTileM, t.row_limit) - t.row0) * p.nb;
@@ -197,7 +208,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
       tma_prefetch_desc(&map_s);
       bool ok = true;
       int kc = 0;  // chunks so far, through all tiles
-      for (int id = blockIdx.x; ok && id < p.tiles; id += step) {
+      for (int id = first_tile; ok && id < last_tile; id += step) {
         const Tile t = tile_at<kFlat>(p, id);
         const int boxes = t.col == kColTiles - 1 ? 1 : kTileN / 64;
         for (int c = 0; c < t.chunks; ++c, ++kc) {
@@ -216,7 +227,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
       const uint32_t a_addr = smem_u32(smem + kOffA), b_addr = smem_u32(smem + kOffB);
       bool ok = true;
       int kc = 0, it = 0;
-      for (int id = blockIdx.x; ok && id < p.tiles; id += step, ++it) {
+      for (int id = first_tile; ok && id < last_tile; id += step, ++it) {
         const Tile t = tile_at<kFlat>(p, id);
         const uint32_t idesc = t.col == kColTiles - 1 ? idesc_zeta : idesc_all;
         const uint32_t acc = tmem + (it & 1) * kTileN;
@@ -226,11 +237,11 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
           const int st = kc % kStages;
           const uint32_t par = (kc / kStages) & 1;
           ok = mbar_wait(&bars->b_full[st], par, abort_flag, p.status, 403) &&
-               mbar_wait(&bars->a_full[kAtOnce ? 0 : st], par, abort_flag, p.status, 402);
+               mbar_wait(&bars->a_full[kAtOnce ? 0 : st], kAtOnce ? 0 : par, abort_flag, p.status, 402);
           if (!ok) break;
           tc_fence_after();
           for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t a = smem_desc(a_addr + st * kABytes + kk * 32, 16, 1024, kSwizzle128);
+            const uint64_t a = smem_desc(a_addr + (kAtOnce ? c : st) * kABytes + kk * 32, 16, 1024, kSwizzle128);
             const uint64_t b = smem_desc(b_addr + st * kBBytes + kk * 2048, 8192, 1024, kSwizzle128);
             mma_f16(acc, a, b, idesc, (c > 0 || kk > 0) ? 1u : 0u);
           }
@@ -366,7 +377,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
     // segments, four rows per instruction.
     uint8_t* const stage = smem + kOffOut + (warp - 4 - 4 * kBuilders) * 4096;
     int n = 0;  // tiles of this accumulator so far
-    for (int id = blockIdx.x + which * step; id < p.tiles; id += 2 * step, ++n) {
+    for (int id = first_tile + which * step; id < last_tile; id += 2 * step, ++n) {
       const Tile t = tile_at<kFlat>(p, id);
       if (!mbar_wait(&bars->acc_full[which], n & 1, abort_flag, p.status, 405)) break;
       tc_fence_after();
@@ -456,8 +467,8 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   // Tiles through the (b, h) boundaries pay with a longer reduction (the keys of every (b, h) a tile touches) and with masks
   // that have to be cut to every row's own keys, tiles inside one (b, h) with padding when Nb is not a multiple of 128.
   // Estimate of either, in half microseconds: rounds of one tile per SM times the cost of a tile, 1.6 + one per chunk of 64
-  // keys inside a (b, h), 2.8 + 1.5 per chunk through the boundaries; where one round does and the masks are made at once,
-  // 1.2 + 1.4 per chunk + one per 32 blocks of a row (its class bytes).  Measured, inside / flat in us: 16 (b, h) of 172 blocks
+  // keys inside a (b, h), 2.8 + 1.5 per chunk through the boundaries; where the masks are made at once, 1.2 + 1.4 per chunk + one
+  // per 32 blocks of a row (its class bytes) + 2 for a second column tile.  Measured, inside / flat in us: 16 (b, h) of 172 blocks
   // 14.5 / 21.7, of 687 80 / 121; 64 of 64 blocks 18.9 / 20.9, of 172 43.5 / 57.8; 512 of 22 blocks 71 / 37, of 64 97 / 97, of 86
   // 119 / 154; with the masks at once 4 (b, h) of 22 blocks 4.7 / 5.6, 10 of 15 5.6 / 6.2, 15 of 64 6.5 / 6.9, 16 of 22 6.3 / 6.2,
   // 12 of 32 6.2 / 5.9, 20 of 15 7.3 / 6.2, 32 of 22 8.5 / 6.3, 64 of 8 12.8 / 5.7.
@@ -476,40 +487,45 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   }
   flat_chunks /= static_cast<double>(probe);
   auto rounds = [](long long tiles, long long ctas) { return static_cast<double>((tiles + ctas - 1) / ctas); };
-  auto time_on = [&](long long ctas, bool flat) {
-    if (flat && tiles_flat <= ctas && most_chunks <= kStages) return 1.2 + 1.4 * most_chunks + nb / 32.0;
-    return flat ? rounds(tiles_flat, ctas) * (2.8 + 1.5 * flat_chunks) : rounds(tiles_inside, ctas) * (1.6 + ceil_div(nb, kChunk));
-  };
   // A CTA of this kernel fills its SM.  Where the whole attention grid finds room on the SMs that are left, it runs beside this
-  // one up to the end of its critical blocks, and what counts is the longer of the two instead of their sum.  That part of the
-  // attention kernel takes 4.5 half microseconds (launch, set-up, phi(Q)) and 1.4 / 1.65 / 2 per step with one / two / three of its CTAs
-  // on an SM.  Both tilings are tried on all SMs, and on those that three attention CTAs to an SM leave (taken when that is a
-  // microsecond shorter).  A whole pass, all SMs and no room / as chosen here in us: 16 heads of 1374 tokens 31.5 / 26.0,
-  // 15 of 3001 in blocks of 128 43.6 / 40.6; tiles inside the (b, h) without / through the boundaries with room: 8 heads of 629
-  // tokens 22.6 / 20.5, of 1374 28.4 / 22.6, of 3000 28.0 / 24.9, 16 of 832 24.9 / 21.9.
+  // one up to the end of its critical blocks, and what counts is the longer of the two instead of their sum; where a part of it
+  // does, that share of the shorter one is saved.  That part of the attention kernel takes 4.5 half microseconds (launch, set-up,
+  // phi(Q)) and 1.4 / 1.65 / 2 per step with one / two / three of its CTAs on an SM.  All forms are tried on all SMs, and those of any
+  // grid also on the SMs that three attention CTAs to an SM leave (taken when that is a microsecond shorter).  A whole pass in
+  // us: 15 (b, h) of 3001 tokens in blocks of 128 on all SMs 43.6, on 28 40.6; tiles inside the (b, h) / as chosen here: 16 heads of
+  // 1374 tokens 33.3 / 26.0, 8 of 629 22.6 / 20.5, of 1374 28.4 / 22.6, of 3000 28.0 / 24.9, 16 of 832 24.9 / 21.9, with room for a part
+  // 12 of 4748 in blocks of 128 46.3 / 43.2, 16 of 4122 53.4 / 51.2.
   struct Choice {
     bool flat;
-    long long ctas;
+    int cols;  // masks at once: column tiles to a CTA; else 0
+    long long grid;
     double own, both;
   };
-  auto choice = [&](bool flat, long long ctas) {
-    const double own = time_on(ctas, flat);
-    const long long left = sms - std::min(ctas, flat ? tiles_flat : tiles_inside);
+  auto choice = [&](bool flat, int cols, long long ctas) {
+    Choice c{flat, cols, 0, 0.0, 0.0};
+    if (cols > 0) {
+      c.grid = row_tiles * ceil_div(kColTiles, cols);
+      c.own = c.grid <= ctas && most_chunks <= kStages ? 1.2 + 1.4 * most_chunks + nb / 32.0 + 2.0 * (cols - 1) : 1e30;
+    } else {
+      c.grid = std::min(ctas, flat ? tiles_flat : tiles_inside);
+      c.own = flat ? rounds(tiles_flat, ctas) * (2.8 + 1.5 * flat_chunks) : rounds(tiles_inside, ctas) * (1.6 + ceil_div(nb, kChunk));
+    }
+    const long long left = sms - c.grid;
     const bool beside = left * kAttentionCtasPerSm >= attention_ctas;
     const long long per_sm = beside ? (attention_ctas + left - 1) / left : kAttentionCtasPerSm;
     const double other = steps == 0 ? 0.0 : 4.5 + steps * (per_sm <= 1 ? 1.4 : per_sm == 2 ? 1.65 : 2.0);
-    return Choice{flat, ctas, own, beside ? std::max(own, other) : own + other};
+    c.both = beside ? std::max(c.own, other) : c.own + other - std::min(c.own, other) * std::max(left, 0ll) / sms;
+    return c;
   };
-  Choice best = choice(false, sms);
-  const Choice through = choice(true, sms);
-  if (through.both < best.both || (through.both == best.both && through.own < best.own)) best = through;
+  Choice best = choice(false, 0, sms);
+  for (const Choice& c : {choice(true, 0, sms), choice(true, 1, sms), choice(true, 2, sms)})
+    if (c.both < best.both || (c.both == best.both && c.own < best.own)) best = c;
   const long long spare = sms - ceil_div(attention_ctas, kAttentionCtasPerSm);
   if (steps > 0 && spare > 0) {
-    for (const Choice& c : {choice(false, spare), choice(true, spare)})
+    for (const Choice& c : {choice(false, 0, spare), choice(true, 0, spare)})
       if (c.both + 2.0 < best.both) best = c;
   }
   const bool flat = best.flat;
-  const long long ctas = best.ctas;
   AggregateParams p;
   p.cls = cls;
   p.nb = nb;
@@ -520,12 +536,12 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   p.g16 = g16;
   p.zeta = zeta;
   p.status = device_status;
-  const bool one = p.tiles <= ctas;
-  auto* const kernel = flat ? (one && most_chunks <= kStages ? aggregate_mma_kernel<true, true> : aggregate_mma_kernel<true, false>)
-                            : (one ? aggregate_mma_kernel<false, true> : aggregate_mma_kernel<false, false>);
+  p.cols = best.cols;
+  auto* const kernel = flat ? (best.cols > 0 ? aggregate_mma_kernel<true, true> : aggregate_mma_kernel<true, false>)
+                            : (p.tiles == best.grid ? aggregate_mma_kernel<false, true> : aggregate_mma_kernel<false, false>);
   st = ensure_dynamic_smem(kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
-  return launch_dependent(kernel, dim3(static_cast<unsigned>(std::min<long long>(p.tiles, ctas))), kThreads, static_cast<int>(kSmemBytes), stream,
+  return launch_dependent(kernel, dim3(static_cast<unsigned>(best.grid)), kThreads, static_cast<int>(kSmemBytes), stream,
                           map_s, p);
 }
 

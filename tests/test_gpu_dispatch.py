@@ -280,11 +280,13 @@ def test_aggregation_tiles_of_persistent_ctas(batch, heads, blocks):
     full_parity(wl, wk.make_inputs(wl), query_blocks=pu.sample_blocks(wl, [0, heads - 1], min(150, batch * blocks)))
 
 
-@pytest.mark.parametrize("batch,heads,blocks", [(3, 43, 1), (32, 32, 1), (23, 3, 5), (16, 4, 15), (28, 1, 36), (9, 3, 37), (6, 19, 9)])
+@pytest.mark.parametrize("batch,heads,blocks", [(3, 43, 1), (32, 32, 1), (23, 3, 5), (16, 4, 15), (28, 1, 36), (9, 3, 37), (6, 19, 9),
+                                                 (32, 64, 1), (31, 7, 5), (16, 4, 22), (41, 7, 7), (64, 4, 8), (3, 683, 1)])
 def test_aggregation_tiles_whose_masks_are_made_at_once(batch, heads, blocks):
-    """One tile per CTA through the (b, h) boundaries: 129 rows, 1024 rows (the most that are one tile per SM), rows that start at
-    every byte of a word, tiles that begin and end inside a sequence, and 1026 rows, where the tiles are two to a CTA again.
-    The same output from class bytes at odd addresses."""
+    """Tiles through the (b, h) boundaries, one or two to a CTA: 129 rows, 1024 rows (the most that are one tile per SM), rows that
+    start at every byte of a word, tiles that begin and end inside a sequence, 1026 rows, where there are more tiles than SMs,
+    up to 2048 rows, where there are twice as many, tiles of one to four chunks (two tiles then go once or twice around the ring), and
+    2049 rows, where the general form follows.  The same output from class bytes at odd addresses."""
     wl = small_workload(f"once{blocks}", batch=batch, heads=heads, tokens=blocks * 64 - 7, crit=0.0 if blocks == 1 else 0.2,
                         neg=0.0 if blocks < 3 else 0.3)
     inputs = wk.make_inputs(wl)
