@@ -126,14 +126,13 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
   }
   const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   constexpr bool kAtOnce = kFlat && kOne, kShare = !kFlat && kOne;
-  // the CTA's tiles: first, first + step, ... below last
-  int first_tile = blockIdx.x, last_tile = p.tiles, step = gridDim.x;
-  if (kAtOnce) {
-    const int groups = (kColTiles + p.cols - 1) / p.cols, rt = first_tile / groups;
-    first_tile = rt * kColTiles + (first_tile - rt * groups) * p.cols;
-    last_tile = min(first_tile + p.cols, (rt + 1) * kColTiles);
-    step = 1;
-  }
+  // The CTA's tiles: first_id(), first_id() + step, ... below last_tile.  (first_id() reads the block's number in the roles themselves: from
+  // a copy made ahead of them the compiler no longer sees that it is not negative, 1.8 KB of code and 0.3 us more.)
+  const int groups = kAtOnce ? (kColTiles + p.cols - 1) / p.cols : 1, row_tile = blockIdx.x / groups;
+  const int first_at_once = row_tile * kColTiles + (blockIdx.x - row_tile * groups) * p.cols;
+  auto first_id = [&]() -> int { return kAtOnce ? first_at_once : blockIdx.x; };
+  const int last_tile = kAtOnce ? min(first_at_once + p.cols, (row_tile + 1) * kColTiles) : p.tiles;
+  const int step = kAtOnce ? 1 : static_cast<int>(gridDim.x);
   constexpr int kAtOnceThreads = (kBuilders + kDrainers) * 128;  // (the storing warps have nothing else to do yet)
 
   if (threadIdx.x == 0) {
@@ -154,7 +153,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
     tmem_relinquish();
   }
   if (kAtOnce && warp >= 4) {
-    const uint32_t bytes = tile_at<kFlat>(p, first_tile).chunks * kABytes;
+    const uint32_t bytes = tile_at<kFlat>(p, first_id()).chunks * kABytes;
     for (uint32_t at = (threadIdx.x - 128) * 16; at < bytes; at += kAtOnceThreads * 16) sts128(smem_u32(smem + kOffA) + at, 0u, 0u, 0u, 0u);
   }
   tc_fence_before();
@@ -169,7 +168,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
 
   if (kAtOnce && warp >= 4) {
     // The class bytes of the tile's rows, in the aligned words that hold them, two words to a thread and turn.
-    const Tile t = tile_at<kFlat>(p, first_tile);
+    const Tile t = tile_at<kFlat>(p, first_id());
     const char* const first = reinterpret_cast<const char*>(p.cls) + static_cast<long long>(t.row0) * p.nb;
     const int ahead = static_cast<int>(reinterpret_cast<intptr_t>(first) & 3);  // bytes of the first word before the tile's
     const int bytes = (min(t.row0 + kTileM, t.row_limit) - t.row0) * p.nb;
@@ -208,7 +207,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
       tma_prefetch_desc(&map_s);
       bool ok = true;
       int kc = 0;  // chunks so far, through all tiles
-      for (int id = first_tile; ok && id < last_tile; id += step) {
+      for (int id = first_id(); ok && id < last_tile; id += step) {
         const Tile t = tile_at<kFlat>(p, id);
         const int boxes = t.col == kColTiles - 1 ? 1 : kTileN / 64;
         for (int c = 0; c < t.chunks; ++c, ++kc) {
@@ -227,7 +226,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
       const uint32_t a_addr = smem_u32(smem + kOffA), b_addr = smem_u32(smem + kOffB);
       bool ok = true;
       int kc = 0, it = 0;
-      for (int id = first_tile; ok && id < last_tile; id += step, ++it) {
+      for (int id = first_id(); ok && id < last_tile; id += step, ++it) {
         const Tile t = tile_at<kFlat>(p, id);
         const uint32_t idesc = t.col == kColTiles - 1 ? idesc_zeta : idesc_all;
         const uint32_t acc = tmem + (it & 1) * kTileN;
@@ -377,7 +376,7 @@ aggregate_mma_kernel(const __grid_constant__ CUtensorMap map_s, const AggregateP
     // segments, four rows per instruction.
     uint8_t* const stage = smem + kOffOut + (warp - 4 - 4 * kBuilders) * 4096;
     int n = 0;  // tiles of this accumulator so far
-    for (int id = first_tile + which * step; id < last_tile; id += 2 * step, ++n) {
+    for (int id = first_id() + which * step; id < last_tile; id += 2 * step, ++n) {
       const Tile t = tile_at<kFlat>(p, id);
       if (!mbar_wait(&bars->acc_full[which], n & 1, abort_flag, p.status, 405)) break;
       tc_fence_after();
