@@ -420,6 +420,21 @@ def test_codes_next_to_rounding_boundaries_at_scales_that_take_a_second_correcti
     assert np.array_equal(got_scales.cpu().numpy().view(np.uint32).ravel(), scales.view(np.uint32).ravel())
 
 
+@pytest.mark.parametrize("block,crit,read", [(64, 0.1, False), (64, 0.2, True), (128, 0.1, True), (64, 0.0, False)])
+def test_key_norms_are_made_for_more_than_one_step(block, crit, read):
+    """The largest norms of the key blocks spare the maxima of a tile's steps after the first: they are written where there is
+    one (one critical block of 128 tokens is two steps)."""
+    wl = small_workload("norms", heads=2, tokens=10 * block, block=block, crit=crit, neg=0.3)
+    inputs = wk.make_inputs(wl)
+    eng, out = pu.run_gpu(inputs, wl)
+    start = lt.lite3r_workspace_layout(eng.shape, wl.crit, wl.neg)[3] + 2 * 10 * block * 64 * 2  # behind the fp16 values
+    norms = eng.workspace[start:start + 2 * 10 * 4].view(torch.float32)
+    norms.fill_(float("nan"))
+    again = eng.forward(torch.from_numpy(inputs["proj"]).cuda(), out=torch.empty_like(out))
+    assert torch.equal(again, out)
+    assert torch.isnan(norms).all() if not read else (norms > 0).all()
+
+
 @pytest.mark.parametrize("block", [64, 128])
 @pytest.mark.parametrize("climb", [7.9, 8.1, 14.8, 15.2, 15.95, 16.1, 40.0])
 def test_attention_with_and_without_a_row_maximum(climb, block):
