@@ -24,7 +24,7 @@
 // its first scores are then under way while the softmax warps write this tile's output, and what lies between two tiles
 // of a CTA (5.5 k clocks of 13 k: launch, barriers, TMEM allocation, first loads) is paid once.  Barriers are never
 // re-initialised: rings and parities run on a count through all tiles.
-// The code (48 KB) is kept below the instruction cache's limit (at 62 KB the same kernel is 8 % slower): waits with their
+// The code (50 KB) is kept below the instruction cache's limit (at 62 KB the same kernel is 8 % slower): waits with their
 // rare part out of line, loops not unrolled, warp-uniform values made known to the compiler.
 // P is carried in fp16 (not e4m3): one e4m3 term has a 2.6 % rounding error per probability, which alone is ten
 // times the output tolerance.  V travels as the dequantised value in fp16 (2^-12 relative rounding).
@@ -107,7 +107,7 @@ struct AttnParams {
   const float* zeta;    // [B*H*Nb][64]
   void* out;
   long long out_stride_b, out_stride_h, out_stride_n;
-  int heads, tokens, nb, tiles_per_head, k_crit, k_marg, phi, out_dtype;
+  int heads, tokens, nb, tiles_per_head, k_crit, phi, out_dtype;
   // output through TMA stores (map_o): position of the token / head / batch dimension among the map's dimensions
   // 1..3 (they are ordered by stride); tma_out = 0: plain stores
   int tma_out, dim_token, dim_head, dim_batch;
@@ -238,7 +238,10 @@ __device__ __forceinline__ int taken_cta(uint32_t answer) {
   return ok != 0 ? static_cast<int>(x) : -1;
 }
 
-template <int BS>
+// kLinear: there are marginal blocks, and with them phi(Q), G, zeta and the norms of the key blocks.  An instance of its own without
+// them (39 KB of code instead of 47 to 50): tiles of one or two steps, which one instance for both had made 2 to 5 % longer when the
+// norm bound came in, 64 x 16 (b, h) of two blocks 42.4 -> 41.1 us a pass, 32 x 16 of 301 tokens 49.2 -> 47.7; dense rows 734 -> 727.
+template <int BS, bool kLinear>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_g,
@@ -262,7 +265,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // (a shuffle from lane 0 tells the compiler that a value is the same in all lanes)
   const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int steps = p.k_crit * kStepsPerBlock;
-  const int v_steps = steps + (p.k_marg > 0 ? 1 : 0);  // V-ring entries of a tile: the steps' V tiles, then G
+  const int v_steps = steps + (kLinear ? 1 : 0);  // V-ring entries of a tile: the steps' V tiles, then G
   // a tile's (b, h) and its query blocks (the second of an odd pair is a copy that is not stored)
   struct Tile {
     int bh, i_q[2];
@@ -353,7 +356,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       };
       if (it > 0) {  // the previous tile's last Q K^T and phi(Q) have read the Q tile
         if (steps > 0) ok = wait_all(&bars->s_full[(kc - 1) % kStages], ((kc - 1) / kStages) & 1, 104);
-        if (p.k_marg > 0) ok = ok && wait_all(&bars->phi_full, (it - 1) & 1, 105);
+        if (kLinear) ok = ok && wait_all(&bars->phi_full, (it - 1) & 1, 105);
         if (!ok) break;
       }
       if (leader && v_steps > 0) {  // (a tile without products has no reader of Q: the copy could outlive the CTA)
@@ -426,7 +429,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         for (int hf = 0; hf < kHalves; ++hf) jv[hf] = jk[hf];
       }
-      if (ok && p.k_marg > 0) {
+      if (ok && kLinear) {
         // The aggregated summaries follow the last V tile through its ring.  G and zeta come from the kernel enqueued
         // just before this one, which may still be running when this kernel was launched to overlap with it: everything
         // above reads older results only.
@@ -491,7 +494,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
       }
       if (!ok) break;
-      if (p.k_marg > 0) {  // the release of the last scores, which the linear product takes up, passes by here
+      if (kLinear) {  // the release of the last scores, which the linear product takes up, passes by here
         ok = __all_sync(0xFFFFFFFFu, mbar_wait_far<1>(&bars->s_free, sc & 1, abort_flag, p.status, 208));
         ++sc;
         if (!ok) break;
@@ -528,7 +531,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
       }
       if (!ok) break;
-      if (p.k_marg > 0) {
+      if (kLinear) {
         // phi(Q) G into the score columns (released by the softmax threads: this step's probabilities, waited for above,
         // were made from the last scores)
         const int st = vc % kStages;
@@ -589,7 +592,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // chunk c ^ ((r >> 1) & 3)).  The loops over chunks are not unrolled: the kernel's code has to stay within the
     // instruction cache.
     float q_norm = INFINITY;  // norm of the query row in units of the codes (not known without a linear branch)
-    if (p.k_marg > 0) {
+    if (kLinear) {
       const float sq = __ldg(p.q_scales + bh_rows + iq);
       if (!(ok = mbar_wait_far(&bars->q_full, it & 1, abort_flag, p.status, 307))) break;
       // the previous tile's output rows, staged where this warp's rows of phi(q) go, must have been read
@@ -685,7 +688,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // to the largest fp16 number).
       // Queries and keys of ordinary size pass it in all but the first steps of a tile (91 % of the steps at 22 key blocks,
       // 99.9 % at 687), which then go without the maximum, its vote and the wait for both.
-      if (!__all_sync(0xFFFFFFFFu, __fmul_ru(q_norm, __uint_as_float(scal.y)) <= __fadd_rd(m_ref, kHeadroom))) {
+      if (!kLinear || !__all_sync(0xFFFFFFFFu, __fmul_ru(q_norm, __uint_as_float(scal.y)) <= __fadd_rd(m_ref, kHeadroom))) {
         // row maximum of the raw scores (c > 0 commutes with max), eight independent chains; a step without any valid key
         // (second half of a short last block) leaves the reference where it is
         float mx[8];
@@ -737,7 +740,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // zeta_i arrives with the aggregated summaries behind the last V tile
     const int v_last = vc + v_steps - 1;  // the tile's last product
     float den = 0.f;
-    if (p.k_marg > 0) {
+    if (kLinear) {
       if (!(ok = mbar_wait_far(&bars->v_full[v_last % kStages], (v_last / kStages) & 1, abort_flag, p.status, 308))) break;
       const uint32_t zeta = smem_u32(smem + kOffZeta) + (it & 1) * 512 + hf * 256;
       uint64_t den2[2] = {0ull, 0ull};  // bit pattern of (0.f, 0.f)
@@ -770,10 +773,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // 128B swizzle.
     const int bb = tile.bh / p.heads, h = tile.bh - bb * p.heads;
     const float inv_l = steps > 0 ? 1.f / l : 0.f;
-    const float l_scale = p.k_marg > 0 ? 1.f / den : 0.f;
+    const float l_scale = kLinear ? 1.f / den : 0.f;
     const bool wide = p.out_dtype == LITE3R_F32;
     const bool to_bf16 = p.out_dtype == LITE3R_BF16;
-    if (p.k_marg == 0) {  // the previous tile's rows must have been read (next to a linear branch phi(q) has waited for that)
+    if (!kLinear) {  // the previous tile's rows must have been read (next to a linear branch phi(q) has waited for that)
       if (lane == 0) bulk_wait_group_read0();
       __syncwarp();
     }
@@ -787,16 +790,16 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         __syncwarp();
       }
       tmem_wait_ld();
-      if (p.k_marg > 0 && half == 1) {  // the linear product has been read: the score columns are free for the next tile
+      if (kLinear && half == 1) {  // the linear product has been read: the score columns are free for the next tile
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->s_free);
       }
-      if (steps == 0 || p.k_marg == 0) {  // without a critical block O, without a linear branch its product was never written
+      if (steps == 0 || !kLinear) {  // without a critical block O, without a linear branch its product was never written
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
           if (steps == 0) v[k] = 0u;
-          if (p.k_marg == 0) u[k] = 0u;
+          if (!kLinear) u[k] = 0u;
         }
       }
       const uint64_t inv2 = pack_f32x2(inv_l, inv_l), lin2 = pack_f32x2(l_scale, l_scale);
@@ -956,11 +959,11 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   p.nb = nb;
   p.tiles_per_head = BS == 64 ? (nb + 1) / 2 : nb;
   p.k_crit = a.k_crit;
-  p.k_marg = a.k_marg;
   p.phi = a.phi;
   p.out_dtype = a.out_dtype;
   p.status = a.device_status;
-  st = ensure_dynamic_smem(attention_kernel<BS>, static_cast<int>(kSmemBytes));
+  auto* const kernel = a.k_marg > 0 ? attention_kernel<BS, true> : attention_kernel<BS, false>;
+  st = ensure_dynamic_smem(kernel, static_cast<int>(kSmemBytes));
   if (st != LITE3R_OK) return st;
   const int ctas = s.batch * s.heads * p.tiles_per_head;
   int sms = 0;
@@ -972,7 +975,7 @@ lite3r_status launch(const AttentionLaunch& a, cudaStream_t stream) {
   // With a linear branch the launch before this one is the aggregation, whose results are needed only at a tile's end: the
   // kernel then runs beside it and waits for its completion itself.  Otherwise it waits before it reads anything.
   p.wait_first = a.overlap_prior ? 0 : 1;
-  return launch_dependent(attention_kernel<BS>, dim3(static_cast<unsigned>(ctas)), kThreads, static_cast<int>(kSmemBytes), stream,
+  return launch_dependent(kernel, dim3(static_cast<unsigned>(ctas)), kThreads, static_cast<int>(kSmemBytes), stream,
                           map_q, map_k, map_v, map_g, map_o, p);
 }
 
