@@ -466,8 +466,8 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   // Tiles through the (b, h) boundaries pay with a longer reduction (the keys of every (b, h) a tile touches) and with masks
   // that have to be cut to every row's own keys, tiles inside one (b, h) with padding when Nb is not a multiple of 128.
   // Estimate of either, in half microseconds: rounds of one tile per SM times the cost of a tile, 1.6 + one per chunk of 64
-  // keys inside a (b, h), 2.8 + 1.5 per chunk through the boundaries; where the masks are made at once, 1.2 + 1.4 per chunk + one
-  // per 32 blocks of a row (its class bytes) + 2 for a second column tile.  Measured, inside / flat in us: 16 (b, h) of 172 blocks
+  // keys inside a (b, h), 2.8 + 1.5 per chunk through the boundaries and 1.2 per chunk once for the first masks; where the masks are
+  // made at once, 1.2 + 1.4 per chunk + one per 32 blocks of a row (its class bytes) + 3 for a second column tile.  Measured, inside / flat in us: 16 (b, h) of 172 blocks
   // 14.5 / 21.7, of 687 80 / 121; 64 of 64 blocks 18.9 / 20.9, of 172 43.5 / 57.8; 512 of 22 blocks 71 / 37, of 64 97 / 97, of 86
   // 119 / 154; with the masks at once 4 (b, h) of 22 blocks 4.7 / 5.6, 10 of 15 5.6 / 6.2, 15 of 64 6.5 / 6.9, 16 of 22 6.3 / 6.2,
   // 12 of 32 6.2 / 5.9, 20 of 15 7.3 / 6.2, 32 of 22 8.5 / 6.3, 64 of 8 12.8 / 5.7.
@@ -488,7 +488,7 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
   auto rounds = [](long long tiles, long long ctas) { return static_cast<double>((tiles + ctas - 1) / ctas); };
   // A CTA of this kernel fills its SM.  Where the whole attention grid finds room on the SMs that are left, it runs beside this
   // one up to the end of its critical blocks, and what counts is the longer of the two instead of their sum; where a part of it
-  // does, that share of the shorter one is saved.  That part of the attention kernel takes 4.5 half microseconds (launch, set-up,
+  // does, 0.7 of that share of the shorter one is saved.  That part of the attention kernel takes 4.5 half microseconds (launch, set-up,
   // phi(Q)) and 1.4 / 1.65 / 2 per step with one / two / three of its CTAs on an SM.  All forms are tried on all SMs, and those of any
   // grid also on the SMs that three attention CTAs to an SM leave (taken when that is a microsecond shorter).  A whole pass in
   // us: 15 (b, h) of 3001 tokens in blocks of 128 on all SMs 43.6, on 28 40.6; tiles inside the (b, h) / as chosen here: 16 heads of
@@ -504,16 +504,16 @@ lite3r_status launch_aggregate(const __nv_bfloat16* hws, const signed char* cls,
     Choice c{flat, cols, 0, 0.0, 0.0};
     if (cols > 0) {
       c.grid = row_tiles * ceil_div(kColTiles, cols);
-      c.own = c.grid <= ctas && most_chunks <= kStages ? 1.2 + 1.4 * most_chunks + nb / 32.0 + 2.0 * (cols - 1) : 1e30;
+      c.own = c.grid <= ctas && most_chunks <= kStages ? 1.2 + 1.4 * most_chunks + nb / 32.0 + 3.0 * (cols - 1) : 1e30;
     } else {
       c.grid = std::min(ctas, flat ? tiles_flat : tiles_inside);
-      c.own = flat ? rounds(tiles_flat, ctas) * (2.8 + 1.5 * flat_chunks) : rounds(tiles_inside, ctas) * (1.6 + ceil_div(nb, kChunk));
+      c.own = flat ? rounds(tiles_flat, ctas) * (2.8 + 1.5 * flat_chunks) + 1.2 * flat_chunks : rounds(tiles_inside, ctas) * (1.6 + ceil_div(nb, kChunk));
     }
     const long long left = sms - c.grid;
     const bool beside = left * kAttentionCtasPerSm >= attention_ctas;
     const long long per_sm = beside ? (attention_ctas + left - 1) / left : kAttentionCtasPerSm;
     const double other = steps == 0 ? 0.0 : 4.5 + steps * (per_sm <= 1 ? 1.4 : per_sm == 2 ? 1.65 : 2.0);
-    c.both = beside ? std::max(c.own, other) : c.own + other - std::min(c.own, other) * std::max(left, 0ll) / sms;
+    c.both = beside ? std::max(c.own, other) : c.own + other - 0.7 * std::min(c.own, other) * std::max(left, 0ll) / sms;
     return c;
   };
   Choice best = choice(false, 0, sms);
