@@ -1299,11 +1299,18 @@ lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r
   }
   // Rows of more than 80 blocks: approximate scores as 16-bit places.  Its fixed part is larger than that of the 64-bit keys
   // (16 heads of 65 blocks: 9.1 against 8.3 us), the share of every entry smaller: 512 heads of 86 blocks 92.5 against 97.0
-  // us, 64 of 172 28 against 38.6, 16 of 687 61 against 108.  Sixteen rows per CTA wherever they fit (some 6300 blocks;
-  // two heads of 2147 blocks, where eight rows would be twice as many CTAs: 75 against 105 us), else eight.
+  // us, 64 of 172 28 against 38.6, 16 of 687 61 against 108.  Eight rows per CTA where that is at most one CTA per SM: such a
+  // CTA is done sooner (alone 1 head of 313 blocks 10.3 against 11.6 us, 5 of 129 7.6 against 8.1, 8 of 129 7.6 against 8.2) and, with half
+  // the registers, starts beside the CTAs of the summaries instead of behind them (a pass of 5 heads of 129 blocks 44.8 against 47.9 us, of
+  // 2 of 313 53.6 against 58.9).  Else sixteen where they fit (some 6300 blocks; 8 heads of 172 blocks 8.8 against 9.7 us, two of
+  // 2147 71 against 102), else eight.
   constexpr int kShortRow = 80;
   if (nb > kShortRow && nb <= kMostBlocks) {
-    if (plan_compact_smem_bytes(nb, 16) <= kCompactLimit) return launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream);
+    int sms = 0;
+    const lite3r_status st = sm_count(&sms);
+    if (st != LITE3R_OK) return st;
+    const bool sixteen = static_cast<long long>(s.batch) * s.heads * ceil_div(nb, 8) > sms;
+    if (sixteen && plan_compact_smem_bytes(nb, 16) <= kCompactLimit) return launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream);
     if (plan_compact_smem_bytes(nb, 8) <= kCompactLimit) return launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream);
   }
   if (nb <= kShortRow) return launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream);

@@ -229,6 +229,24 @@ def test_plan_from_places_equals_plan_from_exact_keys(blocks, block):
         lt.lite3r_plan_variant(0)
 
 
+def test_plan_rows_per_cta_around_one_cta_per_sm():
+    """Eight rows per CTA as long as that is one CTA per SM, sixteen from one row more on: the same plan as from 64-bit keys."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for blocks in (8 * sms, 8 * sms + 1):
+        wl = small_workload(f"rows{blocks}", heads=1, tokens=blocks * 64 - 9, crit=0.05, neg=0.6)
+        inputs = wk.make_inputs(wl)
+        eng, _ = pu.run_gpu(inputs, wl)
+        (_, grid, threads, _), = launches(eng.make_plan)
+        assert (threads, grid[0]) == ((256, sms) if blocks == 8 * sms else (512, -(-blocks // 16)))
+        got = [t.clone() for t in (eng.plan.cls, eng.plan.crit_idx, eng.plan.marg_idx)]
+        try:
+            lt.lite3r_plan_variant(1)
+            eng.make_plan()
+        finally:
+            lt.lite3r_plan_variant(0)
+        assert all(torch.equal(x, y) for x, y in zip(got, (eng.plan.cls, eng.plan.crit_idx, eng.plan.marg_idx)))
+
+
 @pytest.mark.parametrize("blocks", [13592, 13593])
 def test_plan_of_the_longest_rows(blocks):
     """The longest row that fits as 16-bit places and the first that gets one row per CTA (from there on the kernel that the
