@@ -592,8 +592,10 @@ __device__ __forceinline__ void mma_m16n8k16(float (&c)[4], const uint4& a, uint
 // integers, so one instruction compares two of them; an entry past the row's end holds a NaN, which fails every comparison.
 constexpr int kPlaceMid = 16024, kPlaceSpan = 14990, kPlaceLow = 1024, kPlaceHigh = 31030;
 constexpr int kNever = 0x7C00, kTopPlace = 0x7BFF;  // above every place; place of an entry found to be critical
-constexpr int kListed = 64;                         // entries of a threshold range that are decided from a list
+constexpr int kListed = 32;                         // entries of a threshold range that are decided from a list (64: up to 60 against 35 us, figures as below)
+constexpr int kPicked = 256;                        // indices of undecided entries at a time (eight per lane)
 constexpr int kFewListed = 14;                      // with more than this in its bucket the range is narrowed first
+constexpr int kFinest = 0x7F7F;                     // finer places: their top 128 stay free, as 0xFFFF is what lies past a row's end
 
 // Pitch of a row of places: 16-byte aligned, and eight rows on different banks for 4-byte accesses (an odd multiple of 16
 // bytes).
@@ -631,9 +633,9 @@ __device__ __forceinline__ void append_if(int*& dst, int v, uint32_t flag) {
 //   Phase B (one warp per row): the bucket of a 256-bucket histogram between the row's extremes that holds the k-th
 //     largest place; when it is too full, a second histogram inside that bucket, one counter per place; then the entries of
 //     the bucket and a margin on both sides as a list (up to kListed, in any order), ranked by comparing all pairs, first
-//     by place, then, inside the margin, by exact key and index.  Longer lists (ties, rows without places) go to the radix
-//     select, which recomputes keys pass by pass.  What was decided is written back over the places, so that the class of
-//     every entry is a comparison with two thresholds.
+//     by place, then, inside the margin, by exact key and index.  Longer lists get finer places from exact scores, and what
+//     is equal then too (ties, rows without places) goes to the radix select, which recomputes keys pass by pass.  What was
+//     decided is written back over the places, so that the class of every entry is a comparison with two thresholds.
 //   Phase C (same warp): eight entries per lane and turn: class bytes (stored as aligned 8-byte words, shifted over from the
 //     neighbouring lane where the row's address is not a multiple of eight) and the ascending lists, whose positions
 //     come from one warp scan of the lanes' counts.
@@ -647,14 +649,14 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
                                                                        signed char* __restrict__ cls, int* __restrict__ crit_idx,
                                                                        int* __restrict__ marg_idx) {
   static_assert(R == 8 || R == 16, "rows of one tensor product");
-  static_assert(kBuckets * 4 >= 2 * kListed * 8 && R * kBuckets * 4 >= 4096, "undecided entries and query operands take the histograms' place");
+  static_assert(kBuckets * 4 >= 2 * kListed * 8 && kPicked * 2 >= 2 * kListed * 4 && R * kBuckets * 4 >= 4096, "undecided entries and query operands take the histograms' place");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int pitch = place_pitch(nb);
   unsigned short* s_place = reinterpret_cast<unsigned short*>(smem_raw);                              // [R][pitch]
   unsigned int* s_hist = reinterpret_cast<unsigned int*>(s_place + static_cast<size_t>(R) * pitch);   // [R][kBuckets]
   uint4* s_a = reinterpret_cast<uint4*>(s_hist);  // [2][4][32] query operands (hi, lo) of phase A, ahead of the histograms
-  unsigned int* s_list = s_hist + R * kBuckets;                                                          // [R][2][kListed]
-  int* s_q = reinterpret_cast<int*>(s_list + R * 2 * kListed);                                        // [R][64]
+  unsigned int* s_list = s_hist + R * kBuckets;                                                          // [R][2][kListed], or [R][kPicked] halves
+  int* s_q = reinterpret_cast<int*>(s_list + R * kPicked / 2);                                         // [R][64]
   unsigned int* s_range = reinterpret_cast<unsigned int*>(s_q + R * kHeadDim);                        // [R][R] lowest | highest << 16
   __shared__ float s_sum[R];
   __shared__ unsigned s_kmax[R];
@@ -795,7 +797,7 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
   const uint4* const row8 = reinterpret_cast<const uint4*>(row);  // eight places
   const int chunks = (nb + 7) >> 3;
   unsigned int* const hist = s_hist + warp * kBuckets;
-  unsigned int* const list_c = s_list + warp * 2 * kListed;  // index | place << 16 | selected << 31
+  unsigned int* const list_c = s_list + warp * kPicked / 2;  // index | place << 16 | selected << 31
   unsigned int* const list_m = list_c + kListed;
   const int4* const q4 = reinterpret_cast<const int4*>(s_q + warp * kHeadDim);
   const int margin = no_places ? 0x7FFF : 1;
@@ -805,11 +807,12 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
   const int low = static_cast<int>(__reduce_min_sync(0xFFFFFFFFu, range & 0xFFFFu)), high = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, range >> 16));
 
   // the ranking score from an exact dot product (same expression as in plan_kernel)
-  auto exact_order_key = [&](long long dot, int j) -> unsigned long long {
+  auto exact_score = [&](long long dot, int j) -> double {
     const int valid = min(block, tokens - j * block);
     const double num = static_cast<double>(dot) * static_cast<double>(__ldg(k_scales + bh_rows + j));
-    return order_key((valid == block ? num * inv_block : num / static_cast<double>(valid)) + 0.0);  // block is a power of two
+    return (valid == block ? num * inv_block : num / static_cast<double>(valid)) + 0.0;  // block is a power of two
   };
+  auto exact_order_key = [&](long long dot, int j) -> unsigned long long { return order_key(exact_score(dot, j)); };
   auto dot4 = [](const int4& a, const int4& b) -> long long {
     return static_cast<long long>(a.x) * b.x + static_cast<long long>(a.y) * b.y + static_cast<long long>(a.z) * b.z +
            static_cast<long long>(a.w) * b.w;
@@ -880,12 +883,11 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
   __syncwarp();
 
   // A selection: entries whose place is above t_hi are selected, those in [t_lo, t_hi] are decided one by one (from a list
-  // or, `recompute`, by passes over the row), the rest are not.
+  // or, `recompute`, by their finer places), the rest are not.
   struct Chosen {
     int k, t_lo, t_hi;
     int above, bucket_hi;  // entries with a place above bucket_hi
     bool open, recompute;  // something is to be decided; too many entries for a list
-    Selection s;           // (recompute)
   };
   auto begin = [&](int k) -> Chosen {
     Chosen r;
@@ -991,7 +993,7 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
   // Decides the listed entries of both selections side by side, kPer entries per lane: first those of the critical list,
   // then those of the other.  The selected ones are marked (bit 31).
   unsigned long long* const u_key = reinterpret_cast<unsigned long long*>(hist);        // [2 kListed], over the histogram
-  const int m_c = cc.recompute ? 0 : n_c, m_m = cm.recompute ? 0 : n_m;
+  const int m_c = cc.recompute || cm.recompute ? 0 : n_c, m_m = cc.recompute || cm.recompute ? 0 : n_m;
   auto decide = [&](auto per) {
     constexpr int kPer = decltype(per)::value;
     // the lists are read four entries at a time, the shorter one as far as the longer one goes
@@ -1112,9 +1114,7 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
     __syncwarp();
   };
   __syncwarp();
-  if (m_c + m_m > 64)
-    decide(std::integral_constant<int, 4>{});
-  else if (m_c + m_m > 32)
+  if (m_c + m_m > 32)
     decide(std::integral_constant<int, 2>{});
   else if (m_c + m_m > 0)
     decide(std::integral_constant<int, 1>{});
@@ -1124,42 +1124,159 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
   // `mark`: as the upper end of the critical range its entries have all been decided.
   const int thr_c = cc.t_hi + 1, mark = max(thr_c - 1, 0), thr_m = min(cm.t_hi + 1, mark);
   if (cc.recompute || cm.recompute) {
-    auto resolve = [&](Chosen& r) {
-      if (!r.recompute) return;
+    // Ranges too full for a list (one key block of a much larger scale than the others, scores that differ by little): every
+    // entry of a range gets its exact score once, eight lanes to an entry, and with it a finer place inside the range, 0 ..
+    // kFinest, kept in place of the coarse one under bit 15.  The rounding is the same function of every exact score, so only
+    // equal finer places are undecided; two histograms find the one at the threshold, and where it is not selected or left
+    // as a whole, the radix select its share.  Ranges that overlap are treated as one.  With lists of 64 and longer ones left to
+    // the radix select, which recomputed the keys in each of its passes, one lane to a key: 16 heads of 687 blocks of Gaussian
+    // keys with one token 30 times larger 1095 -> 179 us, of 172 blocks 83 -> 35, 10 times larger (clustered keys) 312 -> 112 and 28 -> 27,
+    // keys and queries within 2 % of one value 248 -> 130 and 25 -> 25; of 2147 blocks clustered keys as they are 1063 -> 770.
+    const int l8 = lane & 7, group = lane >> 3;
+    const bool apart = cc.open && cm.open && cm.t_hi < cc.t_lo;
+    unsigned short* const picked = reinterpret_cast<unsigned short*>(list_c);  // [kPicked], over both lists
+    for (int turn = 0; turn < 2; ++turn) {
+      const bool has_c = turn == 0 && cc.open, has_m = cm.open && apart == (turn == 1);
+      if (!has_c && !has_m) continue;
+      const int lo = has_m ? cm.t_lo : cc.t_lo, hi = has_c ? cc.t_hi : cm.t_hi;
+      const double per_place = static_cast<double>(kFinest) / static_cast<double>(hi - lo + 2);
+      const double slope = static_cast<double>(places_per_unit(warp)) * 0x1p-19 * per_place;  // (a place is score * unit * 2^-19)
+      const double offset = static_cast<double>(kPlaceMid - lo + 1) * per_place;
+      const __half2 from = as_half2(static_cast<uint32_t>(lo) * 0x10001u), end = as_half2(static_cast<uint32_t>(hi + 1) * 0x10001u);
+      clear_hist();
       int above = 0;
-      for (int j = lane; j < nb; j += 32) above += static_cast<int>(row[j]) > r.t_hi ? 1 : 0;
+      for (int c0 = 0; c0 < chunks; c0 += 32) {
+        const uint4 v = chunk(c0 + lane);
+        const uint32_t words[4] = {v.x, v.y, v.z, v.w};
+        uint32_t ge[4], gt[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          gt[w] = __hge2_mask(as_half2(words[w]), end);
+          ge[w] = __hge2_mask(as_half2(words[w]), from) & ~gt[w];
+        }
+        above += __popc(mask_bits(gt[0], gt[1], gt[2], gt[3]));
+        uint32_t bits = mask_bits(ge[0], ge[1], ge[2], ge[3]);
+        int at = __popc(bits);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int up = __shfl_up_sync(0xFFFFFFFFu, at, o);
+          if (lane >= o) at += up;
+        }
+        const int total = __shfl_sync(0xFFFFFFFFu, at, 31);
+        at -= __popc(bits);
+        for (; bits != 0u; bits &= bits - 1u) picked[at++] = static_cast<unsigned short>(8 * (c0 + lane) + __ffs(static_cast<int>(bits)) - 1);
+        __syncwarp();
+        for (int e0 = 0; e0 < total; e0 += 32) {
+          long long dot = 0;  // of entry e0 + 4 l8 + group
+#pragma unroll 2
+          for (int t = 0; t < 8 && e0 + 4 * t < total; ++t) {
+            const int j = picked[min(e0 + 4 * t + group, total - 1)];
+            const int4* const k4 = reinterpret_cast<const int4*>(k_colsum + (bh_rows + j) * kHeadDim);
+            long long part = dot4(q4[l8], __ldg(k4 + l8)) + dot4(q4[l8 + 8], __ldg(k4 + l8 + 8));
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
+            if (l8 == t) dot = part;
+          }
+          const int own = e0 + 4 * l8 + group;
+          if (own < total) {
+            const int j = picked[own];
+            const int fine = no_places ? 0 : min(max(__double2int_rd(fma(exact_score(dot, j), slope, offset)), 0), kFinest);
+            row[j] = static_cast<unsigned short>(0x8000 | fine);
+            atomicAdd(&hist[255 - (fine >> 7)], 1u);
+          }
+          __syncwarp();
+        }
+      }
       above = __reduce_add_sync(0xFFFFFFFFu, above);
-      radix_select([&](int c, unsigned long long& key) {
-        const int f = row[c];
-        if (f < r.t_lo || f > r.t_hi) return false;
-        key = exact_key(c);
-        return true;
-      }, nb, r.k - above, hist, lane, r.s);
-    };
-    resolve(cc);
-    resolve(cm);
-    int tie_c = 0, tie_m = 0;
-    for (int j0 = 0; j0 < nb; j0 += 32) {
-      const int j = j0 + lane;
-      const int f = j < nb ? row[j] : -2;
-      const bool range_m = f >= cm.t_lo && f <= cm.t_hi;
-      const bool at_c = cc.recompute && f >= cc.t_lo && f <= cc.t_hi, at_m = cm.recompute && range_m;
-      const unsigned long long key = at_c || at_m ? exact_key(j) : 0ull;
-      const unsigned long long kc = key & cc.s.mask, km = key & cm.s.mask;
-      const bool eq_c = at_c && kc == cc.s.prefix, eq_m = at_m && km == cm.s.prefix;
-      const unsigned b_eq_c = __ballot_sync(0xFFFFFFFFu, eq_c), b_eq_m = __ballot_sync(0xFFFFFFFFu, eq_m);
-      const bool sel_c = at_c && (kc > cc.s.prefix || (eq_c && tie_c + __popc(b_eq_c & below) < cc.s.take));
-      const bool sel_m = at_m && (km > cm.s.prefix || (eq_m && tie_m + __popc(b_eq_m & below) < cm.s.take));
-      tie_c += __popc(b_eq_c);
-      tie_m += __popc(b_eq_m);
-      if (sel_c)
-        row[j] = kTopPlace;
-      else if (at_m)
-        row[j] = static_cast<unsigned short>(sel_m ? mark : 0);
-      else if (at_c && !range_m)
-        row[j] = static_cast<unsigned short>(mark);
+      __syncwarp();
+      // finer places above at_c are critical, else above at_m marginal; equal to one that is open: `take` of them are
+      int at_c = has_c ? 0 : 0x8000, at_m = has_m ? 0 : -1, take_c = cc.k - above, take_m = cm.k - above;
+      {
+        int count[8], before, after;
+        levels_of(32, count, before, after);
+        auto find = [&](int& at, int& take) {  // the highest finer place of the counter
+          const int src = __ffs(static_cast<int>(__ballot_sync(0xFFFFFFFFu, before < take && take <= after))) - 1;
+          const unsigned found = __shfl_sync(0xFFFFFFFFu, level_at(count, before, take), src);
+          at = ((255 - 8 * src - static_cast<int>(found & 7u)) << 7) + 127;
+          take -= static_cast<int>(found >> 17);
+        };
+        if (has_c) find(at_c, take_c);
+        if (has_m) find(at_m, take_m);
+      }
+      clear_hist();
+      for (int c0 = 0; c0 < chunks; c0 += 32) {
+        const uint4 v = chunk(c0 + lane);
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {  // (neither a coarse place nor what lies past the end is within 128 below a counter's highest)
+          const int fine = half_of(v, x) ^ 0x8000;
+          const unsigned d_c = static_cast<unsigned>(at_c - fine), d_m = static_cast<unsigned>(at_m - fine);
+          count_if(counters + (d_c << 2), has_c && d_c < 128u);
+          count_if(counters + 512 + (d_m << 2), has_m && d_m < 128u);
+        }
+      }
+      __syncwarp();
+      bool open_c = false, open_m = false;
+      {
+        int count[8], before, after;
+        levels_of(16, count, before, after);  // lanes 0-15: the first selection's counters, 16-31 the second's
+        const int k = lane < 16 ? take_c : take_m;
+        const unsigned found = level_at(count, before, k);
+        const unsigned where = __ballot_sync(0xFFFFFFFFu, before < k && k <= after);
+        auto enter = [&](int& at, int& take, int base) -> bool {
+          const int src = __ffs(static_cast<int>((where >> base) & 0xFFFFu)) - 1;
+          const unsigned f = __shfl_sync(0xFFFFFFFFu, found, base + src);
+          at -= 8 * src + static_cast<int>(f & 7u);
+          take -= static_cast<int>(f >> 17);
+          if (take < static_cast<int>((f >> 3) & 0x3FFFu)) return true;
+          --at;  // all of them
+          return false;
+        };
+        if (has_c) open_c = enter(at_c, take_c, 0);
+        if (has_m) open_m = enter(at_m, take_m, 16);
+      }
+      __syncwarp();
+      if (open_c || open_m) {
+        Selection sel[2] = {};
+        for (int w = 0; w < 2; ++w) {
+          if (!(w == 0 ? open_c : open_m)) continue;
+          const int code = 0x8000 | (w == 0 ? at_c : at_m);
+          radix_select([&](int c, unsigned long long& key) {
+            if (row[c] != code) return false;
+            key = exact_key(c);
+            return true;
+          }, nb, w == 0 ? take_c : take_m, hist, lane, sel[w]);
+        }
+        int tie_c = 0, tie_m = 0;
+        for (int j0 = 0; j0 < nb; j0 += 32) {
+          const int j = j0 + lane;
+          const int fine = j < nb ? row[j] ^ 0x8000 : -1;
+          const bool of_c = open_c && fine == at_c, of_m = open_m && fine == at_m;
+          if (!__any_sync(0xFFFFFFFFu, of_c || of_m)) continue;
+          const unsigned long long key = of_c || of_m ? exact_key(j) : 0ull;
+          const unsigned long long kc = key & sel[0].mask, km = key & sel[1].mask;
+          const bool eq_c = of_c && kc == sel[0].prefix, eq_m = of_m && km == sel[1].prefix;
+          const unsigned b_eq_c = __ballot_sync(0xFFFFFFFFu, eq_c), b_eq_m = __ballot_sync(0xFFFFFFFFu, eq_m);
+          const bool sel_c = of_c && (kc > sel[0].prefix || (eq_c && tie_c + __popc(b_eq_c & below) < sel[0].take));
+          const bool sel_m = of_m && (km > sel[1].prefix || (eq_m && tie_m + __popc(b_eq_m & below) < sel[1].take));
+          tie_c += __popc(b_eq_c);
+          tie_m += __popc(b_eq_m);
+          if (of_c || of_m) row[j] = static_cast<unsigned short>(sel_c ? kTopPlace : (sel_m || !of_m ? mark : 0));
+        }
+        __syncwarp();
+      }
+      for (int c0 = 0; c0 < chunks; c0 += 32) {
+        const uint4 v = chunk(c0 + lane);
+        uint32_t words[4] = {v.x, v.y, v.z, v.w};
+        auto settled = [&](uint32_t p) -> uint32_t {
+          const int fine = static_cast<int>(p) - 0x8000;
+          return fine < 0 || p == 0xFFFFu ? p : (fine > at_c ? kTopPlace : (fine > at_m ? mark : 0));
+        };
+#pragma unroll
+        for (int w = 0; w < 4; ++w) words[w] = settled(words[w] & 0xFFFFu) | settled(words[w] >> 16) << 16;
+        if (c0 + lane < chunks) reinterpret_cast<uint4*>(row)[c0 + lane] = make_uint4(words[0], words[1], words[2], words[3]);
+      }
+      __syncwarp();
     }
-    __syncwarp();
   }
   // the marginal list first: an entry of both lists that is not critical keeps what that one says
   for (int o = 0; o < m_m; o += 32) {
@@ -1240,7 +1357,7 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
 
 constexpr int kMostBlocks = 16383;  // (counts are packed into 14 bits)
 size_t plan_compact_smem_bytes(int nb, int rows) {
-  return static_cast<size_t>(rows) * (place_pitch(nb) * 2 + kBuckets * 4 + 2 * kListed * 4 + kHeadDim * 4 + rows * 4);
+  return static_cast<size_t>(rows) * (place_pitch(nb) * 2 + kBuckets * 4 + kPicked * 2 + kHeadDim * 4 + rows * 4);
 }
 
 template <int R>

@@ -229,6 +229,65 @@ def test_plan_from_places_equals_plan_from_exact_keys(blocks, block):
         lt.lite3r_plan_variant(0)
 
 
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("blocks", [200, 257, 520])
+def test_plan_ranges_too_full_for_a_list(blocks, block):
+    """Key blocks of a scale far above the others' and scores that differ by little leave most of a row in a few of the 16-bit
+    places: more undecided entries at a threshold than a list holds, both thresholds among the same ones, ties that the exact
+    keys leave, for critical and marginal blocks at once or one after the other.  The same plan bit for bit as from 64-bit
+    keys of every entry."""
+    g = np.random.default_rng(blocks)
+    wl = small_workload(f"full{blocks}", heads=5, tokens=(blocks - 1) * block + 3, block=block, src_dtype="f32")
+    inputs = wk.make_inputs(wl)
+    q, k = inputs["q"], inputs["k"]
+    k[:, 0, 3 * block + 1] *= 30.0
+    k[:, 1, 3 * block + 1] *= 1000.0
+    q[:, 2], k[:, 2] = (1.0 + 0.01 * g.standard_normal((2, 1) + q[:, 2].shape[1:])).astype(np.float32)
+    period = 5 * block
+    k[:, 3] = k[:, 3, np.arange(wl.tokens) % period]  # every block again and again
+    k[:, 3, 3 * block + 1] *= 300.0
+    k[:, 4, 3 * block + 1] *= 8.0
+    try:
+        for crit, neg in ((0.1, 0.6), (0.0, 0.4), (0.3, 0.7), (0.05, 0.0), (0.3, 0.69), (0.01, 0.98)):
+            plans = []
+            for variant in (1, 3, 2):
+                lt.lite3r_plan_variant(variant)
+                eng, _ = pu.run_gpu(inputs, wl, crit=crit, neg=neg)
+                plans.append([t.cpu().numpy() for t in (eng.plan.cls, eng.plan.crit_idx, eng.plan.marg_idx)])
+            for other in plans[1:]:
+                assert all(np.array_equal(a, b) for a, b in zip(plans[0], other)), (crit, neg)
+    finally:
+        lt.lite3r_plan_variant(0)
+
+
+@pytest.mark.parametrize("times", [10.0, 30.0])
+def test_plan_time_with_one_large_key(times):
+    """One key token that much larger than the others (an attention sink) leaves fewer places to all other blocks.  687 blocks
+    took 4.4 and 15 times as long with it; with exact scores made once per undecided entry it is less than three times."""
+    shape = lt.Shape(1, 16, 687 * 64, 64, 64)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, k = (torch.randn((1, 16, shape.tokens, 64), device="cuda", generator=g) for _ in range(2))
+    q8, k8, plan = lt.alloc_fp8(shape, "cuda"), lt.alloc_fp8(shape, "cuda"), lt.alloc_plan(shape, 0.05, 0.75, "cuda")
+    lt.lite3r_quantize_fp8(q, shape, q8)
+
+    def shortest():
+        lt.lite3r_quantize_fp8(k, shape, k8)
+        best = float("inf")
+        for _ in range(6):
+            start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            start.record()
+            for _ in range(10):
+                lt.lite3r_sla_plan(q8, k8, shape, 0.05, 0.75, plan)
+            end.record()
+            end.synchronize()
+            best = min(best, start.elapsed_time(end))
+        return best
+
+    plain = shortest()
+    k[:, :, 7 * 64 + 3] *= times
+    assert shortest() < 3.0 * plain
+
+
 def test_plan_rows_per_cta_around_one_cta_per_sm():
     """Eight rows per CTA as long as that is one CTA per SM, sixteen from one row more on: the same plan as from 64-bit keys."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
