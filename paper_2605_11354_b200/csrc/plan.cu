@@ -588,14 +588,31 @@ __device__ __forceinline__ void mma_m16n8k16(float (&c)[4], const uint4& a, uint
 
 // Places: what a score becomes in shared memory, two bytes instead of an eight-byte key.  The row's scores lie within
 // +-448 S max_j scale^K_j with S = sum_d |colsum^Q_d| 2^-10; this interval is mapped linearly to the integers
-// kPlaceLow .. kPlaceHigh.  All of them are bit patterns of normal, finite fp16 numbers, which are ordered like the
+// kPlaceLow .. kPlaceHigh.  Where up to kLarge key blocks have more than twice the scale that is usual in the row, the
+// interval is that of the others; their own places, the interval's ends where they lie outside it, come from exact scores, as
+// approximate ones are as much less exact as their scales are larger.  All of them are bit patterns of normal, finite fp16 numbers, which are ordered like the
 // integers, so one instruction compares two of them; an entry past the row's end holds a NaN, which fails every comparison.
 constexpr int kPlaceMid = 16024, kPlaceSpan = 14990, kPlaceLow = 1024, kPlaceHigh = 31030;
 constexpr int kNever = 0x7C00, kTopPlace = 0x7BFF;  // above every place; place of an entry found to be critical
 constexpr int kListed = 32;                         // entries of a threshold range that are decided from a list (64: up to 60 against 35 us, figures as below)
+constexpr int kLarge = 32;                          // key blocks of large scale (one per lane)
 constexpr int kPicked = 256;                        // indices of undecided entries at a time (eight per lane)
 constexpr int kFewListed = 14;                      // with more than this in its bucket the range is narrowed first
 constexpr int kFinest = 0x7F7F;                     // finer places: their top 128 stay free, as 0xFFFF is what lies past a row's end
+
+__device__ __forceinline__ long long dot4(const int4& a, const int4& b) {
+  return static_cast<long long>(a.x) * b.x + static_cast<long long>(a.y) * b.y + static_cast<long long>(a.z) * b.z +
+         static_cast<long long>(a.w) * b.w;
+}
+
+// Place of a key block of large scale from its exact score.
+__device__ __forceinline__ int place_of(const int4* q4, const int* k_colsum, const float* k_scale, int valid, float unit) {
+  long long dot = 0;
+#pragma unroll 4
+  for (int d = 0; d < kHeadDim / 4; ++d) dot += dot4(q4[d], __ldg(reinterpret_cast<const int4*>(k_colsum) + d));
+  const double score = static_cast<double>(dot) * static_cast<double>(__ldg(k_scale)) / static_cast<double>(valid);
+  return min(max(__double2int_rn(fma(score, static_cast<double>(unit) * 0x1p-19, static_cast<double>(kPlaceMid))), kPlaceLow), kPlaceHigh);
+}
 
 // Pitch of a row of places: 16-byte aligned, and eight rows on different banks for 4-byte accesses (an odd multiple of 16
 // bytes).
@@ -660,6 +677,9 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
   unsigned int* s_range = reinterpret_cast<unsigned int*>(s_q + R * kHeadDim);                        // [R][R] lowest | highest << 16
   __shared__ float s_sum[R];
   __shared__ unsigned s_kmax[R];
+  __shared__ float s_top;
+  __shared__ int s_large_count;
+  __shared__ unsigned short s_large[kLarge];
 
   const int row_tiles = (nb + R - 1) / R;
   const int bh = blockIdx.x / row_tiles;
@@ -690,13 +710,21 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
     const int2 qv = __ldg(reinterpret_cast<const int2*>(q_colsum + (bh_rows + min(i0 + warp, nb - 1)) * kHeadDim) + lane);
     *reinterpret_cast<int2*>(s_q + warp * kHeadDim + 2 * lane) = qv;
     const unsigned sum_q = __reduce_add_sync(0xFFFFFFFFu, static_cast<unsigned>(abs(qv.x)) + static_cast<unsigned>(abs(qv.y)));
-    unsigned kmax = 0u;  // bits of the largest scale: scales are not negative, and what is not a number counts as the largest
-    for (int j = warp * 32; j < nb; j += R * 32) kmax = max(kmax, __float_as_uint(__ldg(k_scales + bh_rows + min(j + lane, nb - 1))));
+    // bits of the largest scale and sum of the upper bits: scales are not negative, and what is not a number counts as the largest
+    unsigned kmax = 0u, ksum = 0u;
+    for (int j = warp * 32; j < nb; j += R * 32) {
+      const unsigned bits = j + lane < nb ? __float_as_uint(__ldg(k_scales + bh_rows + j + lane)) : 0u;
+      kmax = max(kmax, bits);
+      ksum += bits >> 14;
+    }
     kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
+    ksum = __reduce_add_sync(0xFFFFFFFFu, ksum);
     if (lane == 0) {
       s_sum[warp] = static_cast<float>(sum_q) * 0x1p-10f;
       s_kmax[warp] = kmax;
+      s_list[warp] = ksum;
     }
+    if (threadIdx.x == 0) s_large_count = 0;
     if (warp < 4) {  // operands of k-step `warp`
       uint4 hi = make_uint4(0u, 0u, 0u, 0u), lo = hi;
       auto load_row = [&](int r) {
@@ -715,10 +743,26 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
     }
   }
   __syncthreads();
-  const float k_top = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, lane < R ? s_kmax[lane] : 0u));
+  float k_top = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, lane < R ? s_kmax[lane] : 0u));
+  {
+    // Twice the value whose bits are the mean of the scales' bits, about twice their geometric mean, tells large ones.  Costs 0.3 us at
+    // 16 heads of 172 blocks, 0.8 at 687; with one token of Gaussian keys 30 times larger 35 -> 18.5 and 180 -> 102 us.
+    const unsigned ksum = __reduce_add_sync(0xFFFFFFFFu, lane < R ? s_list[lane] : 0u);
+    const float most = __uint_as_float(static_cast<unsigned>(static_cast<float>(ksum) * __fdividef(16384.f, static_cast<float>(nb))) + 0x00800000u);
+    if (k_top > most) {  // (the same for the whole CTA)
+      for (int j = threadIdx.x; j < nb; j += R * 32) {
+        if (__ldg(k_scales + bh_rows + j) > most) {
+          const int at = atomicAdd(&s_large_count, 1);
+          if (at < kLarge) s_large[at] = static_cast<unsigned short>(j);
+        }
+      }
+      __syncthreads();
+      if (s_large_count <= kLarge) k_top = most;
+    }
+  }
   // places per unit of a row's score; 0: the row has no places
-  auto places_per_unit = [&](int r) {
-    const float reach = 448.f * s_sum[r] * k_top;
+  auto places_per_unit = [&](int r, float top) {
+    const float reach = 448.f * s_sum[r] * top;
     return reach > 0.f && reach < 0x1p126f ? __fdividef(static_cast<float>(kPlaceSpan), reach) : 0.f;
   };
   {
@@ -727,7 +771,7 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
     uint32_t lo2[kHalves], hi2[kHalves];
 #pragma unroll
     for (int r = 0; r < kHalves; ++r) {
-      unit[r] = places_per_unit(8 * r + g);
+      unit[r] = places_per_unit(8 * r + g, k_top);
       lo2[r] = 0x7BFF7BFFu;
       hi2[r] = 0u;
     }
@@ -787,7 +831,9 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
       if (t4 == 0) s_range[warp * R + 8 * r + g] = min(lo2[r] & 0xFFFFu, lo2[r] >> 16) | (max(hi2[r] & 0xFFFFu, hi2[r] >> 16) << 16);
     }
   }
-  const bool no_places = places_per_unit(warp) == 0.f;
+  const bool no_places = places_per_unit(warp, k_top) == 0.f;
+  const int large = s_large_count;
+  if (threadIdx.x == 0) s_top = k_top;
   __syncthreads();
   const int i = i0 + warp;
   if (i >= nb) return;
@@ -804,7 +850,7 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
   const double inv_block = 1.0 / static_cast<double>(block);
   const unsigned below = (1u << lane) - 1u;
   const unsigned range = lane < R ? s_range[lane * R + warp] : 0x0000FFFFu;
-  const int low = static_cast<int>(__reduce_min_sync(0xFFFFFFFFu, range & 0xFFFFu)), high = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, range >> 16));
+  int low = static_cast<int>(__reduce_min_sync(0xFFFFFFFFu, range & 0xFFFFu)), high = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, range >> 16));
 
   // the ranking score from an exact dot product (same expression as in plan_kernel)
   auto exact_score = [&](long long dot, int j) -> double {
@@ -813,10 +859,6 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
     return (valid == block ? num * inv_block : num / static_cast<double>(valid)) + 0.0;  // block is a power of two
   };
   auto exact_order_key = [&](long long dot, int j) -> unsigned long long { return order_key(exact_score(dot, j)); };
-  auto dot4 = [](const int4& a, const int4& b) -> long long {
-    return static_cast<long long>(a.x) * b.x + static_cast<long long>(a.y) * b.y + static_cast<long long>(a.z) * b.z +
-           static_cast<long long>(a.w) * b.w;
-  };
   auto exact_key = [&](int j) -> unsigned long long {  // of entry j, by one lane
     const int4* const k4 = reinterpret_cast<const int4*>(k_colsum + (bh_rows + j) * kHeadDim);
     long long dot = 0;
@@ -824,6 +866,14 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
     for (int d = 0; d < kHeadDim / 4; ++d) dot += dot4(q4[d], __ldg(k4 + d));
     return exact_order_key(dot, j);
   };
+  if (large > 0 && large <= kLarge) {  // places of the key blocks of large scale, from their exact scores
+    const int j = s_large[min(lane, large - 1)];
+    const int place = place_of(q4, k_colsum + (bh_rows + j) * kHeadDim, k_scales + bh_rows + j, min(block, tokens - j * block), places_per_unit(warp, s_top));
+    row[j] = static_cast<unsigned short>(place);
+    low = min(low, __reduce_min_sync(0xFFFFFFFFu, place));
+    high = max(high, __reduce_max_sync(0xFFFFFFFFu, place));
+    __syncwarp();
+  }
 
   auto half_of = [](const uint4& v, int x) -> int {
     const uint32_t w = x < 2 ? v.x : (x < 4 ? v.y : (x < 6 ? v.z : v.w));
@@ -1131,7 +1181,8 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
     // as a whole, the radix select its share.  Ranges that overlap are treated as one.  With lists of 64 and longer ones left to
     // the radix select, which recomputed the keys in each of its passes, one lane to a key: 16 heads of 687 blocks of Gaussian
     // keys with one token 30 times larger 1095 -> 179 us, of 172 blocks 83 -> 35, 10 times larger (clustered keys) 312 -> 112 and 28 -> 27,
-    // keys and queries within 2 % of one value 248 -> 130 and 25 -> 25; of 2147 blocks clustered keys as they are 1063 -> 770.
+    // keys and queries within 2 % of one value 248 -> 130 and 25 -> 25; of 2147 blocks clustered keys as they are 1063 -> 770
+    // (one large key in a row no longer leads here).
     const int l8 = lane & 7, group = lane >> 3;
     const bool apart = cc.open && cm.open && cm.t_hi < cc.t_lo;
     unsigned short* const picked = reinterpret_cast<unsigned short*>(list_c);  // [kPicked], over both lists
@@ -1140,7 +1191,7 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
       if (!has_c && !has_m) continue;
       const int lo = has_m ? cm.t_lo : cc.t_lo, hi = has_c ? cc.t_hi : cm.t_hi;
       const double per_place = static_cast<double>(kFinest) / static_cast<double>(hi - lo + 2);
-      const double slope = static_cast<double>(places_per_unit(warp)) * 0x1p-19 * per_place;  // (a place is score * unit * 2^-19)
+      const double slope = static_cast<double>(places_per_unit(warp, s_top)) * 0x1p-19 * per_place;  // (a place is score * unit * 2^-19)
       const double offset = static_cast<double>(kPlaceMid - lo + 1) * per_place;
       const __half2 from = as_half2(static_cast<uint32_t>(lo) * 0x10001u), end = as_half2(static_cast<uint32_t>(hi + 1) * 0x10001u);
       clear_hist();

@@ -232,12 +232,12 @@ def test_plan_from_places_equals_plan_from_exact_keys(blocks, block):
 @pytest.mark.parametrize("block", [64, 128])
 @pytest.mark.parametrize("blocks", [200, 257, 520])
 def test_plan_ranges_too_full_for_a_list(blocks, block):
-    """Key blocks of a scale far above the others' and scores that differ by little leave most of a row in a few of the 16-bit
-    places: more undecided entries at a threshold than a list holds, both thresholds among the same ones, ties that the exact
+    """Many key blocks of a scale far above the others' and scores that differ by little leave most of a row in a few of the 16-bit
+    places (up to 32 such key blocks are placed by themselves): more undecided entries at a threshold than a list holds, both thresholds among the same ones, ties that the exact
     keys leave, for critical and marginal blocks at once or one after the other.  The same plan bit for bit as from 64-bit
     keys of every entry."""
     g = np.random.default_rng(blocks)
-    wl = small_workload(f"full{blocks}", heads=5, tokens=(blocks - 1) * block + 3, block=block, src_dtype="f32")
+    wl = small_workload(f"full{blocks}", heads=8, tokens=(blocks - 1) * block + 3, block=block, src_dtype="f32")
     inputs = wk.make_inputs(wl)
     q, k = inputs["q"], inputs["k"]
     k[:, 0, 3 * block + 1] *= 30.0
@@ -246,7 +246,9 @@ def test_plan_ranges_too_full_for_a_list(blocks, block):
     period = 5 * block
     k[:, 3] = k[:, 3, np.arange(wl.tokens) % period]  # every block again and again
     k[:, 3, 3 * block + 1] *= 300.0
-    k[:, 4, 3 * block + 1] *= 8.0
+    for head, large, times in ((4, 32, 50.0), (5, 33, 50.0), (6, 40, 2000.0)):  # as many as have their places made exactly, and more
+        k[:, head, 5 * block:(5 + large) * block:block] *= times
+    k[:, 7, -1] *= 100.0  # the last block, of three tokens
     try:
         for crit, neg in ((0.1, 0.6), (0.0, 0.4), (0.3, 0.7), (0.05, 0.0), (0.3, 0.69), (0.01, 0.98)):
             plans = []
@@ -263,7 +265,7 @@ def test_plan_ranges_too_full_for_a_list(blocks, block):
 @pytest.mark.parametrize("times", [10.0, 30.0])
 def test_plan_time_with_one_large_key(times):
     """One key token that much larger than the others (an attention sink) leaves fewer places to all other blocks.  687 blocks
-    took 4.4 and 15 times as long with it; with exact scores made once per undecided entry it is less than three times."""
+    took 4.4 and 15 times as long with it; placed by itself it leaves the others theirs, and the time is 1.25 times."""
     shape = lt.Shape(1, 16, 687 * 64, 64, 64)
     g = torch.Generator(device="cuda").manual_seed(5)
     q, k = (torch.randn((1, 16, shape.tokens, 64), device="cuda", generator=g) for _ in range(2))
@@ -285,7 +287,7 @@ def test_plan_time_with_one_large_key(times):
 
     plain = shortest()
     k[:, :, 7 * 64 + 3] *= times
-    assert shortest() < 3.0 * plain
+    assert shortest() < 2.0 * plain
 
 
 def test_plan_rows_per_cta_around_one_cta_per_sm():
