@@ -514,6 +514,28 @@ def test_key_norms_are_made_for_more_than_one_step(block, crit, read):
     assert torch.isnan(norms).all() if not read else (norms > 0).all()
 
 
+@pytest.mark.parametrize("block,blocks", [(64, 65), (128, 129)])
+def test_key_norms_are_the_largest_of_each_block(block, blocks):
+    """One large key in every block, in every row of it in turn (the last block has five), so that each warp, lane and row that
+    takes part in the maximum decides it once; queries of very different length inside a warp.  The norms against those of
+    the codes, the output against the oracle."""
+    g = np.random.default_rng(block)
+    wl = small_workload(f"norm{block}", heads=2, tokens=(blocks - 1) * block + 5, block=block, crit=0.1, neg=0.3, src_dtype="f32")
+    inputs = wk.make_inputs(wl)
+    for head in range(2):
+        row = np.arange(blocks) * block + (np.arange(blocks) if head == 0 else block - 1 - np.arange(blocks)) % block
+        row[-1] = (blocks - 1) * block + (4 if head == 0 else 0)
+        inputs["k"][:, head, row] *= 12.0
+    inputs["q"] *= np.exp(1.5 * g.standard_normal((1, 2, wl.tokens, 1)) - 1.5).astype(np.float32)
+    eng, out = full_parity(wl, inputs, query_blocks=pu.sample_blocks(wl, [0, 1], 24))
+    start = lt.lite3r_workspace_layout(eng.shape, wl.crit, wl.neg)[3] + 2 * blocks * block * 64 * 2  # behind the fp16 values
+    norms = eng.workspace[start:start + 2 * blocks * 4].view(torch.float32).view(2, blocks)
+    codes = eng.k8.codes.view(torch.float8_e4m3fn).double().view(2, blocks, block, 64)
+    want = codes.pow(2).sum(-1).amax(-1).sqrt()
+    # 64 squares and their sums in single precision, halved by the root, and the root's own rounding
+    torch.testing.assert_close(norms.double(), want, rtol=34 * 2.0 ** -24, atol=0.0)
+
+
 @pytest.mark.parametrize("block", [64, 128])
 @pytest.mark.parametrize("climb", [7.9, 8.1, 14.8, 15.2, 15.95, 16.1, 40.0])
 def test_attention_with_and_without_a_row_maximum(climb, block):
