@@ -33,7 +33,7 @@
 //
 // Warp roles (256 threads): warp 0 = TMA producer, warp 1 = Q K^T issuer, warp 2 = P V issuer (and the linear product)
 // (all lanes run the loops, one elected lane issues; all waits block on mbarriers in the order in which the events
-// occur), warp 3 idle, warps 4-7 = softmax.  The control warps give registers back (setmaxnreg) so that a softmax
+// occur), warp 3 fetches the tensor maps, warps 4-7 = softmax.  The control warps give registers back (setmaxnreg) so that a softmax
 // thread can hold a whole row of scores next to its probabilities.
 // Every wait is bounded (1 s); on expiry the CTA sets *device_status and all roles leave their loops.
 #include <atomic>
@@ -331,8 +331,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // instructions take their operands from); one elected lane issues.
     const bool leader = elect_one();
     const uint32_t answer = smem_u32(smem + kOffNext);
-    // Key blocks and their scales are fetched 32 steps at a time, lane l holding those of step 32 c + l, and handed
-    // to the issuing lane by a shuffle: no global load sits in the per-step path.
+    // Key blocks are fetched 32 steps at a time, lane l holding those of step 32 c + l, and handed to the issuing lane by a
+    // shuffle; the scalars made from their scales go to the softmax threads through shared memory: no global load sits in the
+    // per-step path.
     int jl[2] = {0, 0};
     // The K cursor runs one step ahead of the V cursor (Q K^T of step t+1 is issued under the exponentials of step t, before
     // P V of step t): the events the two wait for alternate in time in exactly this order, so blocking waits lose nothing.
@@ -686,8 +687,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // |q . k| <= |q| |k| bounds the step's scores, also as computed: the second word allows for the roundings before, and the
       // product and the sum here are rounded to the safe side (references beyond 2^24 are further apart than what 2^15 leaves
       // to the largest fp16 number).
-      // Queries and keys of ordinary size pass it in all but the first steps of a tile (91 % of the steps at 22 key blocks,
-      // 99.9 % at 687), which then go without the maximum, its vote and the wait for both.
+      // Queries and keys of ordinary size pass it in most steps after a tile's first, which has no reference yet (92 % of those at 22
+      // key blocks, six steps to a tile, 99.7 % at 687, 34 steps); they go without the maximum, its vote and the wait for both.
       if (!kLinear || !__all_sync(0xFFFFFFFFu, __fmul_ru(q_norm, __uint_as_float(scal.y)) <= __fadd_rd(m_ref, kHeadroom))) {
         // row maximum of the raw scores (c > 0 commutes with max), eight independent chains; a step without any valid key
         // (second half of a short last block) leaves the reference where it is

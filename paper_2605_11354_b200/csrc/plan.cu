@@ -1406,10 +1406,11 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
   if (late_wait) sm100::wait_for_prior_grid();
 }
 
-constexpr int kMostBlocks = 16383;  // (counts are packed into 14 bits)
-size_t plan_compact_smem_bytes(int nb, int rows) {
+constexpr size_t kSmemLimit = 227 * 1024, kCompactLimit = kSmemLimit - 256;  // (the kernel from places has static shared memory, too)
+constexpr size_t plan_compact_smem_bytes(int nb, int rows) {
   return static_cast<size_t>(rows) * (place_pitch(nb) * 2 + kBuckets * 4 + kPicked * 2 + kHeadDim * 4 + rows * 4);
 }
+static_assert(plan_compact_smem_bytes(1 << 14, 8) > kCompactLimit, "counts are packed into 14 bits");
 
 template <int R>
 lite3r_status launch_compact(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r_shape& s, const Counts& c,
@@ -1457,11 +1458,10 @@ lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r
                           const lite3r_plan& plan, bool beside_prior, cudaStream_t stream) {
   const int late_wait = beside_prior ? 1 : 0;
   const int nb = ceil_div(s.tokens, s.block);
-  constexpr size_t kLimit = 227 * 1024, kCompactLimit = kLimit - 256;  // (that kernel has static shared memory, too)
   switch (g_plan_variant.load(std::memory_order_relaxed)) {  // forced by a test; sizes that do not fit are refused
-    case 1: return plan_smem_bytes(nb, 8) <= kLimit ? launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
-    case 2: return plan_compact_smem_bytes(nb, 8) <= kCompactLimit && nb <= kMostBlocks ? launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
-    case 3: return plan_compact_smem_bytes(nb, 16) <= kCompactLimit && nb <= kMostBlocks ? launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 1: return plan_smem_bytes(nb, 8) <= kSmemLimit ? launch_rows<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 2: return plan_compact_smem_bytes(nb, 8) <= kCompactLimit ? launch_compact<8>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
+    case 3: return plan_compact_smem_bytes(nb, 16) <= kCompactLimit ? launch_compact<16>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
     case 4: return nb <= kLongestRow ? launch_rows<1>(q, k, s, c, plan, nb, late_wait, stream) : LITE3R_ERR_UNSUPPORTED;
     default: break;
   }
@@ -1473,7 +1473,7 @@ lite3r_status launch_plan(const lite3r_fp8& q, const lite3r_fp8& k, const lite3r
   // 2 of 313 53.6 against 58.9).  Else sixteen where they fit (some 6300 blocks; 8 heads of 172 blocks 8.8 against 9.7 us, two of
   // 2147 71 against 102), else eight.
   constexpr int kShortRow = 80;
-  if (nb > kShortRow && nb <= kMostBlocks) {
+  if (nb > kShortRow) {
     int sms = 0;
     const lite3r_status st = sm_count(&sms);
     if (st != LITE3R_OK) return st;
