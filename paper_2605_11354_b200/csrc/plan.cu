@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(R * 32, 32 / R) plan_compact_kernel(const int*
     // 16 heads of 172 blocks, 0.8 at 687; with one token of Gaussian keys 30 times larger 35 -> 18.5 and 180 -> 102 us.
     const unsigned ksum = __reduce_add_sync(0xFFFFFFFFu, lane < R ? s_list[lane] : 0u);
     const float most = __uint_as_float(static_cast<unsigned>(static_cast<float>(ksum) * __fdividef(16384.f, static_cast<float>(nb))) + 0x00800000u);
-    if (k_top > most) {  // (the same for the whole CTA)
+    if (k_top > most && k_top < INFINITY) {  // (the same for the whole CTA; next to an infinite scale the row has no places)
       for (int j = threadIdx.x; j < nb; j += R * 32) {
         if (__ldg(k_scales + bh_rows + j) > most) {
           const int at = atomicAdd(&s_large_count, 1);

@@ -262,6 +262,28 @@ def test_plan_ranges_too_full_for_a_list(blocks, block):
         lt.lite3r_plan_variant(0)
 
 
+@pytest.mark.parametrize("scale", [float("inf"), float("nan"), 3e38, 0.0])
+def test_plan_with_extreme_scales(scale):
+    """A key block whose scale is not finite, next to overflow or zero, for ordinary queries and a block of zeros (zero times
+    infinity among its scores): the same plan bit for bit as from 64-bit keys of every entry."""
+    wl = small_workload("extreme", heads=2, tokens=140 * 64 - 7, crit=0.1, neg=0.6)
+    inputs = wk.make_inputs(wl)
+    inputs["q"][:, 0, 3 * 64:4 * 64] = 0.0
+    eng, _ = pu.run_gpu(inputs, wl)
+    eng.k8.scales[0, 0, 9] = scale
+    plans = []
+    try:
+        for variant in (1, 3, 2):
+            lt.lite3r_plan_variant(variant)
+            eng.plan.cls.fill_(-1)
+            eng.make_plan()
+            plans.append([t.cpu().numpy().copy() for t in (eng.plan.cls, eng.plan.crit_idx, eng.plan.marg_idx)])
+    finally:
+        lt.lite3r_plan_variant(0)
+    for other in plans[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(plans[0], other))
+
+
 @pytest.mark.parametrize("times", [10.0, 30.0])
 def test_plan_time_with_one_large_key(times):
     """One key token that much larger than the others (an attention sink) leaves fewer places to all other blocks.  687 blocks
