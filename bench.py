@@ -34,11 +34,11 @@ FP8_OVER_BF16 = 2.0  # nominal dense ratio (4.5 vs 2.25 PFLOP/s)
 # DRAM bytes (read + write) of one launch, keyed by (workload, kernel), from the ncu captures summarised under
 # profiles/; a kernel that changed since its capture has no entry.
 DRAM_BYTES_PER_LAUNCH = {
-    ("vggt8", "attention"): 82429952,
-    ("vggt8", "plan"): 1504768,
-    ("vggt8", "quantize_qkv"): 72324096,
-    ("vggt8", "summary"): 23750912,
-    ("vggt8", "aggregation"): 23407616,
+    ("vggt8", "attention"): 82962176,
+    ("vggt8", "plan"): 1495552,
+    ("vggt8", "quantize_qkv"): 72603904,
+    ("vggt8", "summary"): 23819264,
+    ("vggt8", "aggregation"): 23404544,
 }
 
 
